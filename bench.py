@@ -522,7 +522,7 @@ def run_ours(args):
     peak, peak_kind = measured_peaks()
     stage_ms = {k: v[0] for k, v in stages.items()}
     dom = max(("resample", "fwd_x", "fwd_y", "zmac", "inv_y", "inv_x"), key=lambda k: stage_ms[k])
-    classes = f.length_classes()
+    classes = f.transform_classes()
     launches_of = [(cp, min(f.batch, cnt - b * f.batch)) for cp, cnt in classes
                    for b in range(-(-cnt // f.batch))]
     nbatches = len(launches_of)
@@ -701,7 +701,7 @@ def run_large(args):
         "higher_is_better": True, "dtype": "f32", "precision": args.precision, "data": "synthetic",
         "config": {"workload": f"256^3 pair, {R} rotations, {args.precision.upper()}",
                    "padding": PADDING[args.pad_mode],
-                   "fft_classes": [{"fft": list(cp), "rotations": n} for cp, n in f.length_classes()],
+                   "fft_classes": [{"fft": list(cp), "rotations": n} for cp, n in f.transform_classes()],
                    "batch": f.batch,
                    "device_bytes": f.fixed_bytes + f.workspace_bytes},
         "seconds": dt,
@@ -879,7 +879,7 @@ def main():
     ap.add_argument("--batch", type=int, default=0)
     ap.add_argument("--precision", choices=("fp32", "bf16", "fp16"), default="fp32")
     ap.add_argument("--pad-mode", choices=("bound", "full"), default="bound")
-    ap.add_argument("--autotune", choices=("on", "off"), default="on",
+    ap.add_argument("--autotune", choices=("on", "off"), default="off",
                     help="time both radix splits of each FFT pass on the first launch group "
                          "at new lengths (warm-up) and keep the faster")
     ap.add_argument("--tensor-cores", choices=("on", "off"), default="on",

@@ -115,8 +115,15 @@ typedef enum {
  * correlation lives, so its slot holds exactly its own value; shifts outside
  * the range are invalid and reported as such, as with FULL.  Scores agree
  * with FULL up to FP32 rounding.  The call synchronises its stream once to
- * read the ranges, and once more for each further set of lengths, whose
- * fixed spectra it recomputes (about the cost of one rotation each). */
+ * read the ranges; each further set of lengths costs the recomputation of the
+ * fixed spectra (about one rotation).
+ * These are the lengths cs_ngf_info.pad and cs_ngf_length_sets report.  In the
+ * FP32 form without autotuning the transforms themselves are shorter where the
+ * masks leave slabs empty: both volumes are cut to their masks' boxes (the
+ * masked channels vanish outside), with slabs [a0, a1] of M_A and [b0, b1] of
+ * the rotated mask the correlation lives on [b0 - a1, b1 - a0], and
+ * P >= max(b1 - a0 - lo, hi - b0 + a1) + 1 keeps the admitted shifts
+ * alias-free (cs_ngf_transform_sets reports those lengths). */
 typedef enum {
   CS_NGF_PAD_FULL = 0,  /* P >= 2n - 1 on every call */
   CS_NGF_PAD_BOUND = 1  /* per call, the shortest length the shift bound allows (default) */
@@ -164,7 +171,7 @@ typedef struct {
 
 typedef struct {
   int32_t dims[3];              /* nz, ny, nx */
-  int32_t pad[3];               /* FFT lengths in use (those of the last call) */
+  int32_t pad[3];               /* FFT lengths (those the last call's shift ranges give) */
   int32_t batch;                /* rotations per launch group */
   int64_t sum_mask_a;           /* sum of M_A */
   int64_t fixed_bytes;          /* device bytes of the fixed spectra */
@@ -299,7 +306,7 @@ int64_t cs_ngf_launch_count(void);
  * wrong results: serialise them.
  * Errors: EINVAL, ECUDA (detail in cs_ngf_last_error()). */
 #define CS_NGF_NOALLOC_MAX_DIM 32
-#define CS_NGF_NOALLOC_SCRATCH_BYTES 14583552
+#define CS_NGF_NOALLOC_SCRATCH_BYTES 14582016
 cs_ngf_status cs_ngf_score_rotations_noalloc(const float* A, const uint8_t* maskA, const float* B,
                                              const uint8_t* maskB, const int32_t dims[3],
                                              float eps, float gamma, const double* quats,
@@ -433,6 +440,11 @@ cs_ngf_status cs_ngf_get_info(const cs_ngf_fixed* f, cs_ngf_info* info);
  * and counts [cap] (rotations scored with those lengths; either may be NULL)
  * and returns the number of sets (0 for a NULL handle or before any call). */
 int32_t cs_ngf_length_sets(const cs_ngf_fixed* f, int32_t cap, int32_t* pads, int32_t* counts);
+
+/* The FFT lengths the last scoring call's transforms ran at, in the same form:
+ * those of cs_ngf_length_sets, or shorter ones where the masks' boxes allow
+ * (cs_ngf_pad_mode). */
+int32_t cs_ngf_transform_sets(const cs_ngf_fixed* f, int32_t cap, int32_t* pads, int32_t* counts);
 
 /* Autotuning choices of this process (cs_ngf_config.autotune), one entry per
  * FFT pass, length, input kind and storage form timed so far. */

@@ -32,7 +32,7 @@ EXPORTED = (
     "cs_ngf_server_default_config", "cs_ngf_server_create", "cs_ngf_server_submit",
     "cs_ngf_server_cancel", "cs_ngf_server_wait", "cs_ngf_server_stats", "cs_ngf_server_destroy",
     "cs_ngf_search_default_config", "cs_ngf_global_align", "cs_ngf_length_sets",
-    "cs_ngf_tuning", "cs_ngf_tuning_reset", "cs_ngf_plan_lengths",
+    "cs_ngf_tuning", "cs_ngf_tuning_reset", "cs_ngf_plan_lengths", "cs_ngf_transform_sets",
 )
 
 MAX_LEVELS = 8
@@ -126,6 +126,8 @@ _lib.cs_ngf_tuning_reset.argtypes = []
 _lib.cs_ngf_tuning_reset.restype = None
 _lib.cs_ngf_length_sets.argtypes = [ctypes.c_void_p, _i32, ctypes.c_void_p, ctypes.c_void_p]
 _lib.cs_ngf_length_sets.restype = _i32
+_lib.cs_ngf_transform_sets.argtypes = [_vp, _i32, ctypes.c_void_p, ctypes.c_void_p]
+_lib.cs_ngf_transform_sets.restype = _i32
 _lib.cs_ngf_auto_pad.argtypes = [_i32]
 _lib.cs_ngf_auto_pad.restype = _i32
 _lib.cs_ngf_update_fixed.argtypes = [_vp, _vp, _vp, _vp]
@@ -328,16 +330,24 @@ class Fixed:
 
     @property
     def pad(self):
-        """FFT lengths (z, y, x) in use: those of the last call (bound-limited
-        padding may shorten them below max_pad)."""
+        """FFT lengths (z, y, x) the last call's shift ranges give (bound-limited
+        padding may shorten them below max_pad; see transform_classes)."""
         return tuple(self._info().pad)
 
     def length_classes(self):
-        """[((Pz, Py, Px), rotations)] of the last scoring call, in the order scored."""
-        n = int(_lib.cs_ngf_length_sets(self._h, 0, None, None))
+        """[((Pz, Py, Px), rotations)] the overlap rule gave in the last scoring call."""
+        return self._sets(_lib.cs_ngf_length_sets)
+
+    def transform_classes(self):
+        """[((Pz, Py, Px), rotations)] the last scoring call's transforms ran at, in
+        the order scored: length_classes(), or shorter where the masks' boxes allow."""
+        return self._sets(_lib.cs_ngf_transform_sets)
+
+    def _sets(self, call):
+        n = int(call(self._h, 0, None, None))
         pads = (ctypes.c_int32 * (3 * max(n, 1)))()
         counts = (ctypes.c_int32 * max(n, 1))()
-        _lib.cs_ngf_length_sets(self._h, n, pads, counts)
+        call(self._h, n, pads, counts)
         return [((pads[3 * c], pads[3 * c + 1], pads[3 * c + 2]), int(counts[c])) for c in range(n)]
 
     @property

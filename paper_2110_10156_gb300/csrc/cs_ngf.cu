@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -34,6 +35,8 @@ cs_ngf_status fail(cs_ngf_status s, const std::string& msg) {
 }  // namespace detail
 }  // namespace csngf
 
+using csngf::detail::ClassGeom;
+using csngf::detail::Plan;
 using csngf::detail::fail;
 
 namespace {
@@ -122,7 +125,7 @@ struct Stage {
     if (f->profiling && cudaEventCreate(&a) == cudaSuccess) cudaEventRecord(a, st);
   }
   ~Stage() {
-    if (!f->capturing) g_launches.fetch_add(1, std::memory_order_relaxed);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
     if (a) {
       cudaEvent_t b = nullptr;
       if (cudaEventCreate(&b) == cudaSuccess) {
@@ -189,28 +192,19 @@ void free_handle(cs_ngf_fixed* f) {
   cudaFree(f->margA);
   cudaFree(f->margB);
   cudaFree(f->bounds);
-  cudaFree(f->thr);
   cudaFree(f->keys);
   cudaFree(f->tc_err);
   cudaFree(f->zx);
-  for (int a = 0; a < 3; ++a) {
-    bool dup = false;
-    for (int b = 0; b < a; ++b) dup |= (f->tw[b] == f->tw[a]);
-    if (!dup) cudaFree(f->tw[a]);
-  }
   if (f->rot_ev) cudaEventSynchronize(f->rot_ev);
   if (f->order_ev) cudaEventDestroy(f->order_ev);
   for (auto& sp : f->spans) { cudaEventDestroy(sp.a); cudaEventDestroy(sp.b); }
-  if (f->gexec) cudaGraphExecDestroy(f->gexec);
-  for (auto& gs : f->graphs) cudaGraphExecDestroy(gs.exec);
+  cudaFree(f->boxA);
+  cudaFree(f->allm);
   cudaFree(f->allb);
   cudaFreeHost(f->allb_h);
   cudaFree(f->perm_d);
   cudaFree(f->perm_score);
   cudaFree(f->perm_shift);
-  cudaFree(f->rot_slot);
-  cudaFree(f->slot_score);
-  cudaFree(f->slot_shift);
   cudaFreeHost(f->rot_h);
   cudaFree(f->rot_d);
   if (f->rot_ev) cudaEventDestroy(f->rot_ev);
@@ -223,19 +217,7 @@ void free_handle(cs_ngf_fixed* f) {
   delete f;
 }
 
-// twiddle table exp(-2 pi i m / P), m < P, into dst (at least P entries);
-// synchronous, so no kernel may still read dst
-cs_ngf_status fill_twiddles(int P, float2* dst) {
-  std::vector<float2> h(P);
-  for (int m = 0; m < P; ++m) {
-    h[m].x = (float)ctw::cos2pi(m, P);
-    h[m].y = (float)(-ctw::sin2pi(m, P));
-  }
-  CS_CUDA(cudaMemcpy(dst, h.data(), sizeof(float2) * P, cudaMemcpyHostToDevice));
-  return CS_NGF_OK;
-}
-
-// upload R rotation matrices (host FP64 quaternions) to f->rot_d
+// upload R rotation matrices (host FP64 quaternions) to f->rot_d, boxes empty
 cs_ngf_status upload_rotations(cs_ngf_fixed* f, const double* quats, int R, cudaStream_t st) {
   if (!quats) return fail(CS_NGF_EINVAL, "quats is NULL");
   for (int r = 0; r < R; ++r) {
@@ -254,7 +236,7 @@ cs_ngf_status upload_rotations(cs_ngf_fixed* f, const double* quats, int R, cuda
     f->rot_d = nullptr;
     f->rot_cap = 0;
     const int cap = std::max(R, 64);
-    CS_CUDA(cudaMallocHost((void**)&f->rot_h, sizeof(RotMat) * cap));
+    CS_CUDA(cudaMallocHost((void**)&f->rot_h, sizeof(RotIn) * cap));
     CS_CUDA(dalloc(&f->rot_d, (size_t)cap));
     f->rot_cap = cap;
   }
@@ -262,9 +244,10 @@ cs_ngf_status upload_rotations(cs_ngf_fixed* f, const double* quats, int R, cuda
   for (int r = 0; r < R; ++r) {
     double Rm[9];
     quat_to_rotmat(quats + 4 * r, Rm);
-    for (int i = 0; i < 9; ++i) f->rot_h[r].m[i] = (float)Rm[i];
+    f->rot_h[r] = RotIn{};
+    for (int i = 0; i < 9; ++i) f->rot_h[r].m.m[i] = (float)Rm[i];
   }
-  CS_CUDA(cudaMemcpyAsync(f->rot_d, f->rot_h, sizeof(RotMat) * R, cudaMemcpyHostToDevice, st));
+  CS_CUDA(cudaMemcpyAsync(f->rot_d, f->rot_h, sizeof(RotIn) * R, cudaMemcpyHostToDevice, st));
   CS_CUDA(cudaEventRecord(f->rot_ev, st));
   return CS_NGF_OK;
 }
@@ -345,15 +328,15 @@ bool needs_tuning(const cs_ngf_fixed* f) {
   return false;
 }
 
-// launch FFT pass k of nb volumes with split variant v
-void launch_pass(cs_ngf_fixed* f, int k, int v, int nb, float* map, cudaStream_t st) {
+// launch FFT pass k of the nb rotations at rot with split variant v
+void launch_pass(cs_ngf_fixed* f, int k, int v, const RotIn* rot, int nb, float* map, cudaStream_t st) {
   const Geo& g = f->g;
   switch (k) {
-    case 0: CS_DISPATCH(g.Px, launch_fwd_x<PP>(f->Bh, f->Mh, f->F02, f->tw[2], g, nb, st, v)); break;
-    case 1: CS_DISPATCH(g.Py, launch_fwd_y<PP>(f->F02, f->F13, f->tw[1], g, nb, st, v)); break;
-    case 2: CS_DISPATCH(g.Pz, launch_zmac<PP>(f->F13, f->UV, f->F02, f->tw[0], g, nb, f->bounds, st, v)); break;
-    case 3: CS_DISPATCH(g.Py, launch_inv_y<PP>(f->F02, f->F13, f->tw[1], g, nb, f->bounds, st, v)); break;
-    default: CS_DISPATCH(g.Px, launch_inv_x<PP>(f->F13, f->thr, f->keys, map, f->tw[2], g, nb, f->bounds, st, v)); break;
+    case 0: CS_DISPATCH(g.Px, launch_fwd_x<PP>(f->Bh, f->Mh, f->F02, rot, g, nb, st, v)); break;
+    case 1: CS_DISPATCH(g.Py, launch_fwd_y<PP>(f->F02, f->F13, g, nb, st, v)); break;
+    case 2: CS_DISPATCH(g.Pz, launch_zmac<PP>(f->F13, f->UV, f->F02, g, nb, rot, st, v)); break;
+    case 3: CS_DISPATCH(g.Py, launch_inv_y<PP>(f->F02, f->F13, g, nb, rot, st, v)); break;
+    default: CS_DISPATCH(g.Px, launch_inv_x<PP>(f->F13, f->keys, map, g, nb, rot, st, v)); break;
   }
 }
 
@@ -364,7 +347,7 @@ const char* const kPassName[kPasses] = {"fwd_x", "fwd_y", "zmac", "inv_y", "inv_
 // its output is what the next pass reads.  A pass is repeatable: it reads
 // buffers it does not write, except the x inverse's per-rotation maxima,
 // which are cleared before the final run.
-cs_ngf_status tune_pass(cs_ngf_fixed* f, int k, int nb, cudaStream_t st) {
+cs_ngf_status tune_pass(cs_ngf_fixed* f, int k, const RotIn* rot, int nb, cudaStream_t st) {
   const TuneKey key = tune_key(f, k);
   float best[2] = {0.0f, 0.0f};
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -374,7 +357,7 @@ cs_ngf_status tune_pass(cs_ngf_fixed* f, int k, int nb, cudaStream_t st) {
   for (int v = 0; v < 2 && !s; ++v)
     for (int rep = 0; rep < 2 && !s; ++rep) {
       cudaEventRecord(e0, st);
-      { Stage sp(f, 1 + k, st); launch_pass(f, k, v, nb, nullptr, st); }
+      { Stage sp(f, 1 + k, st); launch_pass(f, k, v, rot, nb, nullptr, st); }
       cudaEventRecord(e1, st);
       if ((s = check_launch(kPassName[k]))) break;
       float ms = 0.0f;
@@ -392,13 +375,14 @@ cs_ngf_status tune_pass(cs_ngf_fixed* f, int k, int nb, cudaStream_t st) {
   }
   f->vars[k] = choice;
   if (k == 4) CS_CUDA(cudaMemsetAsync(f->keys, 0, sizeof(unsigned long long) * nb, st));
-  { Stage sp(f, 1 + k, st); launch_pass(f, k, choice, nb, nullptr, st); }
+  { Stage sp(f, 1 + k, st); launch_pass(f, k, choice, rot, nb, nullptr, st); }
   return check_launch(kPassName[k]);
 }
 
 // the FFT passes for nb volumes already resampled into f->Bh / f->Mh; with
 // tune, passes whose two splits have no choice yet are timed first
-cs_ngf_status run_transforms(cs_ngf_fixed* f, int nb, float* map, cudaStream_t st, bool tune = false) {
+cs_ngf_status run_transforms(cs_ngf_fixed* f, const RotIn* rot, int nb, float* map, cudaStream_t st,
+                             bool tune = false) {
   for (int k = 0; k < kPasses; ++k) {
     if (tune && !map) {
       const TuneKey key = tune_key(f, k);
@@ -408,11 +392,11 @@ cs_ngf_status run_transforms(cs_ngf_fixed* f, int nb, float* map, cudaStream_t s
         untuned = g_tune.find(key) == g_tune.end();
       }
       if (untuned) {
-        if (cs_ngf_status s = tune_pass(f, k, nb, st)) return s;
+        if (cs_ngf_status s = tune_pass(f, k, rot, nb, st)) return s;
         continue;
       }
     }
-    { Stage sp(f, 1 + k, st); launch_pass(f, k, f->vars[k], nb, map, st); }
+    { Stage sp(f, 1 + k, st); launch_pass(f, k, f->vars[k], rot, nb, map, st); }
     if (cs_ngf_status s = check_launch(kPassName[k])) return s;
   }
   return CS_NGF_OK;
@@ -424,150 +408,112 @@ cs_ngf_status pack_floating(cs_ngf_fixed* f, const float* B, const uint8_t* MB, 
   return check_launch("pack");
 }
 
-// score nb rotations whose matrices are at rot (device), with the floating
-// volume already packed in f->BQ, f->C8; results to out_score[nb], out_shift[nb][3]
-cs_ngf_status score_batch_ptrs(cs_ngf_fixed* f, const RotMat* rot, int nb, float* out_score,
-                               int32_t* out_shift, float* map, cudaStream_t st, bool tune = false) {
+// score rotations [r0, r0 + nb) of the uploaded set, with the floating volume
+// already packed in f->BQ, f->C8.  With bound-limited padding plan_classes has
+// counted the masks and uploaded the boxes; with full padding they are counted
+// here, and the boxes are the whole volume.
+cs_ngf_status score_batch(cs_ngf_fixed* f, int r0, int nb, float* best_score, int32_t* best_shift,
+                          float* map, cudaStream_t st, bool tune = false) {
   const Geo& g = f->g;
-  const size_t nmarg = (size_t)g.nz + g.ny + g.nx;
-  CS_CUDA(cudaMemsetAsync(f->msum, 0, sizeof(int) * nb, st));
+  RotIn* rot = f->rot_d + r0;
   CS_CUDA(cudaMemsetAsync(f->keys, 0, sizeof(unsigned long long) * nb, st));
-  CS_CUDA(cudaMemsetAsync(f->margB, 0, sizeof(int) * nmarg * nb, st));
-  {
-    Stage sp(f, 0, st);
-    k_resample<<<resample_grid(g, nb), 128, 0, st>>>(f->BQ, f->C8, rot, g, f->Bh, f->Mh, f->msum, f->margB);
+  if (f->pad_mode == CS_NGF_PAD_BOUND) {
+    {
+      Stage sp(f, 0, st);
+      k_resample_box<<<resample_box_grid(g, nb), 128, 0, st>>>(f->BQ, f->C8, rot, g, f->Bh, f->Mh);
+    }
+    if (cs_ngf_status s = check_launch("resample")) return s;
+  } else {
+    const size_t nmarg = (size_t)g.nz + g.ny + g.nx;
+    CS_CUDA(cudaMemsetAsync(f->msum, 0, sizeof(int) * nb, st));
+    CS_CUDA(cudaMemsetAsync(f->margB, 0, sizeof(int) * nmarg * nb, st));
+    {
+      Stage sp(f, 0, st);
+      k_resample<<<resample_grid(g, nb), 128, 0, st>>>(f->BQ, f->C8, rot, g, f->Bh, f->Mh, f->msum, f->margB);
+    }
+    if (cs_ngf_status s = check_launch("resample")) return s;
+    {
+      Stage sp(f, 7, st);
+      k_shift_bounds<<<dim3((unsigned)nb, 3u), 512, 0, st>>>(f->margA, f->margB, f->msum, f->sumA,
+                                                             f->gamma, g, f->bounds);
+    }
+    if (cs_ngf_status s = check_launch("shift bounds")) return s;
+    const double pvol = (double)g.Px * (double)g.Py * (double)g.Pz;
+    {
+      Stage sp(f, 7, st);
+      k_full_boxes<<<(nb + 127) / 128, 128, 0, st>>>(f->bounds, f->sumA, f->gamma, g, pvol, nb, rot);
+    }
+    if (cs_ngf_status s = check_launch("boxes")) return s;
   }
-  if (cs_ngf_status s = check_launch("resample")) return s;
-  const double pvol = (double)g.Px * (double)g.Py * (double)g.Pz;
-  {
-    Stage sp(f, 7, st);
-    k_thresholds<<<(nb + 127) / 128, 128, 0, st>>>(f->msum, f->sumA, f->gamma, pvol, nb, f->thr);
-  }
-  if (cs_ngf_status s = check_launch("thresholds")) return s;
-  {
-    Stage sp(f, 7, st);
-    k_shift_bounds<<<dim3((unsigned)nb, 3u), 512, 0, st>>>(f->margA, f->margB, f->msum, f->sumA,
-                                                           f->gamma, g, f->bounds);
-  }
-  if (cs_ngf_status s = check_launch("shift bounds")) return s;
   if (map) {
     Stage sp(f, 7, st);
     k_fill<<<256, 256, 0, st>>>(map, (long long)g.vz * g.vy * g.vx, -INFINITY);
   }
-  if (cs_ngf_status s = run_transforms(f, nb, map, st, tune)) return s;
+  if (cs_ngf_status s = run_transforms(f, rot, nb, map, st, tune)) return s;
   {
     Stage sp(f, 7, st);
-    k_finalize<<<(nb + 127) / 128, 128, 0, st>>>(f->keys, nb, g, out_score, out_shift);
+    k_finalize<<<(nb + 127) / 128, 128, 0, st>>>(f->keys, nb, g, best_score + r0, best_shift + 3 * (size_t)r0);
   }
   return check_launch("finalize");
 }
 
-constexpr int kKernelsPerBatch = 9;   // resample, thresholds, bounds, 5 passes, finalize
-
-cs_ngf_status score_batch(cs_ngf_fixed* f, int r0, int nb, float* best_score, int32_t* best_shift,
-                          float* map, cudaStream_t st, bool tune = false) {
-  return score_batch_ptrs(f, f->rot_d + r0, nb, best_score + r0, best_shift + 3 * (size_t)r0, map, st,
-                          tune);
-}
-
-// capture the full-batch launch sequence once (on a private stream; the
-// graph is then replayed on the caller's stream)
-cs_ngf_status ensure_graph(cs_ngf_fixed* f) {
-  if (f->gexec && !std::equal(f->vars, f->vars + kPasses, f->gexec_vars)) {   // captured with other splits
-    cudaGraphExecDestroy(f->gexec);
-    f->gexec = nullptr;
-  }
-  if (f->gexec) return CS_NGF_OK;
-  std::copy(f->vars, f->vars + kPasses, f->gexec_vars);
-  if (!f->rot_slot) {
-    CS_CUDA(dalloc(&f->rot_slot, (size_t)f->batch));
-    CS_CUDA(dalloc(&f->slot_score, (size_t)f->batch));
-    CS_CUDA(dalloc(&f->slot_shift, (size_t)f->batch * 3));
-  }
-  cudaStream_t cs = nullptr;
-  CS_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-  cudaGraph_t graph = nullptr;
-  cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-  cs_ngf_status st = CS_NGF_OK;
-  if (e == cudaSuccess) {
-    f->capturing = true;
-    st = score_batch_ptrs(f, f->rot_slot, f->batch, f->slot_score, f->slot_shift, nullptr, cs);
-    f->capturing = false;
-    e = cudaStreamEndCapture(cs, &graph);
-  }
-  if (e == cudaSuccess && st == CS_NGF_OK) e = cudaGraphInstantiate(&f->gexec, graph, 0);
-  if (graph) cudaGraphDestroy(graph);
-  cudaStreamDestroy(cs);
-  if (st != CS_NGF_OK) return st;
-  if (e != cudaSuccess) {
-    f->gexec = nullptr;
-    return fail(CS_NGF_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-  }
-  return CS_NGF_OK;
-}
-
-// Section 3.1 A side: NGF channels of A times M_A, forward FFTs, weights -> f->UV
-cs_ngf_status run_fixed(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cudaStream_t st) {
+// Section 3.1 A side at the lengths in use: NGF channels of A times M_A over
+// its mask's box, forward FFTs, weights -> f->UV
+cs_ngf_status run_spectra(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cudaStream_t st) {
   Geo g = f->g;
   g.store = kStoreF32;            // the fixed spectra are always computed in FP32
   for (int j = 0; j < 4; ++j) g.scale0[j] = g.scale1[j] = 1.0f;
-  { Stage sp(f, 6, st); k_copy_in<<<1024, 256, 0, st>>>(A, MA, g.nvox, f->Bh, f->Mh); }
-  if (cs_ngf_status s = check_launch("copy_in")) return s;
-  CS_CUDA(cudaMemsetAsync(f->msum, 0, sizeof(int), st));
-  { Stage sp(f, 6, st); k_mask_sum<<<1024, 256, 0, st>>>(f->Mh, g.nvox, f->msum); }
-  if (cs_ngf_status s = check_launch("mask_sum")) return s;
-  CS_CUDA(cudaMemsetAsync(f->margA, 0, sizeof(int) * ((size_t)g.nz + g.ny + g.nx), st));
-  { Stage sp(f, 6, st); k_marginals<<<1024, 256, 0, st>>>(f->Mh, g, f->margA); }
-  if (cs_ngf_status s = check_launch("marginals")) return s;
-  { Stage sp(f, 6, st); CS_DISPATCH(g.Px, launch_fwd_x<PP>(f->Bh, f->Mh, f->F02, f->tw[2], g, 1, st)); }
+  g.ez = f->extA[0]; g.ey = f->extA[1]; g.ex = f->extA[2];
+  f->spectra_ok = g.ez <= g.Pz && g.ey <= g.Py && g.ex <= g.Px;
+  if (!f->spectra_ok) return CS_NGF_OK;   // lengths of another volume: the next call sets its own
+  { Stage sp(f, 6, st); CS_DISPATCH(g.Px, launch_fwd_x<PP>(A, MA, f->F02, f->boxA, g, 1, st)); }
   if (cs_ngf_status s = check_launch("fwd_x (fixed)")) return s;
-  { Stage sp(f, 6, st); CS_DISPATCH(g.Py, launch_fwd_y<PP>(f->F02, f->F13, f->tw[1], g, 1, st)); }
+  { Stage sp(f, 6, st); CS_DISPATCH(g.Py, launch_fwd_y<PP>(f->F02, f->F13, g, 1, st)); }
   if (cs_ngf_status s = check_launch("fwd_y (fixed)")) return s;
-  { Stage sp(f, 6, st); CS_DISPATCH(g.Pz, launch_prep_z<PP>(f->F13, f->UV, f->tw[0], g, st)); }
-  if (cs_ngf_status s = check_launch("prep_z")) return s;
-  int sumA = 0;
-  CS_CUDA(cudaMemcpyAsync(&sumA, f->msum, sizeof(int), cudaMemcpyDeviceToHost, st));
-  CS_CUDA(cudaStreamSynchronize(st));
-  if (sumA != f->sumA) {                 // the captured threshold launch holds sum(M_A)
-    if (f->gexec) cudaGraphExecDestroy(f->gexec);
-    f->gexec = nullptr;
-    for (auto& gs : f->graphs) cudaGraphExecDestroy(gs.exec);
-    f->graphs.clear();
-  }
-  f->sumA = sumA;
-  return CS_NGF_OK;
+  { Stage sp(f, 6, st); CS_DISPATCH(g.Pz, launch_prep_z<PP>(f->F13, f->UV, g, st)); }
+  return check_launch("prep_z");
 }
 
-// switch the handle to FFT lengths pad (each <= alloc_pad): twiddles, fixed
-// spectra at the new lengths, and a new graph on the next full launch group
-cs_ngf_status set_pads(cs_ngf_fixed* f, const int pad[3], cudaStream_t st) {
-  Geo& g = f->g;
-  const int cur[3] = {g.Pz, g.Py, g.Px};
-  if (cur[0] == pad[0] && cur[1] == pad[1] && cur[2] == pad[2]) return CS_NGF_OK;
-  CS_CUDA(cudaStreamSynchronize(st));            // nothing may still read the old tables
-  for (int a = 0; a < 3; ++a)
-    if (cur[a] != pad[a])
-      if (cs_ngf_status s = fill_twiddles(pad[a], f->tw[a])) return s;
-  // the captured launches hold the lengths: keep this graph for a later
-  // return to them, and take the one of the new lengths if there is one
-  if (f->gexec) {
-    cs_ngf_fixed::GraphSlot gs{{g.Pz, g.Py, g.Px}, {0, 0, 0, 0, 0}, f->gexec};
-    std::copy(f->gexec_vars, f->gexec_vars + kPasses, gs.vars);
-    f->graphs.push_back(gs);
+// a new fixed volume: slab counts of its mask, its box, and the spectra at the
+// lengths in use; synchronises st
+cs_ngf_status load_fixed(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cudaStream_t st) {
+  const Geo& g = f->g;
+  const int n[3] = {g.nz, g.ny, g.nx};
+  std::vector<int> marg((size_t)g.nz + g.ny + g.nx);
+  CS_CUDA(cudaMemsetAsync(f->margA, 0, sizeof(int) * marg.size(), st));
+  { Stage sp(f, 6, st); k_marginals<<<(unsigned)g.nz, 256, 0, st>>>(MA, g, f->margA); }
+  if (cs_ngf_status s = check_launch("marginals")) return s;
+  CS_CUDA(cudaMemcpyAsync(marg.data(), f->margA, sizeof(int) * marg.size(), cudaMemcpyDeviceToHost, st));
+  CS_CUDA(cudaStreamSynchronize(st));
+  f->sumA = 0;
+  for (int z = 0; z < g.nz; ++z) f->sumA += marg[z];
+  RotIn box{};
+  const int* m = marg.data();
+  for (int a = 0; a < 3; m += n[a], ++a) {
+    int lo = 0, hi = n[a] - 1;
+    while (lo < hi && !m[lo]) ++lo;
+    while (hi > lo && !m[hi]) --hi;
+    f->a0[a] = lo;
+    f->a1[a] = hi;
+    box.b.org[a] = f->boxed ? lo : 0;
+    f->extA[a] = f->pad_mode == CS_NGF_PAD_BOUND ? hi + 1 - box.b.org[a] : n[a];
   }
-  f->gexec = nullptr;
-  for (size_t i = 0; i < f->graphs.size(); ++i)
-    if (std::equal(pad, pad + 3, f->graphs[i].pad)) {
-      f->gexec = f->graphs[i].exec;
-      std::copy(f->graphs[i].vars, f->graphs[i].vars + kPasses, f->gexec_vars);
-      f->graphs.erase(f->graphs.begin() + (long)i);
-      break;
-    }
-  g.Pz = pad[0];
-  g.Py = pad[1];
-  g.Px = pad[2];
+  CS_CUDA(cudaMemcpyAsync(f->boxA, &box, sizeof(RotIn), cudaMemcpyHostToDevice, st));
+  return run_spectra(f, A, MA, st);
+}
+
+// switch the handle to a class's FFT lengths (each <= alloc_pad), box extents
+// and shift windows, with the fixed spectra at the new lengths
+cs_ngf_status set_class_impl(cs_ngf_fixed* f, const ClassGeom& c, cudaStream_t st) {
+  Geo& g = f->g;
+  g.ez = c.ext[0]; g.ey = c.ext[1]; g.ex = c.ext[2];
+  g.wz = c.win[0]; g.wy = c.win[1];
+  if (f->spectra_ok && g.Pz == c.pad[0] && g.Py == c.pad[1] && g.Px == c.pad[2]) return CS_NGF_OK;
+  g.Pz = c.pad[0];
+  g.Py = c.pad[1];
+  g.Px = c.pad[2];
   resolve_variants(f);
-  return run_fixed(f, f->A_keep, f->MA_keep, st);
+  return run_spectra(f, f->A_keep, f->MA_keep, st);
 }
 
 // FP16 form: per channel field, the power of two that keeps the field's
@@ -597,18 +543,21 @@ int length_for(int need, int cap) {
 cs_ngf_status ensure_rotation_buffers(cs_ngf_fixed* f, int R) {
   if (R <= f->allb_cap) return CS_NGF_OK;
   CS_CUDA(cudaDeviceSynchronize());              // the old buffers may still be read
+  cudaFree(f->allm);
   cudaFree(f->allb);
   cudaFreeHost(f->allb_h);
   cudaFree(f->perm_d);
   cudaFree(f->perm_score);
   cudaFree(f->perm_shift);
-  f->allb = f->perm_d = f->allb_h = nullptr;
+  f->allm = f->perm_d = nullptr;
+  f->allb = f->allb_h = nullptr;
   f->perm_score = nullptr;
   f->perm_shift = nullptr;
   f->allb_cap = 0;
   const int cap = std::max(R, 64);
-  CS_CUDA(dalloc(&f->allb, (size_t)cap * 6));
-  CS_CUDA(cudaMallocHost((void**)&f->allb_h, sizeof(int) * 6 * (size_t)cap));
+  CS_CUDA(dalloc(&f->allm, (size_t)cap * (1 + (size_t)f->g.nz + f->g.ny + f->g.nx)));
+  CS_CUDA(dalloc(&f->allb, (size_t)cap));
+  CS_CUDA(cudaMallocHost((void**)&f->allb_h, sizeof(RotBounds) * (size_t)cap));
   CS_CUDA(dalloc(&f->perm_d, (size_t)cap));
   CS_CUDA(dalloc(&f->perm_score, (size_t)cap));
   CS_CUDA(dalloc(&f->perm_shift, (size_t)cap * 3));
@@ -616,43 +565,62 @@ cs_ngf_status ensure_rotation_buffers(cs_ngf_fixed* f, int R) {
   return CS_NGF_OK;
 }
 
-// Section 3.2 shift bounds of each of the R uploaded rotations (the same
-// counts and bound the launch groups compute, from the floating volume
-// pack_floating prepared) into f->allb_h [R][6]; synchronises st
+// Section 3.2 shift bounds and mask slabs of each of the R uploaded rotations
+// (from the floating volume pack_floating prepared) into f->allb_h [R];
+// synchronises st
 cs_ngf_status rotation_bounds(cs_ngf_fixed* f, int R, cudaStream_t st) {
   if (cs_ngf_status s = ensure_rotation_buffers(f, R)) return s;
   const Geo& g = f->g;
   const size_t nmarg = (size_t)g.nz + g.ny + g.nx;
-  for (int r0 = 0; r0 < R; r0 += f->batch) {
-    const int nb = std::min(f->batch, R - r0);
-    CS_CUDA(cudaMemsetAsync(f->msum, 0, sizeof(int) * nb, st));
-    CS_CUDA(cudaMemsetAsync(f->margB, 0, sizeof(int) * nmarg * nb, st));
-    {
-      Stage sp(f, 0, st);
-      k_mask_counts<<<resample_grid(g, nb), 128, 0, st>>>(f->C8, f->rot_d + r0, g, f->msum, f->margB);
-    }
-    if (cs_ngf_status s = check_launch("mask counts")) return s;
-    {
-      Stage sp(f, 7, st);
-      k_shift_bounds<<<dim3((unsigned)nb, 3u), 512, 0, st>>>(f->margA, f->margB, f->msum, f->sumA,
-                                                             f->gamma, g, f->allb + 6 * (size_t)r0);
-    }
-    if (cs_ngf_status s = check_launch("shift bounds")) return s;
+  int* msum = f->allm;
+  int* marg = f->allm + R;
+  CS_CUDA(cudaMemsetAsync(f->allm, 0, sizeof(int) * (size_t)R * (1 + nmarg), st));
+  const int most = 65535 / (int)resample_grid(g, 1).z;      // rotations a grid's z dimension holds
+  for (int r0 = 0; r0 < R; r0 += most) {
+    const int nb = std::min(most, R - r0);
+    Stage sp(f, 0, st);
+    k_mask_counts<<<resample_grid(g, nb), 128, 0, st>>>(f->C8, f->rot_d + r0, g, msum + r0, marg + nmarg * r0);
   }
-  CS_CUDA(cudaMemcpyAsync(f->allb_h, f->allb, sizeof(int) * 6 * (size_t)R, cudaMemcpyDeviceToHost, st));
+  if (cs_ngf_status s = check_launch("mask counts")) return s;
+  {
+    Stage sp(f, 7, st);
+    k_shift_bounds<<<dim3((unsigned)R, 3u), 512, 0, st>>>(f->margA, marg, msum, f->sumA, f->gamma, g, f->allb);
+  }
+  if (cs_ngf_status s = check_launch("shift bounds")) return s;
+  CS_CUDA(cudaMemcpyAsync(f->allb_h, f->allb, sizeof(RotBounds) * (size_t)R, cudaMemcpyDeviceToHost, st));
   CS_CUDA(cudaStreamSynchronize(st));
   return CS_NGF_OK;
 }
 
-// FFT lengths one rotation needs: per axis the shortest supported P >=
-// n + max(-chi_lo, chi_hi) over its admitted shifts; false if it admits none
-bool rotation_lengths(const int dims[3], const int max_pad[3], const int* b, int pad[3]) {
-  if (b[0] > b[1] || b[2] > b[3] || b[4] > b[5]) return false;
-  for (int a = 0; a < 3; ++a) {
-    const int n = dims[a], lo = b[2 * a], hi = b[2 * a + 1];
-    pad[a] = length_for(n + std::max(n - 1 - lo, hi - (n - 1)), max_pad[a]);
+// FFT lengths a rotation needs, and whether it admits any shift
+struct Need { int pad[3]; bool any; };
+
+// the overlap rule: per axis the shortest supported P >= n + max(-chi_lo,
+// chi_hi) over the admitted shifts (slots lo, hi)
+Need rule_need(const int dims[3], const int max_pad[3], const int lo[3], const int hi[3]) {
+  Need q{{0, 0, 0}, lo[0] <= hi[0] && lo[1] <= hi[1] && lo[2] <= hi[2]};
+  for (int a = 0; a < 3 && q.any; ++a) {
+    const int n = dims[a];
+    q.pad[a] = length_for(n + std::max(n - 1 - lo[a], hi[a] - (n - 1)), max_pad[a]);
   }
-  return true;
+  return q;
+}
+
+// the same with both volumes cut to their masks' boxes, slabs [a0, a1] of the
+// fixed and [b0, b1] of the rotated one: the linear correlation lives on chi
+// in [b0 - a1, b1 - a0], so the admitted shifts are alias-free from
+// max(b1 - a0 - chi_lo, chi_hi - (b0 - a1)) + 1 points on, and both boxes must
+// fit.  150^3 with foreground masks: 138..164 points per axis against 182..207.
+Need box_need(const cs_ngf_fixed* f, const RotBounds& b) {
+  const int dims[3] = {f->g.nz, f->g.ny, f->g.nx};
+  Need q{{0, 0, 0}, b.lo[0] <= b.hi[0] && b.lo[1] <= b.hi[1] && b.lo[2] <= b.hi[2]};
+  for (int a = 0; a < 3 && q.any; ++a) {
+    const int clo = b.lo[a] - (dims[a] - 1), chi = b.hi[a] - (dims[a] - 1);
+    const int alias = std::max(b.b1[a] - f->a0[a] - clo, chi - b.b0[a] + f->a1[a]) + 1;
+    q.pad[a] = length_for(std::max(alias, std::max(b.b1[a] - b.b0[a], f->a1[a] - f->a0[a]) + 1),
+                          f->alloc_pad[a]);
+  }
+  return q;
 }
 
 cs_ngf_status check_volume_args(const cs_ngf_fixed* f, const float* B, const uint8_t* MB) {
@@ -661,37 +629,23 @@ cs_ngf_status check_volume_args(const cs_ngf_fixed* f, const float* B, const uin
   return CS_NGF_OK;
 }
 
-// rotations [r0_begin, r0_begin + n) of the uploaded set; full launch groups
-// replay the captured graph, a short tail is launched directly
+// rotations [r0_begin, r0_begin + n) of the uploaded set in launch groups
 cs_ngf_status score_range_impl(cs_ngf_fixed* f, int r0_begin, int n, float* best_score,
                                int32_t* best_shift, cudaStream_t st) {
   const int end = r0_begin + n;
   for (int r0 = r0_begin; r0 < end; r0 += f->batch) {
-    const int nb = std::min(f->batch, end - r0);
-    if (needs_tuning(f)) {                       // first group at these lengths: time the splits
-      if (cs_ngf_status s = score_batch(f, r0, nb, best_score, best_shift, nullptr, st, true)) return s;
-      continue;
-    }
-    if (nb == f->batch && !f->profiling) {
-      if (cs_ngf_status s = ensure_graph(f)) return s;
-      CS_CUDA(cudaMemcpyAsync(f->rot_slot, f->rot_d + r0, sizeof(RotMat) * nb, cudaMemcpyDeviceToDevice, st));
-      CS_CUDA(cudaGraphLaunch(f->gexec, st));
-      CS_CUDA(cudaMemcpyAsync(best_score + r0, f->slot_score, sizeof(float) * nb, cudaMemcpyDeviceToDevice, st));
-      CS_CUDA(cudaMemcpyAsync(best_shift + 3 * (size_t)r0, f->slot_shift, sizeof(int32_t) * 3 * nb,
-                              cudaMemcpyDeviceToDevice, st));
-      g_launches.fetch_add(kKernelsPerBatch, std::memory_order_relaxed);
-    } else if (cs_ngf_status s = score_batch(f, r0, nb, best_score, best_shift, nullptr, st)) {
+    // the first group at new lengths times the splits (autotuning)
+    if (cs_ngf_status s = score_batch(f, r0, std::min(f->batch, end - r0), best_score, best_shift, nullptr, st,
+                                      needs_tuning(f)))
       return s;
-    }
   }
   return CS_NGF_OK;
 }
 
 // Bound-limited padding per rotation: each rotation's own shortest lengths;
 // rotations that need the same lengths form one class, scored together.  A
-// class costs a fixed-spectra recomputation, a stream synchronisation and
-// (once per handle) a graph capture, about kClassCost rotations of its own
-// size; so two classes merge, with lengths raised to cover both, while the
+// class costs a fixed-spectra recomputation and a partial launch group, about
+// kClassCost rotations of its own size; so two classes merge, with lengths raised to cover both, while the
 // cheapest merge adds less transform volume than that (and while there are
 // more than kMaxClasses).  Rotations admitting no shift join the first
 // class.  The classes do not depend on the launch-group size, so results
@@ -702,16 +656,14 @@ struct LengthClass { int pad[3]; std::vector<int> rot; };
 
 double class_volume(const int* p) { return (double)p[0] * p[1] * p[2]; }
 
-// dims, max_pad: the volume and the largest lengths; cur: the lengths in use
-// (their class goes first); bounds [R][6]: each rotation's admitted shift
-// slots {lo_z, hi_z, lo_y, hi_y, lo_x, hi_x}
-std::vector<LengthClass> length_classes(const int dims[3], const int max_pad[3], const int cur[3],
-                                        int R, const int* bounds) {
+// cur: the lengths in use (their class goes first); none: lengths when no
+// rotation admits a shift
+std::vector<LengthClass> length_classes(const std::vector<Need>& need, const int none_pad[3], const int cur[3]) {
   std::vector<LengthClass> cls;
   std::vector<int> none;
-  for (int r = 0; r < R; ++r) {
-    int p[3];
-    if (!rotation_lengths(dims, max_pad, bounds + 6 * (size_t)r, p)) { none.push_back(r); continue; }
+  for (int r = 0; r < (int)need.size(); ++r) {
+    const int* p = need[r].pad;
+    if (!need[r].any) { none.push_back(r); continue; }
     size_t k = 0;
     while (k < cls.size() && !std::equal(p, p + 3, cls[k].pad)) ++k;
     if (k == cls.size()) cls.push_back({{p[0], p[1], p[2]}, {}});
@@ -741,11 +693,7 @@ std::vector<LengthClass> length_classes(const int dims[3], const int max_pad[3],
     std::sort(cls[bc].rot.begin(), cls[bc].rot.end());
     cls.erase(cls.begin() + (long)bd);
   }
-  if (cls.empty()) {
-    LengthClass lc;
-    for (int a = 0; a < 3; ++a) lc.pad[a] = length_for(dims[a], max_pad[a]);
-    cls.push_back(lc);
-  }
+  if (cls.empty()) cls.push_back({{none_pad[0], none_pad[1], none_pad[2]}, {}});
   cls[0].rot.insert(cls[0].rot.end(), none.begin(), none.end());
   std::sort(cls[0].rot.begin(), cls[0].rot.end());
   // start with the lengths in use (no recomputation), then the larger classes
@@ -757,45 +705,77 @@ std::vector<LengthClass> length_classes(const int dims[3], const int max_pad[3],
   return cls;
 }
 
-// Length classes of the R uploaded rotations (floating volume packed by
-// pack_floating):
-// bounds (synchronises st), classes, and the rotation matrices re-uploaded
-// in class order when there is more than one.  perm[i] = original index of
-// the i-th rotation in class order (empty if the order is unchanged); class
-// c covers [ends[c-1], ends[c]) with lengths pads[c].  Without bound-limited
-// padding: one class with the lengths in use.
-cs_ngf_status plan_classes(cs_ngf_fixed* f, int R, cudaStream_t st,
-                           std::vector<int>& perm, std::vector<int>& ends, std::vector<int>& pads) {
-  perm.clear();
-  ends.assign(1, R);
-  pads.assign({f->g.Pz, f->g.Py, f->g.Px});
-  f->length_sets = 1;
-  f->last_pads = pads;
-  f->last_counts.assign(1, R);
-  if (f->pad_mode != CS_NGF_PAD_BOUND) return CS_NGF_OK;
+// Classes of the R uploaded rotations (floating volume packed by
+// pack_floating): bounds (synchronises st), length classes by the overlap rule
+// (reported) and, for a boxed handle, by the boxes (scored), and the rotations
+// re-uploaded in class order with their boxes.
+cs_ngf_status plan_classes_impl(cs_ngf_fixed* f, int R, cudaStream_t st, Plan& plan) {
+  const Geo& g = f->g;
+  const int dims[3] = {g.nz, g.ny, g.nx};
+  plan.perm.clear();
+  plan.cls.clear();
+  if (f->pad_mode != CS_NGF_PAD_BOUND) {
+    plan.cls.push_back({{g.Pz, g.Py, g.Px}, {g.nz, g.ny, g.nx}, {g.vz, g.vy, g.vx}, R});
+    f->length_sets = 1;
+    f->last_pads.assign({g.Pz, g.Py, g.Px});
+    f->last_counts.assign(1, R);
+    f->run_pads = f->last_pads;
+    f->run_counts = f->last_counts;
+    return CS_NGF_OK;
+  }
   if (cs_ngf_status s = rotation_bounds(f, R, st)) return s;
-  const int dims[3] = {f->g.nz, f->g.ny, f->g.nx}, cur[3] = {f->g.Pz, f->g.Py, f->g.Px};
-  std::vector<LengthClass> cls = length_classes(dims, f->alloc_pad, cur, R, f->allb_h);
+  const RotBounds* bounds = f->allb_h;
+  int none_pad[3];
+  for (int a = 0; a < 3; ++a) none_pad[a] = length_for(dims[a], f->alloc_pad[a]);
+  std::vector<Need> need(R);
+  for (int r = 0; r < R; ++r) need[r] = rule_need(dims, f->alloc_pad, bounds[r].lo, bounds[r].hi);
+  std::vector<LengthClass> cls = length_classes(need, none_pad, f->rule_pad);
   f->length_sets = (int)cls.size();
-  ends.clear();
-  pads.clear();
+  f->last_pads.clear();
   f->last_counts.clear();
-  int k = 0;
   for (const auto& c : cls) {
-    k += (int)c.rot.size();
-    ends.push_back(k);
-    pads.insert(pads.end(), c.pad, c.pad + 3);
+    f->last_pads.insert(f->last_pads.end(), c.pad, c.pad + 3);
     f->last_counts.push_back((int)c.rot.size());
   }
-  f->last_pads = pads;
-  if (cls.size() == 1) return CS_NGF_OK;
-  // the stream is idle (rotation_bounds waited for it): rot_h is free
-  std::vector<RotMat> orig(f->rot_h, f->rot_h + R);
-  perm.reserve(R);
-  k = 0;
-  for (const auto& c : cls)
-    for (int r : c.rot) { f->rot_h[k++] = orig[r]; perm.push_back(r); }
-  CS_CUDA(cudaMemcpyAsync(f->rot_d, f->rot_h, sizeof(RotMat) * R, cudaMemcpyHostToDevice, st));
+  std::copy(cls.back().pad, cls.back().pad + 3, f->rule_pad);
+  if (f->boxed) {
+    const int cur[3] = {g.Pz, g.Py, g.Px};
+    for (int r = 0; r < R; ++r) need[r] = box_need(f, bounds[r]);
+    cls = length_classes(need, none_pad, cur);
+  }
+  f->run_pads.clear();
+  f->run_counts.clear();
+  std::vector<RotMat> mats(R);
+  for (int r = 0; r < R; ++r) mats[r] = f->rot_h[r].m;   // the stream is idle: rot_h is free
+  int k = 0;
+  for (const auto& c : cls) {
+    ClassGeom q{{c.pad[0], c.pad[1], c.pad[2]}, {1, 1, 1}, {1, 1, 1}, 0};
+    const double pvol = (double)q.pad[0] * (double)q.pad[1] * (double)q.pad[2];
+    for (int r : c.rot) {
+      const RotBounds& b = bounds[r];
+      RotIn& in = f->rot_h[k++];
+      in.m = mats[r];
+      if (cls.size() > 1) plan.perm.push_back(r);
+      for (int a = 0; a < 3; ++a) {
+        in.b.lo[a] = in.b.org[a] = in.b.m0[a] = 0;
+        in.b.hi[a] = -1;
+        if (!need[r].any) continue;
+        in.b.lo[a] = b.lo[a];
+        in.b.hi[a] = b.hi[a];
+        in.b.org[a] = f->boxed ? b.b0[a] : 0;
+        const int chi = b.lo[a] - (dims[a] - 1) + (f->boxed ? f->a0[a] - b.b0[a] : 0);
+        in.b.m0[a] = (chi % q.pad[a] + q.pad[a]) % q.pad[a];
+        q.ext[a] = std::max(q.ext[a], b.b1[a] + 1 - in.b.org[a]);
+        q.win[a] = std::max(q.win[a], b.hi[a] - b.lo[a] + 1);
+      }
+      in.b.thr = overlap_threshold(f->sumA, b.msum, f->gamma, pvol);
+    }
+    q.end = k;
+    plan.cls.push_back(q);
+    f->run_pads.insert(f->run_pads.end(), q.pad, q.pad + 3);
+    f->run_counts.push_back((int)c.rot.size());
+  }
+  CS_CUDA(cudaMemcpyAsync(f->rot_d, f->rot_h, sizeof(RotIn) * R, cudaMemcpyHostToDevice, st));
   CS_CUDA(cudaEventRecord(f->rot_ev, st));
   return CS_NGF_OK;
 }
@@ -806,22 +786,25 @@ cs_ngf_status score_all(cs_ngf_fixed* f, const float* B, const uint8_t* MB, cons
   if (!best_score || !best_shift) return fail(CS_NGF_EINVAL, "output pointer is NULL");
   if (cs_ngf_status s = upload_rotations(f, quats, R, st)) return s;
   if (cs_ngf_status s = pack_floating(f, B, MB, st)) return s;
-  std::vector<int> perm, ends, pads;
-  if (cs_ngf_status s = plan_classes(f, R, st, perm, ends, pads)) return s;
-  if (perm.empty()) {
-    if (cs_ngf_status s = set_pads(f, pads.data(), st)) return s;
-    return score_range_impl(f, 0, R, best_score, best_shift, st);
+  Plan plan;
+  if (cs_ngf_status s = plan_classes_impl(f, R, st, plan)) return s;
+  // classes one after another; with several, into the handle's buffers, then
+  // scattered to the caller's order
+  const bool mixed = !plan.perm.empty();
+  float* score = mixed ? f->perm_score : best_score;
+  int32_t* shift = mixed ? f->perm_shift : best_shift;
+  if (mixed) {
+    int* perm_h = reinterpret_cast<int*>(f->allb_h);   // pinned staging; the bounds are spent
+    std::copy(plan.perm.begin(), plan.perm.end(), perm_h);
+    CS_CUDA(cudaMemcpyAsync(f->perm_d, perm_h, sizeof(int) * R, cudaMemcpyHostToDevice, st));
   }
-  // classes one after another into the handle's buffers, then scattered to
-  // the caller's order
-  std::copy(perm.begin(), perm.end(), f->allb_h);   // pinned staging; the bounds are spent
-  CS_CUDA(cudaMemcpyAsync(f->perm_d, f->allb_h, sizeof(int) * R, cudaMemcpyHostToDevice, st));
   int r0 = 0;
-  for (size_t c = 0; c < ends.size(); ++c) {
-    if (cs_ngf_status s = set_pads(f, pads.data() + 3 * c, st)) return s;
-    if (cs_ngf_status s = score_range_impl(f, r0, ends[c] - r0, f->perm_score, f->perm_shift, st)) return s;
-    r0 = ends[c];
+  for (const ClassGeom& c : plan.cls) {
+    if (cs_ngf_status s = set_class_impl(f, c, st)) return s;
+    if (cs_ngf_status s = score_range_impl(f, r0, c.end - r0, score, shift, st)) return s;
+    r0 = c.end;
   }
+  if (!mixed) return CS_NGF_OK;
   { Stage sp(f, 7, st); k_scatter_results<<<(R + 255) / 256, 256, 0, st>>>(f->perm_d, f->perm_score, f->perm_shift, R, best_score, best_shift); }
   return check_launch("scatter results");
 }
@@ -907,12 +890,11 @@ cs_ngf_status score_range(cs_ngf_fixed* f, int r0, int n, float* best_score, int
                           cudaStream_t st) {
   return ::score_range_impl(f, r0, n, best_score, best_shift, st);
 }
-cs_ngf_status plan_classes(cs_ngf_fixed* f, int R, cudaStream_t st,
-                           std::vector<int>& perm, std::vector<int>& ends, std::vector<int>& pads) {
-  return ::plan_classes(f, R, st, perm, ends, pads);
+cs_ngf_status plan_classes(cs_ngf_fixed* f, int R, cudaStream_t st, Plan& plan) {
+  return ::plan_classes_impl(f, R, st, plan);
 }
-cs_ngf_status set_lengths(cs_ngf_fixed* f, const int pad[3], cudaStream_t st) {
-  return ::set_pads(f, pad, st);
+cs_ngf_status set_class(cs_ngf_fixed* f, const ClassGeom& c, cudaStream_t st) {
+  return ::set_class_impl(f, c, st);
 }
 cs_ngf_status resolve_pads(const int32_t dims[3], const cs_ngf_config& cfg, int pad[3]) {
   return ::resolve_pads_impl(dims, cfg, pad);
@@ -920,13 +902,11 @@ cs_ngf_status resolve_pads(const int32_t dims[3], const cs_ngf_config& cfg, int 
 size_t handle_bytes(const int32_t dims[3], const int pad[3], int batch, int measure, int precision,
                     int tensor_cores) {
   const Sizes z = ::sizes_for(dims, pad, measure, precision, tensor_cores);
-  size_t tw = 0;
-  for (int a = 0; a < 3; ++a) tw += (size_t)pad[a] * sizeof(float2);
   const size_t nmarg = (size_t)dims[0] + dims[1] + dims[2];
   const size_t keep = (size_t)dims[0] * dims[1] * dims[2] * 5;    // A, M_A copies (bound-limited padding)
   return z.uv_elems * sizeof(float2) + keep + (size_t)batch * z.per_rot + z.shared_ws +
-         (size_t)batch * (sizeof(int) + sizeof(float) + sizeof(unsigned long long) + 6 * sizeof(int)) +
-         (size_t)(batch + 1) * nmarg * sizeof(int) + tw;
+         (size_t)batch * (sizeof(int) + sizeof(unsigned long long) + sizeof(RotBounds)) + sizeof(RotIn) +
+         (size_t)(batch + 1) * nmarg * sizeof(int);
 }
 }  // namespace detail
 }  // namespace csngf
@@ -1025,9 +1005,15 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
   g.store = cfg.precision == CS_NGF_BF16 ? kStoreBF16 : cfg.precision == CS_NGF_FP16 ? kStoreF16 : kStoreF32;
   set_field_scales(g);
   g.tc = cfg.tensor_cores;
-  for (int a = 0; a < 3; ++a) f->alloc_pad[a] = pad[a];
+  g.ez = g.nz; g.ey = g.ny; g.ex = g.nx;
+  g.wz = g.vz; g.wy = g.vy;
+  for (int a = 0; a < 3; ++a) f->alloc_pad[a] = f->rule_pad[a] = pad[a];
   f->pad_mode = cfg.pad_mode;
   f->autotune = cfg.autotune;
+  // The 16-bit forms round the packed spectra, whose values follow the lengths
+  // and the origin, and the tuner times the splits of the rule's lengths: both
+  // keep those lengths, with only the far empty slabs left out.
+  f->boxed = f->pad_mode == CS_NGF_PAD_BOUND && g.store == kStoreF32 && f->autotune == 0;
   resolve_variants(f);
 
   const Sizes sz = sizes_for(dims, pad, cfg.measure, cfg.precision, cfg.tensor_cores);
@@ -1066,8 +1052,8 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
   const size_t nmarg = (size_t)g.nz + g.ny + g.nx;
   CS_TRYC(dalloc(&f->margA, nmarg));
   CS_TRYC(dalloc(&f->margB, (size_t)batch * nmarg));
-  CS_TRYC(dalloc(&f->bounds, (size_t)batch * 6));
-  CS_TRYC(dalloc(&f->thr, (size_t)batch));
+  CS_TRYC(dalloc(&f->bounds, (size_t)batch));
+  CS_TRYC(dalloc(&f->boxA, (size_t)1));
   CS_TRYC(dalloc(&f->keys, (size_t)batch));
   if (sz.zx_elems) {
     CS_TRYC(dalloc(&f->zx, (size_t)batch * sz.zx_elems));
@@ -1079,10 +1065,6 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
   g.tc_err = f->tc_err;
   f->fixed_bytes = uv_elems * sizeof(float2);
   f->workspace_bytes = (size_t)batch * per_rot + shared_ws;
-  for (int a = 0; a < 3; ++a) {                 // one table per axis: the lengths may part
-    CS_TRYC(dalloc(&f->tw[a], (size_t)pad[a]));
-    CS_TRY(fill_twiddles(pad[a], f->tw[a]));
-  }
   if (f->pad_mode == CS_NGF_PAD_BOUND) {
     CS_TRYC(dalloc(&f->A_keep, (size_t)g.nvox));
     CS_TRYC(dalloc(&f->MA_keep, (size_t)g.nvox));
@@ -1092,7 +1074,7 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
   }
 
   // A side into the new handle
-  CS_TRY(run_fixed(f, A, maskA, st));
+  CS_TRY(load_fixed(f, A, maskA, st));
   CS_TRYC(cudaEventRecord(f->order_ev, st));
 #undef CS_TRY
 #undef CS_TRYC
@@ -1180,9 +1162,9 @@ cs_ngf_status cs_ngf_score_map(cs_ngf_fixed* f, const float* B, const uint8_t* m
   if (cs_ngf_status s = ensure_results(f, 1)) return s;
   if (cs_ngf_status s = upload_rotations(f, quat, 1, st)) return s;
   if (cs_ngf_status s = pack_floating(f, B, maskB, st)) return s;
-  std::vector<int> perm, ends, pads;
-  if (cs_ngf_status s = plan_classes(f, 1, st, perm, ends, pads)) return s;
-  if (cs_ngf_status s = set_pads(f, pads.data(), st)) return s;
+  Plan plan;
+  if (cs_ngf_status s = plan_classes_impl(f, 1, st, plan)) return s;
+  if (cs_ngf_status s = set_class_impl(f, plan.cls[0], st)) return s;
   return score_batch(f, 0, 1, f->res_score, f->res_shift, map, st);
 }
 
@@ -1205,7 +1187,7 @@ cs_ngf_status cs_ngf_resample(cs_ngf_fixed* f, const float* B, const uint8_t* ma
 cs_ngf_status cs_ngf_get_info(const cs_ngf_fixed* f, cs_ngf_info* info) {
   if (!f || !info) return fail(CS_NGF_EINVAL, "handle or info is NULL");
   info->dims[0] = f->g.nz; info->dims[1] = f->g.ny; info->dims[2] = f->g.nx;
-  info->pad[0] = f->g.Pz; info->pad[1] = f->g.Py; info->pad[2] = f->g.Px;
+  for (int a = 0; a < 3; ++a) info->pad[a] = f->rule_pad[a];
   info->batch = f->batch;
   info->sum_mask_a = f->sumA;
   info->fixed_bytes = (int64_t)f->fixed_bytes;
@@ -1228,7 +1210,15 @@ int32_t cs_ngf_plan_lengths(const int32_t dims[3], const int32_t max_pad[3], con
       return -1;
   const int d[3] = {dims[0], dims[1], dims[2]}, m[3] = {max_pad[0], max_pad[1], max_pad[2]};
   const int c[3] = {cur_pad ? cur_pad[0] : 0, cur_pad ? cur_pad[1] : 0, cur_pad ? cur_pad[2] : 0};
-  const std::vector<LengthClass> cls = length_classes(d, m, c, R, bounds);
+  int none_pad[3];
+  for (int a = 0; a < 3; ++a) none_pad[a] = length_for(d[a], m[a]);
+  std::vector<Need> need(R);
+  for (int r = 0; r < R; ++r) {
+    const int32_t* b = bounds + 6 * (size_t)r;
+    const int lo[3] = {b[0], b[2], b[4]}, hi[3] = {b[1], b[3], b[5]};
+    need[r] = rule_need(d, m, lo, hi);
+  }
+  const std::vector<LengthClass> cls = length_classes(need, none_pad, c);
   int k = 0;
   for (size_t i = 0; i < cls.size(); ++i) {
     if ((int)i < cap) {
@@ -1268,15 +1258,23 @@ void cs_ngf_tuning_reset(void) {
   g_tune.clear();
 }
 
-int32_t cs_ngf_length_sets(const cs_ngf_fixed* f, int32_t cap, int32_t* pads, int32_t* counts) {
-  if (!f) return 0;
-  const int n = (int)f->last_counts.size();
+static int32_t copy_sets(const std::vector<int>& p, const std::vector<int>& k, int32_t cap, int32_t* pads,
+                         int32_t* counts) {
+  const int n = (int)k.size();
   for (int c = 0; c < n && c < cap; ++c) {
     if (pads)
-      for (int a = 0; a < 3; ++a) pads[3 * c + a] = f->last_pads[3 * (size_t)c + a];
-    if (counts) counts[c] = f->last_counts[c];
+      for (int a = 0; a < 3; ++a) pads[3 * c + a] = p[3 * (size_t)c + a];
+    if (counts) counts[c] = k[c];
   }
   return n;
+}
+
+int32_t cs_ngf_length_sets(const cs_ngf_fixed* f, int32_t cap, int32_t* pads, int32_t* counts) {
+  return f ? copy_sets(f->last_pads, f->last_counts, cap, pads, counts) : 0;
+}
+
+int32_t cs_ngf_transform_sets(const cs_ngf_fixed* f, int32_t cap, int32_t* pads, int32_t* counts) {
+  return f ? copy_sets(f->run_pads, f->run_counts, cap, pads, counts) : 0;
 }
 
 cs_ngf_status cs_ngf_update_fixed(cs_ngf_fixed* f, const float* A, const uint8_t* maskA, void* stream) {
@@ -1290,7 +1288,7 @@ cs_ngf_status cs_ngf_update_fixed(cs_ngf_fixed* f, const float* A, const uint8_t
     CS_CUDA(cudaMemcpyAsync(f->A_keep, A, sizeof(float) * f->g.nvox, cudaMemcpyDeviceToDevice, st));
     CS_CUDA(cudaMemcpyAsync(f->MA_keep, maskA, (size_t)f->g.nvox, cudaMemcpyDeviceToDevice, st));
   }
-  return run_fixed(f, A, maskA, st);
+  return load_fixed(f, A, maskA, st);
 }
 
 cs_ngf_status cs_ngf_set_profiling(cs_ngf_fixed* f, int32_t on) {

@@ -152,7 +152,7 @@ __device__ __forceinline__ void resample_voxel(const float4* __restrict__ BQ,
 template <bool MONLY>
 __device__ __forceinline__ void resample_block(const float4* __restrict__ BQ,
                                                const uint8_t* __restrict__ C8,
-                                               const RotMat* __restrict__ rot, const Geo& g,
+                                               const RotIn* __restrict__ rot, const Geo& g,
                                                float* __restrict__ Bh, uint8_t* __restrict__ Mh,
                                                int* __restrict__ msum, int* __restrict__ marg) {
   constexpr int RZ = kResampleZGroups, ZB = 4 * RZ;    // z-planes per block
@@ -163,7 +163,7 @@ __device__ __forceinline__ void resample_block(const float4* __restrict__ BQ,
   const int x = blockIdx.x * 8 + tx;
   const int y = blockIdx.y * 4 + ty;
   __shared__ int zs[ZB], ys[4][4], xs[4][8], cs[4];
-  const RotMat R = rot[r];
+  const RotMat R = rot[r].m;
   const SampleRow sr = sample_row(R, g, x, y);
   const bool xy_ok = x < g.nx && y < g.ny;
   const long long plane = (long long)g.nx * g.ny;
@@ -226,60 +226,135 @@ __device__ __forceinline__ void resample_block(const float4* __restrict__ BQ,
 
 __global__ void __launch_bounds__(128)
 k_resample(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8,
-           const RotMat* __restrict__ rot, Geo g, float* __restrict__ Bh, uint8_t* __restrict__ Mh,
+           const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh, uint8_t* __restrict__ Mh,
            int* __restrict__ msum, int* __restrict__ marg) {
   resample_block<false>(BQ, C8, rot, g, Bh, Mh, msum, marg);
 }
 
 __global__ void __launch_bounds__(128)
-k_mask_counts(const uint8_t* __restrict__ C8, const RotMat* __restrict__ rot, Geo g,
+k_mask_counts(const uint8_t* __restrict__ C8, const RotIn* __restrict__ rot, Geo g,
               int* __restrict__ msum, int* __restrict__ marg) {
   resample_block<true>(nullptr, C8, rot, g, nullptr, nullptr, msum, marg);
 }
 
-__global__ void k_marginals(const uint8_t* __restrict__ M, Geo g, int* __restrict__ marg) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.nvox;
-       i += (long long)gridDim.x * blockDim.x) {
-    if (!M[i]) continue;
-    const int x = (int)(i % g.nx);
-    const int y = (int)((i / g.nx) % g.ny);
-    const int z = (int)(i / ((long long)g.nx * g.ny));
-    atomicAdd(&marg[z], 1);
-    atomicAdd(&marg[g.nz + y], 1);
-    atomicAdd(&marg[g.nz + g.ny + x], 1);
+// The voxels the x pass reads: each rotation's box of Geo::ez x ey x ex voxels
+// and one voxel around it (the gradient's neighbours), clipped to the volume.
+// The counts are known by then, so nothing is reduced.  At 150^3 with a
+// foreground mask the box holds 0.4 of the volume.
+__global__ void __launch_bounds__(128)
+k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8,
+               const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh, uint8_t* __restrict__ Mh) {
+  constexpr int RZ = kResampleZGroups, ZB = 4 * RZ;
+  const int ztiles = (g.ez + 2 + ZB - 1) / ZB;
+  const int r = blockIdx.z / ztiles, zt = blockIdx.z - r * ztiles;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const RotBox& b = rot[r].b;
+  const int x = b.org[2] - 1 + blockIdx.x * 8 + (lane & 7);
+  const int y = b.org[1] - 1 + blockIdx.y * 4 + (lane >> 3);
+  if (x < 0 || y < 0 || x >= min(g.nx, b.org[2] + g.ex + 1) || y >= min(g.ny, b.org[1] + g.ey + 1)) return;
+  const int z_end = min(g.nz, b.org[0] + g.ez + 1);
+  const RotMat R = rot[r].m;
+  const SampleRow sr = sample_row(R, g, x, y);
+  const long long plane = (long long)g.nx * g.ny;
+  int z = b.org[0] - 1 + zt * ZB + wid;
+  long long idx = (long long)r * g.nvox + (long long)z * plane + (long long)y * g.nx + x;
+#pragma unroll 1
+  for (int k = 0; k < RZ; ++k, z += 4, idx += 4 * plane) {
+    if (z < 0 || z >= z_end) continue;
+    float val;
+    uint8_t m;
+    resample_voxel(BQ, C8, R, sr, g, z, val, m);
+    Bh[idx] = val;
+    Mh[idx] = m;
   }
 }
 
-// block (rotation r, axis a); thread per shift slot v
+// block per z-plane: warps take rows; the x counts collect in shared memory
+__global__ void __launch_bounds__(256) k_marginals(const uint8_t* __restrict__ M, Geo g, int* __restrict__ marg) {
+  __shared__ int xs[256];
+  __shared__ int zs;
+  const int t = threadIdx.x, lane = t & 31, z = blockIdx.x;
+  xs[t] = 0;
+  if (t == 0) zs = 0;
+  __syncthreads();
+  const uint8_t* P = M + (long long)z * g.nx * g.ny;
+  for (int y = t >> 5; y < g.ny; y += 8) {
+    int c = 0;
+    for (int x = lane; x < g.nx; x += 32)
+      if (P[y * g.nx + x]) {
+        ++c;
+        atomicAdd(&xs[x], 1);
+      }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0 && c) {
+      atomicAdd(&marg[g.nz + y], c);
+      atomicAdd(&zs, c);
+    }
+  }
+  __syncthreads();
+  if (t == 0) marg[z] = zs;
+  if (t < g.nx && xs[t]) atomicAdd(&marg[g.nz + g.ny + t], xs[t]);
+}
+
+// block (rotation r, axis a); thread per shift slot v, then per slab
 __global__ void k_shift_bounds(const int* __restrict__ margA, const int* __restrict__ margB,
                                const int* __restrict__ msumB, int sumA, float gamma, Geo g,
-                               int* __restrict__ bounds) {
+                               RotBounds* __restrict__ bounds) {
   const int r = blockIdx.x, a = blockIdx.y;
   const int n = a == 0 ? g.nz : (a == 1 ? g.ny : g.nx);
   const int off = a == 0 ? 0 : (a == 1 ? g.nz : g.nz + g.ny);
-  const int* ma = margA + off;
   const int* mb = margB + (long long)r * (g.nz + g.ny + g.nx) + off;
   const int mn = min(sumA, msumB[r]);
   double t = ceil((double)gamma * (double)mn);
   if (t < 1.0) t = 1.0;
-  const long long thr = (long long)t;
-  __shared__ int lo_s, hi_s;
-  if (threadIdx.x == 0) { lo_s = 0x7fffffff; hi_s = -1; }
+  const int thr = (int)t;                       // at most the mask sum, < 2^31
+  __shared__ int sa[256], sb[256], lo_s, hi_s, b0_s, b1_s;
+  if (threadIdx.x == 0) { lo_s = b0_s = 0x7fffffff; hi_s = b1_s = -1; }
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    sa[i] = margA[off + i];
+    sb[i] = mb[i];
+  }
   __syncthreads();
   for (int v = threadIdx.x; v < 2 * n - 1; v += blockDim.x) {
     const int c = v - (n - 1);
-    long long u = 0;
-    for (int i = max(0, -c); i < min(n, n - c); ++i) u += min(ma[i], mb[i + c]);
+    int u = 0;                                  // at most a mask sum
+    for (int i = max(0, -c); i < min(n, n - c); ++i) u += min(sa[i], sb[i + c]);
     if (u >= thr) {
       atomicMin(&lo_s, v);
       atomicMax(&hi_s, v);
     }
+    if (v < n && sb[v]) {
+      atomicMin(&b0_s, v);
+      atomicMax(&b1_s, v);
+    }
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    bounds[r * 6 + 2 * a] = lo_s;
-    bounds[r * 6 + 2 * a + 1] = hi_s;
+    bounds[r].lo[a] = lo_s;
+    bounds[r].hi[a] = hi_s;
+    bounds[r].b0[a] = b0_s;
+    bounds[r].b1[a] = b1_s;
+    if (a == 0) bounds[r].msum = msumB[r];
   }
+}
+
+__global__ void k_full_boxes(const RotBounds* __restrict__ bounds, int sumA, float gamma, Geo g,
+                             double pvol, int nrot, RotIn* __restrict__ rot) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= nrot) return;
+  const RotBounds& s = bounds[r];
+  RotBox& b = rot[r].b;
+  const int n[3] = {g.nz, g.ny, g.nx}, P[3] = {g.Pz, g.Py, g.Px};
+  const bool none = s.lo[0] > s.hi[0] || s.lo[1] > s.hi[1] || s.lo[2] > s.hi[2];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    b.lo[a] = none ? 0 : s.lo[a];
+    b.hi[a] = none ? -1 : s.hi[a];
+    b.org[a] = 0;
+    const int chi = b.lo[a] - (n[a] - 1);       // of slot lo, > -P
+    b.m0[a] = chi < 0 ? chi + P[a] : chi;
+  }
+  b.thr = overlap_threshold(sumA, s.msum, gamma, pvol);
 }
 
 __global__ void k_scatter_results(const int* __restrict__ perm, const float* __restrict__ score,
@@ -306,16 +381,6 @@ __global__ void k_mask_sum(const uint8_t* __restrict__ M, long long n, int* __re
     c += M[i] ? 1 : 0;
   for (int off = 16; off > 0; off >>= 1) c += __shfl_down_sync(0xffffffffu, c, off);
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
-}
-
-__global__ void k_thresholds(const int* __restrict__ msumB, int sumA, float gamma, double pvol,
-                             int nrot, float* __restrict__ thr) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrot) return;
-  const int mn = min(sumA, msumB[r]);
-  double t = ceil((double)gamma * (double)mn);
-  if (t < 1.0) t = 1.0;
-  thr[r] = (float)((t - 0.5) * pvol);
 }
 
 __global__ void k_finalize(const unsigned long long* __restrict__ keys, int nrot, Geo g,

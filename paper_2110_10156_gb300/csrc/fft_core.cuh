@@ -53,6 +53,22 @@ constexpr double sin2pi(long e, long R) {
 }
 }  // namespace ctw
 
+// exp(-2 pi i m / P), m < P, as a constant table of the module (rounded from
+// FP64), so that a change of FFT length uploads nothing and waits for nothing
+template <int P>
+struct TwTable { float2 w[P]; };
+template <int P>
+constexpr TwTable<P> make_twiddles() {
+  TwTable<P> t{};
+  for (int m = 0; m < P; ++m) {
+    t.w[m].x = (float)ctw::cos2pi(m, P);
+    t.w[m].y = (float)(-ctw::sin2pi(m, P));
+  }
+  return t;
+}
+template <int P>
+__device__ const TwTable<P> kTw = make_twiddles<P>();
+
 // ---------------------------------------------------------------- complex
 // Complex add and subtract as one paired FP32 instruction (add/sub.rn.f32x2:
 // each lane rounds exactly as a scalar add), half the issue slots of two adds.

@@ -13,7 +13,8 @@
 
 struct cs_ngf_fixed {
   using Geo = csngf::Geo;
-  using RotMat = csngf::RotMat;
+  using RotIn = csngf::RotIn;
+  using RotBounds = csngf::RotBounds;
   int device = 0;
   Geo g{};
   float eps = 1e-5f, gamma = 0.5f;
@@ -26,26 +27,35 @@ struct cs_ngf_fixed {
   int pad_mode = 0;
   float* A_keep = nullptr;     // copies of A and M_A: the fixed spectra are
   uint8_t* MA_keep = nullptr;  // recomputed when the lengths in use change
-  // per-rotation shift bounds of a call and its rotations regrouped by FFT
-  // lengths (bound-limited padding), grown on demand to the call's R
-  int* allb = nullptr;         // device [R][6]
-  int* allb_h = nullptr;       // pinned host copy
+  RotIn* boxA = nullptr;       // device: the fixed volume's box (origin)
+  int extA[3] = {0, 0, 0};     // its extents in use, and the slabs [a0, a1] its mask holds
+  int a0[3] = {0, 0, 0}, a1[3] = {-1, -1, -1};
+  // per-rotation mask counts and bounds of a call and its rotations regrouped
+  // by FFT lengths (bound-limited padding), grown on demand to the call's R
+  int* allm = nullptr;         // device [R][1 + nz + ny + nx]: sums, then slab counts
+  RotBounds* allb = nullptr;   // device [R]
+  RotBounds* allb_h = nullptr; // pinned host copy
   int* perm_d = nullptr;       // device: original index of each regrouped rotation
   float* perm_score = nullptr; // device results in regrouped order
   int32_t* perm_shift = nullptr;
   int allb_cap = 0;
-  int length_sets = 1;         // sets of FFT lengths the last scoring call used
-  std::vector<int> last_pads;  // their lengths [3 per set] and rotation counts
-  std::vector<int> last_counts;
+  // lengths the overlap rule gives (n + max(-lo, hi)): those of the last class
+  // reported, the sets of the last scoring call and their rotation counts
+  int rule_pad[3] = {0, 0, 0};
+  int length_sets = 1;
+  std::vector<int> last_pads, last_counts;
+  // transform lengths of the last scoring call's launch classes (see
+  // csngf::detail::ClassGeom) and their rotation counts
+  std::vector<int> run_pads, run_counts;
+  // transforms take only the masks' boxes, at lengths as short as those allow
+  // (the FP32 form with bound-limited padding and the built-in splits)
+  bool boxed = false;
+  bool spectra_ok = false;     // UV holds A's spectra at g.Pz, Py, Px
   // split variant of each FFT pass at the lengths in use (fwd_x, fwd_y, zmac,
   // inv_y, inv_x): 0 unless autotuning chose the alternative (autotune 1) or
   // the alternatives are requested outright (autotune 2)
   int autotune = 0;
   int vars[5] = {0, 0, 0, 0, 0};
-  int gexec_vars[5] = {0, 0, 0, 0, 0};   // the variants gexec was captured with
-  // one captured graph per set of FFT lengths (all reference the same buffers)
-  struct GraphSlot { int pad[3]; int vars[5]; cudaGraphExec_t exec; };
-  std::vector<GraphSlot> graphs;
   size_t f02_elems = 0, f13_elems = 0;
   float2* UV = nullptr;
   float* Bh = nullptr;
@@ -57,15 +67,13 @@ struct cs_ngf_fixed {
   int* msum = nullptr;
   int* margA = nullptr;        // slab counts of M_A per axis [nz | ny | nx]
   int* margB = nullptr;        // the same for each rotated mask of a batch
-  int* bounds = nullptr;       // per rotation of a batch: shift slots that can be valid
-  float* thr = nullptr;
+  RotBounds* bounds = nullptr; // per rotation of a batch (full padding)
   unsigned long long* keys = nullptr;
   int* tc_err = nullptr;       // set by a tensor-core pass that stopped on its bounded wait
   float2* zx = nullptr;        // X of the tensor-core z pass (reduced-precision forms), per launch group
-  float2* tw[3] = {nullptr, nullptr, nullptr};   // z, y, x
   // rotation matrices: pinned host staging + device copy, grown on demand
-  RotMat* rot_h = nullptr;
-  RotMat* rot_d = nullptr;
+  RotIn* rot_h = nullptr;
+  RotIn* rot_d = nullptr;
   int rot_cap = 0;
   cudaEvent_t rot_ev = nullptr;
   // host-buffer entry point staging
@@ -75,14 +83,7 @@ struct cs_ngf_fixed {
   int32_t* res_shift = nullptr;
   int res_cap = 0;
   size_t fixed_bytes = 0, workspace_bytes = 0;
-  // one captured CUDA graph for a full batch, replayed per batch; the batch's
-  // rotation matrices and results go through fixed slots
-  cudaGraphExec_t gexec = nullptr;
-  RotMat* rot_slot = nullptr;
-  float* slot_score = nullptr;
-  int32_t* slot_shift = nullptr;
-  bool capturing = false;
-  // per-stage CUDA-event timing (cs_ngf_set_profiling); disables graph replay
+  // per-stage CUDA-event timing (cs_ngf_set_profiling)
   bool profiling = false;
   struct Span { int stage; cudaEvent_t a, b; };
   std::vector<Span> spans;
@@ -100,22 +101,26 @@ namespace detail {
 
 // record the calling thread's error detail (cs_ngf_last_error) and return s
 cs_ngf_status fail(cs_ngf_status s, const std::string& msg);
-// host FP64 quaternions -> FP32 matrices in f->rot_d[0..R)
+// host FP64 quaternions -> FP32 matrices in f->rot_h[0..R) and f->rot_d[0..R)
 cs_ngf_status upload_rotations(cs_ngf_fixed* f, const double* quats, int R, cudaStream_t st);
 // (B, M_B) -> f->BQ, f->C8 for the following score calls
 cs_ngf_status pack_floating(cs_ngf_fixed* f, const float* B, const uint8_t* MB, cudaStream_t st);
+// Rotations scored together: FFT lengths, box extents and shift windows per
+// axis (z, y, x), and the end of the class in the call's regrouped order.
+struct ClassGeom { int pad[3], ext[3], win[3], end; };
+struct Plan {
+  std::vector<int> perm;         // original index of the i-th regrouped rotation (empty: unchanged)
+  std::vector<ClassGeom> cls;
+};
 // Bound-limited padding (pad_mode CS_NGF_PAD_BOUND): the R uploaded
 // rotations of the floating volume packed by pack_floating, grouped into
-// classes by the FFT lengths their admitted shifts need.  Synchronises `st`.  perm[i] is the
-// original index of the i-th rotation in class order (empty: order
-// unchanged; otherwise the device matrices are re-uploaded in that order);
-// class c covers [ends[c-1], ends[c]) and uses lengths pads[3c..3c+2].  In
-// other modes: one class with the lengths in use.
-cs_ngf_status plan_classes(cs_ngf_fixed* f, int R, cudaStream_t st,
-                           std::vector<int>& perm, std::vector<int>& ends, std::vector<int>& pads);
-// switch the handle to FFT lengths pad (recomputing the fixed spectra if they
-// change; synchronises `st` then)
-cs_ngf_status set_lengths(cs_ngf_fixed* f, const int pad[3], cudaStream_t st);
+// classes by the FFT lengths their admitted shifts need, their boxes uploaded
+// in class order.  Synchronises `st`.  In full mode: one class with the
+// lengths in use.
+cs_ngf_status plan_classes(cs_ngf_fixed* f, int R, cudaStream_t st, Plan& plan);
+// switch the handle to a class's geometry (recomputing the fixed spectra if
+// the FFT lengths change)
+cs_ngf_status set_class(cs_ngf_fixed* f, const ClassGeom& c, cudaStream_t st);
 // score rotations [r0, r0 + n) of the uploaded set into best_score / best_shift
 // (device, indexed from r0), in launch groups of f->batch
 cs_ngf_status score_range(cs_ngf_fixed* f, int r0, int n, float* best_score, int32_t* best_shift,

@@ -16,10 +16,13 @@
 //   Bh, Mh   [r][z][y][x]                     float / uint8
 //   F0       [r][j][z][y][kx]     j < nf       x transformed
 //   F1       [r][j][kx][z][ky]                  x, y transformed
-//   F2       [r][kx][vz][ky]                    Z = X + iY after the z inverse
-//   F3       [r][vz][vy][kx]                    after the y inverse
+//   F2       [r][kx][dz][ky]                    Z = X + iY after the z inverse
+//   F3       [r][dz][dy][kx]                    after the y inverse
 //   UV       [2nch+1][kx <= Px/2][ky][kz]      fixed-volume weights (prepare)
-// vz, vy, vx index the shift chi = v - (n - 1) in [-(n-1), n-1].
+// z, y of F0 and F1 count from the rotation's box origin (RotBox::org) and run
+// over the class's extents (Geo::ez, ey); dz, dy count from the first shift
+// slot that can be valid (RotBox::lo) over the class's windows (Geo::wz, wy).
+// A shift slot v stands for the shift chi = v - (n - 1) in [-(n-1), n-1].
 //
 // Packed channel pairs (Eq. 2, squared measure): j=0 (xx, yy), j=1 (zz, xy),
 // j=2 (xz, yz), j=3 (mask, 0).  Eq. 3 (unsquared measure): j=0 (x, y),
@@ -37,6 +40,8 @@ struct Geo {
   int nz, ny, nx;       // volume dims
   int Pz, Py, Px;       // FFT lengths per axis
   int vz, vy, vx;       // 2n - 1 shift extents
+  int ez, ey, ex;       // box extents transformed per axis (n: the whole volume)
+  int wz, wy;           // shift slots kept per axis after the inverse (2n - 1: all)
   float eps2;           // eps^2 (Eq. 1)
   long long nvox;       // nz*ny*nx
   int nch;              // packed channel fields: 3 (Eq. 2, squared) or 2 (Eq. 3, unsquared)
@@ -106,6 +111,28 @@ struct Fields {
 // per-rotation matrix (row-major, acts on (x, y, z)), rounded to FP32 on the host
 struct RotMat { float m[9]; };
 
+// What bounds one rotation, per axis (z, y, x).  The masked channels of a
+// rotated volume vanish outside its mask's box, so the forward transforms take
+// the box [org, org + e) only, e the extents of Geo, with the box's origin at
+// transform index 0 (the fixed volume likewise, with its own origin).  Output
+// index m of the circular correlation then stands for the shift slots
+// v = lo + ((m - m0) mod P), m0 the output index of slot lo; the slots in
+// [lo, hi] can be valid (lo > hi: none).  thr: the overlap threshold in FFT
+// units, (max(1, ceil(gamma min(sum M_A, sum M_hat))) - 1/2) Pz Py Px.
+struct RotBox { int lo[3], hi[3], org[3], m0[3]; float thr; };
+struct RotIn { RotMat m; RotBox b; };
+
+// slab counts of a rotated mask reduced per axis: the shift slots [lo, hi] whose
+// slab bound reaches the overlap threshold (lo > hi: none), the first and last
+// slab that holds a mask voxel (b0 > b1: none), and the mask's sum
+struct RotBounds { int lo[3], hi[3], b0[3], b1[3], msum; };
+
+// window index of transform output m (slot lo + it), < P; valid up to hi - lo
+__device__ __forceinline__ int window_index(int m, int m0, int P) {
+  const int d = m - m0;
+  return d < 0 ? d + P : d;
+}
+
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
 // orderable key: larger score -> larger key; equal score -> smaller index wins
@@ -124,31 +151,44 @@ __device__ __forceinline__ unsigned long long make_key(float s, unsigned lin) {
 // C8: nvox entries each).
 __global__ void k_pack_floating(const float* __restrict__ B, const uint8_t* __restrict__ MB, Geo g,
                                 float4* __restrict__ BQ, uint8_t* __restrict__ C8);
+// k_resample: the whole volume, mask counts into msum and marg (marg may be
+// nullptr); grid resample_grid.  k_resample_box: only the voxels the x pass
+// reads, each rotation's box and one voxel around it; grid resample_box_grid.
 __global__ void k_resample(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8,
-                           const RotMat* __restrict__ rot, Geo g, float* __restrict__ Bh,
+                           const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh,
                            uint8_t* __restrict__ Mh, int* __restrict__ msum, int* __restrict__ marg);
+__global__ void k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8,
+                               const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh,
+                               uint8_t* __restrict__ Mh);
 // The rotated masks alone, counted into msum and marg as k_resample counts
 // them (the same decisions from the same corner codes, no volumes written):
 // the pre-pass that bounds the shifts of a whole call.  Grid: resample_grid.
-__global__ void k_mask_counts(const uint8_t* __restrict__ C8, const RotMat* __restrict__ rot, Geo g,
+__global__ void k_mask_counts(const uint8_t* __restrict__ C8, const RotIn* __restrict__ rot, Geo g,
                               int* __restrict__ msum, int* __restrict__ marg);
 constexpr int kResampleZGroups = 8;            // z-plane groups of 4 per resample block
 inline dim3 resample_grid(const Geo& g, int nrot) {
   return dim3((unsigned)((g.nx + 7) / 8), (unsigned)((g.ny + 3) / 4),
               (unsigned)(((g.nz + 4 * kResampleZGroups - 1) / (4 * kResampleZGroups)) * nrot));
 }
+inline dim3 resample_box_grid(const Geo& g, int nrot) {
+  return dim3((unsigned)((g.ex + 2 + 7) / 8), (unsigned)((g.ey + 2 + 3) / 4),
+              (unsigned)(((g.ez + 2 + 4 * kResampleZGroups - 1) / (4 * kResampleZGroups)) * nrot));
+}
 
 // ----------------------------------------------------------------- shift bounds
-// Marginal mask counts per axis, [nz | ny | nx] per volume (marg in k_resample
-// fills them for each rotated mask; k_marginals for the fixed mask).  For a
+// Marginal mask counts per axis, [nz | ny | nx] per volume (k_mask_counts and
+// k_resample fill them for each rotated mask; k_marginals for the fixed mask).  For a
 // shift chi, N(chi) <= sum_i min(a_i, b_{i + chi_axis}) over the slabs of any
 // axis, so shifts whose slab bound is below the Section 3.2 overlap threshold
 // are invalid; k_shift_bounds keeps, per rotation and axis, the range of shift
-// slots that can be valid ([lo, hi] in v = chi + n - 1; lo > hi: none).
+// slots that can be valid and the slabs that hold mask voxels.
 __global__ void k_marginals(const uint8_t* __restrict__ M, Geo g, int* __restrict__ marg);
 __global__ void k_shift_bounds(const int* __restrict__ margA, const int* __restrict__ margB,
                                const int* __restrict__ msumB, int sumA, float gamma, Geo g,
-                               int* __restrict__ bounds);
+                               RotBounds* __restrict__ bounds);
+// full padding: the boxes of a launch group (origin 0) from its bounds
+__global__ void k_full_boxes(const RotBounds* __restrict__ bounds, int sumA, float gamma, Geo g,
+                             double pvol, int nrot, RotIn* __restrict__ rot);
 __global__ void k_fill(float* __restrict__ p, long long n, float v);
 // results scored in a regrouped order back to the caller's: entry i belongs
 // to rotation perm[i]
@@ -159,9 +199,13 @@ __global__ void k_scatter_results(const int* __restrict__ perm, const float* __r
 // sum of a uint8 mask (for the fixed volume)
 __global__ void k_mask_sum(const uint8_t* __restrict__ M, long long n, int* __restrict__ out);
 
-// per-rotation overlap threshold in FFT units: (max(1, ceil(gamma min(sA, sB))) - 0.5) * Pz Py Px
-__global__ void k_thresholds(const int* __restrict__ msumB, int sumA, float gamma, double pvol,
-                             int nrot, float* __restrict__ thr);
+// overlap threshold in FFT units: (max(1, ceil(gamma min(sA, sB))) - 0.5) * Pz Py Px
+__host__ __device__ inline float overlap_threshold(int sumA, int sumB, float gamma, double pvol) {
+  const int mn = sumA < sumB ? sumA : sumB;
+  double t = ceil((double)gamma * (double)mn);
+  if (t < 1.0) t = 1.0;
+  return (float)((t - 0.5) * pvol);
+}
 
 // decode per-rotation keys into (score, shift)
 __global__ void k_finalize(const unsigned long long* __restrict__ keys, int nrot, Geo g,
@@ -175,20 +219,16 @@ __global__ void k_copy_in(const float* __restrict__ A, const uint8_t* __restrict
 // F0 / F1 are laid out by Fields<g.store> (FP32 everywhere when g.store == kStoreF32).
 // v: split variant of the length P (SplitV<P, v>; 0 = the built-in one, 1 =
 // the alternative where P has one, chosen by the autotuner)
-template <int P> void launch_fwd_x(const float* Bh, const uint8_t* Mh, void* F0, const float2* tw,
+// rot: the launch group's rotations (matrices and boxes)
+template <int P> void launch_fwd_x(const float* Bh, const uint8_t* Mh, void* F0, const RotIn* rot,
                                    Geo g, int nrot, cudaStream_t st, int v = 0);
-template <int P> void launch_fwd_y(const void* F0, void* F1, const float2* tw, Geo g, int nrot,
+template <int P> void launch_fwd_y(const void* F0, void* F1, Geo g, int nrot, cudaStream_t st, int v = 0);
+template <int P> void launch_zmac(const void* F1, const float2* UV, float2* F2, Geo g, int nrot,
+                                  const RotIn* rot, cudaStream_t st, int v = 0);
+template <int P> void launch_prep_z(const float2* F1, float2* UV, Geo g, cudaStream_t st);
+template <int P> void launch_inv_y(const float2* F2, float2* F3, Geo g, int nrot, const RotIn* rot,
                                    cudaStream_t st, int v = 0);
-template <int P> void launch_zmac(const void* F1, const float2* UV, float2* F2, const float2* tw,
-                                  Geo g, int nrot, const int* bounds, cudaStream_t st, int v = 0);
-template <int P> void launch_prep_z(const float2* F1, float2* UV, const float2* tw, Geo g,
-                                    cudaStream_t st);
-template <int P> void launch_inv_y(const float2* F2, float2* F3, const float2* tw, Geo g, int nrot,
-                                   const int* bounds, cudaStream_t st, int v = 0);
-template <int P> void launch_inv_x(const float2* F3, const float* thr, unsigned long long* keys,
-                                   float* map, const float2* tw, Geo g, int nrot, const int* bounds,
-                                   cudaStream_t st, int v = 0);
-// bounds: per rotation {lo_z, hi_z, lo_y, hi_y, lo_x, hi_x} shift slots that can
-// be valid, or nullptr for the full range
+template <int P> void launch_inv_x(const float2* F3, unsigned long long* keys, float* map, Geo g, int nrot,
+                                   const RotIn* rot, cudaStream_t st, int v = 0);
 
 }  // namespace csngf

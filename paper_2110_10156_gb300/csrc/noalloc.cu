@@ -6,8 +6,7 @@
 // under a strict device-memory budget.  cs_ngf_score_rotations_noalloc serves
 // them.  It runs the same kernels as cs_ngf_score_rotations, one rotation at a
 // time, but all of its scratch memory (the fixed-volume spectra, the resampled
-// volume, the FFT intermediates, the twiddle tables and the per-rotation
-// result key) lives in one file-scope device array of fixed size, g_scratch.
+// volume, the FFT intermediates and the per-rotation result key) lives in one file-scope device array of fixed size, g_scratch.
 // Every GPU that loads this library holds that array until the process exits.
 #include <cuda_runtime.h>
 
@@ -42,7 +41,6 @@ constexpr size_t kVolBytes = align256((size_t)kNaMaxDim * kNaMaxDim * kNaMaxDim 
 constexpr size_t kMaskBytes = align256((size_t)kNaMaxDim * kNaMaxDim * kNaMaxDim);
 constexpr size_t kBQBytes = align256((size_t)kNaMaxDim * kNaMaxDim * kNaMaxDim * 16);
 constexpr size_t kC8Bytes = align256((size_t)kNaMaxDim * kNaMaxDim * kNaMaxDim);
-constexpr size_t kTwBytes = align256((size_t)3 * kNaMaxPad * 8);
 constexpr size_t kMiscBytes = 256;   // msum[2] (A, B), thr, key, rotation matrix
 
 constexpr size_t kOffUV = 0;
@@ -52,8 +50,7 @@ constexpr size_t kOffBh = kOffF13 + kF13Bytes;
 constexpr size_t kOffMh = kOffBh + kVolBytes;
 constexpr size_t kOffBQ = kOffMh + kMaskBytes;
 constexpr size_t kOffC8 = kOffBQ + kBQBytes;
-constexpr size_t kOffTw = kOffC8 + kC8Bytes;
-constexpr size_t kOffMisc = kOffTw + kTwBytes;
+constexpr size_t kOffMisc = kOffC8 + kC8Bytes;
 constexpr size_t kScratchBytes = kOffMisc + kMiscBytes;
 static_assert(kScratchBytes == (size_t)CS_NGF_NOALLOC_SCRATCH_BYTES, "header states the scratch size");
 
@@ -64,10 +61,8 @@ static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
 struct Misc {
   int msum[2];                 // [0] sum of M_A, [1] sum of the rotated M_B
-  float thr;                   // overlap threshold in FFT units
-  int pad_;
   unsigned long long key;      // best (score, shift) key of the current rotation
-  RotMat rot;                  // the current rotation
+  RotIn rot;                   // the current rotation; its box is the whole volume, every shift
 };
 static_assert(sizeof(Misc) <= kMiscBytes, "misc slice");
 
@@ -88,27 +83,14 @@ cs_ngf_status na_fail(cs_ngf_status s, const std::string& m) {
                                                             cudaGetErrorString(e_));    \
   } while (0)
 
-// FP64 twiddle tables exp(-2 pi i m / P) for the three axes, rounded to FP32
-__global__ void k_na_twiddles(float2* tw, int Pz, int Py, int Px) {
-  const int a = blockIdx.x, m = threadIdx.x;
-  const int P = a == 0 ? Pz : (a == 1 ? Py : Px);
-  if (m >= P) return;
-  double s, c;
-  sincospi(2.0 * (double)m / (double)P, &s, &c);
-  tw[a * kNaMaxPad + m] = make_float2((float)c, (float)(-s));
-}
-
-__global__ void k_na_set_rot(RotMat m, Misc* misc) {
-  misc->rot = m;
+__global__ void k_na_set_rot(RotIn in, Misc* misc) {
+  misc->rot = in;
   misc->msum[1] = 0;
   misc->key = 0ull;
 }
 
 __global__ void k_na_threshold(Misc* misc, float gamma, double pvol) {
-  const int mn = min(misc->msum[0], misc->msum[1]);
-  double t = ceil((double)gamma * (double)mn);
-  if (t < 1.0) t = 1.0;
-  misc->thr = (float)((t - 0.5) * pvol);
+  misc->rot.b.thr = overlap_threshold(misc->msum[0], misc->msum[1], gamma, pvol);
 }
 
 void quat_matrix(const double* q, double* R) {
@@ -225,6 +207,8 @@ extern "C" cs_ngf_status cs_ngf_score_rotations_noalloc(
   g.nz = dims[0]; g.ny = dims[1]; g.nx = dims[2];
   g.Pz = na_pad(g.nz); g.Py = na_pad(g.ny); g.Px = na_pad(g.nx);
   g.vz = 2 * g.nz - 1; g.vy = 2 * g.ny - 1; g.vx = 2 * g.nx - 1;
+  g.ez = g.nz; g.ey = g.ny; g.ex = g.nx;
+  g.wz = g.vz; g.wy = g.vy;
   g.eps2 = eps * eps;
   g.nvox = (long long)g.nz * g.ny * g.nx;
   g.nch = 3;                         // Eq. 2 (squared) measure
@@ -239,24 +223,18 @@ extern "C" cs_ngf_status cs_ngf_score_rotations_noalloc(
   uint8_t* Mh = (uint8_t*)(base + kOffMh);
   float4* BQ = (float4*)(base + kOffBQ);
   uint8_t* C8 = (uint8_t*)(base + kOffC8);
-  float2* tw = (float2*)(base + kOffTw);
   Misc* misc = (Misc*)(base + kOffMisc);
   cudaStream_t st = (cudaStream_t)stream;
 
-  // fixed volume: twiddles, mask sum, forward transforms, weights (all in scratch)
-  k_na_twiddles<<<3, kNaMaxPad, 0, st>>>(tw, g.Pz, g.Py, g.Px);
-  if (cs_ngf_status s = na_launched("twiddles")) return s;
-  const float2* twz = tw;
-  const float2* twy = tw + kNaMaxPad;
-  const float2* twx = tw + 2 * kNaMaxPad;
+  // fixed volume: mask sum, forward transforms, weights (all in scratch)
   NA_CUDA(cudaMemsetAsync(misc, 0, sizeof(Misc), st));
   k_copy_in<<<64, 256, 0, st>>>(A, maskA, g.nvox, Bh, Mh);
   if (cs_ngf_status s = na_launched("copy_in")) return s;
   k_mask_sum<<<64, 256, 0, st>>>(Mh, g.nvox, &misc->msum[0]);
   if (cs_ngf_status s = na_launched("mask_sum")) return s;
-  NA_DISPATCH(g.Px, launch_fwd_x<PP>(Bh, Mh, F02, twx, g, 1, st));
-  NA_DISPATCH(g.Py, launch_fwd_y<PP>(F02, F13, twy, g, 1, st));
-  NA_DISPATCH(g.Pz, launch_prep_z<PP>(F13, UV, twz, g, st));
+  NA_DISPATCH(g.Px, launch_fwd_x<PP>(Bh, Mh, F02, &misc->rot, g, 1, st));
+  NA_DISPATCH(g.Py, launch_fwd_y<PP>(F02, F13, g, 1, st));
+  NA_DISPATCH(g.Pz, launch_prep_z<PP>(F13, UV, g, st));
   if (cs_ngf_status s = na_launched("fixed transforms")) return s;
 
   k_pack_floating<<<64, 256, 0, st>>>(B, maskB, g, BQ, C8);
@@ -265,16 +243,21 @@ extern "C" cs_ngf_status cs_ngf_score_rotations_noalloc(
   for (int r = 0; r < R; ++r) {
     double Rm[9];
     quat_matrix(quats + 4 * r, Rm);
-    RotMat m;
-    for (int i = 0; i < 9; ++i) m.m[i] = (float)Rm[i];
-    k_na_set_rot<<<1, 1, 0, st>>>(m, misc);                 // also zeroes the sum and key
+    RotIn in{};
+    for (int i = 0; i < 9; ++i) in.m.m[i] = (float)Rm[i];
+    const int n[3] = {g.nz, g.ny, g.nx}, P[3] = {g.Pz, g.Py, g.Px};
+    for (int a = 0; a < 3; ++a) {
+      in.b.hi[a] = 2 * n[a] - 2;
+      in.b.m0[a] = P[a] - (n[a] - 1);
+    }
+    k_na_set_rot<<<1, 1, 0, st>>>(in, misc);                 // also zeroes the sum and key
     k_resample<<<resample_grid(g, 1), 128, 0, st>>>(BQ, C8, &misc->rot, g, Bh, Mh, &misc->msum[1], nullptr);
     k_na_threshold<<<1, 1, 0, st>>>(misc, gamma, pvol);
-    NA_DISPATCH(g.Px, launch_fwd_x<PP>(Bh, Mh, F02, twx, g, 1, st));
-    NA_DISPATCH(g.Py, launch_fwd_y<PP>(F02, F13, twy, g, 1, st));
-    NA_DISPATCH(g.Pz, launch_zmac<PP>(F13, UV, F02, twz, g, 1, nullptr, st));
-    NA_DISPATCH(g.Py, launch_inv_y<PP>(F02, F13, twy, g, 1, nullptr, st));
-    NA_DISPATCH(g.Px, launch_inv_x<PP>(F13, &misc->thr, &misc->key, nullptr, twx, g, 1, nullptr, st));
+    NA_DISPATCH(g.Px, launch_fwd_x<PP>(Bh, Mh, F02, &misc->rot, g, 1, st));
+    NA_DISPATCH(g.Py, launch_fwd_y<PP>(F02, F13, g, 1, st));
+    NA_DISPATCH(g.Pz, launch_zmac<PP>(F13, UV, F02, g, 1, &misc->rot, st));
+    NA_DISPATCH(g.Py, launch_inv_y<PP>(F02, F13, g, 1, &misc->rot, st));
+    NA_DISPATCH(g.Px, launch_inv_x<PP>(F13, &misc->key, nullptr, g, 1, &misc->rot, st));
     k_finalize<<<1, 32, 0, st>>>(&misc->key, 1, g, best_score + r, best_shift + 3 * (size_t)r);
     if (cs_ngf_status s = na_launched("rotation")) return s;
   }

@@ -6,23 +6,17 @@
 
 namespace csngf {
 
-// Output index m of a length-P circular correlation -> the shift slot
-// v = chi + n - 1 in [lo, hi] with chi = m or chi = m - P, or -1 if neither
-// lies there.  Slot m sums the linear correlation at every chi = m (mod P);
-// it equals the value at the one chi in [lo, hi] when every other chi of that
-// class lies outside the linear support [-(n-1), n-1], which the caller
-// guarantees by P >= n + max(n-1-lo, hi-(n-1)) (with lo = 0, hi = 2n-2 that
-// is the full linear-correlation length P >= 2n-1).
-__device__ __forceinline__ int shift_slot(int m, int n, int P, int lo, int hi) {
-  const int v1 = m + n - 1;                      // chi = m
-  if (m <= n - 1 && v1 >= lo && v1 <= hi) return v1;
-  const int v2 = m - P + n - 1;                  // chi = m - P
-  if (v2 >= 0 && v2 >= lo && v2 <= hi) return v2;
-  return -1;
-}
+// Output index m of a length-P circular correlation sums the linear
+// correlation over every shift of its residue class mod P.  With the fixed
+// mask on slabs [a0, a1] and the rotated one on [b0, b1] the linear
+// correlation lives on chi in [b0 - a1, b1 - a0], so a slot in the admitted
+// range [lo, hi] holds its one shift whenever
+// P >= max(b1 - a0 - chi_lo, chi_hi - (b0 - a1)) + 1, which the caller
+// guarantees (for masks that fill the volume that is n + max(-chi_lo, chi_hi),
+// and for every shift 2n - 1).
 
-// Forward-transform inputs: a volume side n is zero padded to P.  When
-// n <= P/2 the upper half of every step-1 sequence is zero and step 1 is the
+// Forward-transform inputs: box extents e are zero padded to P.  When
+// e <= P/2 the upper half of every step-1 sequence is zero and step 1 is the
 // pruned form (FourStep::step1_half); otherwise all N1 inputs are read.
 template <class FS, bool HALF>
 struct FwdIn {
@@ -88,7 +82,8 @@ struct FwdXCfg {
 template <int P, int ROWS, int ST, bool HALF, int V>
 __global__ void __launch_bounds__(ROWS * SplitV<P, V>::N2, FwdXCfg<P, HALF, V>::MIN_BLOCKS)
 k_fwd_x(const float* __restrict__ Bh, const uint8_t* __restrict__ Mh, void* __restrict__ F0,
-        const float2* __restrict__ tw, Geo g, long long nrows) {
+        const RotIn* __restrict__ rot, Geo g, long long nrows) {
+  const float2* __restrict__ tw = kTw<P>.w;
   using FS = FourStep<P, true, V>;
   using FI = FwdIn<FS, HALF>;
   constexpr int N1 = FS::N1, N2 = FS::N2, CS = FS::CS, H = FI::NI;
@@ -97,11 +92,13 @@ k_fwd_x(const float* __restrict__ Bh, const uint8_t* __restrict__ Mh, void* __re
   const int lrow = t / N2, n2 = t - lrow * N2;
   const long long grow = (long long)blockIdx.x * ROWS + lrow;
   const bool row_ok = grow < nrows;
-  const long long rz = row_ok ? grow / g.ny : 0;
-  const int y = row_ok ? (int)(grow - rz * g.ny) : 0;
-  const int r = (int)(rz / g.nz), z = (int)(rz - (long long)r * g.nz);
+  const long long rz = row_ok ? grow / g.ey : 0;
+  const int yb = row_ok ? (int)(grow - rz * g.ey) : 0;
+  const int r = (int)(rz / g.ez), zb = (int)(rz - (long long)r * g.ez);
+  const RotBox& bx = rot[r].b;
+  const int z = zb + bx.org[0], y = yb + bx.org[1], ox = bx.org[2];   // voxel of box index (zb, yb, 0)
 
-  // x = N2*n1 + n2 < nx: with nx <= P/2 only n1 < N1/2 can hold data
+  // x = org + N2*n1 + n2 over ex voxels: with ex <= P/2 only n1 < N1/2 can hold data
   constexpr bool NS = !HALF;                  // NGF staged in shared memory
   constexpr int HR = NS ? 1 : H;
   float vx[HR], vy[HR], vz[HR], mm[HR];
@@ -113,17 +110,30 @@ k_fwd_x(const float* __restrict__ Bh, const uint8_t* __restrict__ Mh, void* __re
   const int ym = max(y - 1, 0), yp = min(y + 1, g.ny - 1);
   const int zm = max(z - 1, 0), zp = min(z + 1, g.nz - 1);
   const long long base = (long long)z * sz + (long long)y * sy;
-  const long long rows_per_field = (long long)g.nz * g.ny;
+  const long long rows_per_field = (long long)g.ez * g.ey;
   const int nrot = (int)(nrows / rows_per_field);
   const bool has_partner = !(r & 1) && r + 1 < nrot;
+  // the partner's mask in its own box: offset of its row from M, and its x origin
+  long long pbase = 0;
+  int pox = 0, pnx = 0;
+  if (has_partner) {
+    const RotBox& pb = rot[r + 1].b;
+    const int pz = zb + pb.org[0], py = yb + pb.org[1];
+    pox = pb.org[2];
+    pnx = (pz < g.nz && py < g.ny) ? min(g.ex, g.nx - pox) : 0;
+    pbase = g.nvox + (long long)pz * sz + (long long)py * sy + pox;
+  }
+  const bool in_vol = row_ok && z < g.nz && y < g.ny;
   // per element: the NGF times the mask (m^2 = m, so every Eq. 6 product of
   // two masked components equals the product times m, bit for bit) and the
   // mask pair of the mask field coded as m + 2 m2 (m2: the next rotation's mask)
 #pragma unroll
   for (int n1 = 0; n1 < H; ++n1) {
-    const int x = N2 * n1 + n2;
+    const int xb = N2 * n1 + n2, x = xb + ox;
     float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (row_ok && x < g.nx) {
+    const float m2 = xb < pnx && M[pbase + xb] ? 2.0f : 0.0f;
+    q.w = m2;
+    if (in_vol && xb < g.ex && x < g.nx) {
       const int xm = max(x - 1, 0), xp = min(x + 1, g.nx - 1);
       const float gx = 0.5f * (__ldg(&Vol[base + xp]) - __ldg(&Vol[base + xm]));
       const float gy = 0.5f * (__ldg(&Vol[(long long)z * sz + (long long)yp * sy + x]) -
@@ -132,7 +142,6 @@ k_fwd_x(const float* __restrict__ Bh, const uint8_t* __restrict__ Mh, void* __re
                                __ldg(&Vol[(long long)zm * sz + (long long)y * sy + x]));
       const float inv = rsqrtf(gx * gx + gy * gy + gz * gz + g.eps2);
       const float m = M[base + x] ? 1.0f : 0.0f;
-      const float m2 = (has_partner && M[g.nvox + base + x]) ? 2.0f : 0.0f;
       q = make_float4(m * (gx * inv), m * (gy * inv), m * (gz * inv), m + m2);
     }
     if constexpr (NS) {
@@ -197,11 +206,11 @@ k_fwd_x(const float* __restrict__ Bh, const uint8_t* __restrict__ Mh, void* __re
       if (gr < nrows && !skip_row) {
         float2 u[N2];
         FS::template step2<-1>(u, ex + lr * CS, k1);
-        const long long rz2 = gr / g.ny;
-        const int y2 = (int)(gr - rz2 * g.ny);
-        const int r2 = (int)(rz2 / g.nz), z2 = (int)(rz2 - (long long)r2 * g.nz);
+        const long long rz2 = gr / g.ey;
+        const int y2 = (int)(gr - rz2 * g.ey);
+        const int r2 = (int)(rz2 / g.ez), z2 = (int)(rz2 - (long long)r2 * g.ez);
         char* fld = Fields<ST>::field(F0, g, rows_per_field * P, r2, j);
-        const long long row = ((long long)z2 * g.ny + y2) * P;
+        const long long row = ((long long)z2 * g.ey + y2) * P;
         const float sc = field_scale(g.scale0, j);
         if (j == g.nch) {
 #pragma unroll
@@ -217,32 +226,32 @@ k_fwd_x(const float* __restrict__ Bh, const uint8_t* __restrict__ Mh, void* __re
 }
 
 template <int P, bool HALF, int V>
-void launch_fwd_x_t(const float* Bh, const uint8_t* Mh, void* F0, const float2* tw, Geo g, int nrot,
+void launch_fwd_x_t(const float* Bh, const uint8_t* Mh, void* F0, const RotIn* rot, Geo g, int nrot,
                     cudaStream_t st) {
   constexpr int N2 = SplitV<P, V>::N2;
   constexpr int ROWS = FwdXCfg<P, HALF, V>::ROWS;
-  const long long nrows = (long long)nrot * g.nz * g.ny;
+  const long long nrows = (long long)nrot * g.ez * g.ey;
   const size_t smem = FwdXCfg<P, HALF, V>::smem_bytes;
   const unsigned blocks = (unsigned)((nrows + ROWS - 1) / ROWS);
   auto go = [&](auto kern) {
     set_smem(kern, smem);
-    kern<<<blocks, ROWS * N2, smem, st>>>(Bh, Mh, F0, tw, g, nrows);
+    kern<<<blocks, ROWS * N2, smem, st>>>(Bh, Mh, F0, rot, g, nrows);
   };
   by_store(g.store, [&](auto st) { go(k_fwd_x<P, ROWS, decltype(st)::value, HALF, V>); });
 }
 
 template <int P>
-void launch_fwd_x(const float* Bh, const uint8_t* Mh, void* F0, const float2* tw, Geo g, int nrot,
+void launch_fwd_x(const float* Bh, const uint8_t* Mh, void* F0, const RotIn* rot, Geo g, int nrot,
                   cudaStream_t st, int v) {
   by_split<P>(v, [&](auto vc) {
     constexpr int V = decltype(vc)::value;
-    if (2 * g.nx <= P) launch_fwd_x_t<P, true, V>(Bh, Mh, F0, tw, g, nrot, st);
-    else launch_fwd_x_t<P, false, V>(Bh, Mh, F0, tw, g, nrot, st);
+    if (2 * g.ex <= P) launch_fwd_x_t<P, true, V>(Bh, Mh, F0, rot, g, nrot, st);
+    else launch_fwd_x_t<P, false, V>(Bh, Mh, F0, rot, g, nrot, st);
   });
 }
 
 // ---------------------------------------------------------------------------
-// fwd_y: y-axis FFT of every column of F0 (rows y >= ny are zero); the output
+// fwd_y: y-axis FFT of every column of F0 (rows y >= ey are zero); the output
 // is transposed so that ky is contiguous for the z pass.
 // Block: W consecutive kx of one (r, j, z) plane.
 // ---------------------------------------------------------------------------
@@ -270,8 +279,8 @@ template <int P, int V> struct FwdYCfg {
 
 template <int P, int W, int ST, bool HALF, int V>
 __global__ void __launch_bounds__(W * SplitV<P, V>::N2, FwdYCfg<P, V>::MIN_BLOCKS)
-k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, const float2* __restrict__ tw,
-        Geo g) {
+k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, Geo g) {
+  const float2* __restrict__ tw = kTw<P>.w;
   using FS = FourStep<P, true, V>;
   using FI = FwdIn<FS, HALF>;
   constexpr int N1 = FS::N1, N2 = FS::N2, CS = FS::CS;
@@ -279,9 +288,9 @@ k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, const float2* __rest
   const int t = threadIdx.x;
   // kx tiles run fastest over the grid, so the blocks that read the two halves
   // of a 128-byte line of F0 run together and the second one hits in L2
-  const long long plane = blockIdx.y;                // ((r * nf) + j) * nz + z
-  const long long rj = plane / g.nz;
-  const int z = (int)(plane - rj * g.nz);
+  const long long plane = blockIdx.y;                // ((r * nf) + j) * ez + z
+  const long long rj = plane / g.ez;
+  const int z = (int)(plane - rj * g.ez);
   const int r = (int)(rj / g.nf), j = (int)(rj - (long long)r * g.nf);
   const bool is_mask = j == g.nch;
   if (is_mask && (r & 1)) return;                    // paired into the even rotation's mask field
@@ -289,22 +298,22 @@ k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, const float2* __rest
   {
     const int col = t % W, n2 = t / W;
     const int kx = kx0 + col;
-    const char* src = Fields<ST>::field(F0, g, (long long)g.nz * g.ny * g.Px, r, j);
+    const char* src = Fields<ST>::field(F0, g, (long long)g.ez * g.ey * g.Px, r, j);
     const float isc = 1.0f / field_scale(g.scale0, j);
-    const long long zoff = (long long)z * g.ny * g.Px;
-    float2 v[FI::NI];                     // y < ny: with ny <= P/2 the upper half is zero
+    const long long zoff = (long long)z * g.ey * g.Px;
+    float2 v[FI::NI];                     // y < ey: with ey <= P/2 the upper half is zero
     if (is_mask) {
 #pragma unroll
       for (int n1 = 0; n1 < FI::NI; ++n1) {
         const int y = N2 * n1 + n2;
-        v[n1] = (y < g.ny && kx < g.Px) ? Fields<ST>::get(src, zoff + (long long)y * g.Px + kx, true, isc)
+        v[n1] = (y < g.ey && kx < g.Px) ? Fields<ST>::get(src, zoff + (long long)y * g.Px + kx, true, isc)
                                         : make_float2(0.f, 0.f);
       }
     } else {
 #pragma unroll
       for (int n1 = 0; n1 < FI::NI; ++n1) {
         const int y = N2 * n1 + n2;
-        v[n1] = (y < g.ny && kx < g.Px) ? Fields<ST>::get(src, zoff + (long long)y * g.Px + kx, false, isc)
+        v[n1] = (y < g.ey && kx < g.Px) ? Fields<ST>::get(src, zoff + (long long)y * g.Px + kx, false, isc)
                                         : make_float2(0.f, 0.f);
       }
     }
@@ -317,8 +326,8 @@ k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, const float2* __rest
     if (kx < g.Px) {
       float2 u[N2];
       FS::template step2<-1>(u, ex + col * CS, k1);
-      char* dst = Fields<ST>::field(F1, g, (long long)g.nz * g.Px * P, r, j);
-      const long long row = ((long long)kx * g.nz + z) * P;       // [kx][z][ky]
+      char* dst = Fields<ST>::field(F1, g, (long long)g.ez * g.Px * P, r, j);
+      const long long row = ((long long)kx * g.ez + z) * P;       // [kx][z][ky]
       const float sc = field_scale(g.scale1, j);
       if (is_mask) {
 #pragma unroll
@@ -332,15 +341,15 @@ k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, const float2* __rest
 }
 
 template <int P, int V>
-void launch_fwd_y_t(const void* F0, void* F1, const float2* tw, Geo g, int nrot, cudaStream_t st) {
+void launch_fwd_y_t(const void* F0, void* F1, Geo g, int nrot, cudaStream_t st) {
   constexpr int W = FwdYCfg<P, V>::W, N2 = SplitV<P, V>::N2;
   const size_t smem = FwdYCfg<P, V>::smem_bytes;
-  dim3 grid((unsigned)((g.Px + W - 1) / W), (unsigned)(nrot * g.nf * g.nz));   // y: at most 32 * 4 * 256
+  dim3 grid((unsigned)((g.Px + W - 1) / W), (unsigned)(nrot * g.nf * g.ez));   // y: at most 32 * 4 * 256
   auto go = [&](auto kern) {
     set_smem(kern, smem);
-    kern<<<grid, W * N2, smem, st>>>(F0, F1, tw, g);
+    kern<<<grid, W * N2, smem, st>>>(F0, F1, g);
   };
-  const bool half = 2 * g.ny <= P;
+  const bool half = 2 * g.ey <= P;
   by_store(g.store, [&](auto sf) {
     constexpr int ST = decltype(sf)::value;
     half ? go(k_fwd_y<P, W, ST, true, V>) : go(k_fwd_y<P, W, ST, false, V>);
@@ -348,8 +357,8 @@ void launch_fwd_y_t(const void* F0, void* F1, const float2* tw, Geo g, int nrot,
 }
 
 template <int P>
-void launch_fwd_y(const void* F0, void* F1, const float2* tw, Geo g, int nrot, cudaStream_t st, int v) {
-  by_split<P>(v, [&](auto vc) { launch_fwd_y_t<P, decltype(vc)::value>(F0, F1, tw, g, nrot, st); });
+void launch_fwd_y(const void* F0, void* F1, Geo g, int nrot, cudaStream_t st, int v) {
+  by_split<P>(v, [&](auto vc) { launch_fwd_y_t<P, decltype(vc)::value>(F0, F1, g, nrot, st); });
 }
 
 // ---------------------------------------------------------------------------
@@ -411,7 +420,8 @@ struct ZmacCfg {
 template <int P, int ST, bool HALF, int V>
 __global__ void __launch_bounds__(ZmacCfg<P, HALF, V>::NT, ZmacCfg<P, HALF, V>::MIN_BLOCKS)
 k_zmac(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __restrict__ F2,
-       const float2* __restrict__ tw, Geo g, int nrot, const int* __restrict__ bounds) {
+       Geo g, int nrot, const RotIn* __restrict__ rot) {
+  const float2* __restrict__ tw = kTw<P>.w;
   using C = ZmacCfg<P, HALF, V>;
   using FS = typename C::FS;
   using FI = FwdIn<FS, HALF>;
@@ -443,37 +453,37 @@ k_zmac(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __res
   const bool ok1 = pk1 < g.Py;
   const int ky1 = c1 < W ? pk1 : (g.Py - pk1) % g.Py;
   const int kx1 = c1 < W ? kx : mkx;
-  const long long col_off = (long long)kx1 * g.nz * g.Py + ky1;   // F1 is [r][j][kx][z][ky]
+  const long long col_off = (long long)kx1 * g.ez * g.Py + ky1;   // F1 is [r][j][kx][z][ky]
   // step-2 role: column c2 (fastest), k1
   const bool has2 = t < NC * N1;
   const int c2 = t % NC, k1 = t / NC;
 
-  // z = N2*n1 + n2 < nz (with nz <= P/2 only n1 < N1/2).  Field inputs are copied
+  // z = N2*n1 + n2 < ez (with ez <= P/2 only n1 < N1/2).  Field inputs are copied
   // asynchronously (cp.async) two fields ahead into this thread's own slots of
   // two stages: no registers are held meanwhile.  Slots outside the volume are
   // zero once and never copied to.  Fields run in the order (r, j), j < nfr(r).
 #pragma unroll
   for (int n1 = 0; n1 < H; ++n1) {
     const int z = N2 * n1 + n2;
-    if (!(ok1 && z < g.nz)) stage[n1 * NT + t] = stage[(H + n1) * NT + t] = make_float2(0.f, 0.f);
+    if (!(ok1 && z < g.ez)) stage[n1 * NT + t] = stage[(H + n1) * NT + t] = make_float2(0.f, 0.f);
   }
   auto nfr = [&](int r) { return (r & 1) ? g.nch : g.nf; };  // an odd rotation's mask came with its partner
   int pr = 0, pj = 0;                         // next field to copy
   auto fetch = [&](float2* buf) {             // copies field (pr, pj), if any, and advances
     if (pr < nrot) {
-      const char* src = Fields<ST>::field(F1, g, g.nz * plane_stride, pr, pj);
+      const char* src = Fields<ST>::field(F1, g, g.ez * plane_stride, pr, pj);
       if (ST == kStoreF32 || pj == g.nch) {
 #pragma unroll
         for (int n1 = 0; n1 < H; ++n1) {
           const int z = N2 * n1 + n2;
-          if (ok1 && z < g.nz)
+          if (ok1 && z < g.ez)
             cp_async8(buf + n1 * NT + t, src + (col_off + (long long)z * g.Py) * 8);
         }
       } else {
 #pragma unroll
         for (int n1 = 0; n1 < H; ++n1) {
           const int z = N2 * n1 + n2;
-          if (ok1 && z < g.nz)
+          if (ok1 && z < g.ez)
             cp_async4(buf + n1 * NT + t, src + (col_off + (long long)z * g.Py) * 4);
         }
       }
@@ -652,12 +662,12 @@ k_zmac(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __res
         const int kx2 = c2 < W ? kx : mkx;
         float2 u[N2];
         FS::template step2<1>(u, ex + c2 * CS, k1);
-        float2* dst = F2 + ((long long)r * g.Px + kx2) * g.vz * g.Py + ky2;   // [r][kx][vz][ky]
-        const int lo = bounds ? bounds[6 * r] : 0, hi = bounds ? bounds[6 * r + 1] : g.vz - 1;
+        float2* dst = F2 + ((long long)r * g.Px + kx2) * g.wz * g.Py + ky2;   // [r][kx][dz][ky]
+        const int m0 = rot[r].b.m0[0], last = rot[r].b.hi[0] - rot[r].b.lo[0];
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) {
-          const int vz = shift_slot(k1 + N1 * k2, g.nz, P, lo, hi);
-          if (vz >= 0) dst[(long long)vz * g.Py] = u[k2];
+          const int dz = window_index(k1 + N1 * k2, m0, P);
+          if (dz <= last) dst[(long long)dz * g.Py] = u[k2];
         }
       }
     }
@@ -666,14 +676,14 @@ k_zmac(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __res
 }
 
 template <int P, bool HALF, int V>
-void launch_zmac_t(const void* F1, const float2* UV, float2* F2, const float2* tw, Geo g, int nrot,
-                   const int* bounds, cudaStream_t st) {
+void launch_zmac_t(const void* F1, const float2* UV, float2* F2, Geo g, int nrot, const RotIn* rot,
+                   cudaStream_t st) {
   using C = ZmacCfg<P, HALF, V>;
   dim3 grid((unsigned)((g.Py + C::W - 1) / C::W), (unsigned)(g.Px / 2 + 1));
   by_store(g.store, [&](auto sf) {
     constexpr int ST = decltype(sf)::value;
     set_smem(k_zmac<P, ST, HALF, V>, C::smem_bytes);
-    k_zmac<P, ST, HALF, V><<<grid, C::NT, C::smem_bytes, st>>>(F1, UV, F2, tw, g, nrot, bounds);
+    k_zmac<P, ST, HALF, V><<<grid, C::NT, C::smem_bytes, st>>>(F1, UV, F2, g, nrot, rot);
   });
 }
 
@@ -684,22 +694,22 @@ void launch_zmac_t(const void* F1, const float2* UV, float2* F2, const float2* t
 namespace csngf {
 
 template <int P>
-void launch_zmac(const void* F1, const float2* UV, float2* F2, const float2* tw, Geo g, int nrot,
-                 const int* bounds, cudaStream_t st, int v) {
+void launch_zmac(const void* F1, const float2* UV, float2* F2, Geo g, int nrot, const RotIn* rot,
+                 cudaStream_t st, int v) {
   by_split<P>(v, [&](auto vc) {
     constexpr int V = decltype(vc)::value;
-    const bool half = 2 * g.nz <= P;
+    const bool half = 2 * g.ez <= P;
     if (g.tc && g.store != kStoreF32) {          // reduced-precision forms: tensor-core z DFT
       bool done = false;
       by_store(g.store, [&](auto sf) {
         constexpr int ST = decltype(sf)::value;
-        done = half ? launch_zsplit_t<P, ST, true, V>(F1, UV, F2, tw, g, nrot, bounds, st)
-                    : launch_zsplit_t<P, ST, false, V>(F1, UV, F2, tw, g, nrot, bounds, st);
+        done = half ? launch_zsplit_t<P, ST, true, V>(F1, UV, F2, g, nrot, rot, st)
+                    : launch_zsplit_t<P, ST, false, V>(F1, UV, F2, g, nrot, rot, st);
       });
       if (done) return;
     }
-    if (half) launch_zmac_t<P, true, V>(F1, UV, F2, tw, g, nrot, bounds, st);
-    else launch_zmac_t<P, false, V>(F1, UV, F2, tw, g, nrot, bounds, st);
+    if (half) launch_zmac_t<P, true, V>(F1, UV, F2, g, nrot, rot, st);
+    else launch_zmac_t<P, false, V>(F1, UV, F2, g, nrot, rot, st);
   });
 }
 
@@ -712,8 +722,8 @@ void launch_zmac(const void* F1, const float2* UV, float2* F2, const float2* tw,
 // ---------------------------------------------------------------------------
 template <int P, int W, bool HALF>
 __global__ void __launch_bounds__(2 * W * Split<P>::N2)
-k_prep_z(const float2* __restrict__ F1, float2* __restrict__ UV, const float2* __restrict__ tw,
-         Geo g) {
+k_prep_z(const float2* __restrict__ F1, float2* __restrict__ UV, Geo g) {
+  const float2* __restrict__ tw = kTw<P>.w;
   using FS = FourStep<P>;
   using FI = FwdIn<FS, HALF>;
   constexpr int N1 = FS::N1, N2 = FS::N2, CS = FS::CS;
@@ -738,12 +748,12 @@ k_prep_z(const float2* __restrict__ F1, float2* __restrict__ UV, const float2* _
     float wa = 1.f, wb = 1.f;
     if (g.nch == 3) { wa = j == 2 ? 2.f : 1.f; wb = j == 0 ? 1.f : 2.f; }
     else { wb = j == 0 ? 1.f : 0.f; }
-    const float2* src = F1 + (long long)j * g.nz * plane_stride;   // [j][kx][z][ky]
-    float2 v[FI::NI];                     // z < nz: with nz <= P/2 the upper half is zero
+    const float2* src = F1 + (long long)j * g.ez * plane_stride;   // [j][kx][z][ky]
+    float2 v[FI::NI];                     // z < ez: with ez <= P/2 the upper half is zero
 #pragma unroll
     for (int n1 = 0; n1 < FI::NI; ++n1) {
       const int z = N2 * n1 + n2;
-      v[n1] = (ok1 && z < g.nz) ? src[((long long)kx1 * g.nz + z) * g.Py + ky1]
+      v[n1] = (ok1 && z < g.ez) ? src[((long long)kx1 * g.ez + z) * g.Py + ky1]
                                 : make_float2(0.f, 0.f);
     }
     FI::template step1<-1>(v, ex + c1 * CS, n2, tw);
@@ -787,44 +797,41 @@ k_prep_z(const float2* __restrict__ F1, float2* __restrict__ UV, const float2* _
 }
 
 template <int P>
-void launch_prep_z(const float2* F1, float2* UV, const float2* tw, Geo g, cudaStream_t st) {
+void launch_prep_z(const float2* F1, float2* UV, Geo g, cudaStream_t st) {
   constexpr int W = 8, N2 = Split<P>::N2;
   const size_t smem = (size_t)2 * W * FourStep<P>::CS * sizeof(float2);
   dim3 grid((unsigned)((g.Py + W - 1) / W), (unsigned)(g.Px / 2 + 1));
   auto go = [&](auto kern) {
     set_smem(kern, smem);
-    kern<<<grid, 2 * W * N2, smem, st>>>(F1, UV, tw, g);
+    kern<<<grid, 2 * W * N2, smem, st>>>(F1, UV, g);
   };
-  if (2 * g.nz <= P) go(k_prep_z<P, W, true>);
+  if (2 * g.ez <= P) go(k_prep_z<P, W, true>);
   else go(k_prep_z<P, W, false>);
 }
 
 // ---------------------------------------------------------------------------
-// inv_y: y-axis inverse FFT of every (vz, kx) row of F2, keeping 2ny-1 shift
-// rows, transposed so kx is contiguous.  Block: W consecutive kx rows.
+// inv_y: y-axis inverse FFT of every (dz, kx) row of F2, keeping the window's
+// shift rows, transposed so kx is contiguous.  Block: W consecutive kx rows.
 // ---------------------------------------------------------------------------
 template <int P, int W, int V>
 __global__ void __launch_bounds__(W * SplitV<P, V>::N2)
-k_inv_y(const float2* __restrict__ F2, float2* __restrict__ F3, const float2* __restrict__ tw,
-        Geo g, const int* __restrict__ bounds) {
+k_inv_y(const float2* __restrict__ F2, float2* __restrict__ F3, Geo g, const RotIn* __restrict__ rot) {
+  const float2* __restrict__ tw = kTw<P>.w;
   using FS = FourStep<P, true, V>;
   constexpr int N1 = FS::N1, N2 = FS::N2, CS = FS::CS;
   extern __shared__ float2 ex[];
   const int t = threadIdx.x;
-  const long long plane = blockIdx.x;               // r * vz + vz_i
+  const long long plane = blockIdx.x;               // r * wz + dz
   const int kx0 = blockIdx.y * W;
-  const int r = (int)(plane / g.vz), vzi = (int)(plane - (long long)r * g.vz);
-  int lo_y = 0, hi_y = g.vy - 1;
-  if (bounds) {                                      // planes outside the shift bound: nothing to do
-    if (vzi < bounds[6 * r] || vzi > bounds[6 * r + 1]) return;
-    lo_y = bounds[6 * r + 2];
-    hi_y = bounds[6 * r + 3];
-  }
+  const int r = (int)(plane / g.wz), dz = (int)(plane - (long long)r * g.wz);
+  const RotBox& b = rot[r].b;
+  if (dz > b.hi[0] - b.lo[0]) return;                // past this rotation's window
+  const int m0 = b.m0[1], last = b.hi[1] - b.lo[1];
   {
     const int row = t / N2, n2 = t - row * N2;
     const int kx = kx0 + row;
     float2 v[N1];
-    const float2* src = F2 + (((long long)r * g.Px + kx) * g.vz + vzi) * (long long)P;   // [r][kx][vz][ky]
+    const float2* src = F2 + (((long long)r * g.Px + kx) * g.wz + dz) * (long long)P;   // [r][kx][dz][ky]
 #pragma unroll
     for (int n1 = 0; n1 < N1; ++n1)
       v[n1] = (kx < g.Px) ? src[N2 * n1 + n2] : make_float2(0.f, 0.f);
@@ -837,86 +844,84 @@ k_inv_y(const float2* __restrict__ F2, float2* __restrict__ F3, const float2* __
     if (kx < g.Px) {
       float2 u[N2];
       FS::template step2<1>(u, ex + col * CS, k1);
-      float2* dst = F3 + plane * (long long)g.vy * g.Px + kx;
+      float2* dst = F3 + plane * (long long)g.wy * g.Px + kx;
 #pragma unroll
       for (int k2 = 0; k2 < N2; ++k2) {
-        const int vy = shift_slot(k1 + N1 * k2, g.ny, P, lo_y, hi_y);
-        if (vy >= 0) dst[(long long)vy * g.Px] = u[k2];
+        const int dy = window_index(k1 + N1 * k2, m0, P);
+        if (dy <= last) dst[(long long)dy * g.Px] = u[k2];
       }
     }
   }
 }
 
 template <int P>
-void launch_inv_y(const float2* F2, float2* F3, const float2* tw, Geo g, int nrot, const int* bounds,
-                  cudaStream_t st, int v) {
+void launch_inv_y(const float2* F2, float2* F3, Geo g, int nrot, const RotIn* rot, cudaStream_t st,
+                  int v) {
   by_split<P>(v, [&](auto vc) {
     constexpr int V = decltype(vc)::value;
     constexpr int W = 16, N2 = SplitV<P, V>::N2;
     const size_t smem = (size_t)W * FourStep<P, true, V>::CS * sizeof(float2);
     set_smem(k_inv_y<P, W, V>, smem);
-    dim3 grid((unsigned)(nrot * g.vz), (unsigned)((g.Px + W - 1) / W));
-    k_inv_y<P, W, V><<<grid, W * N2, smem, st>>>(F2, F3, tw, g, bounds);
+    dim3 grid((unsigned)(nrot * g.wz), (unsigned)((g.Px + W - 1) / W));
+    k_inv_y<P, W, V><<<grid, W * N2, smem, st>>>(F2, F3, g, rot);
   });
 }
 
 // ---------------------------------------------------------------------------
-// inv_x: x-axis inverse FFT of every (vz, vy) row of F3; at each valid shift
+// inv_x: x-axis inverse FFT of every (dz, dy) row of F3; at each valid shift
 // s = X / N (Eq. 5) where N >= the minimum overlap, and the block's argmax is
 // folded into the rotation's key with one atomicMax.  Optionally writes the
-// score map (-inf where invalid).  Block: ROWS consecutive vy of one plane.
+// score map (-inf where invalid).  Block: ROWS consecutive dy of one plane.
 // ---------------------------------------------------------------------------
 template <int P, int ROWS, int V>
 __global__ void __launch_bounds__((ROWS * SplitV<P, V>::N2 + 31) / 32 * 32)
-k_inv_x(const float2* __restrict__ F3, const float* __restrict__ thr,
-        unsigned long long* __restrict__ keys, float* __restrict__ map,
-        const float2* __restrict__ tw, Geo g, const int* __restrict__ bounds) {
+k_inv_x(const float2* __restrict__ F3, unsigned long long* __restrict__ keys, float* __restrict__ map,
+        Geo g, const RotIn* __restrict__ rot) {
+  const float2* __restrict__ tw = kTw<P>.w;
   using FS = FourStep<P, true, V>;
   constexpr int N1 = FS::N1, N2 = FS::N2, CS = FS::CS, NT = (ROWS * N2 + 31) / 32 * 32;
   extern __shared__ float2 ex[];
   __shared__ unsigned long long red[NT / 32];
   const int t = threadIdx.x;
-  const int plane = blockIdx.y;                       // r * vz + vz_i
-  const int r = plane / g.vz, vzi = plane - r * g.vz;
-  const int vy0 = blockIdx.x * ROWS;
-  int lo_y = 0, hi_y = g.vy - 1, lo_x = 0, hi_x = g.vx - 1;
-  if (bounds) {                                      // outside the shift bound: nothing to do
-    const int* b = bounds + 6 * r;
-    if (vzi < b[0] || vzi > b[1] || vy0 > b[3] || vy0 + ROWS - 1 < b[2]) return;
-    lo_y = b[2]; hi_y = b[3]; lo_x = b[4]; hi_x = b[5];
-  }
+  const int plane = blockIdx.y;                       // r * wz + dz
+  const int r = plane / g.wz, dz = plane - r * g.wz;
+  const int dy0 = blockIdx.x * ROWS;
+  const RotBox& b = rot[r].b;
+  const int ny_w = b.hi[1] - b.lo[1] + 1, last = b.hi[2] - b.lo[2], m0 = b.m0[2];
+  if (dz > b.hi[0] - b.lo[0] || dy0 >= ny_w) return;   // past this rotation's window
   if (t < ROWS * N2) {
     const int lrow = t / N2, n2 = t - lrow * N2;
-    const int vyi = vy0 + lrow;
-    const float2* src = F3 + ((long long)plane * g.vy + vyi) * P;
+    const int dy = dy0 + lrow;
+    const float2* src = F3 + ((long long)plane * g.wy + dy) * P;
     float2 v[N1];
 #pragma unroll
     for (int n1 = 0; n1 < N1; ++n1)
-      v[n1] = (vyi < g.vy) ? src[N2 * n1 + n2] : make_float2(0.f, 0.f);
+      v[n1] = (dy < ny_w) ? src[N2 * n1 + n2] : make_float2(0.f, 0.f);
     FS::template step1<1>(v, ex + lrow * CS, n2, tw);
   }
   __syncthreads();
   unsigned long long best = 0ull;
   if (t < ROWS * N1) {
     const int lr = t / N1, k1 = t - lr * N1;
-    const int vyi = vy0 + lr;
-    if (vyi < g.vy && vyi >= lo_y && vyi <= hi_y) {
+    const int dy = dy0 + lr;
+    if (dy < ny_w) {
       float2 u[N2];
       FS::template step2<1>(u, ex + lr * CS, k1);
-      const float th = thr[r];
-      const unsigned row_lin = ((unsigned)vzi * (unsigned)g.vy + (unsigned)vyi) * (unsigned)g.vx;
+      const float th = b.thr;
+      const unsigned row_lin = ((unsigned)(b.lo[0] + dz) * (unsigned)g.vy + (unsigned)(b.lo[1] + dy)) *
+                                   (unsigned)g.vx + (unsigned)b.lo[2];
 #pragma unroll
       for (int k2 = 0; k2 < N2; ++k2) {
-        const int vxi = shift_slot(k1 + N1 * k2, g.nx, P, lo_x, hi_x);
-        if (vxi >= 0) {
+        const int dx = window_index(k1 + N1 * k2, m0, P);
+        if (dx <= last) {
           const float2 zz = u[k2];
           float s = __int_as_float(0xff800000);
           if (zz.y >= th) {
             s = __fdiv_rn(zz.x, zz.y);
-            const unsigned long long key = make_key(s, row_lin + (unsigned)vxi);
+            const unsigned long long key = make_key(s, row_lin + (unsigned)dx);
             best = key > best ? key : best;
           }
-          if (map) map[(long long)row_lin + vxi] = s;
+          if (map) map[(long long)row_lin + dx] = s;
         }
       }
     }
@@ -930,36 +935,36 @@ k_inv_x(const float2* __restrict__ F3, const float* __restrict__ thr,
   if ((t & 31) == 0) red[t >> 5] = best;
   __syncthreads();
   if (t == 0) {
-    unsigned long long b = 0ull;
-    for (int w = 0; w < NT / 32; ++w) b = red[w] > b ? red[w] : b;
-    if (b) atomicMax(&keys[r], b);
+    unsigned long long top = 0ull;
+    for (int w = 0; w < NT / 32; ++w) top = red[w] > top ? red[w] : top;
+    if (top) atomicMax(&keys[r], top);
   }
 }
 
 template <int P>
-void launch_inv_x(const float2* F3, const float* thr, unsigned long long* keys, float* map,
-                  const float2* tw, Geo g, int nrot, const int* bounds, cudaStream_t st, int v) {
+void launch_inv_x(const float2* F3, unsigned long long* keys, float* map, Geo g, int nrot, const RotIn* rot,
+                  cudaStream_t st, int v) {
   by_split<P>(v, [&](auto vc) {
     constexpr int V = decltype(vc)::value;
     constexpr int N2 = SplitV<P, V>::N2;
     constexpr int ROWS = (256 / N2) > 0 ? (256 / N2) : 1;
     const size_t smem = (size_t)ROWS * FourStep<P, true, V>::CS * sizeof(float2);
     set_smem(k_inv_x<P, ROWS, V>, smem);
-    dim3 grid((unsigned)((g.vy + ROWS - 1) / ROWS), (unsigned)(nrot * g.vz));
-    k_inv_x<P, ROWS, V><<<grid, (ROWS * N2 + 31) / 32 * 32, smem, st>>>(F3, thr, keys, map, tw, g, bounds);
+    dim3 grid((unsigned)((g.wy + ROWS - 1) / ROWS), (unsigned)(nrot * g.wz));
+    k_inv_x<P, ROWS, V><<<grid, (ROWS * N2 + 31) / 32 * 32, smem, st>>>(F3, keys, map, g, rot);
   });
 }
 
 #define CSNGF_INSTANTIATE_PASSES(P)                                                              \
-  template void launch_fwd_x<P>(const float*, const uint8_t*, void*, const float2*, Geo, int,    \
+  template void launch_fwd_x<P>(const float*, const uint8_t*, void*, const RotIn*, Geo, int,     \
                                 cudaStream_t, int);                                              \
-  template void launch_fwd_y<P>(const void*, void*, const float2*, Geo, int, cudaStream_t, int); \
-  template void launch_zmac<P>(const void*, const float2*, float2*, const float2*, Geo, int,      \
-                               const int*, cudaStream_t, int);                                   \
-  template void launch_prep_z<P>(const float2*, float2*, const float2*, Geo, cudaStream_t);      \
-  template void launch_inv_y<P>(const float2*, float2*, const float2*, Geo, int, const int*,     \
-                                cudaStream_t, int);                                              \
-  template void launch_inv_x<P>(const float2*, const float*, unsigned long long*, float*,        \
-                                const float2*, Geo, int, const int*, cudaStream_t, int);
+  template void launch_fwd_y<P>(const void*, void*, Geo, int, cudaStream_t, int);                \
+  template void launch_zmac<P>(const void*, const float2*, float2*, Geo, int, const RotIn*,      \
+                               cudaStream_t, int);                                               \
+  template void launch_prep_z<P>(const float2*, float2*, Geo, cudaStream_t);                     \
+  template void launch_inv_y<P>(const float2*, float2*, Geo, int, const RotIn*, cudaStream_t,    \
+                                int);                                                            \
+  template void launch_inv_x<P>(const float2*, unsigned long long*, float*, Geo, int,            \
+                                const RotIn*, cudaStream_t, int);
 
 }  // namespace csngf

@@ -87,9 +87,7 @@ struct Job {
   Slot* slot = nullptr;
   cudaStream_t stream = nullptr;
   int cursor = 0;
-  // bound-limited padding: rotations in class order (perm[i] = original
-  // index; empty = unchanged), class c ends at class_end[c], lengths class_pad
-  std::vector<int> perm, class_end, class_pad;
+  csngf::detail::Plan plan;         // rotations in class order, scored class by class
   size_t cls = 0;
   std::deque<cudaEvent_t> inflight;
   cudaEvent_t done_ev = nullptr;
@@ -201,11 +199,9 @@ cs_ngf_status setup_job(cs_ngf_server* sv, Job* j, Slot* slot, bool fresh) {
   if (cs_ngf_status s = csngf::detail::upload_rotations(slot->f, j->quats.data(), j->R, st)) return s;
   if (cs_ngf_status s = csngf::detail::pack_floating(slot->f, slot->dB, slot->dMB, st)) return s;
   // FFT lengths per class of rotations (bound-limited padding), first class set up
-  if (cs_ngf_status s = csngf::detail::plan_classes(slot->f, j->R, st, j->perm, j->class_end,
-                                                    j->class_pad))
-    return s;
+  if (cs_ngf_status s = csngf::detail::plan_classes(slot->f, j->R, st, j->plan)) return s;
   j->cls = 0;
-  return csngf::detail::set_lengths(slot->f, j->class_pad.data(), st);
+  return csngf::detail::set_class(slot->f, j->plan.cls[0], st);
 }
 
 void finish_job(cs_ngf_server* sv, Job* j) {
@@ -340,14 +336,14 @@ void worker_loop(cs_ngf_server* sv) {
         // launch groups stay inside a class; the next class switches lengths
         // (which waits for this job's groups in flight)
         bool next_class = false;
-        while (j->cls + 1 < j->class_end.size() && j->cursor >= j->class_end[j->cls]) {
+        while (j->cls + 1 < j->plan.cls.size() && j->cursor >= j->plan.cls[j->cls].end) {
           ++j->cls;
           next_class = true;
         }
-        const int n = std::min(s->f->batch, j->class_end[j->cls] - j->cursor);
+        const int n = std::min(s->f->batch, j->plan.cls[j->cls].end - j->cursor);
         lk.unlock();
         cs_ngf_status st = CS_NGF_OK;
-        if (next_class) st = csngf::detail::set_lengths(s->f, j->class_pad.data() + 3 * j->cls, j->stream);
+        if (next_class) st = csngf::detail::set_class(s->f, j->plan.cls[j->cls], j->stream);
         if (!st) st = csngf::detail::score_range(s->f, j->cursor, n, s->d_score, s->d_shift, j->stream);
         cudaEvent_t ev = nullptr;
         if (!st) st = cuda_status(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "event");
@@ -396,14 +392,14 @@ void worker_loop(cs_ngf_server* sv) {
         }
         const int n = j->cursor;
         Slot* s = j->slot;
-        if (j->perm.empty()) {
+        if (j->plan.perm.empty()) {
           j->out_score.assign(s->h_score, s->h_score + n);
           j->out_shift.assign(s->h_shift, s->h_shift + 3 * (size_t)n);
         } else {                              // back to submission order
           j->out_score.assign((size_t)j->R, -INFINITY);
           j->out_shift.assign(3 * (size_t)j->R, 0);
           for (int i = 0; i < n; ++i) {
-            const int r = j->perm[i];
+            const int r = j->plan.perm[i];
             j->out_score[r] = s->h_score[i];
             for (int a = 0; a < 3; ++a) j->out_shift[3 * (size_t)r + a] = s->h_shift[3 * (size_t)i + a];
           }

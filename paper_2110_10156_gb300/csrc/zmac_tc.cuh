@@ -78,7 +78,8 @@ struct ZxTcCfg {
 template <int P, int ST>
 __global__ void __launch_bounds__(ZxTcCfg<P>::NT, 1)
 k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __restrict__ Xg,
-        const float2* __restrict__ tw, Geo g, int nrot, int KP) {
+        Geo g, int nrot, int KP) {
+  const float2* __restrict__ tw = kTw<P>.w;
   using C = ZxTcCfg<P>;
   constexpr int W = C::W, NT = C::NT, TILE = W * P, HF = C::HF;
   const int NB = g.nch * 4 * W;                    // MMA N: (field, primary/mirror, column, re/im)
@@ -98,7 +99,7 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
   const int mkx = (g.Px - kx) % g.Px;
   const long long hx = g.Px / 2 + 1;
   const long long S7 = hx * g.Py * (long long)P;
-  const long long E = (long long)g.nz * g.Px * g.Py;
+  const long long E = (long long)g.ez * g.Px * g.Py;
 
   for (uint32_t q = t; q < 2 * stageB / 16; q += NT)
     reinterpret_cast<uint4*>(Bs)[q] = make_uint4(0u, 0u, 0u, 0u);
@@ -116,7 +117,7 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
   for (int m = warp; m < 128; m += NT / 32)
     for (int k = lane; k < KP; k += 32) {
       float cv = 0.f, sv = 0.f;
-      if (m <= HF && k < g.nz) {
+      if (m <= HF && k < g.ez) {
         const float2 w = __ldg(&tw[(m * k) % P]);   // exp(-2 pi i m k / P)
         cv = w.x;
         sv = -w.y;
@@ -139,8 +140,8 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
   const bool prim = item < 2;
   const int cm = item - 2;
   const bool okc = t < 10 * ZSTEP && (prim ? ky0 + 4 * item < g.Py : ky0 + cm < g.Py);
-  const long long srow = prim ? (long long)kx * g.nz * g.Py + ky0 + 4 * item
-                              : (long long)mkx * g.nz * g.Py + (g.Py - (ky0 + cm)) % g.Py;
+  const long long srow = prim ? (long long)kx * g.ez * g.Py + ky0 + 4 * item
+                              : (long long)mkx * g.ez * g.Py + (g.Py - (ky0 + cm)) % g.Py;
   const int nrow = prim ? 8 * item : 16 + 2 * cm;
   auto fetch_b = [&](int r, int s) {
     if (r < nrot && okc) {
@@ -150,10 +151,10 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
         const int n = j * 4 * W + nrow;
         unsigned char* dcol = B0 + (uint32_t)(n / 8) * sbo + (n % 8) * 2;
         if (prim) {
-          for (int z = zr0; z < g.nz; z += ZSTEP)
+          for (int z = zr0; z < g.ez; z += ZSTEP)
             cp_async16(dcol + (z / 8) * 128 + (z % 8) * 16, src + (srow + (long long)z * g.Py) * 4);
         } else {
-          for (int z = zr0; z < g.nz; z += ZSTEP)
+          for (int z = zr0; z < g.ez; z += ZSTEP)
             cp_async4(dcol + (z / 8) * 128 + (z % 8) * 16, src + (srow + (long long)z * g.Py) * 4);
         }
       }
@@ -281,8 +282,8 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
 template <int P, int ST, bool HALF, int V>
 __global__ void __launch_bounds__(ZinvCfg<P, V>::NT, 2)
 k_zinv(const void* __restrict__ F1, const float2* __restrict__ Xg, const float2* __restrict__ UV,
-       float2* __restrict__ F2, const float2* __restrict__ tw, Geo g, int nrot,
-       const int* __restrict__ bounds) {
+       float2* __restrict__ F2, Geo g, int nrot, const RotIn* __restrict__ rot) {
+  const float2* __restrict__ tw = kTw<P>.w;
   using C = ZinvCfg<P, V>;
   using FS = typename C::FS;
   using FI = FwdIn<FS, HALF>;
@@ -299,14 +300,14 @@ k_zinv(const void* __restrict__ F1, const float2* __restrict__ Xg, const float2*
   const bool self_mirror = (2 * kx) % g.Px == 0;
   const long long hx = g.Px / 2 + 1;
   const long long S7 = hx * g.Py * (long long)P;
-  const long long E = (long long)g.nz * g.Px * g.Py;
+  const long long E = (long long)g.ez * g.Px * g.Py;
   auto slot = [](int kz) { return (kz / N1) * FS::RS + kz % N1; };
   const int c1 = t % NC, n2 = t / NC;
   const int pk1 = ky0 + (c1 < W ? c1 : c1 - W);
   const bool ok1 = pk1 < g.Py;
   const int ky1 = c1 < W ? pk1 : (g.Py - pk1) % g.Py;
   const int kx1 = c1 < W ? kx : mkx;
-  const long long col_off = (long long)kx1 * g.nz * g.Py + ky1;
+  const long long col_off = (long long)kx1 * g.ez * g.Py + ky1;
   const bool has2 = t < NC * N1;
   const int c2 = t % NC, k1 = t / NC;
 
@@ -326,7 +327,7 @@ k_zinv(const void* __restrict__ F1, const float2* __restrict__ Xg, const float2*
     for (int n1 = 0; n1 < HI; ++n1) {
       const int z = N2 * n1 + n2;
       mv[n1] = make_float2(0.f, 0.f);
-      if (r < nrot && ok1 && z < g.nz) {
+      if (r < nrot && ok1 && z < g.ez) {
         const float2* src = reinterpret_cast<const float2*>(Fields<ST>::field(F1, g, E, r, g.nch));
         mv[n1] = __ldg(&src[col_off + (long long)z * g.Py]);
       }
@@ -411,12 +412,12 @@ k_zinv(const void* __restrict__ F1, const float2* __restrict__ Xg, const float2*
         const int kx2 = c2 < W ? kx : mkx;
         float2 u[N2];
         FS::template step2<1>(u, ex + c2 * CS, k1);
-        float2* dst = F2 + ((long long)r * g.Px + kx2) * g.vz * g.Py + ky2;   // [r][kx][vz][ky]
-        const int lo = bounds ? bounds[6 * r] : 0, hi = bounds ? bounds[6 * r + 1] : g.vz - 1;
+        float2* dst = F2 + ((long long)r * g.Px + kx2) * g.wz * g.Py + ky2;   // [r][kx][dz][ky]
+        const int m0 = rot[r].b.m0[0], last = rot[r].b.hi[0] - rot[r].b.lo[0];
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) {
-          const int vz = shift_slot(k1 + N1 * k2, g.nz, P, lo, hi);
-          if (vz >= 0) dst[(long long)vz * g.Py] = u[k2];
+          const int dz = window_index(k1 + N1 * k2, m0, P);
+          if (dz <= last) dst[(long long)dz * g.Py] = u[k2];
         }
       }
     }
@@ -428,15 +429,15 @@ k_zinv(const void* __restrict__ F1, const float2* __restrict__ Xg, const float2*
 // precision form and shared memory allow it; false otherwise (the caller then
 // runs k_zmac)
 template <int P, int ST, bool HALF, int V>
-bool launch_zsplit_t(const void* F1, const float2* UV, float2* F2, const float2* tw, Geo g, int nrot,
-                     const int* bounds, cudaStream_t st) {
+bool launch_zsplit_t(const void* F1, const float2* UV, float2* F2, Geo g, int nrot, const RotIn* rot,
+                     cudaStream_t st) {
   using C1 = ZxTcCfg<P>;
   using C2 = ZinvCfg<P, V>;
   if constexpr (!C1::OK || ST == kStoreF32) {
     return false;
   } else {
     if (!g.zx) return false;
-    const int KP = (g.nz + 15) / 16 * 16;
+    const int KP = (g.ez + 15) / 16 * 16;
     const int NB = g.nch * 4 * C1::W;
     if (NB > 128 || NB % 16 != 0) return false;
     const size_t b1 = C1::bytes(KP, NB, 2 * g.nch);
@@ -444,10 +445,10 @@ bool launch_zsplit_t(const void* F1, const float2* UV, float2* F2, const float2*
     const size_t s1 = std::max<size_t>(b1, 120 * 1024);   // one block per SM: all of its tensor memory
     set_smem(k_zx_tc<P, ST>, s1);
     dim3 grid((unsigned)((g.Py + C1::W - 1) / C1::W), (unsigned)(g.Px / 2 + 1));
-    k_zx_tc<P, ST><<<grid, C1::NT, s1, st>>>(F1, UV, g.zx, tw, g, nrot, KP);
+    k_zx_tc<P, ST><<<grid, C1::NT, s1, st>>>(F1, UV, g.zx, g, nrot, KP);
     const size_t s2 = ((size_t)C2::NC * C2::FS::CS + (size_t)C2::W * P + P) * sizeof(float2);
     set_smem(k_zinv<P, ST, HALF, V>, s2);
-    k_zinv<P, ST, HALF, V><<<grid, C2::NT, s2, st>>>(F1, g.zx, UV, F2, tw, g, nrot, bounds);
+    k_zinv<P, ST, HALF, V><<<grid, C2::NT, s2, st>>>(F1, g.zx, UV, F2, g, nrot, rot);
     return true;
   }
 }

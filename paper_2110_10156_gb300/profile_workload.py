@@ -115,7 +115,7 @@ def classify_rotations(f, B, MB, quats) -> dict:
     out = {}
     for i in range(len(quats)):
         f.score_rotations(B, MB, quats[i:i + 1])
-        (cp, _), = f.length_classes()
+        (cp, _), = f.transform_classes()
         out.setdefault(tuple(cp), []).append(i)
     return out
 
@@ -183,7 +183,7 @@ def main(argv=None) -> int:
     for _ in range(args.repeat):
         sc, sh = f.score_rotations(B, MB, quats)
     torch.cuda.synchronize()
-    print(f"dims {p.A.shape} classes {f.length_classes()} batch {f.batch} best {float(sc.max()):.6f}")
+    print(f"dims {p.A.shape} classes {f.transform_classes()} batch {f.batch} best {float(sc.max()):.6f}")
     f.release()
     return 0
 
