@@ -855,10 +855,11 @@ Sizes sizes_for(const int32_t dims[3], const int pad[3], int measure, int precis
   z.f13_elems = (std::max((nch * cb + 8) * E1, vz * vy * Px * 8) + 7) / 8;
   z.fixed_f02 = nf * E0;                                            // one rotation, FP32 (A side)
   z.fixed_f13 = nf * E1;
-  z.zx_elems = (tensor_cores && precision != CS_NGF_FP32) ? (Px / 2 + 1) * Py * Pz : 0;
+  const size_t Py8 = (Py + 7) / 8 * 8;                              // the z pass's tiles of 8 columns
+  z.zx_elems = (tensor_cores && precision != CS_NGF_FP32) ? (Px / 2 + 1) * Py8 * Pz : 0;
   z.per_rot = (z.f02_elems + z.f13_elems + z.zx_elems) * sizeof(float2) + nvox * 5;
   z.shared_ws = nvox * (sizeof(float4) + 1);                       // BQ, C8
-  z.uv_elems = (2 * nch + 1) * (Px / 2 + 1) * Py * Pz;
+  z.uv_elems = (2 * nch + 1) * (Px / 2 + 1) * Py8 * Pz;
   return z;
 }
 

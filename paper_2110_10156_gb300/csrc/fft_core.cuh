@@ -307,7 +307,8 @@ struct FourStep {
   }
 
   // v holds x[N2*n1 + n2] for n1 = 0..N1-1; writes twiddled N1-point outputs
-  template <int S, bool TS = false>
+  // (exchange elements lie W apart: callers with W sequences interleaved)
+  template <int S, bool TS = false, int W = 1>
   __device__ __forceinline__ static void step1(float2 (&v)[N1], float2* ex_seq, int n2,
                                                const float2* __restrict__ twN) {
     Dft<N1, S>::run(v);
@@ -315,7 +316,7 @@ struct FourStep {
     for (int k1 = 0; k1 < N1; ++k1) {
       float2 w = twl<TS>(&twN[n2 * k1]);
       if (S > 0) w.y = -w.y;
-      ex_seq[n2 * RS + k1] = (k1 == 0) ? v[k1] : cmul(v[k1], w);
+      ex_seq[(n2 * RS + k1) * W] = (k1 == 0) ? v[k1] : cmul(v[k1], w);
     }
   }
 
@@ -323,7 +324,7 @@ struct FourStep {
   // of data zero-padded from length <= N/2): the N1-point DFT splits into two
   // N1/2-point DFTs, X[2m] = DFT(x)[m], X[2m+1] = DFT(x * W_N1^n)[m].
   static constexpr int H = N1 / 2;
-  template <int S, bool TS = false>
+  template <int S, bool TS = false, int W = 1>
   __device__ __forceinline__ static void step1_half(float2 (&v)[H], float2* ex_seq, int n2,
                                                     const float2* __restrict__ twN) {
     static_assert(N1 % 2 == 0, "half-zero step needs an even N1");
@@ -340,8 +341,8 @@ struct FourStep {
       const int ke = 2 * m, ko = 2 * m + 1;
       float2 we = twl<TS>(&twN[n2 * ke]), wo = twl<TS>(&twN[n2 * ko]);
       if (S > 0) { we.y = -we.y; wo.y = -wo.y; }
-      ex_seq[n2 * RS + ke] = (m == 0) ? e[m] : cmul(e[m], we);
-      ex_seq[n2 * RS + ko] = cmul(o[m], wo);
+      ex_seq[(n2 * RS + ke) * W] = (m == 0) ? e[m] : cmul(e[m], we);
+      ex_seq[(n2 * RS + ko) * W] = cmul(o[m], wo);
     }
   }
 

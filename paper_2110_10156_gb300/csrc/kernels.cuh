@@ -18,7 +18,7 @@
 //   F1       [r][j][kx][z][ky]                  x, y transformed
 //   F2       [r][kx][dz][ky]                    Z = X + iY after the z inverse
 //   F3       [r][dz][dy][kx]                    after the y inverse
-//   UV       [2nch+1][kx <= Px/2][ky][kz]      fixed-volume weights (prepare)
+//   UV       [kx <= Px/2][ky/8][2nch+1][kz][ky%8]  fixed-volume weights (prepare)
 // z, y of F0 and F1 count from the rotation's box origin (RotBox::org) and run
 // over the class's extents (Geo::ez, ey); dz, dy count from the first shift
 // slot that can be valid (RotBox::lo) over the class's windows (Geo::wz, wy).
@@ -57,7 +57,7 @@ struct Geo {
   // set to 1 by a tensor-core pass whose bounded wait for its own MMAs ran out
   // (it then stops and returns); nullptr: not reported
   int* tc_err;
-  // X of the tensor-core z pass, [r][kx <= Px/2][ky][kz] per launch group
+  // X of the tensor-core z pass, [r][kx <= Px/2][ky/8][kz][ky%8] per launch group
   // (the handle allocates it with the tensor-core forms); nullptr: the z pass
   // runs as one kernel
   float2* zx;

@@ -27,6 +27,12 @@ struct FwdIn {
     if constexpr (HALF) FS::template step1_half<S, TS>(v, ex_seq, n2, twN);
     else FS::template step1<S, TS>(v, ex_seq, n2, twN);
   }
+  // the same to an exchange whose elements lie W apart, twiddles in shared memory
+  template <int S, int W>
+  __device__ __forceinline__ static void step1w(float2 (&v)[NI], float2* ex_row, int n2, const float2* tws) {
+    if constexpr (HALF) FS::template step1_half<S, true, W>(v, ex_row - n2 * FS::RS * W, n2, tws);
+    else FS::template step1<S, true, W>(v, ex_row - n2 * FS::RS * W, n2, tws);
+  }
 };
 
 // calls f with the storage form of the channel fields as a compile-time constant
@@ -47,6 +53,19 @@ static void by_split(int v, F&& f) {
     }
   }
   f(std::integral_constant<int, 0>{});
+}
+
+// calls f with whether a box extent e fills at most half the length (where the
+// split's first factor is even, so that the pruned first step exists)
+template <int P, int V, class F>
+static void by_half(int e, F&& f) {
+  if constexpr (SplitV<P, V>::N1 % 2 == 0) {
+    if (2 * e <= P) {
+      f(std::true_type{});
+      return;
+    }
+  }
+  f(std::false_type{});
 }
 
 template <class K>
@@ -245,8 +264,9 @@ void launch_fwd_x(const float* Bh, const uint8_t* Mh, void* F0, const RotIn* rot
                   cudaStream_t st, int v) {
   by_split<P>(v, [&](auto vc) {
     constexpr int V = decltype(vc)::value;
-    if (2 * g.ex <= P) launch_fwd_x_t<P, true, V>(Bh, Mh, F0, rot, g, nrot, st);
-    else launch_fwd_x_t<P, false, V>(Bh, Mh, F0, rot, g, nrot, st);
+    by_half<P, V>(g.ex, [&](auto hc) {
+      launch_fwd_x_t<P, decltype(hc)::value, V>(Bh, Mh, F0, rot, g, nrot, st);
+    });
   });
 }
 
@@ -349,10 +369,9 @@ void launch_fwd_y_t(const void* F0, void* F1, Geo g, int nrot, cudaStream_t st) 
     set_smem(kern, smem);
     kern<<<grid, W * N2, smem, st>>>(F0, F1, g);
   };
-  const bool half = 2 * g.ey <= P;
   by_store(g.store, [&](auto sf) {
     constexpr int ST = decltype(sf)::value;
-    half ? go(k_fwd_y<P, W, ST, true, V>) : go(k_fwd_y<P, W, ST, false, V>);
+    by_half<P, V>(g.ey, [&](auto hc) { go(k_fwd_y<P, W, ST, decltype(hc)::value, V>); });
   });
 }
 
@@ -361,334 +380,9 @@ void launch_fwd_y(const void* F0, void* F1, Geo g, int nrot, cudaStream_t st, in
   by_split<P>(v, [&](auto vc) { launch_fwd_y_t<P, decltype(vc)::value>(F0, F1, g, nrot, st); });
 }
 
-// ---------------------------------------------------------------------------
-// zmac: for W columns (kx, ky) and their mirrors (-kx, -ky):
-//   z-axis FFT of the four packed fields,
-//   X(k) = sum_j U_j(k) H_j(k) + V_j(k) conj(H_j(-k))   (six weighted channels)
-//   Y(k) = U_3(k) H_3(k)                                 (mask correlation)
-//   z-axis inverse FFT of Z = X + iY at k and of conj(X) + i conj(Y) at -k,
-// keeping the 2nz-1 shift planes.  Loops over the batch's rotations so the
-// fixed spectra tile stays in L2.
-// ---------------------------------------------------------------------------
-// shared memory of a zmac block with W primary columns (see ZmacCfg)
-template <int P, bool HALF, int V>
-constexpr size_t zmac_smem_base(int W) {
-  const int NI = HALF ? SplitV<P, V>::N1 / 2 : SplitV<P, V>::N1;
-  const size_t cs = 2 * W < 16 ? FourStep<P, true, V>::CS : FourStep<P, false, V>::CS;
-  return ((size_t)7 * W * P + (size_t)2 * W * cs + (size_t)2 * NI * (2 * W * SplitV<P, V>::N2)) *
-         sizeof(float2);
-}
-
-template <int P, bool HALF, int V>
-struct ZmacCfg {
-  // primary columns per block: the block's tile of the seven fixed spectra
-  // (7 * W * P complex values) stays in shared memory for the whole batch;
-  // 8 columns where the tile, the exchange and two input stages fit (at most
-  // 227 KB per block), else 4
-  static constexpr int W =
-      (P <= 320 && zmac_smem_base<P, HALF, V>(8) + P * sizeof(float2) <= 232448) ? 8 : 4;
-  static constexpr int NT = 2 * W * SplitV<P, V>::N2;
-  // exchange rows unpadded when 16 columns fill a half-warp (natural order)
-  static constexpr bool PAD = 2 * W < 16;
-  using FS = FourStep<P, PAD, V>;
-  static constexpr int NI = FwdIn<FS, HALF>::NI;   // staged inputs per thread and field
-  // shared memory: fixed-spectra tile [7][W][P], transform exchange [2W][CS],
-  // two stages of field inputs [2][NI][NT] and, where it does not cost a
-  // second block per SM, the twiddle table [P] (else twiddles come from L1)
-  static constexpr size_t smem_base = zmac_smem_base<P, HALF, V>(W);
-  static constexpr bool fits2(size_t b) { return 2 * (b + 1024) <= 228 * 1024; }   // per-block reserve
-  static constexpr bool TWS = fits2(smem_base + P * sizeof(float2)) || !fits2(smem_base);
-  static constexpr size_t smem_one = smem_base + (TWS ? P * sizeof(float2) : 0);
-  // a second exchange buffer, used by alternate fields, where it fits without
-  // costing a block per SM: the next field's first step then need not wait
-  // for this field's multiply-accumulate to finish reading
-  static constexpr size_t ex_bytes = (size_t)2 * W * FS::CS * sizeof(float2);
-  static constexpr int EXB =
-      (smem_one + ex_bytes <= 232448 && fits2(smem_one + ex_bytes) == fits2(smem_one)) ? 2 : 1;
-  static constexpr size_t smem_bytes = smem_one + (EXB - 1) * ex_bytes;
-  // Registers per thread when B blocks share an SM: each of the SM's four
-  // sub-partitions holds 16384 registers and the warps placed on it, at most
-  // ceil(B * warps / 4) of them (allocation in multiples of 8 per thread).
-  static constexpr int regs_for(int B) {
-    return (16384 / (32 * ((B * ((NT + 31) / 32) + 3) / 4))) / 8 * 8;
-  }
-  // two blocks per SM where shared memory allows it and each thread still
-  // keeps at least 128 registers
-  static constexpr int MIN_BLOCKS = (fits2(smem_bytes) && regs_for(2) >= 128) ? 2 : 1;
-};
-
-template <int P, int ST, bool HALF, int V>
-__global__ void __launch_bounds__(ZmacCfg<P, HALF, V>::NT, ZmacCfg<P, HALF, V>::MIN_BLOCKS)
-k_zmac(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __restrict__ F2,
-       Geo g, int nrot, const RotIn* __restrict__ rot) {
-  const float2* __restrict__ tw = kTw<P>.w;
-  using C = ZmacCfg<P, HALF, V>;
-  using FS = typename C::FS;
-  using FI = FwdIn<FS, HALF>;
-  constexpr int W = C::W;
-  constexpr int N1 = FS::N1, N2 = FS::N2, CS = FS::CS, H = C::NI;
-  constexpr int NC = 2 * W, NT = C::NT, MI = (W * P + NT - 1) / NT;
-  constexpr int TILE = W * P;                 // complex values per fixed-spectra tile
-  extern __shared__ __align__(16) float2 smem[];
-  float2* uvs = smem;                         // [7][W][P] fixed-spectra weights
-  constexpr int EXB = C::EXB;
-  float2* ex0 = smem + 7 * TILE;              // [EXB][NC][CS] transform exchange
-  float2* stage = ex0 + EXB * NC * CS;        // [2][H][NT] inputs of the next two fields
-                                              // (each thread uses only its own slots)
-  float2* tws = stage + 2 * H * NT;           // [P] twiddles
-  // a transformed column stays in the exchange slots of the four-step split:
-  // X[kz] with kz = k1 + N1*k2 sits at k2*RS + k1
-  auto slot = [](int kz) { return (kz / N1) * FS::RS + kz % N1; };
-  const int t = threadIdx.x;
-  const int kx = blockIdx.y, ky0 = blockIdx.x * W;
-  const int mkx = (g.Px - kx) % g.Px;
-  const bool self_mirror = (2 * kx) % g.Px == 0;
-  const long long hx = g.Px / 2 + 1;
-  const long long S7 = hx * g.Py * (long long)P;
-  const long long plane_stride = (long long)g.Px * g.Py;
-
-  // step-1 role: column c1 (fastest), n2
-  const int c1 = t % NC, n2 = t / NC;
-  const int pk1 = ky0 + (c1 < W ? c1 : c1 - W);
-  const bool ok1 = pk1 < g.Py;
-  const int ky1 = c1 < W ? pk1 : (g.Py - pk1) % g.Py;
-  const int kx1 = c1 < W ? kx : mkx;
-  const long long col_off = (long long)kx1 * g.ez * g.Py + ky1;   // F1 is [r][j][kx][z][ky]
-  // step-2 role: column c2 (fastest), k1
-  const bool has2 = t < NC * N1;
-  const int c2 = t % NC, k1 = t / NC;
-
-  // z = N2*n1 + n2 < ez (with ez <= P/2 only n1 < N1/2).  Field inputs are copied
-  // asynchronously (cp.async) two fields ahead into this thread's own slots of
-  // two stages: no registers are held meanwhile.  Slots outside the volume are
-  // zero once and never copied to.  Fields run in the order (r, j), j < nfr(r).
-#pragma unroll
-  for (int n1 = 0; n1 < H; ++n1) {
-    const int z = N2 * n1 + n2;
-    if (!(ok1 && z < g.ez)) stage[n1 * NT + t] = stage[(H + n1) * NT + t] = make_float2(0.f, 0.f);
-  }
-  auto nfr = [&](int r) { return (r & 1) ? g.nch : g.nf; };  // an odd rotation's mask came with its partner
-  int pr = 0, pj = 0;                         // next field to copy
-  auto fetch = [&](float2* buf) {             // copies field (pr, pj), if any, and advances
-    if (pr < nrot) {
-      const char* src = Fields<ST>::field(F1, g, g.ez * plane_stride, pr, pj);
-      if (ST == kStoreF32 || pj == g.nch) {
-#pragma unroll
-        for (int n1 = 0; n1 < H; ++n1) {
-          const int z = N2 * n1 + n2;
-          if (ok1 && z < g.ez)
-            cp_async8(buf + n1 * NT + t, src + (col_off + (long long)z * g.Py) * 8);
-        }
-      } else {
-#pragma unroll
-        for (int n1 = 0; n1 < H; ++n1) {
-          const int z = N2 * n1 + n2;
-          if (ok1 && z < g.ez)
-            cp_async4(buf + n1 * NT + t, src + (col_off + (long long)z * g.Py) * 4);
-        }
-      }
-      if (++pj == nfr(pr)) { pj = 0; ++pr; }
-    }
-    cp_async_commit();                         // one group per call, empty or not
-  };
-  // this thread's staged inputs of field j from buf, once all but the most
-  // recent copy group have landed
-  auto take = [&](float2 (&v)[H], const float2* buf, int j) {
-    if (ST == kStoreF32 || j == g.nch) {
-#pragma unroll
-      for (int n1 = 0; n1 < H; ++n1) v[n1] = buf[n1 * NT + t];
-    } else if (ST == kStoreBF16) {
-#pragma unroll
-      for (int n1 = 0; n1 < H; ++n1)
-        v[n1] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(buf + n1 * NT + t));
-    } else {                                   // FP16: undo the field's power-of-two scale
-      const float isc = 1.0f / field_scale(g.scale1, j);
-#pragma unroll
-      for (int n1 = 0; n1 < H; ++n1) {
-        const float2 h = __half22float2(*reinterpret_cast<const __half2*>(buf + n1 * NT + t));
-        v[n1] = make_float2(h.x * isc, h.y * isc);
-      }
-    }
-  };
-  // the block's fixed-spectra tile: 7 contiguous runs of W*P values (rows
-  // ky0..ky0+W-1 are contiguous in [kx][ky][kz]), copied asynchronously as the
-  // first copy group; rows past Py are zero
-  {
-    const int valid = min(W, g.Py - ky0) * P;
-    for (int a = 0; a < 2 * g.nch + 1; ++a) {
-      const float2* src = UV + a * S7 + ((long long)kx * g.Py + ky0) * P;
-      float2* dst = uvs + a * TILE;
-      for (int q = t; q < TILE / 2; q += NT) {
-        if (2 * q < valid) cp_async16(dst + 2 * q, src + 2 * q);
-        else reinterpret_cast<float4*>(dst)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-    cp_async_commit();
-  }
-  fetch(stage);
-  fetch(stage + H * NT);
-  constexpr bool TWS = C::TWS;
-  if constexpr (TWS)
-    for (int q = t; q < P; q += NT) tws[q] = __ldg(&tw[q]);
-  const float2* twz = TWS ? tws : tw;
-  __syncthreads();                            // twiddles visible to all (the tile is
-                                              // waited for with the first field)
-
-  // Y of an odd rotation is formed with its partner's mask field and carried
-  // in Yn: live only from that product to the next rotation's start
-  float2 Y[MI], Yn[MI];
-  int f = 0;                                  // field counter: stage f & 1
-  for (int r = 0; r < nrot; ++r) {
-    float2 X[MI];
-#pragma unroll
-    for (int m = 0; m < MI; ++m) {
-      X[m] = make_float2(0.f, 0.f);
-      Y[m] = (r & 1) ? Yn[m] : make_float2(0.f, 0.f);
-    }
-    // Eq. 7-8: the weighted channel products (separated through the mirror
-    // column) and the mask product of field j, transformed in exb,
-    // accumulated in registers
-    auto mac = [&](int j, const float2* exb) {
-      if (j < g.nch) {
-        const float2* Us = uvs + (2 * j) * TILE;
-        const float2* Vs = uvs + (2 * j + 1) * TILE;
-#pragma unroll
-        for (int m = 0; m < MI; ++m) {
-          const int i = t + NT * m;
-          if (i < TILE) {
-            const int c = i / P, kz = i - c * P;
-            const float2 h = exb[c * CS + slot(kz)];
-            const float2 hm = cconj(exb[(W + c) * CS + slot(kz == 0 ? 0 : P - kz)]);
-            X[m] = cadd(X[m], cadd(cmul(Us[i], h), cmul(Vs[i], hm)));
-          }
-        }
-      } else {
-        // the mask pair (M_r, M_{r+1}): M_r = (h + hm)/2, M_{r+1} = -i (h - hm)/2
-        const float2* Ms = uvs + 2 * g.nch * TILE;
-#pragma unroll
-        for (int m = 0; m < MI; ++m) {
-          const int i = t + NT * m;
-          if (i < TILE) {
-            const int c = i / P, kz = i - c * P;
-            const float2 h = exb[c * CS + slot(kz)];
-            const float2 hm = cconj(exb[(W + c) * CS + slot(kz == 0 ? 0 : P - kz)]);
-            const float2 U = Ms[i];
-            Y[m] = cmul(U, cscale(cadd(h, hm), 0.5f));
-            const float2 d = cscale(csub(h, hm), 0.5f);
-            Yn[m] = cmul(U, make_float2(d.y, -d.x));
-          }
-        }
-      }
-    };
-    // step 2 of one column sequence (column cc, k1), in place: the outputs
-    // X[k1 + N1*k2] go to the slots k2*RS + k1 this thread has just read, so
-    // no other thread's reads are overtaken
-    auto step2_at = [&](float2* exb, int cc, int kk) {
-      float2 u[N2];
-      FS::template step2<-1>(u, exb + cc * CS, kk);
-#pragma unroll
-      for (int k2 = 0; k2 < N2; ++k2) exb[cc * CS + k2 * FS::RS + kk] = u[k2];
-    };
-#pragma unroll 1
-    for (int j = 0; j < nfr(r);) {
-      if (EXB == 2 && j + 1 < nfr(r)) {
-        // two fields at once, in the two exchanges: both first steps, one
-        // barrier, both second steps spread over all threads, one barrier,
-        // both products, one barrier
-        float2* ex1 = ex0 + NC * CS;
-        cp_async_wait_all();                   // both fields' inputs have landed
-        {
-          float2 v[H];
-          take(v, stage + (f & 1) * H * NT, j);
-          FI::template step1<-1, TWS>(v, ex0 + c1 * CS, n2, twz);
-          take(v, stage + ((f + 1) & 1) * H * NT, j + 1);
-          FI::template step1<-1, TWS>(v, ex1 + c1 * CS, n2, twz);
-        }
-        __syncthreads();                       // (also orders this thread's reads of the
-                                               //  stages before the next copies into them)
-        fetch(stage + (f & 1) * H * NT);       // the next two fields
-        fetch(stage + ((f + 1) & 1) * H * NT);
-        for (int w = t; w < 2 * NC * N1; w += NT) {
-          const int q = w < NC * N1 ? w : w - NC * N1;
-          step2_at(w < NC * N1 ? ex0 : ex1, q % NC, q / NC);
-        }
-        __syncthreads();
-        mac(j, ex0);
-        mac(j + 1, ex1);
-        __syncthreads();
-        j += 2;
-        f += 2;
-      } else {
-        float2* buf = stage + (f & 1) * H * NT;
-        cp_async_wait_one();                   // all but the most recent copy group
-        float2 v[H];
-        take(v, buf, j);
-        FI::template step1<-1, TWS>(v, ex0 + c1 * CS, n2, twz);
-        __syncthreads();                       // (also orders this thread's reads of buf
-                                               //  before the next copies into it)
-        fetch(buf);                            // two fields ahead
-        if (has2) step2_at(ex0, c2, k1);
-        __syncthreads();
-        mac(j, ex0);
-        __syncthreads();
-        ++j;
-        ++f;
-      }
-    }
-    float2* ex = ex0;                         // the rotation's inverse
-    // Z = X + iY at k, conj(X) + i conj(Y) at -k
-#pragma unroll
-    for (int m = 0; m < MI; ++m) {
-      const int i = t + NT * m;
-      if (i < TILE) {
-        const int c = i / P, kz = i - c * P;
-        ex[c * CS + slot(kz)] = make_float2(X[m].x - Y[m].y, X[m].y + Y[m].x);
-        ex[(W + c) * CS + slot(kz == 0 ? 0 : P - kz)] = make_float2(X[m].x + Y[m].y, Y[m].x - X[m].y);
-      }
-    }
-    __syncthreads();
-    {
-      float2 v[N1];
-#pragma unroll
-      for (int n1 = 0; n1 < N1; ++n1) v[n1] = ex[c1 * CS + slot(N2 * n1 + n2)];
-      __syncthreads();
-      FS::template step1<1, TWS>(v, ex + c1 * CS, n2, twz);
-    }
-    __syncthreads();
-    if (has2 && !(c2 >= W && self_mirror)) {
-      const int pk2 = ky0 + (c2 < W ? c2 : c2 - W);
-      if (pk2 < g.Py) {
-        const int ky2 = c2 < W ? pk2 : (g.Py - pk2) % g.Py;
-        const int kx2 = c2 < W ? kx : mkx;
-        float2 u[N2];
-        FS::template step2<1>(u, ex + c2 * CS, k1);
-        float2* dst = F2 + ((long long)r * g.Px + kx2) * g.wz * g.Py + ky2;   // [r][kx][dz][ky]
-        const int m0 = rot[r].b.m0[0], last = rot[r].b.hi[0] - rot[r].b.lo[0];
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) {
-          const int dz = window_index(k1 + N1 * k2, m0, P);
-          if (dz <= last) dst[(long long)dz * g.Py] = u[k2];
-        }
-      }
-    }
-    __syncthreads();
-  }
-}
-
-template <int P, bool HALF, int V>
-void launch_zmac_t(const void* F1, const float2* UV, float2* F2, Geo g, int nrot, const RotIn* rot,
-                   cudaStream_t st) {
-  using C = ZmacCfg<P, HALF, V>;
-  dim3 grid((unsigned)((g.Py + C::W - 1) / C::W), (unsigned)(g.Px / 2 + 1));
-  by_store(g.store, [&](auto sf) {
-    constexpr int ST = decltype(sf)::value;
-    set_smem(k_zmac<P, ST, HALF, V>, C::smem_bytes);
-    k_zmac<P, ST, HALF, V><<<grid, C::NT, C::smem_bytes, st>>>(F1, UV, F2, g, nrot, rot);
-  });
-}
-
 }  // namespace csngf
 
+#include "zpass.cuh"
 #include "zmac_tc.cuh"
 
 namespace csngf {
@@ -696,117 +390,31 @@ namespace csngf {
 template <int P>
 void launch_zmac(const void* F1, const float2* UV, float2* F2, Geo g, int nrot, const RotIn* rot,
                  cudaStream_t st, int v) {
+  float2* W = const_cast<float2*>(UV);            // written in the prepare mode only
   by_split<P>(v, [&](auto vc) {
     constexpr int V = decltype(vc)::value;
-    const bool half = 2 * g.ez <= P;
-    if (g.tc && g.store != kStoreF32) {          // reduced-precision forms: tensor-core z DFT
-      bool done = false;
-      by_store(g.store, [&](auto sf) {
-        constexpr int ST = decltype(sf)::value;
-        done = half ? launch_zsplit_t<P, ST, true, V>(F1, UV, F2, g, nrot, rot, st)
-                    : launch_zsplit_t<P, ST, false, V>(F1, UV, F2, g, nrot, rot, st);
-      });
-      if (done) return;
-    }
-    if (half) launch_zmac_t<P, true, V>(F1, UV, F2, g, nrot, rot, st);
-    else launch_zmac_t<P, false, V>(F1, UV, F2, g, nrot, rot, st);
-  });
-}
-
-// ---------------------------------------------------------------------------
-// prep_z (fixed volume, once): z-axis FFT of A's packed fields, channel
-// separation via the mirror column, and the weights
-//   U_j = (w_a conj(A_a) - i w_b conj(A_b)) / 2,  V_j = (w_a conj(A_a) + i w_b conj(A_b)) / 2
-// for the channel fields j < nch (channels a, b of the pair with their Eq. 6
-// weights, or Eq. 3 weights), and conj(A_mask) last, stored for kx <= Px/2.
-// ---------------------------------------------------------------------------
-template <int P, int W, bool HALF>
-__global__ void __launch_bounds__(2 * W * Split<P>::N2)
-k_prep_z(const float2* __restrict__ F1, float2* __restrict__ UV, Geo g) {
-  const float2* __restrict__ tw = kTw<P>.w;
-  using FS = FourStep<P>;
-  using FI = FwdIn<FS, HALF>;
-  constexpr int N1 = FS::N1, N2 = FS::N2, CS = FS::CS;
-  constexpr int NC = 2 * W, NT = NC * N2, MI = (W * P + NT - 1) / NT;
-  extern __shared__ float2 ex[];
-  const int t = threadIdx.x;
-  const int kx = blockIdx.y, ky0 = blockIdx.x * W;
-  const int mkx = (g.Px - kx) % g.Px;
-  const long long hx = g.Px / 2 + 1;
-  const long long S7 = hx * g.Py * (long long)P;
-  const int c1 = t % NC, n2 = t / NC;
-  const int pk1 = ky0 + (c1 < W ? c1 : c1 - W);
-  const bool ok1 = pk1 < g.Py;
-  const int ky1 = c1 < W ? pk1 : (g.Py - pk1) % g.Py;
-  const int kx1 = c1 < W ? kx : mkx;
-  const bool has2 = t < NC * N1;
-  const int c2 = t % NC, k1 = t / NC;
-  const long long plane_stride = (long long)g.Px * g.Py;
-#pragma unroll 1
-  for (int j = 0; j < g.nf; ++j) {
-    // Eq. 6 weights: squared (1,1), (1,2), (2,2); unsquared (Eq. 3) (1,1), (1,0)
-    float wa = 1.f, wb = 1.f;
-    if (g.nch == 3) { wa = j == 2 ? 2.f : 1.f; wb = j == 0 ? 1.f : 2.f; }
-    else { wb = j == 0 ? 1.f : 0.f; }
-    const float2* src = F1 + (long long)j * g.ez * plane_stride;   // [j][kx][z][ky]
-    float2 v[FI::NI];                     // z < ez: with ez <= P/2 the upper half is zero
-#pragma unroll
-    for (int n1 = 0; n1 < FI::NI; ++n1) {
-      const int z = N2 * n1 + n2;
-      v[n1] = (ok1 && z < g.ez) ? src[((long long)kx1 * g.ez + z) * g.Py + ky1]
-                                : make_float2(0.f, 0.f);
-    }
-    FI::template step1<-1>(v, ex + c1 * CS, n2, tw);
-    __syncthreads();
-    float2 u[N2];
-    if (has2) FS::template step2<-1>(u, ex + c2 * CS, k1);
-    __syncthreads();
-    if (has2) {
-#pragma unroll
-      for (int k2 = 0; k2 < N2; ++k2) ex[c2 * CS + k1 + N1 * k2] = u[k2];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < MI; ++m) {
-      const int i = t + NT * m;
-      if (i < W * P) {
-        const int c = i / P, kz = i - c * P;
-        const int ky = ky0 + c;
-        if (ky < g.Py) {
-          const float2 h = ex[c * CS + kz];
-          const long long o = ((long long)kx * g.Py + ky) * P + kz;
-          if (j < g.nch) {
-            const float2 hm = cconj(ex[(W + c) * CS + (kz == 0 ? 0 : P - kz)]);
-            // A_a = (h + hm)/2, A_b = -i (h - hm)/2
-            const float2 Aa = cscale(cadd(h, hm), 0.5f);
-            const float2 d = cscale(csub(h, hm), 0.5f);
-            const float2 Ab = make_float2(d.y, -d.x);
-            const float2 ca = cscale(cconj(Aa), wa);
-            const float2 cb = cscale(cconj(Ab), wb);
-            const float2 icb = make_float2(-cb.y, cb.x);          // i * cb
-            UV[(2 * j) * S7 + o] = cscale(csub(ca, icb), 0.5f);
-            UV[(2 * j + 1) * S7 + o] = cscale(cadd(ca, icb), 0.5f);
-          } else {
-            UV[2 * g.nch * S7 + o] = cconj(h);
+    by_store(g.store, [&](auto sf) {
+      constexpr int ST = decltype(sf)::value;
+      by_half<P, V>(g.ez, [&](auto hc) {
+        constexpr bool HALF = decltype(hc)::value;
+        // reduced-precision forms: the channels' z DFT on the tensor cores
+        if constexpr (ST != kStoreF32) {
+          if (g.tc && launch_zx_tc<P, ST>(F1, UV, g, nrot, st)) {
+            launch_zpass_t<P, ST, HALF, V, kZFromX>(F1, W, g.zx, F2, g, nrot, rot, st);
+            return;
           }
         }
-      }
-    }
-    __syncthreads();
-  }
+        launch_zpass_t<P, ST, HALF, V, kZFull>(F1, W, nullptr, F2, g, nrot, rot, st);
+      });
+    });
+  });
 }
 
 template <int P>
 void launch_prep_z(const float2* F1, float2* UV, Geo g, cudaStream_t st) {
-  constexpr int W = 8, N2 = Split<P>::N2;
-  const size_t smem = (size_t)2 * W * FourStep<P>::CS * sizeof(float2);
-  dim3 grid((unsigned)((g.Py + W - 1) / W), (unsigned)(g.Px / 2 + 1));
-  auto go = [&](auto kern) {
-    set_smem(kern, smem);
-    kern<<<grid, 2 * W * N2, smem, st>>>(F1, UV, g);
-  };
-  if (2 * g.ez <= P) go(k_prep_z<P, W, true>);
-  else go(k_prep_z<P, W, false>);
+  by_half<P, 0>(g.ez, [&](auto hc) {
+    launch_zpass_t<P, kStoreF32, decltype(hc)::value, 0, kZPrep>(F1, UV, nullptr, nullptr, g, 1, nullptr, st);
+  });
 }
 
 // ---------------------------------------------------------------------------

@@ -1,13 +1,8 @@
-// z pass of the reduced-precision forms with the forward z-axis DFT of the
-// channel fields on the tensor cores (tcgen05, FP32 accumulation in tensor
-// memory).  Included by passes.cuh; computes exactly what k_zmac computes
-// (Eq. 7-8: the weighted channel products summed in the spectrum, the mask
-// product, one inverse z transform of Z = X + iY), in two kernels:
-//
-//   k_zx_tc  the channel fields' forward transform as a dense real DFT on the
-//            tensor cores and the Eq. 7-8 sum X, written to HBM;
-//   k_zinv   the mask field's FP32 forward transform and Y on the CUDA
-//            cores, Z = X + iY, the inverse and the bound's planes to F2.
+// The channel fields' half of the z pass in the reduced-precision forms: their
+// forward z-axis DFT on the tensor cores (tcgen05, FP32 accumulation in tensor
+// memory) and the Eq. 7-8 sum X, written to HBM.  Included by passes.cuh;
+// k_zpass (kZFromX) reads X, transforms the mask field in FP32 and runs the
+// inverse.
 //
 // The dense DFT: for a column b(z), z < nz, of a packed complex field and
 // kz in [0, P/2]
@@ -31,17 +26,6 @@
 
 namespace csngf {
 
-// the CUDA-core half's block: W primary columns (kx, ky0 .. ky0 + W - 1) and
-// their mirrors, one thread per (column, n2) of the length's radix split
-template <int P, int V>
-struct ZinvCfg {
-  static constexpr int W = 8;
-  static constexpr int NC = 2 * W;
-  static constexpr int N2 = SplitV<P, V>::N2;
-  static constexpr int NT = NC * N2;
-  using FS = FourStep<P, (2 * W < 16), V>;
-};
-
 template <int ST>
 __device__ __forceinline__ void store16(unsigned char* p, float v) {
   if constexpr (ST == kStoreBF16) *reinterpret_cast<__nv_bfloat16*>(p) = __float2bfloat16_rn(v);
@@ -49,15 +33,13 @@ __device__ __forceinline__ void store16(unsigned char* p, float v) {
 }
 
 // ---------------------------------------------------------------------------
-// k_zx_tc forms X, the Eq. 7-8 sum of the weighted channel products, for
-// every column of the half spectrum kx <= P/2, in HBM; k_zinv reads it.  X
-// costs one write and one read of hx * Py * Pz complex values per rotation;
-// in exchange the tensor-core kernel double-buffers its operands and keeps no
-// CUDA-core transform in its per-rotation chain.
-// X layout: [r][kx <= P/2][ky][kz] (kz contiguous).
+// X costs one write and one read of a half spectrum of complex values per
+// rotation; in exchange the tensor-core kernel double-buffers its operands and
+// keeps no CUDA-core transform in its per-rotation chain.
+// X layout: [r][kx <= P/2][ky / 8][kz][ky % 8].
 //
 // k_zx_tc, per block: one kx, W = 8 ky columns and their mirrors, every
-// rotation of the launch; the cos / sin tiles and the block's U_j, V_j stay
+// rotation of the launch; the cos / sin tiles and the block's weights stay
 // in shared memory.  Rotation r + 1's MMAs run while rotation r's products
 // are summed; rotation r + 2's operand is copied (cp.async) as soon as
 // rotation r's MMAs are done.  16 warps, four per tensor-memory lane quarter.
@@ -83,7 +65,7 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
   using C = ZxTcCfg<P>;
   constexpr int W = C::W, NT = C::NT, TILE = W * P, HF = C::HF;
   const int NB = g.nch * 4 * W;                    // MMA N: (field, primary/mirror, column, re/im)
-  const int NUV = 2 * g.nch;                       // U_j, V_j
+  const int NUV = 2 * g.nch;                       // weight channels
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char* As = smem_raw;                    // [cos | sin][128][KP], K-major
   const uint32_t tileA = 128u * (uint32_t)KP * 2u;
@@ -97,22 +79,16 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int kx = blockIdx.y, ky0 = blockIdx.x * W;
   const int mkx = (g.Px - kx) % g.Px;
-  const long long hx = g.Px / 2 + 1;
-  const long long S7 = hx * g.Py * (long long)P;
+  const long long tiles = (long long)gridDim.x * gridDim.y, tile = (long long)kx * gridDim.x + blockIdx.x;
   const long long E = (long long)g.ez * g.Px * g.Py;
 
   for (uint32_t q = t; q < 2 * stageB / 16; q += NT)
     reinterpret_cast<uint4*>(Bs)[q] = make_uint4(0u, 0u, 0u, 0u);
-  {
-    const int valid = min(W, g.Py - ky0) * P;
-    for (int a = 0; a < NUV; ++a) {
-      const float2* src = UV + a * S7 + ((long long)kx * g.Py + ky0) * P;
-      float2* dst = uvs + a * TILE;
-      for (int q = t; q < TILE / 2; q += NT) {
-        if (2 * q < valid) cp_async16(dst + 2 * q, src + 2 * q);
-        else reinterpret_cast<float4*>(dst)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
+  // the block's weights, [channel][kz][column] in HBM, transposed so that kz runs
+  // over the lanes
+  for (int q = t; q < NUV * TILE; q += NT) {
+    const int a = q / TILE, i = q - a * TILE, c = i % W, k = i / W;
+    cp_async8(uvs + a * TILE + c * P + k, UV + (tile * (NUV + 1) + a) * TILE + i);
   }
   for (int m = warp; m < 128; m += NT / 32)
     for (int k = lane; k < KP; k += 32) {
@@ -216,7 +192,7 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
     if (t == 0 && r + 1 < nrot) issue(tmem, (r + 1) & 1);
     // (3) Eq. 7-8: X at kz and P - kz of this thread's four primary columns
     const uint32_t trow = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(s * 2 * NB);
-    float2* Xr = Xg + (((long long)r * hx + kx) * g.Py + ky0) * P;
+    float2* Xr = Xg + (r * tiles + tile) * TILE;
     {
       const int ch = cg;                           // primary columns 2 ch, 2 ch + 1
       uint32_t rc[3][4], rs[3][4], rcm[3][4], rsm[3][4];
@@ -231,11 +207,11 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
         }
       tc::wait_ld();
       if (kz_ok) {
+        float2 Xa[2], Xb[2];
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
           const int c = 2 * ch + i;
-          if (ky0 + c >= g.Py) continue;
-          float2 Xa = make_float2(0.f, 0.f), Xb = make_float2(0.f, 0.f);
+          Xa[i] = Xb[i] = make_float2(0.f, 0.f);
 #pragma unroll
           for (int j = 0; j < 3; ++j)
             if (j < g.nch) {
@@ -248,16 +224,20 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
               const float Smi = __uint_as_float(rsm[j][2 * i + 1]) * isc;
               const float2 Hk = make_float2(Cr + Si, Ci - Sr);
               const float2 Hp = make_float2(Cr - Si, Ci + Sr);
-              const float2 Mk = make_float2(Cmr + Smi, Cmi - Smr);
-              const float2 Mp = make_float2(Cmr - Smi, Cmi + Smr);
-              const float2* Uj = uvs + (2 * j) * TILE + c * P;
-              const float2* Vj = uvs + (2 * j + 1) * TILE + c * P;
-              Xa = cadd(Xa, cadd(cmul(Uj[kz], Hk), cmul(Vj[kz], cconj(Mp))));
-              Xb = cadd(Xb, cadd(cmul(Uj[kzm], Hp), cmul(Vj[kzm], cconj(Mk))));
+              const float2 Mk = make_float2(Cmr + Smi, -(Cmi - Smr));   // conjugates of the
+              const float2 Mp = make_float2(Cmr - Smi, -(Cmi + Smr));   // mirror's values
+              const float2* Wa = uvs + (2 * j) * TILE + c * P;
+              const float2* Wb = Wa + TILE;
+              // channels a = H + conj H', b = -i (H - conj H') at kz and P - kz
+              cmac(Xa[i], Wa[kz], cadd(Hk, Mp));
+              cmac(Xa[i], Wb[kz], mul_si<-1>(csub(Hk, Mp)));
+              cmac(Xb[i], Wa[kzm], cadd(Hp, Mk));
+              cmac(Xb[i], Wb[kzm], mul_si<-1>(csub(Hp, Mk)));
             }
-          Xr[c * P + kz] = Xa;
-          if (kzm != kz) Xr[c * P + kzm] = Xb;
         }
+        *reinterpret_cast<float4*>(Xr + kz * W + 2 * ch) = make_float4(Xa[0].x, Xa[0].y, Xa[1].x, Xa[1].y);
+        if (kzm != kz)
+          *reinterpret_cast<float4*>(Xr + kzm * W + 2 * ch) = make_float4(Xb[0].x, Xb[0].y, Xb[1].x, Xb[1].y);
       }
     }
     tc::fence_before_sync();
@@ -272,183 +252,23 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
   if (warp == 0) tc::dealloc(tmem, C::TMEM_COLS);
 }
 
-// the CUDA-core half: mask field forward z transform, Y = conj(M_A^) M_B^,
-// Z = X + iY with X from k_zx_tc, the inverse z transform and the bound's
-// shift planes to F2 (the same arithmetic as k_zmac for these steps)
-// Two blocks per SM (at most 96 registers a thread at the 320-thread 10 x 20
-// split; a few bytes spill): its 40 KB of shared memory allow it, and the
-// extra warps hide the transforms' latency (BF16 z pass 127 -> 114 ms per
-// 1000 rotations of the 150^3 workload).
-template <int P, int ST, bool HALF, int V>
-__global__ void __launch_bounds__(ZinvCfg<P, V>::NT, 2)
-k_zinv(const void* __restrict__ F1, const float2* __restrict__ Xg, const float2* __restrict__ UV,
-       float2* __restrict__ F2, Geo g, int nrot, const RotIn* __restrict__ rot) {
-  const float2* __restrict__ tw = kTw<P>.w;
-  using C = ZinvCfg<P, V>;
-  using FS = typename C::FS;
-  using FI = FwdIn<FS, HALF>;
-  constexpr int W = C::W, NC = C::NC, N1 = FS::N1, N2 = FS::N2, CS = FS::CS, NT = C::NT;
-  constexpr int HI = FI::NI;
-  constexpr int TILE = W * P, MI = (TILE + NT - 1) / NT;
-  extern __shared__ __align__(16) float2 smz[];
-  float2* ex = smz;                                // [NC][CS]
-  float2* Ms = ex + NC * CS;                       // [W][P] the mask weights conj(M_A^)
-  float2* tws = Ms + TILE;                         // [P]
-  const int t = threadIdx.x;
-  const int kx = blockIdx.y, ky0 = blockIdx.x * W;
-  const int mkx = (g.Px - kx) % g.Px;
-  const bool self_mirror = (2 * kx) % g.Px == 0;
-  const long long hx = g.Px / 2 + 1;
-  const long long S7 = hx * g.Py * (long long)P;
-  const long long E = (long long)g.ez * g.Px * g.Py;
-  auto slot = [](int kz) { return (kz / N1) * FS::RS + kz % N1; };
-  const int c1 = t % NC, n2 = t / NC;
-  const int pk1 = ky0 + (c1 < W ? c1 : c1 - W);
-  const bool ok1 = pk1 < g.Py;
-  const int ky1 = c1 < W ? pk1 : (g.Py - pk1) % g.Py;
-  const int kx1 = c1 < W ? kx : mkx;
-  const long long col_off = (long long)kx1 * g.ez * g.Py + ky1;
-  const bool has2 = t < NC * N1;
-  const int c2 = t % NC, k1 = t / NC;
-
-  {
-    const int valid = min(W, g.Py - ky0) * P;
-    const float2* src = UV + 2 * g.nch * S7 + ((long long)kx * g.Py + ky0) * P;
-    for (int q = t; q < TILE / 2; q += NT) {
-      if (2 * q < valid) cp_async16(Ms + 2 * q, src + 2 * q);
-      else reinterpret_cast<float4*>(Ms)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    cp_async_commit();
-  }
-  for (int q = t; q < P; q += NT) tws[q] = __ldg(&tw[q]);
-  float2 mv[HI];
-  auto load_m = [&](int r) {
-#pragma unroll
-    for (int n1 = 0; n1 < HI; ++n1) {
-      const int z = N2 * n1 + n2;
-      mv[n1] = make_float2(0.f, 0.f);
-      if (r < nrot && ok1 && z < g.ez) {
-        const float2* src = reinterpret_cast<const float2*>(Fields<ST>::field(F1, g, E, r, g.nch));
-        mv[n1] = __ldg(&src[col_off + (long long)z * g.Py]);
-      }
-    }
-  };
-  // X of this thread's (column, kz) elements, one rotation ahead
-  float2 xv[MI];
-  auto load_x = [&](int r) {
-#pragma unroll
-    for (int m = 0; m < MI; ++m) {
-      const int i = t + NT * m;
-      xv[m] = make_float2(0.f, 0.f);
-      if (r < nrot && i < TILE) {
-        const int c = i / P, kz = i - c * P;
-        if (ky0 + c < g.Py) xv[m] = __ldg(&Xg[(((long long)r * hx + kx) * g.Py + ky0 + c) * P + kz]);
-      }
-    }
-  };
-  auto step2_at = [&](int cc, int kk) {
-    float2 u[N2];
-    FS::template step2<-1>(u, ex + cc * CS, kk);
-#pragma unroll
-    for (int k2 = 0; k2 < N2; ++k2) ex[cc * CS + k2 * FS::RS + kk] = u[k2];
-  };
-  load_m(0);
-  load_x(0);
-  cp_async_wait_all();
-  __syncthreads();
-
-  float2 Y[MI], Yn[MI];
-#pragma unroll 1
-  for (int r = 0; r < nrot; ++r) {
-    if (!(r & 1)) {
-      FI::template step1<-1, true>(mv, ex + c1 * CS, n2, tws);
-      load_m(r + 2);
-      __syncthreads();
-      if (has2) step2_at(c2, k1);
-      __syncthreads();
-#pragma unroll
-      for (int m = 0; m < MI; ++m) {
-        const int i = t + NT * m;
-        if (i < TILE) {
-          const int c = i / P, kz = i - c * P;
-          const float2 h = ex[c * CS + slot(kz)];
-          const float2 hm = cconj(ex[(W + c) * CS + slot(kz == 0 ? 0 : P - kz)]);
-          const float2 U = Ms[i];
-          Y[m] = cmul(U, cscale(cadd(h, hm), 0.5f));
-          const float2 d = cscale(csub(h, hm), 0.5f);
-          Yn[m] = cmul(U, make_float2(d.y, -d.x));
-        }
-      }
-      __syncthreads();
-    } else {
-#pragma unroll
-      for (int m = 0; m < MI; ++m) Y[m] = Yn[m];
-    }
-    // Z = X + iY at k, conj(X) + i conj(Y) at -k
-#pragma unroll
-    for (int m = 0; m < MI; ++m) {
-      const int i = t + NT * m;
-      if (i < TILE) {
-        const int c = i / P, kz = i - c * P;
-        const float2 X = xv[m];
-        ex[c * CS + slot(kz)] = make_float2(X.x - Y[m].y, X.y + Y[m].x);
-        ex[(W + c) * CS + slot(kz == 0 ? 0 : P - kz)] = make_float2(X.x + Y[m].y, Y[m].x - X.y);
-      }
-    }
-    load_x(r + 1);
-    __syncthreads();
-    {
-      float2 v[N1];
-#pragma unroll
-      for (int n1 = 0; n1 < N1; ++n1) v[n1] = ex[c1 * CS + slot(N2 * n1 + n2)];
-      __syncthreads();
-      FS::template step1<1, true>(v, ex + c1 * CS, n2, tws);
-    }
-    __syncthreads();
-    if (has2 && !(c2 >= W && self_mirror)) {
-      const int pk2 = ky0 + (c2 < W ? c2 : c2 - W);
-      if (pk2 < g.Py) {
-        const int ky2 = c2 < W ? pk2 : (g.Py - pk2) % g.Py;
-        const int kx2 = c2 < W ? kx : mkx;
-        float2 u[N2];
-        FS::template step2<1>(u, ex + c2 * CS, k1);
-        float2* dst = F2 + ((long long)r * g.Px + kx2) * g.wz * g.Py + ky2;   // [r][kx][dz][ky]
-        const int m0 = rot[r].b.m0[0], last = rot[r].b.hi[0] - rot[r].b.lo[0];
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) {
-          const int dz = window_index(k1 + N1 * k2, m0, P);
-          if (dz <= last) dst[(long long)dz * g.Py] = u[k2];
-        }
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// the tensor-core z pass when g.zx (the X buffer) is set and the length,
-// precision form and shared memory allow it; false otherwise (the caller then
-// runs k_zmac)
-template <int P, int ST, bool HALF, int V>
-bool launch_zsplit_t(const void* F1, const float2* UV, float2* F2, Geo g, int nrot, const RotIn* rot,
-                     cudaStream_t st) {
+// the channel sum X into g.zx when the length, precision form and shared memory
+// allow it; false otherwise
+template <int P, int ST>
+bool launch_zx_tc(const void* F1, const float2* UV, Geo g, int nrot, cudaStream_t st) {
   using C1 = ZxTcCfg<P>;
-  using C2 = ZinvCfg<P, V>;
-  if constexpr (!C1::OK || ST == kStoreF32) {
+  if constexpr (!C1::OK) {
     return false;
   } else {
     if (!g.zx) return false;
     const int KP = (g.ez + 15) / 16 * 16;
     const int NB = g.nch * 4 * C1::W;
     if (NB > 128 || NB % 16 != 0) return false;
-    const size_t b1 = C1::bytes(KP, NB, 2 * g.nch);
-    if (b1 > 232448) return false;
-    const size_t s1 = std::max<size_t>(b1, 120 * 1024);   // one block per SM: all of its tensor memory
+    if (C1::bytes((g.nz + 15) / 16 * 16, NB, 2 * g.nch) > 232448) return false;
+    const size_t s1 = std::max<size_t>(C1::bytes(KP, NB, 2 * g.nch), 120 * 1024);   // one block per SM: all of its tensor memory
     set_smem(k_zx_tc<P, ST>, s1);
     dim3 grid((unsigned)((g.Py + C1::W - 1) / C1::W), (unsigned)(g.Px / 2 + 1));
     k_zx_tc<P, ST><<<grid, C1::NT, s1, st>>>(F1, UV, g.zx, g, nrot, KP);
-    const size_t s2 = ((size_t)C2::NC * C2::FS::CS + (size_t)C2::W * P + P) * sizeof(float2);
-    set_smem(k_zinv<P, ST, HALF, V>, s2);
-    k_zinv<P, ST, HALF, V><<<grid, C2::NT, s2, st>>>(F1, g.zx, UV, F2, g, nrot, rot);
     return true;
   }
 }
