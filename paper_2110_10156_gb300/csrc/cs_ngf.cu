@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <iterator>
 #include <map>
 #include <mutex>
 #include <string>
@@ -50,6 +51,10 @@ namespace {
   } while (0)
 
 constexpr int kPads[] = {16, 32, 40, 64, 80, 100, 128, 160, 192, 200, 216, 256, 320, 360, 400, 512};
+
+// the lengths box transforms take: those and the steps between (box_only)
+constexpr int kBoxPads[] = {16, 24, 32, 40, 48, 56, 64, 72, 80, 96, 100, 112, 120, 128, 144, 160, 168, 180, 192,
+                            200, 216, 240, 256, 280, 300, 320, 360, 400, 512};
 
 bool pad_supported(int p) {
   for (int v : kPads)
@@ -157,6 +162,19 @@ struct Stage {
     case 360: { constexpr int PP = 360; CALL; } break;                                  \
     case 400: { constexpr int PP = 400; CALL; } break;                                  \
     case 512: { constexpr int PP = 512; CALL; } break;                                  \
+    case 24: { constexpr int PP = 24; CALL; } break;                                    \
+    case 48: { constexpr int PP = 48; CALL; } break;                                    \
+    case 56: { constexpr int PP = 56; CALL; } break;                                    \
+    case 72: { constexpr int PP = 72; CALL; } break;                                    \
+    case 96: { constexpr int PP = 96; CALL; } break;                                    \
+    case 112: { constexpr int PP = 112; CALL; } break;                                  \
+    case 120: { constexpr int PP = 120; CALL; } break;                                  \
+    case 144: { constexpr int PP = 144; CALL; } break;                                  \
+    case 168: { constexpr int PP = 168; CALL; } break;                                  \
+    case 180: { constexpr int PP = 180; CALL; } break;                                  \
+    case 240: { constexpr int PP = 240; CALL; } break;                                  \
+    case 280: { constexpr int PP = 280; CALL; } break;                                  \
+    case 300: { constexpr int PP = 300; CALL; } break;                                  \
     default: break;                                                                     \
   }
 
@@ -617,8 +635,8 @@ Need box_need(const cs_ngf_fixed* f, const RotBounds& b) {
   for (int a = 0; a < 3 && q.any; ++a) {
     const int clo = b.lo[a] - (dims[a] - 1), chi = b.hi[a] - (dims[a] - 1);
     const int alias = std::max(b.b1[a] - f->a0[a] - clo, chi - b.b0[a] + f->a1[a]) + 1;
-    q.pad[a] = length_for(std::max(alias, std::max(b.b1[a] - b.b0[a], f->a1[a] - f->a0[a]) + 1),
-                          f->alloc_pad[a]);
+    const int points = std::max(alias, std::max(b.b1[a] - b.b0[a], f->a1[a] - f->a0[a]) + 1);
+    q.pad[a] = std::min(*std::lower_bound(std::begin(kBoxPads), std::end(kBoxPads), points), f->alloc_pad[a]);
   }
   return q;
 }
@@ -647,18 +665,19 @@ cs_ngf_status score_range_impl(cs_ngf_fixed* f, int r0_begin, int n, float* best
 // class costs a fixed-spectra recomputation and a partial launch group, about
 // kClassCost rotations of its own size; so two classes merge, with lengths raised to cover both, while the
 // cheapest merge adds less transform volume than that (and while there are
-// more than kMaxClasses).  Rotations admitting no shift join the first
+// more than kMaxClasses; kMaxBoxClasses for the closer spaced box lengths).  Rotations admitting no shift join the first
 // class.  The classes do not depend on the launch-group size, so results
 // stay the same for every even batch.
 constexpr double kClassCost = 4.0;
-constexpr size_t kMaxClasses = 8;
+constexpr size_t kMaxClasses = 8, kMaxBoxClasses = 16;
 struct LengthClass { int pad[3]; std::vector<int> rot; };
 
 double class_volume(const int* p) { return (double)p[0] * p[1] * p[2]; }
 
 // cur: the lengths in use (their class goes first); none: lengths when no
 // rotation admits a shift
-std::vector<LengthClass> length_classes(const std::vector<Need>& need, const int none_pad[3], const int cur[3]) {
+std::vector<LengthClass> length_classes(const std::vector<Need>& need, const int none_pad[3], const int cur[3],
+                                        size_t max_classes = kMaxClasses) {
   std::vector<LengthClass> cls;
   std::vector<int> none;
   for (int r = 0; r < (int)need.size(); ++r) {
@@ -687,7 +706,7 @@ std::vector<LengthClass> length_classes(const std::vector<Need>& need, const int
         }
       }
     const double keep = kClassCost * std::min(class_volume(cls[bc].pad), class_volume(cls[bd].pad));
-    if (best >= keep && cls.size() <= kMaxClasses) break;
+    if (best >= keep && cls.size() <= max_classes) break;
     std::copy(bm, bm + 3, cls[bc].pad);
     cls[bc].rot.insert(cls[bc].rot.end(), cls[bd].rot.begin(), cls[bd].rot.end());
     std::sort(cls[bc].rot.begin(), cls[bc].rot.end());
@@ -741,7 +760,7 @@ cs_ngf_status plan_classes_impl(cs_ngf_fixed* f, int R, cudaStream_t st, Plan& p
   if (f->boxed) {
     const int cur[3] = {g.Pz, g.Py, g.Px};
     for (int r = 0; r < R; ++r) need[r] = box_need(f, bounds[r]);
-    cls = length_classes(need, none_pad, cur);
+    cls = length_classes(need, none_pad, cur, kMaxBoxClasses);
   }
   f->run_pads.clear();
   f->run_counts.clear();

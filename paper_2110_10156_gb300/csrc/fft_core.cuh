@@ -211,11 +211,37 @@ struct Dft<5, S> {
   }
 };
 
+template <int S>
+struct Dft<7, S> {
+  __device__ __forceinline__ static void run(float2 (&v)[7]) {
+    constexpr float c[3] = {(float)ctw::cos2pi(1, 7), (float)ctw::cos2pi(2, 7), (float)ctw::cos2pi(3, 7)};
+    constexpr float s[3] = {(float)ctw::sin2pi(1, 7), (float)ctw::sin2pi(2, 7), (float)ctw::sin2pi(3, 7)};
+    const float2 x0 = v[0];
+    float2 t[3], d[3];
+    sfor<3>([&](auto ic) { constexpr int i = decltype(ic)::value; t[i] = cadd(v[i + 1], v[6 - i]); d[i] = csub(v[i + 1], v[6 - i]); });
+    v[0] = cadd(cadd(x0, t[0]), cadd(t[1], t[2]));
+    sfor<3>([&](auto kc) {                       // X_k = a + S i b, X_{7-k} = a - S i b
+      constexpr int k = decltype(kc)::value + 1;
+      float2 a = x0, b = make_float2(0.f, 0.f);
+      sfor<3>([&](auto ic) {
+        constexpr int i = decltype(ic)::value, e = (i + 1) * k % 7;
+        constexpr float ce = c[(e <= 3 ? e : 7 - e) - 1], se = e <= 3 ? s[e - 1] : -s[6 - e];
+        a = make_float2(a.x + ce * t[i].x, a.y + ce * t[i].y);
+        b = i == 0 ? make_float2(se * d[i].x, se * d[i].y) : make_float2(b.x + se * d[i].x, b.y + se * d[i].y);
+      });
+      const float2 ib = mul_si<S>(b);
+      v[k] = cadd(a, ib);
+      v[7 - k] = csub(a, ib);
+    });
+  }
+};
+
 constexpr int first_factor(int R) {
   return (R % 4 == 0 && R != 4) ? 4
          : (R % 2 == 0 && R != 2) ? 2
          : (R % 5 == 0 && R != 5) ? 5
          : (R % 3 == 0 && R != 3) ? 3
+         : (R % 7 == 0 && R != 7) ? 7
                                   : R;
 }
 
@@ -269,6 +295,19 @@ template <> struct SplitV<320, 0> { static constexpr int N1 = 16, N2 = 20; };
 template <> struct SplitV<360, 0> { static constexpr int N1 = 18, N2 = 20; };
 template <> struct SplitV<400, 0> { static constexpr int N1 = 16, N2 = 25; };
 template <> struct SplitV<512, 0> { static constexpr int N1 = 16, N2 = 32; };
+template <> struct SplitV<24, 0>  { static constexpr int N1 = 4,  N2 = 6; };
+template <> struct SplitV<48, 0>  { static constexpr int N1 = 6,  N2 = 8; };
+template <> struct SplitV<56, 0>  { static constexpr int N1 = 7,  N2 = 8; };
+template <> struct SplitV<72, 0>  { static constexpr int N1 = 8,  N2 = 9; };
+template <> struct SplitV<96, 0>  { static constexpr int N1 = 8,  N2 = 12; };
+template <> struct SplitV<112, 0> { static constexpr int N1 = 8,  N2 = 14; };
+template <> struct SplitV<120, 0> { static constexpr int N1 = 10, N2 = 12; };
+template <> struct SplitV<144, 0> { static constexpr int N1 = 12, N2 = 12; };
+template <> struct SplitV<168, 0> { static constexpr int N1 = 12, N2 = 14; };
+template <> struct SplitV<180, 0> { static constexpr int N1 = 12, N2 = 15; };
+template <> struct SplitV<240, 0> { static constexpr int N1 = 15, N2 = 16; };
+template <> struct SplitV<280, 0> { static constexpr int N1 = 14, N2 = 20; };
+template <> struct SplitV<300, 0> { static constexpr int N1 = 15, N2 = 20; };
 template <> struct SplitV<64, 1>  { static constexpr int N1 = 4,  N2 = 16; };
 template <> struct SplitV<80, 1>  { static constexpr int N1 = 4,  N2 = 20; };
 template <> struct SplitV<128, 1> { static constexpr int N1 = 4,  N2 = 32; };
@@ -283,6 +322,13 @@ template <> struct SplitV<400, 1> { static constexpr int N1 = 20, N2 = 20; };
 constexpr bool has_alt_split(int N) {
   return N == 64 || N == 80 || N == 128 || N == 160 || N == 192 || N == 200 || N == 216 || N == 256 ||
          N == 320 || N == 400;
+}
+// lengths that only box transforms use (FP32, built-in split): steps of about
+// 1/8 between the lengths the ABI offers.  At 150^3 the boxes need 138..164
+// points, which 144, 160 and 168 cover with 0.8 of the volume 160 and 192 take.
+constexpr bool box_only(int N) {
+  return N == 24 || N == 48 || N == 56 || N == 72 || N == 96 || N == 112 || N == 120 || N == 144 ||
+         N == 168 || N == 180 || N == 240 || N == 280 || N == 300;
 }
 template <int N>
 using Split = SplitV<N, 0>;

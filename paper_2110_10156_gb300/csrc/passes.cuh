@@ -36,9 +36,10 @@ struct FwdIn {
 };
 
 // calls f with the storage form of the channel fields as a compile-time constant
-template <class F>
+template <int P, class F>
 static void by_store(int store, F&& f) {
-  if (store == kStoreBF16) f(std::integral_constant<int, kStoreBF16>{});
+  if constexpr (box_only(P)) f(std::integral_constant<int, kStoreF32>{});
+  else if (store == kStoreBF16) f(std::integral_constant<int, kStoreBF16>{});
   else if (store == kStoreF16) f(std::integral_constant<int, kStoreF16>{});
   else f(std::integral_constant<int, kStoreF32>{});
 }
@@ -59,7 +60,7 @@ static void by_split(int v, F&& f) {
 // split's first factor is even, so that the pruned first step exists)
 template <int P, int V, class F>
 static void by_half(int e, F&& f) {
-  if constexpr (SplitV<P, V>::N1 % 2 == 0) {
+  if constexpr (SplitV<P, V>::N1 % 2 == 0 && !box_only(P)) {
     if (2 * e <= P) {
       f(std::true_type{});
       return;
@@ -256,7 +257,7 @@ void launch_fwd_x_t(const float* Bh, const uint8_t* Mh, void* F0, const RotIn* r
     set_smem(kern, smem);
     kern<<<blocks, ROWS * N2, smem, st>>>(Bh, Mh, F0, rot, g, nrows);
   };
-  by_store(g.store, [&](auto st) { go(k_fwd_x<P, ROWS, decltype(st)::value, HALF, V>); });
+  by_store<P>(g.store, [&](auto st) { go(k_fwd_x<P, ROWS, decltype(st)::value, HALF, V>); });
 }
 
 template <int P>
@@ -369,7 +370,7 @@ void launch_fwd_y_t(const void* F0, void* F1, Geo g, int nrot, cudaStream_t st) 
     set_smem(kern, smem);
     kern<<<grid, W * N2, smem, st>>>(F0, F1, g);
   };
-  by_store(g.store, [&](auto sf) {
+  by_store<P>(g.store, [&](auto sf) {
     constexpr int ST = decltype(sf)::value;
     by_half<P, V>(g.ey, [&](auto hc) { go(k_fwd_y<P, W, ST, decltype(hc)::value, V>); });
   });
@@ -393,7 +394,7 @@ void launch_zmac(const void* F1, const float2* UV, float2* F2, Geo g, int nrot, 
   float2* W = const_cast<float2*>(UV);            // written in the prepare mode only
   by_split<P>(v, [&](auto vc) {
     constexpr int V = decltype(vc)::value;
-    by_store(g.store, [&](auto sf) {
+    by_store<P>(g.store, [&](auto sf) {
       constexpr int ST = decltype(sf)::value;
       by_half<P, V>(g.ez, [&](auto hc) {
         constexpr bool HALF = decltype(hc)::value;

@@ -125,3 +125,26 @@ def test_another_fixed_volume_with_a_larger_box(cs):
     s2, c2 = [t.cpu().numpy() for t in g.score_rotations(dev(p.B), dev(p.MB), p.quats)]
     np.testing.assert_array_equal(sc, s2)
     np.testing.assert_array_equal(sh, c2)
+
+
+# lengths only box transforms take (csrc/fft_core.cuh box_only), and their neighbours below
+BOX_LENGTHS = {24: 16, 48: 40, 56: 48, 72: 64, 96: 80, 112: 100, 120: 112, 144: 128, 168: 160, 180: 168,
+               240: 216, 280: 256, 300: 280}
+
+
+@pytest.mark.parametrize("P", sorted(BOX_LENGTHS))
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_box_only_lengths_match_oracle(cs, P, axis):
+    """Full masks admit shifts to half the side, so a side of 2P/3 needs P points;
+    the map and the best shift of both rotations against the oracle."""
+    dims = [7, 9, 6]
+    dims[axis] = max(n for n in range(2, P) if n + n // 2 <= P)
+    p = synth.small_pair(300 + P + axis, tuple(dims), masks="full", n_rot=2)
+    f = cs.prepare_fixed(dev(p.A), dev(p.MA))
+    gmap = f.score_map(dev(p.B), dev(p.MB), [1.0, 0.0, 0.0, 0.0]).cpu().numpy()
+    (ran, _), = f.transform_classes()
+    assert ran[axis] == P
+    check_maps(O.score_map(p.A, p.MA, p.B, p.MB, [1.0, 0.0, 0.0, 0.0])[0], gmap)
+    sc, sh = [t.cpu().numpy() for t in f.score_rotations(dev(p.B), dev(p.MB), p.quats)]
+    for r, q in enumerate(p.quats):
+        check_best_against_map(O.score_map(p.A, p.MA, p.B, p.MB, q)[0], sc[r], sh[r])
