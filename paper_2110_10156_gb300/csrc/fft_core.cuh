@@ -68,6 +68,20 @@ constexpr TwTable<P> make_twiddles() {
 }
 template <int P>
 __device__ const TwTable<P> kTw = make_twiddles<P>();
+// the first step's twiddles exp(-2 pi i k1 n2 / P) as [k1][n2]: lanes over n2 read
+// consecutive entries
+template <int P, int N1, int N2>
+constexpr TwTable<P> make_step_twiddles() {
+  TwTable<P> t{};
+  for (int k = 0; k < N1; ++k)
+    for (int n = 0; n < N2; ++n) {
+      t.w[k * N2 + n].x = (float)ctw::cos2pi((long)k * n, P);
+      t.w[k * N2 + n].y = (float)(-ctw::sin2pi((long)k * n, P));
+    }
+  return t;
+}
+template <int P, int N1, int N2>
+__device__ const TwTable<P> kTwStep = make_step_twiddles<P, N1, N2>();
 
 // ---------------------------------------------------------------- complex
 // Complex add and subtract as one paired FP32 instruction (add/sub.rn.f32x2:
@@ -143,20 +157,76 @@ __device__ __forceinline__ float2 tw_mul(float2 x) {
     return make_float2(x.x * c - x.y * s, x.x * s + x.y * c);
   }
 }
+// a + S i d, a - S i d; a + c t, c t
+template <int S> __device__ __forceinline__ float2 add_si(float2 a, float2 d) { return cadd(a, mul_si<S>(d)); }
+template <int S> __device__ __forceinline__ float2 sub_si(float2 a, float2 d) { return csub(a, mul_si<S>(d)); }
+__device__ __forceinline__ float2 cmad(float2 a, float2 t, float c) { return make_float2(a.x + c * t.x, a.y + c * t.y); }
+
+// Two complex values side by side, x their real and y their imaginary parts:
+// every step of two transforms at once is paired FP32 instructions without
+// moves between lanes, half the issue slots (the z pass: 30 M warp
+// instructions per rotation with one value per step, issue-bound latency at
+// 16 warps per SM).
+struct __align__(16) c2 { float2 x, y; };
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 pa, pb, pr;\n\tmov.b64 pa, {%2, %3};\n\tmov.b64 pb, {%4, %5};\n\t"
+      "mul.rn.f32x2 pr, pa, pb;\n\tmov.b64 {%0, %1}, pr;\n\t}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 r;
+  asm("{\n\t.reg .b64 pa, pb, pc, pr;\n\tmov.b64 pa, {%2, %3};\n\tmov.b64 pb, {%4, %5};\n\t"
+      "mov.b64 pc, {%6, %7};\n\tfma.rn.f32x2 pr, pa, pb, pc;\n\tmov.b64 {%0, %1}, pr;\n\t}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
+}
+__device__ __forceinline__ float2 dup(float s) { return make_float2(s, s); }
+__device__ __forceinline__ c2 cadd(c2 a, c2 b) { return {cadd(a.x, b.x), cadd(a.y, b.y)}; }
+__device__ __forceinline__ c2 csub(c2 a, c2 b) { return {csub(a.x, b.x), csub(a.y, b.y)}; }
+__device__ __forceinline__ c2 cscale(c2 a, float s) { return {mul2(a.x, dup(s)), mul2(a.y, dup(s))}; }
+__device__ __forceinline__ c2 cmad(c2 a, c2 t, float c) { return {fma2(t.x, dup(c), a.x), fma2(t.y, dup(c), a.y)}; }
+template <int S> __device__ __forceinline__ c2 add_si(c2 a, c2 d) {
+  return S < 0 ? c2{cadd(a.x, d.y), csub(a.y, d.x)} : c2{csub(a.x, d.y), cadd(a.y, d.x)};
+}
+template <int S> __device__ __forceinline__ c2 sub_si(c2 a, c2 d) { return add_si<-S>(a, d); }
+// both values times w = (wx, wx), (wy, wy)
+__device__ __forceinline__ c2 cmul(c2 v, c2 w) {
+  const float2 n = make_float2(-w.y.x, -w.y.y);
+  return {fma2(v.y, n, mul2(v.x, w.x)), fma2(v.x, w.y, mul2(v.y, w.x))};
+}
+template <int R, int S, int E>
+__device__ __forceinline__ c2 tw_mul(c2 v) {
+  constexpr int e = ((E % R) + R) % R;
+  if constexpr (e == 0) {
+    return v;
+  } else {
+    constexpr float c = (float)ctw::cos2pi(e, R);
+    constexpr float s = (float)(S * ctw::sin2pi(e, R));
+    if constexpr (2 * e == R) return {mul2(v.x, dup(-1.0f)), mul2(v.y, dup(-1.0f))};
+    else if constexpr (4 * e == R || 4 * e == 3 * R)
+      return s < 0 ? c2{v.y, mul2(v.x, dup(-1.0f))} : c2{mul2(v.y, dup(-1.0f)), v.x};
+    else return {fma2(v.y, dup(-s), mul2(v.x, dup(c))), fma2(v.x, dup(s), mul2(v.y, dup(c)))};
+  }
+}
 
 // ---------------------------------------------------------------- DFTs
+// of R values of T (float2: one complex value, c2: two side by side)
 template <int R, int S>
 struct Dft;
 
 template <int S>
 struct Dft<1, S> {
-  __device__ __forceinline__ static void run(float2 (&)[1]) {}
+  template <class T>
+  __device__ __forceinline__ static void run(T (&)[1]) {}
 };
 
 template <int S>
 struct Dft<2, S> {
-  __device__ __forceinline__ static void run(float2 (&v)[2]) {
-    float2 a = v[0], b = v[1];
+  template <class T>
+  __device__ __forceinline__ static void run(T (&v)[2]) {
+    T a = v[0], b = v[1];
     v[0] = cadd(a, b);
     v[1] = csub(a, b);
   }
@@ -164,74 +234,73 @@ struct Dft<2, S> {
 
 template <int S>
 struct Dft<3, S> {
-  __device__ __forceinline__ static void run(float2 (&v)[3]) {
+  template <class T>
+  __device__ __forceinline__ static void run(T (&v)[3]) {
     constexpr float c1 = (float)ctw::cos2pi(1, 3), s1 = (float)ctw::sin2pi(1, 3);
-    const float2 t = cadd(v[1], v[2]), d = csub(v[1], v[2]);
-    const float2 x0 = v[0];
+    const T t = cadd(v[1], v[2]), d = csub(v[1], v[2]);
+    const T x0 = v[0];
     v[0] = cadd(x0, t);
-    const float2 a = make_float2(x0.x + c1 * t.x, x0.y + c1 * t.y);
-    const float2 ib = mul_si<S>(make_float2(s1 * d.x, s1 * d.y));   // S i sin(2 pi/3) (x1 - x2)
-    // X1 = a + S i b, X2 = a - S i b
-    v[1] = cadd(a, ib);
-    v[2] = csub(a, ib);
+    const T a = cmad(x0, t, c1), b = cscale(d, s1);
+    v[1] = add_si<S>(a, b);                      // a + S i sin(2 pi/3) (x1 - x2)
+    v[2] = sub_si<S>(a, b);
   }
 };
 
 template <int S>
 struct Dft<4, S> {
-  __device__ __forceinline__ static void run(float2 (&v)[4]) {
-    float2 a0 = cadd(v[0], v[2]), a1 = csub(v[0], v[2]);
-    float2 b0 = cadd(v[1], v[3]), b1 = mul_si<S>(csub(v[1], v[3]));
+  template <class T>
+  __device__ __forceinline__ static void run(T (&v)[4]) {
+    T a0 = cadd(v[0], v[2]), a1 = csub(v[0], v[2]);
+    T b0 = cadd(v[1], v[3]), b1 = csub(v[1], v[3]);
     v[0] = cadd(a0, b0);
     v[2] = csub(a0, b0);
-    v[1] = cadd(a1, b1);
-    v[3] = csub(a1, b1);
+    v[1] = add_si<S>(a1, b1);
+    v[3] = sub_si<S>(a1, b1);
   }
 };
 
 template <int S>
 struct Dft<5, S> {
-  __device__ __forceinline__ static void run(float2 (&v)[5]) {
-    constexpr float c1 = (float)ctw::cos2pi(1, 5), c2 = (float)ctw::cos2pi(2, 5);
+  template <class T>
+  __device__ __forceinline__ static void run(T (&v)[5]) {
+    constexpr float c1 = (float)ctw::cos2pi(1, 5), c2_ = (float)ctw::cos2pi(2, 5);
     constexpr float s1 = (float)ctw::sin2pi(1, 5), s2 = (float)ctw::sin2pi(2, 5);
-    float2 t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
-    float2 t3 = csub(v[1], v[4]), t4 = csub(v[2], v[3]);
-    float2 x0 = v[0];
+    T t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
+    T t3 = csub(v[1], v[4]), t4 = csub(v[2], v[3]);
+    T x0 = v[0];
     v[0] = cadd(x0, cadd(t1, t2));
-    float2 a1 = make_float2(x0.x + c1 * t1.x + c2 * t2.x, x0.y + c1 * t1.y + c2 * t2.y);
-    float2 a2 = make_float2(x0.x + c2 * t1.x + c1 * t2.x, x0.y + c2 * t1.y + c1 * t2.y);
-    float2 b1 = make_float2(s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y);
-    float2 b2 = make_float2(s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y);
-    // forward: X1 = a1 - i b1, X4 = a1 + i b1, X2 = a2 - i b2, X3 = a2 + i b2
-    float2 ib1 = mul_si<S>(b1), ib2 = mul_si<S>(b2);   // S i b
-    v[1] = cadd(a1, ib1);
-    v[4] = csub(a1, ib1);
-    v[2] = cadd(a2, ib2);
-    v[3] = csub(a2, ib2);
+    const T a1 = cmad(cmad(x0, t1, c1), t2, c2_), a2 = cmad(cmad(x0, t1, c2_), t2, c1);
+    const T b1 = cmad(cscale(t3, s1), t4, s2), b2 = cmad(cscale(t3, s2), t4, -s1);
+    // X1 = a1 + S i b1, X4 = a1 - S i b1, X2 = a2 + S i b2, X3 = a2 - S i b2
+    v[1] = add_si<S>(a1, b1);
+    v[4] = sub_si<S>(a1, b1);
+    v[2] = add_si<S>(a2, b2);
+    v[3] = sub_si<S>(a2, b2);
   }
 };
 
 template <int S>
 struct Dft<7, S> {
-  __device__ __forceinline__ static void run(float2 (&v)[7]) {
+  template <class T>
+  __device__ __forceinline__ static void run(T (&v)[7]) {
     constexpr float c[3] = {(float)ctw::cos2pi(1, 7), (float)ctw::cos2pi(2, 7), (float)ctw::cos2pi(3, 7)};
     constexpr float s[3] = {(float)ctw::sin2pi(1, 7), (float)ctw::sin2pi(2, 7), (float)ctw::sin2pi(3, 7)};
-    const float2 x0 = v[0];
-    float2 t[3], d[3];
+    const T x0 = v[0];
+    T t[3], d[3];
     sfor<3>([&](auto ic) { constexpr int i = decltype(ic)::value; t[i] = cadd(v[i + 1], v[6 - i]); d[i] = csub(v[i + 1], v[6 - i]); });
     v[0] = cadd(cadd(x0, t[0]), cadd(t[1], t[2]));
     sfor<3>([&](auto kc) {                       // X_k = a + S i b, X_{7-k} = a - S i b
       constexpr int k = decltype(kc)::value + 1;
-      float2 a = x0, b = make_float2(0.f, 0.f);
+      T a = x0, b;
       sfor<3>([&](auto ic) {
         constexpr int i = decltype(ic)::value, e = (i + 1) * k % 7;
         constexpr float ce = c[(e <= 3 ? e : 7 - e) - 1], se = e <= 3 ? s[e - 1] : -s[6 - e];
-        a = make_float2(a.x + ce * t[i].x, a.y + ce * t[i].y);
-        b = i == 0 ? make_float2(se * d[i].x, se * d[i].y) : make_float2(b.x + se * d[i].x, b.y + se * d[i].y);
+        a = cmad(a, t[i], ce);
+        if constexpr (i == 0) b = cscale(d[i], se);
+        else b = cmad(b, d[i], se);
       });
-      const float2 ib = mul_si<S>(b);
-      v[k] = cadd(a, ib);
-      v[7 - k] = csub(a, ib);
+      v[k] = add_si<S>(a, b);
+      v[7 - k] = sub_si<S>(a, b);
     });
   }
 };
@@ -251,11 +320,12 @@ struct Dft {
   static constexpr int A = first_factor(R);
   static constexpr int B = R / A;
   static_assert(A * B == R && A > 1 && B > 1, "unsupported DFT length");
-  __device__ __forceinline__ static void run(float2 (&v)[R]) {
-    float2 t[B][A];
+  template <class T>
+  __device__ __forceinline__ static void run(T (&v)[R]) {
+    T t[B][A];
     sfor<B>([&](auto bc) {
       constexpr int b = decltype(bc)::value;
-      float2 s[A];
+      T s[A];
       sfor<A>([&](auto ac) { constexpr int a = decltype(ac)::value; s[a] = v[B * a + b]; });
       Dft<A, S>::run(s);
       sfor<A>([&](auto kc) {
@@ -265,13 +335,29 @@ struct Dft {
     });
     sfor<A>([&](auto kc) {
       constexpr int ka = decltype(kc)::value;
-      float2 u[B];
+      T u[B];
       sfor<B>([&](auto bc) { constexpr int b = decltype(bc)::value; u[b] = t[b][ka]; });
       Dft<B, S>::run(u);
       sfor<B>([&](auto kb) { constexpr int k = decltype(kb)::value; v[ka + A * k] = u[k]; });
     });
   }
 };
+
+// R-point transform of R/2 values and R/2 zeros: two R/2-point ones,
+// X[2m] = DFT(x)[m], X[2m+1] = DFT(x W_R^n)[m]
+template <int R, int S, class T>
+__device__ __forceinline__ void dft_half(T (&x)[R / 2], T (&v)[R]) {
+  static_assert(R % 2 == 0);
+  T o[R / 2];
+  sfor<R / 2>([&](auto nc) { constexpr int n = decltype(nc)::value; o[n] = tw_mul<R, S, n>(x[n]); });
+  Dft<R / 2, S>::run(x);
+  Dft<R / 2, S>::run(o);
+#pragma unroll
+  for (int m = 0; m < R / 2; ++m) {
+    v[2 * m] = x[m];
+    v[2 * m + 1] = o[m];
+  }
+}
 
 // ---------------------------------------------------------------- four-step
 // N = N1 * N2 with N1 <= N2 (step 2 then has at most one item per thread).
@@ -353,8 +439,7 @@ struct FourStep {
   }
 
   // v holds x[N2*n1 + n2] for n1 = 0..N1-1; writes twiddled N1-point outputs
-  // (exchange elements lie W apart: callers with W sequences interleaved)
-  template <int S, bool TS = false, int W = 1>
+  template <int S, bool TS = false>
   __device__ __forceinline__ static void step1(float2 (&v)[N1], float2* ex_seq, int n2,
                                                const float2* __restrict__ twN) {
     Dft<N1, S>::run(v);
@@ -362,33 +447,7 @@ struct FourStep {
     for (int k1 = 0; k1 < N1; ++k1) {
       float2 w = twl<TS>(&twN[n2 * k1]);
       if (S > 0) w.y = -w.y;
-      ex_seq[(n2 * RS + k1) * W] = (k1 == 0) ? v[k1] : cmul(v[k1], w);
-    }
-  }
-
-  // Same as step1 when the input is zero for n1 >= N1/2 (a forward transform
-  // of data zero-padded from length <= N/2): the N1-point DFT splits into two
-  // N1/2-point DFTs, X[2m] = DFT(x)[m], X[2m+1] = DFT(x * W_N1^n)[m].
-  static constexpr int H = N1 / 2;
-  template <int S, bool TS = false, int W = 1>
-  __device__ __forceinline__ static void step1_half(float2 (&v)[H], float2* ex_seq, int n2,
-                                                    const float2* __restrict__ twN) {
-    static_assert(N1 % 2 == 0, "half-zero step needs an even N1");
-    float2 e[H], o[H];
-    sfor<H>([&](auto nc) {
-      constexpr int n = decltype(nc)::value;
-      e[n] = v[n];
-      o[n] = tw_mul<N1, S, n>(v[n]);
-    });
-    Dft<H, S>::run(e);
-    Dft<H, S>::run(o);
-#pragma unroll
-    for (int m = 0; m < H; ++m) {
-      const int ke = 2 * m, ko = 2 * m + 1;
-      float2 we = twl<TS>(&twN[n2 * ke]), wo = twl<TS>(&twN[n2 * ko]);
-      if (S > 0) { we.y = -we.y; wo.y = -wo.y; }
-      ex_seq[(n2 * RS + ke) * W] = (m == 0) ? e[m] : cmul(e[m], we);
-      ex_seq[(n2 * RS + ko) * W] = cmul(o[m], wo);
+      ex_seq[n2 * RS + k1] = (k1 == 0) ? v[k1] : cmul(v[k1], w);
     }
   }
 

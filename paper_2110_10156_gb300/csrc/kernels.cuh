@@ -14,11 +14,13 @@
 //
 // Data layout (all [slow]...[fast], complex64 = float2):
 //   Bh, Mh   [r][z][y][x]                     float / uint8
-//   F0       [r][j][z][y][kx]     j < nf       x transformed
-//   F1       [r][j][kx][z][ky]                  x, y transformed
-//   F2       [r][kx][dz][ky]                    Z = X + iY after the z inverse
+//   F0       [r][j][z][kx/4][y][kx%4]  j < nf   x transformed
+//   F1       [r][j][kx][p/4][z][p%4]            x, y transformed
+//   F2       [r][kx][dz][p]                     Z = X + iY after the z inverse
 //   F3       [r][dz][dy][kx]                    after the y inverse
-//   UV       [kx <= Px/2][ky/8][2nch+1][kz][ky%8]  fixed-volume weights (prepare)
+//   UV       [kx <= Px/2][p/4][j][kz][p%4][a, b]  fixed-volume weights (zpass.cuh)
+// p orders ky so that a tile of four and the tile of their mirrors -ky are both
+// contiguous (ky_pos).
 // z, y of F0 and F1 count from the rotation's box origin (RotBox::org) and run
 // over the class's extents (Geo::ez, ey); dz, dy count from the first shift
 // slot that can be valid (RotBox::lo) over the class's windows (Geo::wz, wy).
@@ -54,14 +56,25 @@ struct Geo {
   // 1: in the BF16 and FP16 forms the z pass runs the forward z-axis DFT of
   // the channel fields on the tensor cores (k_zmac_tc) where its length allows
   int tc;
-  // set to 1 by a tensor-core pass whose bounded wait for its own MMAs ran out
+  // set to 1 by a z pass whose bounded wait for its own MMAs or copies ran out
   // (it then stops and returns); nullptr: not reported
   int* tc_err;
-  // X of the tensor-core z pass, [r][kx <= Px/2][ky/8][kz][ky%8] per launch group
+  // X of the tensor-core z pass, [r][kx <= Px/2][p/4][kz][p%4] per launch group
   // (the handle allocates it with the tensor-core forms); nullptr: the z pass
   // runs as one kernel
   float2* zx;
 };
+
+// Order of the ky axis in F1, F2 and the weights: first half ky = 0 .. P/2 - 1,
+// second half P/2, P - 1, P - 2, ... P/2 + 1, each half padded to a multiple of
+// four.  Four positions make a tile; the mirrors -ky of a tile's columns are
+// the other half's tile in the same order, except ky = 0 and P/2, their own
+// mirrors (position 0 of a half).
+__host__ __device__ constexpr int ky_half(int P) { return (P / 2 + 3) / 4 * 4; }
+__host__ __device__ constexpr int ky_total(int P) { return 2 * ky_half(P); }
+__host__ __device__ constexpr int ky_pos(int ky, int P) {
+  return 2 * ky < P ? ky : ky_half(P) + (2 * ky == P ? 0 : P - ky);
+}
 
 constexpr int kStoreF32 = 0, kStoreBF16 = 1, kStoreF16 = 2;
 
@@ -91,14 +104,15 @@ struct Fields {
     return (const char*)base + (long long)r * rot_bytes(g, E) + (long long)j * E * CB;
   }
   // scale: the field's storage scale (FP16 form; ignored otherwise)
-  __device__ __forceinline__ static void put(char* f, long long i, float2 v, bool mask, float scale) {
+  // (an index counts one field's values, < 2^27: byte offsets fit 32 bits)
+  __device__ __forceinline__ static void put(char* f, unsigned i, float2 v, bool mask, float scale) {
     if (ST == kStoreBF16 && !mask) reinterpret_cast<__nv_bfloat162*>(f)[i] = __float22bfloat162_rn(v);
     else if (ST == kStoreF16 && !mask)
       reinterpret_cast<__half2*>(f)[i] = __float22half2_rn(make_float2(v.x * scale, v.y * scale));
     else reinterpret_cast<float2*>(f)[i] = v;
   }
   // inv_scale: 1 / the field's storage scale (FP16 form; ignored otherwise)
-  __device__ __forceinline__ static float2 get(const char* f, long long i, bool mask, float inv_scale) {
+  __device__ __forceinline__ static float2 get(const char* f, unsigned i, bool mask, float inv_scale) {
     if (ST == kStoreBF16 && !mask) return __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(f)[i]);
     if (ST == kStoreF16 && !mask) {
       const float2 v = __half22float2(reinterpret_cast<const __half2*>(f)[i]);

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "kernels.cuh"
+#include "tc.cuh"
 
 namespace csngf {
 
@@ -14,26 +15,6 @@ namespace csngf {
 // P >= max(b1 - a0 - chi_lo, chi_hi - (b0 - a1)) + 1, which the caller
 // guarantees (for masks that fill the volume that is n + max(-chi_lo, chi_hi),
 // and for every shift 2n - 1).
-
-// Forward-transform inputs: box extents e are zero padded to P.  When
-// e <= P/2 the upper half of every step-1 sequence is zero and step 1 is the
-// pruned form (FourStep::step1_half); otherwise all N1 inputs are read.
-template <class FS, bool HALF>
-struct FwdIn {
-  static constexpr int NI = HALF ? FS::N1 / 2 : FS::N1;   // step-1 inputs per thread
-  template <int S, bool TS = false>
-  __device__ __forceinline__ static void step1(float2 (&v)[NI], float2* ex_seq, int n2,
-                                               const float2* __restrict__ twN) {
-    if constexpr (HALF) FS::template step1_half<S, TS>(v, ex_seq, n2, twN);
-    else FS::template step1<S, TS>(v, ex_seq, n2, twN);
-  }
-  // the same to an exchange whose elements lie W apart, twiddles in shared memory
-  template <int S, int W>
-  __device__ __forceinline__ static void step1w(float2 (&v)[NI], float2* ex_row, int n2, const float2* tws) {
-    if constexpr (HALF) FS::template step1_half<S, true, W>(v, ex_row - n2 * FS::RS * W, n2, tws);
-    else FS::template step1<S, true, W>(v, ex_row - n2 * FS::RS * W, n2, tws);
-  }
-};
 
 // calls f with the storage form of the channel fields as a compile-time constant
 template <int P, class F>
@@ -56,11 +37,24 @@ static void by_split(int v, F&& f) {
   f(std::integral_constant<int, 0>{});
 }
 
-// calls f with whether a box extent e fills at most half the length (where the
-// split's first factor is even, so that the pruned first step exists)
+// calls f with whether a box extent e fills at most half the length: the upper
+// half of every first-step sequence is then zero and the step is pruned
+// (dft_half; where the split's first factor is even)
 template <int P, int V, class F>
 static void by_half(int e, F&& f) {
   if constexpr (SplitV<P, V>::N1 % 2 == 0 && !box_only(P)) {
+    if (2 * e <= P) {
+      f(std::true_type{});
+      return;
+    }
+  }
+  f(std::false_type{});
+}
+
+// the same for the z pass, whose first step takes the larger factor
+template <int P, int V, class F>
+static void by_half_z(int e, F&& f) {
+  if constexpr (SplitV<P, V>::N2 % 2 == 0 && !box_only(P)) {
     if (2 * e <= P) {
       f(std::true_type{});
       return;
@@ -75,189 +69,216 @@ static void set_smem(K kern, size_t bytes) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-// ---------------------------------------------------------------------------
-// fwd_x: Eq. 1 NGF of the resampled volume, the Eq. 6 channels packed in four
-// complex fields, and the x-axis FFT of every row (zero padded to Px).
-// Block: ROWS rows of one slab; thread (row, n2) gathers x = N2*n1 + n2.
-// ---------------------------------------------------------------------------
-// A thread keeps the NGF (x, y, z, mask) of its step-1 inputs across the
-// four fields: in registers for half-length inputs, in its own slots of
-// shared memory [NI][NT] (float4) for full-length ones, which would spill.
-template <int P, bool HALF, int V>
-struct FwdXCfg {
-  static constexpr int N2 = SplitV<P, V>::N2;
-  static constexpr int ROWS = (256 / N2) > 0 ? (256 / N2) : 1;
-  static constexpr int NT = ROWS * N2;
-  static constexpr int NI = FwdIn<FourStep<P, true, V>, HALF>::NI;
-  static constexpr size_t ex_bytes = ((size_t)ROWS * FourStep<P, true, V>::CS * sizeof(float2) + 15) / 16 * 16;
-  static constexpr size_t smem_bytes = ex_bytes + (HALF ? 0 : (size_t)NI * NT * sizeof(float4));
-  // three blocks per SM (at most 80 registers per thread): the gradient
-  // gathers and the per-field barriers leave the pass latency-bound, and the
-  // extra resident warps hide more of it than the few spilled registers cost
-  // (measured: 200-point lengths 2.13 -> 1.67 ms per 32 rotations, 320-point
-  // half-input lengths 72 -> 65 ms per 1000 rotations; 400 and 320 unchanged)
-  static constexpr int MIN_BLOCKS = 3;
+// Offsets of a second step's outputs in a tiled axis: tiles of four consecutive
+// indices, each with L entries per index ([i / 4][L][i % 4]).  Index k + N1 m for
+// compile-time m advances by N1 L every PER = 4 / gcd(4, N1) steps, so a thread
+// computes PER offsets once.
+__device__ __forceinline__ int tile_off(int i, int L) { return (i >> 2) * 4 * L + (i & 3); }
+template <int N1>
+struct TileRun {
+  static constexpr int PER = N1 % 4 == 0 ? 1 : N1 % 2 == 0 ? 2 : 4;
+  int b[PER], step;
+  __device__ __forceinline__ TileRun(int k, int L) : step(N1 * PER * L) {
+#pragma unroll
+    for (int e = 0; e < PER; ++e) b[e] = tile_off(k + N1 * e, L);
+  }
+  __device__ __forceinline__ int at(int m) const { return b[m % PER] + m / PER * step; }
+};
+// the same for ky = k1 + N1 k2 in the order of ky_pos
+template <int P, int N1, int N2>
+struct KyRun {
+  TileRun<N1> up, down;
+  int k1, L;
+  __device__ __forceinline__ KyRun(int k1_, int L_) : up(k1_, L_), down(N1 - k1_, L_), k1(k1_), L(L_) {}
+  __device__ __forceinline__ int at(int k2) const {
+    if (N1 * (k2 + 1) <= P / 2) return up.at(k2);                       // first half for every k1
+    const int second = ky_half(P) * L + down.at(N2 - 1 - k2);           // P - ky = N1 (N2 - 1 - k2) + N1 - k1
+    if (N1 * k2 > P / 2) return second;
+    const int ky2 = 2 * (k1 + N1 * k2);
+    return ky2 < P ? up.at(k2) : ky2 == P ? ky_half(P) * L : second;
+  }
 };
 
-template <int P, int ROWS, int ST, bool HALF, int V>
-__global__ void __launch_bounds__(ROWS * SplitV<P, V>::N2, FwdXCfg<P, HALF, V>::MIN_BLOCKS)
+// Blocks per SM for the passes: as many as keep at least
+// MINR registers per thread (each of the SM's four sub-partitions holds 16384
+// registers for the warps placed on it) and fit in shared memory.
+constexpr int pass_blocks(int threads, size_t smem, int minr) {
+  int best = 1;
+  for (int b = 2; b <= 8; ++b) {
+    const int per_sub = (b * ((threads + 31) / 32) + 3) / 4;
+    const int regs = (16384 / (32 * per_sub)) / 8 * 8;
+    if (regs >= minr && (size_t)b * (smem + 1024) <= 228 * 1024) best = b;
+  }
+  return best;
+}
+
+// ---------------------------------------------------------------------------
+// fwd_x: Eq. 1 NGF of the resampled volume, the Eq. 6 channels packed in four
+// complex fields, and the x-axis FFT of every row of the box (zero padded to
+// Px).  Block: ROWS rows; thread (row, n2) gathers x = N2*n1 + n2.
+// ---------------------------------------------------------------------------
+// Two fields travel side by side (c2): (j = 0, 1), then (j = 2, mask), half the
+// instructions and half the barriers of one after the other.  The second
+// pair's inputs wait in the thread's own shared-memory slots [NI][NT].
+// What bounds it: the gradient's gathers through L1 (68 % of its throughput
+// before) and their latency.  Most voxels of a box lie outside the mask (two
+// thirds at 150^3), so the masks are read first and a masked-out voxel's
+// gathers go to its row's first voxel, one sector per warp.
+template <int P, bool HALF, int V>
+struct FwdXCfg {
+  static constexpr int N1 = SplitV<P, V>::N1, N2 = SplitV<P, V>::N2;
+  static constexpr int ROWS = 128 / N2 > 0 ? 128 / N2 : 1;
+  static constexpr int NT = ROWS * N2;
+  static constexpr int NI = HALF ? N1 / 2 : N1;
+  // exchange [row][n2][k1] of pairs: odd row length, and rows N1 apart (mod 8),
+  // put eight consecutive lanes of either step in different 16-byte banks
+  static constexpr int RS = N1 | 1, CS0 = N2 * RS, CS = CS0 + ((N1 - CS0) % 8 + 8) % 8;
+  static constexpr size_t smem_bytes = ((size_t)ROWS * CS + (size_t)NI * NT) * sizeof(c2);
+  static constexpr int regs = 4 * (N1 > N2 ? N1 : N2) + 56 < 248 ? 4 * (N1 > N2 ? N1 : N2) + 56 : 248;
+  static constexpr int MIN_BLOCKS = pass_blocks(NT, smem_bytes, regs);
+};
+
+template <int P, int ST, bool HALF, int V>
+__global__ void __launch_bounds__(FwdXCfg<P, HALF, V>::NT, FwdXCfg<P, HALF, V>::MIN_BLOCKS)
 k_fwd_x(const float* __restrict__ Bh, const uint8_t* __restrict__ Mh, void* __restrict__ F0,
-        const RotIn* __restrict__ rot, Geo g, long long nrows) {
-  const float2* __restrict__ tw = kTw<P>.w;
-  using FS = FourStep<P, true, V>;
-  using FI = FwdIn<FS, HALF>;
-  constexpr int N1 = FS::N1, N2 = FS::N2, CS = FS::CS, H = FI::NI;
-  extern __shared__ float2 ex[];
+        const RotIn* __restrict__ rot, Geo g) {
+  using C = FwdXCfg<P, HALF, V>;
+  constexpr int N1 = C::N1, N2 = C::N2, RS = C::RS, CS = C::CS, NI = C::NI, ROWS = C::ROWS, NT = C::NT;
+  extern __shared__ __align__(16) c2 xsm[];
+  c2* ex = xsm;
+  c2* slot = ex + ROWS * CS + threadIdx.x;
   const int t = threadIdx.x;
   const int lrow = t / N2, n2 = t - lrow * N2;
-  const long long grow = (long long)blockIdx.x * ROWS + lrow;
-  const bool row_ok = grow < nrows;
-  const long long rz = row_ok ? grow / g.ey : 0;
-  const int yb = row_ok ? (int)(grow - rz * g.ey) : 0;
-  const int r = (int)(rz / g.ez), zb = (int)(rz - (long long)r * g.ez);
-  const RotBox& bx = rot[r].b;
-  const int z = zb + bx.org[0], y = yb + bx.org[1], ox = bx.org[2];   // voxel of box index (zb, yb, 0)
+  // rows [row0, row0 + ROWS) of one plane of one rotation
+  const int r = blockIdx.z, zb = blockIdx.y, row0 = blockIdx.x * ROWS;
+  const bool even = !(r & 1);
 
-  // x = org + N2*n1 + n2 over ex voxels: with ex <= P/2 only n1 < N1/2 can hold data
-  constexpr bool NS = !HALF;                  // NGF staged in shared memory
-  constexpr int HR = NS ? 1 : H;
-  float vx[HR], vy[HR], vz[HR], mm[HR];
-  float4* ngs = reinterpret_cast<float4*>(reinterpret_cast<char*>(ex) + FwdXCfg<P, HALF, V>::ex_bytes);
-  const int NTX = ROWS * N2;
-  const float* Vol = Bh + (long long)r * g.nvox;
-  const uint8_t* M = Mh + (long long)r * g.nvox;
-  const long long sy = g.nx, sz = (long long)g.nx * g.ny;
-  const int ym = max(y - 1, 0), yp = min(y + 1, g.ny - 1);
-  const int zm = max(z - 1, 0), zp = min(z + 1, g.nz - 1);
-  const long long base = (long long)z * sz + (long long)y * sy;
-  const long long rows_per_field = (long long)g.ez * g.ey;
-  const int nrot = (int)(nrows / rows_per_field);
-  const bool has_partner = !(r & 1) && r + 1 < nrot;
-  // the partner's mask in its own box: offset of its row from M, and its x origin
-  long long pbase = 0;
-  int pox = 0, pnx = 0;
-  if (has_partner) {
-    const RotBox& pb = rot[r + 1].b;
-    const int pz = zb + pb.org[0], py = yb + pb.org[1];
-    pox = pb.org[2];
-    pnx = (pz < g.nz && py < g.ny) ? min(g.ex, g.nx - pox) : 0;
-    pbase = g.nvox + (long long)pz * sz + (long long)py * sy + pox;
-  }
-  const bool in_vol = row_ok && z < g.nz && y < g.ny;
-  // per element: the NGF times the mask (m^2 = m, so every Eq. 6 product of
-  // two masked components equals the product times m, bit for bit) and the
-  // mask pair of the mask field coded as m + 2 m2 (m2: the next rotation's mask)
+  c2 v[N1];
+  {
+    const int yb = row0 + lrow;
+    const RotBox& bx = rot[r].b;
+    const int z = zb + bx.org[0], y = yb + bx.org[1], ox = bx.org[2];   // voxel of box index (zb, yb, 0)
+    // byte offsets into a rotation's volume fit 32 bits (2^24 voxels)
+    const char* Vol = reinterpret_cast<const char*>(Bh + r * g.nvox);
+    const uint8_t* M = Mh + r * g.nvox;
+    const int sy = g.nx, sz = g.nx * g.ny;
+    const bool row_in = yb < g.ey && z < g.nz && y < g.ny;
+    const int nx_ok = row_in ? min(g.ex, g.nx - ox) : 0;
+    const unsigned row = row_in ? z * sz + y * sy : 0u;
+    const unsigned oc = 4 * row, oym = oc - (row_in && y > 0 ? 4 * sy : 0), oyp = oc + (row_in && y + 1 < g.ny ? 4 * sy : 0);
+    const unsigned ozm = oc - (row_in && z > 0 ? 4 * sz : 0), ozp = oc + (row_in && z + 1 < g.nz ? 4 * sz : 0);
+    auto vol = [&](unsigned o) { return __ldg(reinterpret_cast<const float*>(Vol + o)); };
+    // masks are paired across consecutive rotations: the even rotation's mask
+    // field carries (M_r, M_{r+1}), the partner's in its own box
+    unsigned prow = 0;
+    int pnx = 0;
+    if (even && r + 1 < (int)gridDim.z && yb < g.ey) {
+      const RotBox& pb = rot[r + 1].b;
+      const int pz = zb + pb.org[0], py = yb + pb.org[1];
+      if (pz < g.nz && py < g.ny) {
+        pnx = min(g.ex, g.nx - pb.org[2]);
+        prow = (unsigned)g.nvox + pz * sz + py * sy + pb.org[2];
+      }
+    }
+    unsigned mb = 0, pb = 0;
 #pragma unroll
-  for (int n1 = 0; n1 < H; ++n1) {
-    const int xb = N2 * n1 + n2, x = xb + ox;
-    float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    const float m2 = xb < pnx && M[pbase + xb] ? 2.0f : 0.0f;
-    q.w = m2;
-    if (in_vol && xb < g.ex && x < g.nx) {
-      const int xm = max(x - 1, 0), xp = min(x + 1, g.nx - 1);
-      const float gx = 0.5f * (__ldg(&Vol[base + xp]) - __ldg(&Vol[base + xm]));
-      const float gy = 0.5f * (__ldg(&Vol[(long long)z * sz + (long long)yp * sy + x]) -
-                               __ldg(&Vol[(long long)z * sz + (long long)ym * sy + x]));
-      const float gz = 0.5f * (__ldg(&Vol[(long long)zp * sz + (long long)y * sy + x]) -
-                               __ldg(&Vol[(long long)zm * sz + (long long)y * sy + x]));
+    for (int n1 = 0; n1 < NI; ++n1) {
+      const int x = N2 * n1 + n2;
+      if (x < nx_ok && M[row + ox + x]) mb |= 1u << n1;
+      if (x < pnx && M[prow + x]) pb |= 1u << n1;
+    }
+#pragma unroll
+    for (int n1 = 0; n1 < NI; ++n1) {
+      const bool in = mb >> n1 & 1;
+      // x = org + N2*n1 + n2 over ex voxels: with ex <= P/2 only n1 < N1/2 can hold data
+      const int x = ox + N2 * n1 + n2;
+      const unsigned xo = in ? 4 * x : 0;
+      const float gx = 0.5f * (vol(oc + xo + (in && x + 1 < g.nx ? 4 : 0)) - vol(oc + xo - (in && x > 0 ? 4 : 0)));
+      const float gy = 0.5f * (vol(oyp + xo) - vol(oym + xo));
+      const float gz = 0.5f * (vol(ozp + xo) - vol(ozm + xo));
       const float inv = rsqrtf(gx * gx + gy * gy + gz * gz + g.eps2);
-      const float m = M[base + x] ? 1.0f : 0.0f;
-      q = make_float4(m * (gx * inv), m * (gy * inv), m * (gz * inv), m + m2);
-    }
-    if constexpr (NS) {
-      ngs[n1 * NTX + t] = q;
-    } else {
-      vx[n1] = q.x;
-      vy[n1] = q.y;
-      vz[n1] = q.z;
-      mm[n1] = q.w;
+      // the NGF times the mask (m^2 = m: every product of two masked components
+      // equals the product times m, bit for bit)
+      const float X = in ? gx * inv : 0.0f, Y = in ? gy * inv : 0.0f, Z = in ? gz * inv : 0.0f;
+      const float m = even && in ? 1.0f : 0.0f, m2 = pb >> n1 & 1 ? 1.0f : 0.0f;
+      // Eq. 6 products (squared measure): (xx, yy) and (zz, xy), then (xz, yz) and
+      // the mask pair; Eq. 3 (unsquared): (x, y) and (z, 0), then the mask pair
+      if (g.nch == 3) {
+        v[n1] = {make_float2(X * X, Z * Z), make_float2(Y * Y, X * Y)};
+        slot[n1 * NT] = {make_float2(X * Z, m), make_float2(Y * Z, m2)};
+      } else {
+        v[n1] = {make_float2(X, Z), make_float2(Y, 0.0f)};
+        slot[n1 * NT] = {make_float2(0.0f, m), make_float2(0.0f, m2)};
+      }
     }
   }
-  // Masks are paired across consecutive rotations: the even rotation's mask
-  // field carries (M_r, M_{r+1}); an odd rotation has no mask field of its own.
-  const bool odd_block = ((blockIdx.x * (long long)ROWS) / rows_per_field & 1) &&
-                         (blockIdx.x * (long long)ROWS) / rows_per_field ==
-                             (min(blockIdx.x * (long long)ROWS + ROWS, nrows) - 1) / rows_per_field;
 #pragma unroll 1
-  for (int j = 0; j < g.nf; ++j) {
-    if (j == g.nch && odd_block) break;          // uniform over the block
-    // Eq. 6 products (squared measure) or Eq. 3 components (unsquared); the
-    // mask field comes last
-    const int code = j == g.nch ? 3 : (g.nch == 3 ? j : 4 + j);
-    float2 v[H];
-    // this field's inputs, with the field's product chosen at compile time
-    auto inputs = [&](auto cc) {
-      constexpr int CODE = decltype(cc)::value;
+  for (int pair = 0; pair < 2; ++pair) {
+    if (pair) {
+      __syncthreads();                            // the first pair has left the exchange
 #pragma unroll
-      for (int n1 = 0; n1 < H; ++n1) {
-        float X, Y, Z, w;
-        if constexpr (NS) {
-          const float4 q = ngs[n1 * NTX + t];   // this thread's own slot
-          X = q.x; Y = q.y; Z = q.z; w = q.w;
-        } else {
-          X = vx[n1 < HR ? n1 : 0]; Y = vy[n1 < HR ? n1 : 0]; Z = vz[n1 < HR ? n1 : 0];
-          w = mm[n1 < HR ? n1 : 0];
-        }
-        if constexpr (CODE == 0) v[n1] = make_float2(X * X, Y * Y);
-        else if constexpr (CODE == 1) v[n1] = make_float2(Z * Z, X * Y);
-        else if constexpr (CODE == 2) v[n1] = make_float2(X * Z, Y * Z);
-        else if constexpr (CODE == 4) v[n1] = make_float2(X, Y);
-        else if constexpr (CODE == 5) v[n1] = make_float2(Z, 0.0f);
-        else {                                   // mask pair (M_r, M_{r+1}); w = m + 2 m2
-          const float m2 = w >= 2.0f ? 1.0f : 0.0f;
-          v[n1] = (r & 1) ? make_float2(0.0f, 0.0f) : make_float2(w - 2.0f * m2, m2);
-        }
-      }
-    };
-    switch (code) {
-      case 0: inputs(std::integral_constant<int, 0>{}); break;
-      case 1: inputs(std::integral_constant<int, 1>{}); break;
-      case 2: inputs(std::integral_constant<int, 2>{}); break;
-      case 4: inputs(std::integral_constant<int, 4>{}); break;
-      case 5: inputs(std::integral_constant<int, 5>{}); break;
-      default: inputs(std::integral_constant<int, 3>{}); break;
+      for (int n1 = 0; n1 < NI; ++n1) v[n1] = slot[n1 * NT];
     }
-    FI::template step1<-1>(v, ex + lrow * CS, n2, tw);
-    __syncthreads();
-    if (t < ROWS * N1) {
-      const int lr = t / N1, k1 = t - lr * N1;
-      const long long gr = (long long)blockIdx.x * ROWS + lr;
-      const bool skip_row = j == g.nch && ((gr / rows_per_field) & 1);   // odd rotation: no mask field
-      if (gr < nrows && !skip_row) {
-        float2 u[N2];
-        FS::template step2<-1>(u, ex + lr * CS, k1);
-        const long long rz2 = gr / g.ey;
-        const int y2 = (int)(gr - rz2 * g.ey);
-        const int r2 = (int)(rz2 / g.ez), z2 = (int)(rz2 - (long long)r2 * g.ez);
-        char* fld = Fields<ST>::field(F0, g, rows_per_field * P, r2, j);
-        const long long row = ((long long)z2 * g.ey + y2) * P;
-        const float sc = field_scale(g.scale0, j);
-        if (j == g.nch) {
+    if constexpr (HALF) {
+      c2 h[NI];
 #pragma unroll
-          for (int k2 = 0; k2 < N2; ++k2) Fields<ST>::put(fld, row + k1 + N1 * k2, u[k2], true, sc);
+      for (int n1 = 0; n1 < NI; ++n1) h[n1] = v[n1];
+      dft_half<N1, -1>(h, v);
+    } else {
+      Dft<N1, -1>::run(v);
+    }
+    c2* e = ex + lrow * CS + n2 * RS;
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) {
+      const float2 w = __ldg(&kTwStep<P, N1, N2>.w[k1 * N2 + n2]);
+      e[k1] = k1 == 0 ? v[k1] : cmul(v[k1], c2{dup(w.x), dup(w.y)});
+    }
+    __syncthreads();
+    const int lr = t / N1, k1 = t - lr * N1;
+    // the fields of this pair that exist: (0, 1), then (2 if nch == 3, the mask if
+    // the rotation is even)
+    const bool lo = pair == 0 || g.nch == 3, hi = pair == 0 || even;
+    if (t < ROWS * N1 && row0 + lr < g.ey && (lo || hi)) {
+      c2 u[N2];
+      const c2* s = ex + lr * CS + k1;
+#pragma unroll
+      for (int i = 0; i < N2; ++i) u[i] = s[i * RS];
+      Dft<N2, -1>::run(u);
+      const long long E = (long long)g.ez * g.ey * P;
+      const int j0 = 2 * pair, j1 = pair ? g.nch : 1;
+      const int o = zb * P * g.ey + 4 * (row0 + lr);       // [z][kx/4][y][kx%4]
+      const TileRun<N1> run(k1, g.ey);
+      if (lo) {
+        char* f0 = Fields<ST>::field(F0, g, E, r, j0);
+        const float s0 = field_scale(g.scale0, j0);
+#pragma unroll
+        for (int i = 0; i < N2; ++i) Fields<ST>::put(f0, o + run.at(i), make_float2(u[i].x.x, u[i].y.x), false, s0);
+      }
+      if (hi) {
+        char* f1 = Fields<ST>::field(F0, g, E, r, j1);
+        const float s1 = field_scale(g.scale0, j1);
+        if (pair == 0) {
+#pragma unroll
+          for (int i = 0; i < N2; ++i) Fields<ST>::put(f1, o + run.at(i), make_float2(u[i].x.y, u[i].y.y), false, s1);
         } else {
 #pragma unroll
-          for (int k2 = 0; k2 < N2; ++k2) Fields<ST>::put(fld, row + k1 + N1 * k2, u[k2], false, sc);
+          for (int i = 0; i < N2; ++i) Fields<ST>::put(f1, o + run.at(i), make_float2(u[i].x.y, u[i].y.y), true, s1);
         }
       }
     }
-    __syncthreads();
   }
 }
 
 template <int P, bool HALF, int V>
 void launch_fwd_x_t(const float* Bh, const uint8_t* Mh, void* F0, const RotIn* rot, Geo g, int nrot,
                     cudaStream_t st) {
-  constexpr int N2 = SplitV<P, V>::N2;
-  constexpr int ROWS = FwdXCfg<P, HALF, V>::ROWS;
-  const long long nrows = (long long)nrot * g.ez * g.ey;
-  const size_t smem = FwdXCfg<P, HALF, V>::smem_bytes;
-  const unsigned blocks = (unsigned)((nrows + ROWS - 1) / ROWS);
-  auto go = [&](auto kern) {
-    set_smem(kern, smem);
-    kern<<<blocks, ROWS * N2, smem, st>>>(Bh, Mh, F0, rot, g, nrows);
-  };
-  by_store<P>(g.store, [&](auto st) { go(k_fwd_x<P, ROWS, decltype(st)::value, HALF, V>); });
+  using C = FwdXCfg<P, HALF, V>;
+  const dim3 grid((unsigned)((g.ey + C::ROWS - 1) / C::ROWS), (unsigned)g.ez, (unsigned)nrot);
+  by_store<P>(g.store, [&](auto sf) {
+    constexpr int ST = decltype(sf)::value;
+    set_smem(k_fwd_x<P, ST, HALF, V>, C::smem_bytes);
+    k_fwd_x<P, ST, HALF, V><<<grid, C::NT, C::smem_bytes, st>>>(Bh, Mh, F0, rot, g);
+  });
 }
 
 template <int P>
@@ -272,107 +293,119 @@ void launch_fwd_x(const float* Bh, const uint8_t* Mh, void* F0, const RotIn* rot
 }
 
 // ---------------------------------------------------------------------------
-// fwd_y: y-axis FFT of every column of F0 (rows y >= ey are zero); the output
-// is transposed so that ky is contiguous for the z pass.
-// Block: W consecutive kx of one (r, j, z) plane.
+// fwd_y: y-axis FFT of every column of F0 (rows y >= ey are zero), to the z
+// pass's tiles.  Block: one tile of four kx in four z planes of one (r, j).
 // ---------------------------------------------------------------------------
-// Blocks per SM for the single-transform passes: as many as keep at least
-// MINR registers per thread (each of the SM's four sub-partitions holds 16384
-// registers for the warps placed on it) and fit in shared memory.
-constexpr int pass_blocks(int threads, size_t smem, int minr) {
-  int best = 1;
-  for (int b = 2; b <= 8; ++b) {
-    const int per_sub = (b * ((threads + 31) / 32) + 3) / 4;
-    const int regs = (16384 / (32 * per_sub)) / 8 * 8;
-    if (regs >= minr && (size_t)b * (smem + 1024) <= 228 * 1024) best = b;
-  }
-  return best;
-}
+// F0's tiles of four kx are contiguous over y, so a plane's columns arrive as
+// one bulk copy, and four planes make 128-byte pieces of F1's tiles
+// [kx][p/4][z][p%4] (one plane: 32 bytes, 31 against 28 us per rotation at 150^3).
 template <int P, int V> struct FwdYCfg {
-  // 16 columns per block; 8 where the second stage is longer than 20 points
-  // (more registers per thread: smaller blocks keep several per SM)
-  static constexpr int W = SplitV<P, V>::N2 > 20 ? 8 : 16;
-  static constexpr int NT = W * SplitV<P, V>::N2;
-  static constexpr size_t smem_bytes = (size_t)W * FourStep<P, true, V>::CS * sizeof(float2);
-  // the 25- and 32-point second stages need more registers than 16- or 20-point ones
-  static constexpr int MIN_BLOCKS = pass_blocks(NT, smem_bytes, SplitV<P, V>::N2 > 20 ? 80 : 48);
+  static constexpr int N1 = SplitV<P, V>::N1, N2 = SplitV<P, V>::N2, W = 16;
+  static constexpr int NT = W * N2;
+  // exchange [column][n2][k1]: odd rows, and columns 4 rows apart (mod 16), put
+  // four columns of four rows in different banks
+  static constexpr int RS = N1 | 1, CS0 = N2 * RS, CS = CS0 + ((4 * RS - CS0) % 16 + 16) % 16;
+  static constexpr size_t smem_bytes(int ey) { return ((size_t)W * CS + (size_t)W * ey) * sizeof(float2) + 16; }
+  static constexpr int MIN_BLOCKS = pass_blocks(NT, smem_bytes(3 * P / 4), N2 > 20 ? 80 : 48);
 };
 
-template <int P, int W, int ST, bool HALF, int V>
-__global__ void __launch_bounds__(W * SplitV<P, V>::N2, FwdYCfg<P, V>::MIN_BLOCKS)
+template <int P, int ST, bool HALF, int V>
+__global__ void __launch_bounds__(FwdYCfg<P, V>::NT, FwdYCfg<P, V>::MIN_BLOCKS)
 k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, Geo g) {
-  const float2* __restrict__ tw = kTw<P>.w;
-  using FS = FourStep<P, true, V>;
-  using FI = FwdIn<FS, HALF>;
-  constexpr int N1 = FS::N1, N2 = FS::N2, CS = FS::CS;
-  extern __shared__ float2 ex[];
+  using C = FwdYCfg<P, V>;
+  constexpr int N1 = C::N1, N2 = C::N2, W = C::W, RS = C::RS, CS = C::CS, NI = HALF ? N1 / 2 : N1;
+  extern __shared__ __align__(128) float2 ysm[];
+  float2* in = ysm;                                  // [4 z][ey][4 kx] (4-byte values in the 16-bit forms)
+  float2* ex = in + W * g.ey;                        // [W][CS]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(ex + W * CS + (W * CS & 1));
   const int t = threadIdx.x;
-  // kx tiles run fastest over the grid, so the blocks that read the two halves
-  // of a 128-byte line of F0 run together and the second one hits in L2
-  const long long plane = blockIdx.y;                // ((r * nf) + j) * ez + z
-  const long long rj = plane / g.ez;
-  const int z = (int)(plane - rj * g.ez);
-  const int r = (int)(rj / g.nf), j = (int)(rj - (long long)r * g.nf);
+  const int rj = blockIdx.z, z0 = 4 * blockIdx.y;    // rj = r * nf + j
+  const int r = g.nf == 4 ? rj >> 2 : rj / 3, j = rj - r * g.nf;
   const bool is_mask = j == g.nch;
   if (is_mask && (r & 1)) return;                    // paired into the even rotation's mask field
-  const int kx0 = blockIdx.x * W;
-  {
-    const int col = t % W, n2 = t / W;
-    const int kx = kx0 + col;
+  const bool wide = ST == kStoreF32 || is_mask;
+  const int nz = min(4, g.ez - z0);
+  const uint32_t bytes = (uint32_t)g.ey * 4 * (wide ? 8 : 4);   // of one plane's tile
+  if (t == 0) {
     const char* src = Fields<ST>::field(F0, g, (long long)g.ez * g.ey * g.Px, r, j);
+    tc::mbar_init(bar, 1);
+    tc::mbar_init_fence();
+    tc::mbar_expect(bar, nz * bytes);
+    for (int z = 0; z < nz; ++z)
+      tc::bulk_load(reinterpret_cast<char*>(in) + z * bytes,
+                    src + ((long long)(z0 + z) * (g.Px / 4) + blockIdx.x) * bytes, bytes, bar);
+  }
+  __syncthreads();                                   // the barrier is initialised
+  const bool dead = !tc::mbar_wait(bar, 0, kTcWaitNs);
+  {
+    const int kxi = t & 3, n2 = (t >> 2) % N2, zz = t / (4 * N2);
     const float isc = 1.0f / field_scale(g.scale0, j);
-    const long long zoff = (long long)z * g.ey * g.Px;
-    float2 v[FI::NI];                     // y < ey: with ey <= P/2 the upper half is zero
-    if (is_mask) {
+    const int o = (zz * g.ey + n2) * 4 + kxi;
+    float2 v[NI];                                    // y < ey: with ey <= P/2 the upper half is zero
+    auto rows = [&](auto mc) {
 #pragma unroll
-      for (int n1 = 0; n1 < FI::NI; ++n1) {
-        const int y = N2 * n1 + n2;
-        v[n1] = (y < g.ey && kx < g.Px) ? Fields<ST>::get(src, zoff + (long long)y * g.Px + kx, true, isc)
-                                        : make_float2(0.f, 0.f);
-      }
+      for (int n1 = 0; n1 < NI; ++n1)
+        v[n1] = N2 * n1 + n2 < g.ey && zz < nz
+                    ? Fields<ST>::get(reinterpret_cast<const char*>(in), o + 4 * N2 * n1, decltype(mc)::value, isc)
+                    : make_float2(0.f, 0.f);
+    };
+    if (wide) rows(std::true_type{});
+    else rows(std::false_type{});
+    float2* e = ex + (zz * 4 + kxi) * CS + n2 * RS;
+    float2 a[N1];
+    if constexpr (HALF) {
+      dft_half<N1, -1>(v, a);
     } else {
 #pragma unroll
-      for (int n1 = 0; n1 < FI::NI; ++n1) {
-        const int y = N2 * n1 + n2;
-        v[n1] = (y < g.ey && kx < g.Px) ? Fields<ST>::get(src, zoff + (long long)y * g.Px + kx, false, isc)
-                                        : make_float2(0.f, 0.f);
-      }
+      for (int i = 0; i < N1; ++i) a[i] = v[i];
+      Dft<N1, -1>::run(a);
     }
-    FI::template step1<-1>(v, ex + col * CS, n2, tw);
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) {
+      const float2 w = __ldg(&kTwStep<P, N1, N2>.w[k1 * N2 + n2]);
+      e[k1] = k1 == 0 ? a[k1] : cmul(a[k1], w);
+    }
   }
   __syncthreads();
   if (t < W * N1) {
-    const int col = t / N1, k1 = t - col * N1;
-    const int kx = kx0 + col;
-    if (kx < g.Px) {
+    const int k1 = t % N1, kxi = t / N1 & 3, zz = t / (4 * N1);
+    if (zz < nz) {
       float2 u[N2];
-      FS::template step2<-1>(u, ex + col * CS, k1);
-      char* dst = Fields<ST>::field(F1, g, (long long)g.ez * g.Px * P, r, j);
-      const long long row = ((long long)kx * g.ez + z) * P;       // [kx][z][ky]
+      const float2* s = ex + (zz * 4 + kxi) * CS + k1;
+#pragma unroll
+      for (int i = 0; i < N2; ++i) u[i] = s[i * RS];
+      Dft<N2, -1>::run(u);
+      char* dst = Fields<ST>::field(F1, g, (long long)g.ez * g.Px * ky_total(P), r, j);
+      const int row = (4 * blockIdx.x + kxi) * ky_total(P) * g.ez + 4 * (z0 + zz);
+      const KyRun<P, N1, N2> run(k1, g.ez);
       const float sc = field_scale(g.scale1, j);
       if (is_mask) {
 #pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) Fields<ST>::put(dst, row + k1 + N1 * k2, u[k2], true, sc);
+        for (int k2 = 0; k2 < N2; ++k2) Fields<ST>::put(dst, row + run.at(k2), u[k2], true, sc);
       } else {
 #pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) Fields<ST>::put(dst, row + k1 + N1 * k2, u[k2], false, sc);
+        for (int k2 = 0; k2 < N2; ++k2) Fields<ST>::put(dst, row + run.at(k2), u[k2], false, sc);
       }
     }
+  }
+  if (dead) {                                        // the results are invalid; its copies end before the block does
+    if (t == 0 && g.tc_err) atomicExch(g.tc_err, 1);
+    tc::mbar_wait(bar, 0, kTcWaitNs / 4);
   }
 }
 
 template <int P, int V>
 void launch_fwd_y_t(const void* F0, void* F1, Geo g, int nrot, cudaStream_t st) {
-  constexpr int W = FwdYCfg<P, V>::W, N2 = SplitV<P, V>::N2;
-  const size_t smem = FwdYCfg<P, V>::smem_bytes;
-  dim3 grid((unsigned)((g.Px + W - 1) / W), (unsigned)(nrot * g.nf * g.ez));   // y: at most 32 * 4 * 256
-  auto go = [&](auto kern) {
-    set_smem(kern, smem);
-    kern<<<grid, W * N2, smem, st>>>(F0, F1, g);
-  };
+  using C = FwdYCfg<P, V>;
+  const size_t smem = C::smem_bytes(g.ey);
+  const dim3 grid((unsigned)(g.Px / 4), (unsigned)((g.ez + 3) / 4), (unsigned)(nrot * g.nf));
   by_store<P>(g.store, [&](auto sf) {
     constexpr int ST = decltype(sf)::value;
-    by_half<P, V>(g.ey, [&](auto hc) { go(k_fwd_y<P, W, ST, decltype(hc)::value, V>); });
+    by_half<P, V>(g.ey, [&](auto hc) {
+      auto kern = k_fwd_y<P, ST, decltype(hc)::value, V>;
+      set_smem(kern, smem);
+      kern<<<grid, C::NT, smem, st>>>(F0, F1, g);
+    });
   });
 }
 
@@ -396,7 +429,7 @@ void launch_zmac(const void* F1, const float2* UV, float2* F2, Geo g, int nrot, 
     constexpr int V = decltype(vc)::value;
     by_store<P>(g.store, [&](auto sf) {
       constexpr int ST = decltype(sf)::value;
-      by_half<P, V>(g.ez, [&](auto hc) {
+      by_half_z<P, V>(g.ez, [&](auto hc) {
         constexpr bool HALF = decltype(hc)::value;
         // reduced-precision forms: the channels' z DFT on the tensor cores
         if constexpr (ST != kStoreF32) {
@@ -413,7 +446,7 @@ void launch_zmac(const void* F1, const float2* UV, float2* F2, Geo g, int nrot, 
 
 template <int P>
 void launch_prep_z(const float2* F1, float2* UV, Geo g, cudaStream_t st) {
-  by_half<P, 0>(g.ez, [&](auto hc) {
+  by_half_z<P, 0>(g.ez, [&](auto hc) {
     launch_zpass_t<P, kStoreF32, decltype(hc)::value, 0, kZPrep>(F1, UV, nullptr, nullptr, g, 1, nullptr, st);
   });
 }
@@ -440,10 +473,10 @@ k_inv_y(const float2* __restrict__ F2, float2* __restrict__ F3, Geo g, const Rot
     const int row = t / N2, n2 = t - row * N2;
     const int kx = kx0 + row;
     float2 v[N1];
-    const float2* src = F2 + (((long long)r * g.Px + kx) * g.wz + dz) * (long long)P;   // [r][kx][dz][ky]
+    const float2* src = F2 + (((long long)r * g.Px + kx) * g.wz + dz) * (long long)ky_total(P);   // [r][kx][dz][p]
 #pragma unroll
     for (int n1 = 0; n1 < N1; ++n1)
-      v[n1] = (kx < g.Px) ? src[N2 * n1 + n2] : make_float2(0.f, 0.f);
+      v[n1] = (kx < g.Px) ? src[ky_pos(N2 * n1 + n2, P)] : make_float2(0.f, 0.f);
     FS::template step1<1>(v, ex + row * CS, n2, tw);
   }
   __syncthreads();

@@ -18,7 +18,7 @@
 
 namespace csngf {
 
-// wait limit of a tensor-core pass for its own MMAs (they take microseconds)
+// wait limit of a z pass for its own MMAs and copies (they take microseconds)
 constexpr unsigned long long kTcWaitNs = 2000000000ull;
 
 namespace tc {
@@ -118,19 +118,31 @@ __device__ __forceinline__ unsigned long long global_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
+__device__ __forceinline__ bool mbar_try(uint64_t* mbar, uint32_t parity) {
+  uint32_t done = 0;
+  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+               "selp.u32 %0, 1, 0, p;\n}\n"
+               : "=r"(done) : "r"(smem_addr(mbar)), "r"(parity) : "memory");
+  return done != 0;
+}
 // wait for the phase with the given parity to complete, for at most limit_ns;
 // false if it did not
 __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, unsigned long long limit_ns) {
-  const uint32_t a = smem_addr(mbar);
-  uint32_t done = 0;
+  if (mbar_try(mbar, parity)) return true;
   const unsigned long long t0 = global_ns();
-  while (true) {
-    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                 "selp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(done) : "r"(a), "r"(parity) : "memory");
-    if (done) return true;
+  while (!mbar_try(mbar, parity))
     if (global_ns() - t0 > limit_ns) return false;
-  }
+  return true;
+}
+// this phase also waits for `bytes` of bulk copies
+__device__ __forceinline__ void mbar_expect(uint64_t* mbar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(mbar)), "r"(bytes) : "memory");
+}
+// contiguous bulk copy global -> shared (16-byte aligned, bytes a multiple of
+// 16), completing on mbar
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(mbar)) : "memory");
 }
 
 }  // namespace tc

@@ -11,9 +11,9 @@
 //     H(P - kz) = (C.re b - S.im b) + i (C.im b + S.re b)
 // so two M = 128 products (C and S, rows kz, K = z padded to a multiple of
 // 16) give every frequency of every column.  The B operand is a tile of the
-// 16-bit field values as they lie in F1 ([kx][z][ky] with (re, im) pairs):
+// 16-bit field values as they lie in F1 ([kx][p/4][z][p%4] with (re, im) pairs):
 // N-major, its columns (field, primary / mirror, column, re / im), so that
-// the 8 primary columns of a row are two 16-byte copies.  Tensor memory lane
+// the 8 primary columns of a row are two 16-byte copies, their mirrors two more.  Tensor memory lane
 // kz then holds H at kz and P - kz of a column and of its mirror column
 // (-kx, -ky), which is all the multiply-accumulate of that frequency pair
 // needs.  The mask field (the overlap count N) and the inverse stay on the
@@ -36,9 +36,9 @@ __device__ __forceinline__ void store16(unsigned char* p, float v) {
 // X costs one write and one read of a half spectrum of complex values per
 // rotation; in exchange the tensor-core kernel double-buffers its operands and
 // keeps no CUDA-core transform in its per-rotation chain.
-// X layout: [r][kx <= P/2][ky / 8][kz][ky % 8].
+// X layout: [r][kx <= P/2][p/4][kz][p%4].
 //
-// k_zx_tc, per block: one kx, W = 8 ky columns and their mirrors, every
+// k_zx_tc, per block: one kx, W = 8 columns (two tiles) and their mirrors, every
 // rotation of the launch; the cos / sin tiles and the block's weights stay
 // in shared memory.  Rotation r + 1's MMAs run while rotation r's products
 // are summed; rotation r + 2's operand is copied (cp.async) as soon as
@@ -77,18 +77,20 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
   uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 2);
 
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int kx = blockIdx.y, ky0 = blockIdx.x * W;
+  const int kx = blockIdx.y;
   const int mkx = (g.Px - kx) % g.Px;
-  const long long tiles = (long long)gridDim.x * gridDim.y, tile = (long long)kx * gridDim.x + blockIdx.x;
-  const long long E = (long long)g.ez * g.Px * g.Py;
+  const int ntile = 2 * gridDim.x, half = ky_half(g.Py) / 4;   // tiles of four columns
+  const long long E = (long long)g.ez * g.Px * 4 * ntile;
 
   for (uint32_t q = t; q < 2 * stageB / 16; q += NT)
     reinterpret_cast<uint4*>(Bs)[q] = make_uint4(0u, 0u, 0u, 0u);
-  // the block's weights, [channel][kz][column] in HBM, transposed so that kz runs
-  // over the lanes
+  // the block's weights, [tile][field][kz][column][a, b] in HBM, transposed so that
+  // kz runs over the lanes
   for (int q = t; q < NUV * TILE; q += NT) {
-    const int a = q / TILE, i = q - a * TILE, c = i % W, k = i / W;
-    cp_async8(uvs + a * TILE + c * P + k, UV + (tile * (NUV + 1) + a) * TILE + i);
+    const int i = q % (NUV * TILE / 2), h = q / (NUV * TILE / 2);   // entry of the block's tile h
+    const int j = i / TILE, k = i % TILE / 8, c = 4 * h + i % 8 / 2, s = i & 1;
+    cp_async8(uvs + (2 * j + s) * TILE + c * P + k,
+              UV + ((long long)kx * ntile + 2 * blockIdx.x + h) * (NUV + 1) * 4 * P + i);
   }
   for (int m = warp; m < 128; m += NT / 32)
     for (int k = lane; k < KP; k += 32) {
@@ -109,29 +111,30 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
   }
   if (warp == 0) tc::alloc(tslot, C::TMEM_COLS);
 
-  // operand copies of one (field, z) row: two 16-byte runs of primary
-  // columns, 8 mirror values of 4 bytes; thread t takes item t % 10
-  constexpr int ZSTEP = NT / 10;
-  const int item = t % 10, zr0 = t / 10;
-  const bool prim = item < 2;
-  const int cm = item - 2;
-  const bool okc = t < 10 * ZSTEP && (prim ? ky0 + 4 * item < g.Py : ky0 + cm < g.Py);
-  const long long srow = prim ? (long long)kx * g.ez * g.Py + ky0 + 4 * item
-                              : (long long)mkx * g.ez * g.Py + (g.Py - (ky0 + cm)) % g.Py;
-  const int nrow = prim ? 8 * item : 16 + 2 * cm;
+  // operand copies of one (field, z) row: two tiles of primary columns and two
+  // of their mirrors, 16 bytes each (tiles that hold ky = 0 or P/2, which are
+  // their own mirrors: the four mirror values one by one)
+  const int item = t % 4, zr0 = t / 4, tile = 2 * blockIdx.x + (item & 1);
+  const bool prim = item < 2, own = tile == 0 || tile == half;
+  const int mtile = tile < half ? tile + half : tile - half;
+  const long long tz = 4LL * g.ez;                 // values per tile
+  const long long srow = prim ? ((long long)kx * ntile + tile) * tz : ((long long)mkx * ntile + mtile) * tz;
+  const long long sown = ((long long)mkx * ntile + tile) * tz;
   auto fetch_b = [&](int r, int s) {
-    if (r < nrot && okc) {
+    if (r < nrot) {
       unsigned char* B0 = Bs + (size_t)s * stageB;
       for (int j = 0; j < g.nch; ++j) {
         const char* src = Fields<ST>::field(F1, g, E, r, j);
-        const int n = j * 4 * W + nrow;
-        unsigned char* dcol = B0 + (uint32_t)(n / 8) * sbo + (n % 8) * 2;
-        if (prim) {
-          for (int z = zr0; z < g.ez; z += ZSTEP)
-            cp_async16(dcol + (z / 8) * 128 + (z % 8) * 16, src + (srow + (long long)z * g.Py) * 4);
-        } else {
-          for (int z = zr0; z < g.ez; z += ZSTEP)
-            cp_async4(dcol + (z / 8) * 128 + (z % 8) * 16, src + (srow + (long long)z * g.Py) * 4);
+        unsigned char* dcol = B0 + (uint32_t)(j * 4 + item) * sbo;
+        for (int z = zr0; z < g.ez; z += NT / 4) {
+          unsigned char* d = dcol + (z / 8) * 128 + (z % 8) * 16;
+          if (prim || !own) {
+            cp_async16(d, src + (srow + 4 * z) * 4);
+          } else {
+            cp_async4(d, src + (sown + 4 * z) * 4);
+#pragma unroll
+            for (int c = 1; c < 4; ++c) cp_async4(d + 4 * c, src + (srow + 4 * z + c) * 4);
+          }
         }
       }
     }
@@ -192,7 +195,7 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
     if (t == 0 && r + 1 < nrot) issue(tmem, (r + 1) & 1);
     // (3) Eq. 7-8: X at kz and P - kz of this thread's four primary columns
     const uint32_t trow = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(s * 2 * NB);
-    float2* Xr = Xg + (r * tiles + tile) * TILE;
+    float2* Xr = Xg + (((long long)r * gridDim.y + kx) * ntile + 2 * blockIdx.x + (cg >> 1)) * 4 * P + 2 * (cg & 1);
     {
       const int ch = cg;                           // primary columns 2 ch, 2 ch + 1
       uint32_t rc[3][4], rs[3][4], rcm[3][4], rsm[3][4];
@@ -235,9 +238,9 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
               cmac(Xb[i], Wb[kzm], mul_si<-1>(csub(Hp, Mk)));
             }
         }
-        *reinterpret_cast<float4*>(Xr + kz * W + 2 * ch) = make_float4(Xa[0].x, Xa[0].y, Xa[1].x, Xa[1].y);
+        *reinterpret_cast<float4*>(Xr + kz * 4) = make_float4(Xa[0].x, Xa[0].y, Xa[1].x, Xa[1].y);
         if (kzm != kz)
-          *reinterpret_cast<float4*>(Xr + kzm * W + 2 * ch) = make_float4(Xb[0].x, Xb[0].y, Xb[1].x, Xb[1].y);
+          *reinterpret_cast<float4*>(Xr + kzm * 4) = make_float4(Xb[0].x, Xb[0].y, Xb[1].x, Xb[1].y);
       }
     }
     tc::fence_before_sync();
@@ -267,7 +270,7 @@ bool launch_zx_tc(const void* F1, const float2* UV, Geo g, int nrot, cudaStream_
     if (C1::bytes((g.nz + 15) / 16 * 16, NB, 2 * g.nch) > 232448) return false;
     const size_t s1 = std::max<size_t>(C1::bytes(KP, NB, 2 * g.nch), 120 * 1024);   // one block per SM: all of its tensor memory
     set_smem(k_zx_tc<P, ST>, s1);
-    dim3 grid((unsigned)((g.Py + C1::W - 1) / C1::W), (unsigned)(g.Px / 2 + 1));
+    dim3 grid((unsigned)(ky_total(g.Py) / C1::W), (unsigned)(g.Px / 2 + 1));
     k_zx_tc<P, ST><<<grid, C1::NT, s1, st>>>(F1, UV, g.zx, g, nrot, KP);
     return true;
   }

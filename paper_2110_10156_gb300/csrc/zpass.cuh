@@ -15,35 +15,59 @@
 // conj x + i conj y at (-kx, -ky), whose y and x inverses have the numerator as
 // real and the count as imaginary part.
 //
-// Weights (UV): [kx <= Px/2][ky / 8][channel 2 nch + 1][kz][ky % 8].
+// The two channels of a field travel side by side (c2) through the transform;
+// so do X and Y through the inverse.
+//
+// What bounds it: with inputs and weights read where they were needed, the pass
+// waited on memory whatever its arithmetic (45 us per rotation at 150^3 with
+// the transforms, 50 without).  So a tile's inputs and weights arrive by bulk
+// copies one field ahead, issued by one thread: no registers, no address
+// arithmetic, no load instructions in the other warps.
+//
+// Weights (UV): [kx <= Px/2][p / 4] tiles of per field [kz][p % 4][a, b] and
+// the mask's [kz][p % 4].
 #pragma once
+
+#include <algorithm>
+
+#include "tc.cuh"
 
 namespace csngf {
 
-constexpr int kZW = 8;                            // ky columns per block: 64-byte rows of F1
+constexpr int kZW = 4;                            // columns per block: one tile of F1
 
 enum { kZFull = 0, kZFromX = 1, kZPrep = 2 };     // see k_zpass
 
-// Q: rotations a block transforms side by side.  Two share each weight tile,
-// and the mask field that carries both their masks; above 16 points in the
-// second step a thread's X and transform registers no longer leave room for
-// two blocks of two rotations on an SM, and one rotation per block fits three.
+// A block transforms a tile of up to four rotations side by side: they share the
+// weights, and pairs the mask field that carries both their masks.
+//
+// The z transform takes the split's larger factor first (N1 >= N2): X, which
+// stays in registers through all fields, has N2 values per thread, the pair of
+// transforms 2 N1 in the first step and 2 N2 in the second, so that 128
+// registers hold both (10 x 16 with the larger factor last: 168 and spills).
 template <int P, int V, int MODE>
 struct ZCfg {
-  using FS = FourStep<P, true, V>;                // odd row stride: conflict-free for 8-column rows
-  static constexpr int N1 = FS::N1, N2 = FS::N2, W = kZW;
-  static constexpr int Q = (MODE == kZPrep || N2 > 16) ? 1 : 2;
-  static constexpr int NT = Q * W * N2;
-  static constexpr int SEQ = N2 * FS::RS * W;     // one transform per column in exchange, 2 per rotation
-  static constexpr int NWT = MODE == kZFull ? 2 : MODE == kZFromX ? 1 : 0;   // weight tiles held
-  static constexpr size_t smem_bytes = ((size_t)Q * 2 * SEQ + (size_t)NWT * W * P + P) * sizeof(float2);
-  static constexpr int warps = (NT + 31) / 32;
-  // registers a thread needs: X and the transform (2 N2 each) and about 56 more
-  static constexpr int regs = (4 * N2 + 56 + 7) / 8 * 8;
-  static constexpr int fit_regs = 65536 / (warps * 32 * (regs < 255 ? regs : 255));
-  static constexpr int fit_smem = (int)(228 * 1024 / (smem_bytes + 1024));
-  static constexpr int fit = fit_regs < fit_smem ? fit_regs : fit_smem;
-  static constexpr int MIN_BLOCKS = fit < 1 ? 1 : fit > 6 ? 6 : fit;
+  static constexpr int A = SplitV<P, V>::N1, B = SplitV<P, V>::N2;
+  static constexpr int N1 = A > B ? A : B, N2 = A > B ? B : A, W = kZW, QMAX = MODE == kZPrep ? 1 : 4;
+  // exchange [Q][N2][N1 (odd)][W] of pairs: 8 lanes take four columns of two
+  // rows, which an odd row length puts in different banks
+  static constexpr int RS = N1 | 1, SEQ = N2 * RS * W;
+  static constexpr int NWT = MODE == kZFull ? 2 : MODE == kZFromX ? 1 : 0;   // weights: values per column
+  static constexpr size_t wbytes = (size_t)NWT * W * P * sizeof(float2);     // of one buffer, two are held
+  // q rotations of ez planes: exchange, inputs [q][column, mirror][ez][W], weights
+  static constexpr size_t smem_bytes(int q, int ez) {
+    return (size_t)(q * SEQ + P) * sizeof(c2) + (size_t)q * 2 * ez * W * sizeof(float2) + 2 * wbytes + 64;
+  }
+  // as many rotations as two blocks (else one) have room for
+  static constexpr int fit(int blocks, int ez) {
+    int q = QMAX;
+    while (q > 1 && blocks * (smem_bytes(q, ez) + 1024) > 228 * 1024) q /= 2;
+    return q;
+  }
+  static constexpr int fit(int ez) { return 2 * fit(2, ez) > fit(1, ez) ? fit(2, ez) : fit(1, ez); }
+  static constexpr int Q = fit(2 * P / 3);        // what the registers are bounded for: typical boxes
+  static constexpr int regs = 4 * N1 + 2 * N2 + 40 < 248 ? 4 * N1 + 2 * N2 + 40 : 248;
+  static constexpr int MIN_BLOCKS = pass_blocks(Q * W * N1, smem_bytes(Q, 2 * P / 3), regs);
 };
 
 __device__ __forceinline__ void cmac(float2& x, float2 w, float2 u) {
@@ -58,181 +82,232 @@ __device__ __forceinline__ void cmac(float2& x, float2 w, float2 u) {
 // tensor-core half (Xg, laid out as one weight channel).  kZPrep: the fixed
 // volume: the weights w/4 conj(a'), w the Eq. 6 (Eq. 3) weight of the channel,
 // 1 for the mask (1/4: both sides carry a factor 2).
-// Block: 8 ky columns of one kx, the rotations [blockIdx.z * rpb, + rpb).
+// Block: one tile of one kx, the rotations [blockIdx.z * rpb, + rpb).
 template <int P, int ST, bool HALF, int V, int MODE>
-__global__ void __launch_bounds__(ZCfg<P, V, MODE>::NT, ZCfg<P, V, MODE>::MIN_BLOCKS)
+__global__ void __launch_bounds__(ZCfg<P, V, MODE>::Q * kZW * ZCfg<P, V, MODE>::N1,
+                                          ZCfg<P, V, MODE>::MIN_BLOCKS)
 k_zpass(const void* __restrict__ F1, float2* __restrict__ UV, const float2* __restrict__ Xg,
         float2* __restrict__ F2, Geo g, int nrot, int rpb, const RotIn* __restrict__ rot) {
   using C = ZCfg<P, V, MODE>;
-  using FS = typename C::FS;
-  using FI = FwdIn<FS, HALF>;
-  constexpr int N1 = FS::N1, N2 = FS::N2, RS = FS::RS, W = C::W, Q = C::Q, NT = C::NT, SEQ = C::SEQ;
-  constexpr int NI = FI::NI;
-  extern __shared__ __align__(16) float2 zsm[];
-  float2* ex = zsm;                               // [Q][2][N2][RS][W]
-  float2* ws = ex + Q * 2 * SEQ;                  // [NWT][P][W]
-  float2* tws = ws + C::NWT * W * P;              // [P]
+  constexpr int N1 = C::N1, N2 = C::N2, W = C::W, RS = C::RS, SEQ = C::SEQ;
+  constexpr int NI = HALF ? N1 / 2 : N1;
+  constexpr bool kMaskOnly = MODE == kZFromX, kWeights = MODE != kZPrep;
+  const int Q = blockDim.x / (W * N1);            // rotations side by side
   const int t = threadIdx.x;
-  const int kx = blockIdx.y, ky0 = blockIdx.x * W;
-  const int mkx = kx == 0 ? 0 : g.Px - kx;
-  const int c = t % W, ky = ky0 + c;
-  const bool col_ok = ky < g.Py;
-  const int mky = ky == 0 ? 0 : g.Py - ky;
+  extern __shared__ __align__(128) c2 zsm[];
+  c2* ex = zsm;                                   // [Q][N2][RS][W]
+  c2* tw2 = ex + Q * SEQ;                         // [P]
+  float2* ws = reinterpret_cast<float2*>(tw2 + P);                      // [2][P][W][a, b], or the mask's [P][W]
+  float2* stg = ws + 2 * C::wbytes / sizeof(float2);                    // [Q][column, mirror][ez][W]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(stg + Q * 2 * g.ez * W);  // inputs, weights per buffer
+  const int kx = blockIdx.y, mkx = kx == 0 ? 0 : g.Px - kx;
+  const int ntile = gridDim.x, half = ntile / 2, tile = blockIdx.x;
+  const int mtile = tile < half ? tile + half : tile - half;
+  const bool own = tile == 0 || tile == half;     // column 0 is ky = 0 or P/2: its own mirror
+  const int c = t % W, pos = tile * W + c;
   const int q1 = t / (W * N2), n2 = t / W - q1 * N2;   // first-step role
+  const bool has1 = t < Q * W * N2;
   const int q2 = t / (W * N1), k1 = t / W - q2 * N1;   // second-step role
-  const bool has2 = t < Q * W * N1;
   const int nchan = 2 * g.nch + 1;
-  float2* wt = UV + ((long long)kx * gridDim.x + blockIdx.x) * nchan * (P * W);
-  const long long E = (long long)g.ez * g.Px * g.Py;   // F1 is [r][j][kx][z][ky]
-  const long long off_h = (long long)kx * g.ez * g.Py + ky, off_m = (long long)mkx * g.ez * g.Py + mky;
-  for (int i = t; i < P; i += NT) tws[i] = kTw<P>.w[i];
-  // (the first barrier of the loop orders these writes before their reads)
+  float2* wt = UV + ((long long)kx * ntile + tile) * nchan * (P * W);
+  const long long E = (long long)g.ez * g.Px * W * ntile;              // F1 is [r][j][kx][p/4][z][p%4]
+  const long long tz = (long long)g.ez * W;                            // values of a tile
+  const long long off_h = ((long long)kx * ntile + tile) * tz, off_m = ((long long)mkx * ntile + mtile) * tz;
 
-  float2* e1 = ex + (q1 * 2) * SEQ + n2 * RS * W + c;
-  float2* e2 = ex + (q2 * 2) * SEQ + k1 * W + c;
-  float2 X[N2], u[N2];
+  auto fetch_inputs = [&](int r0, int j) {        // one thread: field j of rotations r0 .. r0 + Q - 1
+    const int b = (ST == kStoreF32 || j == g.nch) ? 8 : 4;
+    const uint32_t bytes = (uint32_t)tz * b;
+    int n = 0;
+    for (int q = 0; q < Q; ++q) {
+      const int r = j == g.nch ? (r0 + q) & ~1 : r0 + q;   // a mask field carries rotations 2k and 2k + 1
+      if (r < nrot) ++n;
+    }
+    tc::mbar_expect(&bar[0], 2 * n * bytes);
+    for (int q = 0; q < Q; ++q) {
+      const int r = j == g.nch ? (r0 + q) & ~1 : r0 + q;
+      if (r >= nrot) continue;
+      const char* f = Fields<ST>::field(F1, g, E, r, j);
+      tc::bulk_load(stg + 2 * q * tz, f + off_h * b, bytes, &bar[0]);
+      tc::bulk_load(stg + (2 * q + 1) * tz, f + off_m * b, bytes, &bar[0]);
+    }
+  };
+  auto fetch_weights = [&](int j, int s) {        // one thread: field j's weights
+    const uint32_t bytes = (j == g.nch ? 1 : 2) * P * W * sizeof(float2);
+    tc::mbar_expect(&bar[1 + s], bytes);
+    tc::bulk_load(reinterpret_cast<char*>(ws) + s * C::wbytes, wt + (long long)2 * j * P * W, bytes, &bar[1 + s]);
+  };
 
-  auto load = [&](float2 (&h)[NI], float2 (&m)[NI], int r, int j) {
-    const bool mask = ST == kStoreF32 || j == g.nch;
-    const char* f = Fields<ST>::field(F1, g, E, r, j);
+  const int rbeg = (int)blockIdx.z * rpb, rend = min(nrot, rbeg + rpb);
+  const int jbeg = kMaskOnly ? g.nch : 0;
+  if (t == 0) {
+    for (int i = 0; i < 3; ++i) tc::mbar_init(&bar[i], 1);
+    tc::mbar_init_fence();
+    fetch_inputs(rbeg, jbeg);
+    if (kWeights) fetch_weights(jbeg, 0);
+  }
+  for (int i = t; i < P; i += blockDim.x) tw2[i] = {dup(kTw<P>.w[i].x), dup(kTw<P>.w[i].y)};
+  __syncthreads();                                // the barriers are initialised
+
+  float2 X[N2];
+  int f = 0;                                      // fields so far: buffers and phases of the barriers
+  bool dead = false;                              // a wait ran out: no more waits, results invalid
+  auto wait = [&](int b, int phase) {
+    if (!dead && !tc::mbar_wait(&bar[b], phase & 1, kTcWaitNs)) dead = true;
+  };
+  // channels a', b' at this thread's z; zero past the box
+  auto load = [&](c2 (&v)[NI], const float2* s, int r, int j) {
     const float isc = 1.0f / field_scale(g.scale1, j);
-    const bool ok = col_ok && r < nrot;
-    if (mask) {
+    auto rows = [&](auto mc) {
+      constexpr bool wide = decltype(mc)::value;
 #pragma unroll
       for (int n1 = 0; n1 < NI; ++n1) {
-        const int z = N2 * n1 + n2;
-        h[n1] = m[n1] = make_float2(0.f, 0.f);
-        if (ok && z < g.ez) {
-          h[n1] = Fields<ST>::get(f, off_h + (long long)z * g.Py, true, isc);
-          m[n1] = Fields<ST>::get(f, off_m + (long long)z * g.Py, true, isc);
+        const int i = (N2 * n1 + n2) * W + c;
+        float2 h = make_float2(0.f, 0.f), m = h;
+        if (i < (int)tz) {
+          h = Fields<ST>::get(reinterpret_cast<const char*>(s), i, wide, isc);
+          m = Fields<ST>::get(reinterpret_cast<const char*>(s + tz), i, wide, isc);
+        }
+        v[n1] = {h, m};
+      }
+      if (own && c == 0) {                        // the column's own mirror: the same tile of -kx
+        const char* fld = Fields<ST>::field(F1, g, E, j == g.nch ? r & ~1 : r, j);
+        const long long o = ((long long)mkx * ntile + tile) * tz;
+#pragma unroll
+        for (int n1 = 0; n1 < NI; ++n1) {
+          const int i = (N2 * n1 + n2) * W;
+          v[n1].y = make_float2(0.f, 0.f);
+          if (r < nrot && i < (int)tz) v[n1].y = Fields<ST>::get(fld, o + i, wide, isc);
         }
       }
-    } else {
 #pragma unroll
       for (int n1 = 0; n1 < NI; ++n1) {
-        const int z = N2 * n1 + n2;
-        h[n1] = m[n1] = make_float2(0.f, 0.f);
-        if (ok && z < g.ez) {
-          h[n1] = Fields<ST>::get(f, off_h + (long long)z * g.Py, false, isc);
-          m[n1] = Fields<ST>::get(f, off_m + (long long)z * g.Py, false, isc);
-        }
+        const float2 h = v[n1].x, m = v[n1].y;
+        v[n1] = {cadd(h, m), make_float2(h.y - m.y, m.x - h.x)};
       }
-    }
-  };
-  auto step2 = [&](const float2* e) {             // u[k2] = transform at k1 + N1 k2
-#pragma unroll
-    for (int i = 0; i < N2; ++i) u[i] = e[i * RS * W];
-    Dft<N2, -1>::run(u);
-  };
-  auto fetch_weights = [&](int ch, int n) {       // n channels from ch
-    const float2* src = wt + (long long)ch * P * W;
-    for (int i = t; i < n * P * W / 2; i += NT) cp_async16(ws + 2 * i, src + 2 * i);
-    cp_async_commit();
-  };
-  auto inv1 = [&](float2 (&v)[N2], float2* e) {   // over k2, twiddle, to the exchange
-    Dft<N2, 1>::run(v);
-#pragma unroll
-    for (int i = 0; i < N2; ++i) {
-      const float2 w = tws[i * k1];
-      e[i * RS * W] = i == 0 ? v[i] : cmul(v[i], make_float2(w.x, -w.y));
-    }
+    };
+    if (ST == kStoreF32 || j == g.nch) rows(std::true_type{});
+    else rows(std::false_type{});
   };
 
-  const int rend = min(nrot, ((int)blockIdx.z + 1) * rpb);
 #pragma unroll 1
-  for (int r0 = (int)blockIdx.z * rpb; r0 < rend; r0 += Q) {
+  for (int r0 = rbeg; r0 < rend; r0 += Q) {
 #pragma unroll
     for (int i = 0; i < N2; ++i) X[i] = make_float2(0.f, 0.f);
     const int r2 = r0 + q2;                       // this thread's rotation in the second step
     if constexpr (MODE == kZFromX) {
-      if (has2 && r2 < nrot) {
-        const float2* xs = Xg + (((long long)r2 * gridDim.y + kx) * gridDim.x + blockIdx.x) * (P * W) + k1 * W + c;
+      if (r2 < nrot) {
+        const float2* xs = Xg + (((long long)r2 * gridDim.y + kx) * ntile + tile) * (P * W) + k1 * W + c;
 #pragma unroll
         for (int i = 0; i < N2; ++i) X[i] = __ldg(&xs[i * N1 * W]);
       }
     }
 #pragma unroll 1
-    for (int j = MODE == kZFromX ? g.nch : 0; j <= g.nch; ++j) {
+    for (int j = jbeg; j <= g.nch; ++j, ++f) {
       const bool mask = j == g.nch;
-      const bool two = !mask && !(g.nch == 2 && j == 1);   // Eq. 3: (z, 0) holds one channel
-      __syncthreads();                            // the previous reads of ex and ws are done
-      if constexpr (MODE != kZPrep) fetch_weights(2 * j, MODE == kZFull && two ? 2 : 1);
-      {
-        float2 h[NI], m[NI];
-        // a mask field carries rotations 2k and 2k + 1 as its a and b
-        load(h, m, mask ? (r0 + q1) & ~1 : r0 + q1, j);
+      wait(0, f);
+      __syncthreads();                            // the previous reads of ex are done
+      if (has1) {
+        c2 in[NI];
+        load(in, stg + 2 * q1 * tz, r0 + q1, j);
+        c2* e = ex + (q1 * N2 + n2) * RS * W + c; // this thread's row [k1]
+        c2 v[N1];
+        if constexpr (HALF) {                     // zero for n1 >= N1/2: two N1/2-point transforms
+          dft_half<N1, -1>(in, v);
+        } else {
 #pragma unroll
-        for (int i = 0; i < NI; ++i) {
-          const float2 s = make_float2(h[i].x + m[i].x, h[i].y - m[i].y);
-          const float2 d = make_float2(h[i].y + m[i].y, m[i].x - h[i].x);
-          h[i] = s;
-          m[i] = d;
+          for (int i = 0; i < N1; ++i) v[i] = in[i];
+          Dft<N1, -1>::run(v);
         }
-        if (!mask || !((r0 + q1) & 1)) FI::template step1w<-1, W>(h, e1 + (mask ? SEQ : 0), n2, tws);
-        if (two || (mask && ((r0 + q1) & 1))) FI::template step1w<-1, W>(m, e1 + SEQ, n2, tws);
+#pragma unroll
+        for (int k = 0; k < N1; ++k) e[k * W] = k == 0 ? v[k] : cmul(v[k], tw2[n2 * k]);
       }
-      if constexpr (MODE != kZPrep) cp_async_wait_all();
       __syncthreads();
-      if (!has2) continue;
+      if (t == 0) {                               // the inputs have been read, the other weights' products summed
+        const int nr = mask ? r0 + Q : r0, nj = mask ? jbeg : j + 1;
+        if (nr < rend) {
+          fetch_inputs(nr, nj);
+          if (kWeights) fetch_weights(nj, (f + 1) & 1);
+        }
+      }
+      c2* e = ex + (q2 * N2 * RS + k1) * W + c;   // its column [n2] in the second step
+      c2 u[N2];
+#pragma unroll
+      for (int i = 0; i < N2; ++i) u[i] = e[i * RS * W];
+      if (kWeights) wait(1 + (f & 1), f >> 1);
+      Dft<N2, -1>::run(u);                        // at kz = k1 + N1 i
       if constexpr (MODE == kZPrep) {
         float wa = 0.25f, wb = 0.25f;             // Eq. 6: (1, 1), (1, 2), (2, 2); Eq. 3: (1, 1), (1, 0)
         if (!mask && g.nch == 3) { wa = j == 2 ? 0.5f : 0.25f; wb = j == 0 ? 0.25f : 0.5f; }
-        for (int s = 0; s < (mask ? 1 : 2); ++s) {
-          float2* o = wt + (long long)(2 * j + s) * P * W + k1 * W + c;
-          const float w = s ? wb : wa;
-          if (s == 1 && !two) {
+        if (!mask && g.nch == 2 && j == 1) wb = 0.0f;
+        if (mask) {
+          float2* o = wt + (long long)(2 * j) * P * W + k1 * W + c;
 #pragma unroll
-            for (int i = 0; i < N2; ++i) o[i * N1 * W] = make_float2(0.f, 0.f);
-            continue;
-          }
-          step2(e2 + (mask || s ? SEQ : 0));
+          for (int i = 0; i < N2; ++i) o[i * N1 * W] = make_float2(wa * u[i].x.x, -wa * u[i].y.x);
+        } else {
+          float4* o = reinterpret_cast<float4*>(wt + (long long)(2 * j) * P * W) + k1 * W + c;
 #pragma unroll
-          for (int i = 0; i < N2; ++i) o[i * N1 * W] = make_float2(w * u[i].x, -w * u[i].y);
+          for (int i = 0; i < N2; ++i)
+            o[i * N1 * W] = make_float4(wa * u[i].x.x, -wa * u[i].y.x, wb * u[i].x.y, -wb * u[i].y.y);
         }
-      } else if (!mask) {
-        step2(e2);
+        continue;
+      }
+      const char* wb = reinterpret_cast<const char*>(ws) + (f & 1) * C::wbytes;
+      if (!mask) {
+        const float4* w4 = reinterpret_cast<const float4*>(wb) + k1 * W + c;
 #pragma unroll
-        for (int i = 0; i < N2; ++i) cmac(X[i], ws[(k1 + N1 * i) * W + c], u[i]);
-        if (two) {
-          step2(e2 + SEQ);
-#pragma unroll
-          for (int i = 0; i < N2; ++i) cmac(X[i], ws[(P + k1 + N1 * i) * W + c], u[i]);
+        for (int i = 0; i < N2; ++i) {
+          const float4 w = w4[i * N1 * W];
+          cmac(X[i], make_float2(w.x, w.y), make_float2(u[i].x.x, u[i].y.x));
+          cmac(X[i], make_float2(w.z, w.w), make_float2(u[i].x.y, u[i].y.y));
         }
       } else {
-        // the second step read this thread's own slots only, and the channels'
-        // exchange is free: both inverses start in place
-        step2(e2 + SEQ);
+        // Y from this rotation's mask, then X and Y side by side into the
+        // inverse: over k2, twiddle, back to the slots this thread has read
+        const float2* wm = reinterpret_cast<const float2*>(wb) + k1 * W + c;
+        const bool odd = r2 & 1;
 #pragma unroll
-        for (int i = 0; i < N2; ++i) u[i] = cmul(ws[(k1 + N1 * i) * W + c], u[i]);
-        inv1(u, e2 + SEQ);
-        inv1(X, e2);
+        for (int i = 0; i < N2; ++i) {
+          const float2 Y = cmul(wm[i * N1 * W], odd ? make_float2(u[i].x.y, u[i].y.y) : make_float2(u[i].x.x, u[i].y.x));
+          u[i] = {make_float2(X[i].x, Y.x), make_float2(X[i].y, Y.y)};
+        }
+        Dft<N2, 1>::run(u);
+#pragma unroll
+        for (int i = 0; i < N2; ++i) {
+          c2 w = tw2[i * k1];
+          w.y = make_float2(-w.y.x, -w.y.y);
+          e[i * RS * W] = i == 0 ? u[i] : cmul(u[i], w);
+        }
       }
     }
     if constexpr (MODE == kZPrep) continue;
     __syncthreads();
     const int r1 = r0 + q1;
-    if (r1 < nrot && col_ok) {
-      float2 x[N1], y[N1];
+    if (has1 && r1 < nrot) {                      // (padded positions hold what nobody reads)
+      const c2* e = ex + (q1 * N2 + n2) * RS * W + c;
+      c2 v[N1];
 #pragma unroll
-      for (int i = 0; i < N1; ++i) {
-        x[i] = e1[i * W];
-        y[i] = e1[SEQ + i * W];
-      }
-      Dft<N1, 1>::run(x);
-      Dft<N1, 1>::run(y);
+      for (int i = 0; i < N1; ++i) v[i] = e[i * W];
+      Dft<N1, 1>::run(v);
       const int m0 = rot[r1].b.m0[0], last = rot[r1].b.hi[0] - rot[r1].b.lo[0];
-      float2* d = F2 + ((long long)r1 * g.Px + kx) * g.wz * g.Py + ky;      // [r][kx][dz][ky]
-      float2* dm = F2 + ((long long)r1 * g.Px + mkx) * g.wz * g.Py + mky;
+      const int pp = W * ntile, mpos = own && c == 0 ? pos : mtile * W + c;
+      float2* d = F2 + ((long long)r1 * g.Px + kx) * g.wz * pp + pos;       // [r][kx][dz][p]
+      float2* dm = F2 + ((long long)r1 * g.Px + mkx) * g.wz * pp + mpos;
       const bool self = mkx == kx;                // its mirrors are columns of this kx
 #pragma unroll
       for (int i = 0; i < N1; ++i) {
         const int dz = window_index(N2 * i + n2, m0, P);
-        if (dz <= last) {
-          d[(long long)dz * g.Py] = make_float2(x[i].x - y[i].y, x[i].y + y[i].x);
-          if (!self) dm[(long long)dz * g.Py] = make_float2(x[i].x + y[i].y, y[i].x - x[i].y);
+        if (dz <= last) {                         // x + iy, and conj x + i conj y
+          d[dz * pp] = make_float2(v[i].x.x - v[i].y.y, v[i].y.x + v[i].x.y);
+          if (!self) dm[dz * pp] = make_float2(v[i].x.x + v[i].y.y, v[i].x.y - v[i].y.x);
         }
       }
     }
+  }
+  if (dead && g.tc_err) atomicExch(g.tc_err, 1);
+  if (dead) {                                     // copies that were not waited for, before the block ends
+    tc::mbar_wait(&bar[0], (f - 1) & 1, kTcWaitNs / 4);
+    if (kWeights)
+      for (int l = f - 1; l >= 0 && l >= f - 2; --l) tc::mbar_wait(&bar[1 + (l & 1)], (l >> 1) & 1, kTcWaitNs / 4);
   }
 }
 
@@ -240,15 +315,18 @@ template <int P, int ST, bool HALF, int V, int MODE>
 void launch_zpass_t(const void* F1, float2* UV, const float2* Xg, float2* F2, Geo g, int nrot, const RotIn* rot,
                     cudaStream_t st) {
   using C = ZCfg<P, V, MODE>;
-  const unsigned tiles = (unsigned)((g.Py + C::W - 1) / C::W), nkx = (unsigned)(g.Px / 2 + 1);
+  const unsigned tiles = (unsigned)(ky_total(g.Py) / C::W), nkx = (unsigned)(g.Px / 2 + 1);
+  int q = std::min(C::Q, C::fit(g.ez));           // large boxes leave room for fewer
+  while (q > 1 && q >= 2 * nrot) q /= 2;
   // rotations per block: few enough that the blocks fill the SMs many times
   // over (a short last wave), more where there are blocks to spare (the weights
   // then come from L2)
   const long long cols = (long long)tiles * nkx;
-  int rpb = 2;
-  while (rpb < 8 && cols * ((nrot + 2 * rpb - 1) / (2 * rpb)) >= 152 * C::MIN_BLOCKS * 16) rpb *= 2;
-  set_smem(k_zpass<P, ST, HALF, V, MODE>, C::smem_bytes);
-  k_zpass<P, ST, HALF, V, MODE><<<dim3(tiles, nkx, (unsigned)((nrot + rpb - 1) / rpb)), C::NT, C::smem_bytes, st>>>(
+  int rpb = q;
+  while (rpb < 16 && cols * ((nrot + 2 * rpb - 1) / (2 * rpb)) >= 152 * C::MIN_BLOCKS * 16) rpb *= 2;
+  const size_t smem = C::smem_bytes(q, g.ez);
+  set_smem(k_zpass<P, ST, HALF, V, MODE>, smem);
+  k_zpass<P, ST, HALF, V, MODE><<<dim3(tiles, nkx, (unsigned)((nrot + rpb - 1) / rpb)), q * C::W * C::N1, smem, st>>>(
       F1, UV, Xg, F2, g, nrot, rpb, rot);
 }
 
