@@ -204,6 +204,8 @@ void free_handle(cs_ngf_fixed* f) {
   cudaFree(f->Mh);
   cudaFree(f->BQ);
   cudaFree(f->C8);
+  cudaFree(f->N8);
+  cudaFree(f->mbox);
   cudaFree(f->F02);
   cudaFree(f->F13);
   cudaFree(f->msum);
@@ -426,9 +428,21 @@ cs_ngf_status run_transforms(cs_ngf_fixed* f, const RotIn* rot, int nb, float* m
   return CS_NGF_OK;
 }
 
-// (B, M_B) -> f->BQ, f->C8, shared by every rotation of the call
-cs_ngf_status pack_floating(cs_ngf_fixed* f, const float* B, const uint8_t* MB, cudaStream_t st) {
-  { Stage sp(f, 0, st); k_pack_floating<<<512, 256, 0, st>>>(B, MB, f->g, f->BQ, f->C8); }
+// (B, M_B) -> f->BQ, f->C8, shared by the R rotations of the call; with enough of
+// them (the three passes cost a few rotations' saving), the cells near the mask
+cs_ngf_status pack_floating(cs_ngf_fixed* f, const float* B, const uint8_t* MB, int R, cudaStream_t st) {
+  const Geo& g = f->g;
+  const bool bound = f->pad_mode == CS_NGF_PAD_BOUND;
+  if (bound) CS_CUDA(cudaMemsetAsync(f->mbox, 0x80, sizeof(int) * 6, st));
+  { Stage sp(f, 0, st); k_pack_floating<<<512, 256, 0, st>>>(B, MB, g, f->BQ, f->C8, bound ? f->mbox : nullptr); }
+  f->near = bound && R >= 16;
+  if (f->near) {
+    uint8_t* tmp = f->N8;
+    uint8_t* out = f->N8 + g.nvox;
+    { Stage sp(f, 0, st); k_near_axis<<<1024, 256, 0, st>>>(f->C8, out, g, 2); }
+    { Stage sp(f, 0, st); k_near_axis<<<1024, 256, 0, st>>>(out, tmp, g, 1); }
+    { Stage sp(f, 0, st); k_near_axis<<<1024, 256, 0, st>>>(tmp, out, g, 0); }
+  }
   return check_launch("pack");
 }
 
@@ -444,7 +458,8 @@ cs_ngf_status score_batch(cs_ngf_fixed* f, int r0, int nb, float* best_score, in
   if (f->pad_mode == CS_NGF_PAD_BOUND) {
     {
       Stage sp(f, 0, st);
-      k_resample_box<<<resample_box_grid(g, nb), 128, 0, st>>>(f->BQ, f->C8, rot, g, f->Bh, f->Mh);
+      k_resample_box<<<resample_box_grid(g, nb), 128, 0, st>>>(f->BQ, f->C8, f->near ? f->N8 + g.nvox : nullptr, rot, g,
+                                                               f->Bh, f->Mh);
     }
     if (cs_ngf_status s = check_launch("resample")) return s;
   } else {
@@ -599,11 +614,10 @@ cs_ngf_status rotation_bounds(cs_ngf_fixed* f, int R, cudaStream_t st) {
   int* msum = f->allm;
   int* marg = f->allm + R;
   CS_CUDA(cudaMemsetAsync(f->allm, 0, sizeof(int) * (size_t)R * (1 + nmarg), st));
-  const int most = 65535 / (int)resample_grid(g, 1).z;      // rotations a grid's z dimension holds
-  for (int r0 = 0; r0 < R; r0 += most) {
-    const int nb = std::min(most, R - r0);
+  for (int r0 = 0; r0 < R; r0 += 65535) {
+    const dim3 grid((unsigned)((g.nx + 7) / 8), (unsigned)((g.ny + 3) / 4), (unsigned)std::min(65535, R - r0));
     Stage sp(f, 0, st);
-    k_mask_counts<<<resample_grid(g, nb), 128, 0, st>>>(f->C8, f->rot_d + r0, g, msum + r0, marg + nmarg * r0);
+    k_mask_counts<<<grid, 128, 0, st>>>(f->C8, f->rot_d + r0, g, f->mbox, msum + r0, marg + nmarg * r0);
   }
   if (cs_ngf_status s = check_launch("mask counts")) return s;
   {
@@ -810,7 +824,7 @@ cs_ngf_status score_all(cs_ngf_fixed* f, const float* B, const uint8_t* MB, cons
   if (R <= 0) return fail(CS_NGF_EINVAL, "R must be positive");
   if (!best_score || !best_shift) return fail(CS_NGF_EINVAL, "output pointer is NULL");
   if (cs_ngf_status s = upload_rotations(f, quats, R, st)) return s;
-  if (cs_ngf_status s = pack_floating(f, B, MB, st)) return s;
+  if (cs_ngf_status s = pack_floating(f, B, MB, R, st)) return s;
   Plan plan;
   if (cs_ngf_status s = plan_classes_impl(f, R, st, plan)) return s;
   // classes one after another; with several, into the handle's buffers, then
@@ -883,7 +897,7 @@ Sizes sizes_for(const int32_t dims[3], const int pad[3], int measure, int precis
   z.fixed_f13 = nf * E1;
   z.zx_elems = (tensor_cores && precision != CS_NGF_FP32) ? (Px / 2 + 1) * PyT * Pz : 0;
   z.per_rot = (z.f02_elems + z.f13_elems + z.zx_elems) * sizeof(float2) + nvox * 5;
-  z.shared_ws = nvox * (sizeof(float4) + 1);                       // BQ, C8
+  z.shared_ws = nvox * (sizeof(float4) + 3);                       // BQ, C8, N8
   z.uv_elems = (2 * nch + 1) * (Px / 2 + 1) * PyT * Pz;
   return z;
 }
@@ -909,8 +923,8 @@ namespace detail {
 cs_ngf_status upload_rotations(cs_ngf_fixed* f, const double* q, int R, cudaStream_t st) {
   return ::upload_rotations(f, q, R, st);
 }
-cs_ngf_status pack_floating(cs_ngf_fixed* f, const float* B, const uint8_t* MB, cudaStream_t st) {
-  return ::pack_floating(f, B, MB, st);
+cs_ngf_status pack_floating(cs_ngf_fixed* f, const float* B, const uint8_t* MB, int R, cudaStream_t st) {
+  return ::pack_floating(f, B, MB, R, st);
 }
 cs_ngf_status score_range(cs_ngf_fixed* f, int r0, int n, float* best_score, int32_t* best_shift,
                           cudaStream_t st) {
@@ -1072,6 +1086,8 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
   CS_TRYC(dalloc(&f->Mh, (size_t)batch * g.nvox));
   CS_TRYC(dalloc(&f->BQ, (size_t)g.nvox));
   CS_TRYC(dalloc(&f->C8, (size_t)g.nvox));
+  CS_TRYC(dalloc(&f->N8, (size_t)g.nvox * 2));
+  CS_TRYC(dalloc(&f->mbox, (size_t)6));
   CS_TRYC(dalloc(&f->F02, std::max((size_t)batch * f->f02_elems, sz.fixed_f02)));
   CS_TRYC(dalloc(&f->F13, std::max((size_t)batch * f->f13_elems, sz.fixed_f13)));
   CS_TRYC(dalloc(&f->msum, (size_t)batch));
@@ -1187,7 +1203,7 @@ cs_ngf_status cs_ngf_score_map(cs_ngf_fixed* f, const float* B, const uint8_t* m
   CS_CLAIM(f, st, true);
   if (cs_ngf_status s = ensure_results(f, 1)) return s;
   if (cs_ngf_status s = upload_rotations(f, quat, 1, st)) return s;
-  if (cs_ngf_status s = pack_floating(f, B, maskB, st)) return s;
+  if (cs_ngf_status s = pack_floating(f, B, maskB, 1, st)) return s;
   Plan plan;
   if (cs_ngf_status s = plan_classes_impl(f, 1, st, plan)) return s;
   if (cs_ngf_status s = set_class_impl(f, plan.cls[0], st)) return s;
@@ -1205,7 +1221,7 @@ cs_ngf_status cs_ngf_resample(cs_ngf_fixed* f, const float* B, const uint8_t* ma
   if (cs_ngf_status s = upload_rotations(f, quat, 1, st)) return s;
   CS_CUDA(cudaMemsetAsync(f->msum, 0, sizeof(int), st));
   const Geo& g = f->g;
-  if (cs_ngf_status s = pack_floating(f, B, maskB, st)) return s;
+  if (cs_ngf_status s = pack_floating(f, B, maskB, 1, st)) return s;
   k_resample<<<resample_grid(g, 1), 128, 0, st>>>(f->BQ, f->C8, f->rot_d, g, Bhat, Mhat, f->msum, nullptr);
   return check_launch("resample");
 }

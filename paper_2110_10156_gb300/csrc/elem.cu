@@ -44,8 +44,10 @@ __device__ __forceinline__ float lerp_rn(float a, float b, float t) {
 // base is never on a far face (axis_sample clamps i0 <= n - 2); entries past
 // the volume hold 0.
 __global__ void k_pack_floating(const float* __restrict__ B, const uint8_t* __restrict__ MB, Geo g,
-                                float4* __restrict__ BQ, uint8_t* __restrict__ C8) {
+                                float4* __restrict__ BQ, uint8_t* __restrict__ C8,
+                                int* __restrict__ mbox) {
   const int sy = g.nx, sz = g.nx * g.ny;          // volumes hold < 2^31 voxels
+  int b[6] = {-(1 << 30), -(1 << 30), -(1 << 30), -1, -1, -1};   // -min z, y, x and max of cells with a mask corner
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.nvox;
        i += (long long)gridDim.x * blockDim.x) {
     const int x = (int)(i % g.nx), y = (int)((i / g.nx) % g.ny), z = (int)(i / sz);
@@ -59,6 +61,31 @@ __global__ void k_pack_floating(const float* __restrict__ B, const uint8_t* __re
       for (int k = 0; k < 8; ++k) bits |= (MB[i + o[k]] ? 1u : 0u) << k;
     }
     C8[i] = (uint8_t)bits;
+    if (bits) {
+      b[0] = max(b[0], -z); b[1] = max(b[1], -y); b[2] = max(b[2], -x);
+      b[3] = max(b[3], z); b[4] = max(b[4], y); b[5] = max(b[5], x);
+    }
+  }
+  if (!mbox) return;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const int v = __reduce_max_sync(0xffffffffu, b[k]);
+    if ((threadIdx.x & 31) == 0 && v > (k < 3 ? -(1 << 30) : -1)) atomicMax(&mbox[k], v);
+  }
+}
+
+// out[i] = any of in over the five voxels around i along one axis: three passes
+// mark every cell within two of a cell with a mask corner
+__global__ void k_near_axis(const uint8_t* __restrict__ in, uint8_t* __restrict__ out, Geo g, int axis) {
+  const int n = axis == 0 ? g.nz : (axis == 1 ? g.ny : g.nx);
+  const int st = axis == 0 ? g.nx * g.ny : (axis == 1 ? g.nx : 1);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (int)g.nvox; i += gridDim.x * blockDim.x) {
+    const int k = i / st % n;
+    uint8_t v = 0;
+#pragma unroll
+    for (int o = -2; o <= 2; ++o)
+      if (k + o >= 0 && k + o < n) v |= in[i + o * st];
+    out[i] = v ? 1 : 0;
   }
 }
 
@@ -117,17 +144,19 @@ __device__ __forceinline__ uint8_t mask_voxel(const uint8_t* __restrict__ C8, co
   return mask_decision(__ldg(&C8[b000]), ax.t, ay.t, az.t);
 }
 
-__device__ __forceinline__ void resample_voxel(const float4* __restrict__ BQ,
+// false (nothing set): the sample's cell is not marked in N8
+__device__ __forceinline__ bool resample_voxel(const float4* __restrict__ BQ,
                                                const uint8_t* __restrict__ C8, const RotMat& R,
                                                const SampleRow& sr, const Geo& g, int z, float& val,
-                                               uint8_t& m) {
+                                               uint8_t& m, const uint8_t* __restrict__ N8 = nullptr) {
   AxisSample ax, ay, az;
   sample_axes(R, sr, g, z, ax, ay, az);
+  const int sy = g.nx, sz = g.nx * g.ny;          // volumes hold < 2^31 voxels
+  const int b000 = az.i0 * sz + ay.i0 * sy + ax.i0;
+  if (N8 && !__ldg(&N8[b000])) return false;
   val = 0.0f;
   m = 0;
   if (ax.inside && ay.inside && az.inside) {
-    const int sy = g.nx, sz = g.nx * g.ny;        // volumes hold < 2^31 voxels
-    const int b000 = az.i0 * sz + ay.i0 * sy + ax.i0;
     const float4 q0 = __ldg(&BQ[b000]), q1 = __ldg(&BQ[b000 + sz]);   // z-faces z0, z0 + 1
     const float2 c00 = make_float2(q0.x, q0.y), c01 = make_float2(q0.z, q0.w);
     const float2 c10 = make_float2(q1.x, q1.y), c11 = make_float2(q1.z, q1.w);
@@ -140,6 +169,7 @@ __device__ __forceinline__ void resample_voxel(const float4* __restrict__ BQ,
     val = lerp_exact(v0, v1, az.t);
     m = mask_decision(bits, ax.t, ay.t, az.t);
   }
+  return true;
 }
 
 // Section 3.2 resample.  Block: 8 x 4 voxels per warp (x fastest), so one
@@ -148,8 +178,6 @@ __device__ __forceinline__ void resample_voxel(const float4* __restrict__ BQ,
 // (block: 8 x 4 x 4*RZ voxels).  Mask counts per axis (the slab bound's
 // marginals) are reduced with warp shuffles before one atomic per slot.
 // Grid: (x tiles, y tiles, z tiles * rotations).
-// MONLY: only the rotated mask, counted (no volumes written)
-template <bool MONLY>
 __device__ __forceinline__ void resample_block(const float4* __restrict__ BQ,
                                                const uint8_t* __restrict__ C8,
                                                const RotIn* __restrict__ rot, const Geo& g,
@@ -175,16 +203,12 @@ __device__ __forceinline__ void resample_block(const float4* __restrict__ BQ,
     const int z = zt * ZB + 4 * k + wid;
     int mk = 0;
     if (xy_ok && z < g.nz) {
-      if constexpr (MONLY) {
-        mk = mask_voxel(C8, R, sr, g, z);
-      } else {
-        float val;
-        uint8_t m;
-        resample_voxel(BQ, C8, R, sr, g, z, val, m);
-        Bh[idx] = val;
-        Mh[idx] = m;
-        mk = m;
-      }
+      float val;
+      uint8_t m;
+      resample_voxel(BQ, C8, R, sr, g, z, val, m);
+      Bh[idx] = val;
+      Mh[idx] = m;
+      mk = m;
     }
     c += mk;
     const int wz = __reduce_add_sync(0xffffffffu, mk);      // plane z, this warp's patch
@@ -228,21 +252,99 @@ __global__ void __launch_bounds__(128)
 k_resample(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8,
            const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh, uint8_t* __restrict__ Mh,
            int* __restrict__ msum, int* __restrict__ marg) {
-  resample_block<false>(BQ, C8, rot, g, Bh, Mh, msum, marg);
+  resample_block(BQ, C8, rot, g, Bh, Mh, msum, marg);
 }
 
+// z-planes whose sample points along this thread's (x, y) can lie in the cells
+// [lo, hi] per axis (z, y, x) that hold a mask corner, with a margin for the
+// rounding of the estimate; an axis the line runs almost across only rules
+// whole lines out
+__device__ __forceinline__ void z_range(const RotMat& R, const SampleRow& sr, const Geo& g, const int* lo,
+                                        const int* hi, int& z0, int& z1) {
+  const float c[3] = {0.5f * (float)(g.nx - 1), 0.5f * (float)(g.ny - 1), 0.5f * (float)(g.nz - 1)};
+  float a = -1.0f, b = (float)g.nz;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {                   // x, y, z
+    const float l = (float)lo[2 - i], h = (float)(hi[2 - i] + 1);
+    const float q = sr.s[i] + c[i], d = R.m[3 * i + 2];
+    if (fabsf(d) < 1e-3f) {
+      if (q < l - 1.0f || q > h + 1.0f) b = -2.0f;
+    } else {
+      const float inv = 1.0f / d;
+      const float t0 = (l - 0.01f - q) * inv + c[2], t1 = (h + 0.01f - q) * inv + c[2];
+      a = fmaxf(a, fminf(t0, t1) - 0.05f);
+      b = fminf(b, fmaxf(t0, t1) + 0.05f);
+    }
+  }
+  z0 = max(0, (int)floorf(a));
+  z1 = min(g.nz - 1, (int)ceilf(b));
+}
+
+// Grid: (x tiles, y tiles, rotations).  Block: an 8 x 4 patch of (x, y), its four
+// warps on every fourth plane of the range that can meet the floating mask's
+// box (0.4 of the planes at 150^3 with a foreground mask: 8.4 -> 4 us per
+// rotation).
 __global__ void __launch_bounds__(128)
-k_mask_counts(const uint8_t* __restrict__ C8, const RotIn* __restrict__ rot, Geo g,
+k_mask_counts(const uint8_t* __restrict__ C8, const RotIn* __restrict__ rot, Geo g, const int* __restrict__ mbox,
               int* __restrict__ msum, int* __restrict__ marg) {
-  resample_block<true>(nullptr, C8, rot, g, nullptr, nullptr, msum, marg);
+  __shared__ int zs[256], ys[4][4], xs[4][8], cs[4];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5, r = blockIdx.z;
+  const int tx = lane & 7, ty = lane >> 3;
+  const int x = blockIdx.x * 8 + tx, y = blockIdx.y * 4 + ty;
+  const RotMat R = rot[r].m;
+  const SampleRow sr = sample_row(R, g, x, y);
+  const int lo[3] = {-mbox[0], -mbox[1], -mbox[2]}, hi[3] = {mbox[3], mbox[4], mbox[5]};
+  int z0 = 1 << 30, z1 = -1;
+  if (x < g.nx && y < g.ny && hi[0] >= 0) z_range(R, sr, g, lo, hi, z0, z1);
+  const bool some = z0 <= z1;
+  const int w0 = __reduce_min_sync(0xffffffffu, some ? z0 : 1 << 30);
+  const int w1 = __reduce_max_sync(0xffffffffu, some ? z1 : -1);
+  if (w0 > w1) return;                            // (the four warps of a block agree)
+  for (int z = t; z < g.nz; z += 128) zs[z] = 0;
+  __syncthreads();
+  int c = 0;                                      // this thread's mask voxels
+#pragma unroll 1
+  for (int z = w0 + ((wid - w0) & 3); z <= w1; z += 4) {
+    const int mk = some && z >= z0 && z <= z1 ? mask_voxel(C8, R, sr, g, z) : 0;
+    c += mk;
+    const int wz = __reduce_add_sync(0xffffffffu, mk);
+    if (lane == 0) zs[z] = wz;
+  }
+  int cy = c;                                     // lanes sharing ty: xor over the tx bits
+  cy += __shfl_xor_sync(0xffffffffu, cy, 1);
+  cy += __shfl_xor_sync(0xffffffffu, cy, 2);
+  cy += __shfl_xor_sync(0xffffffffu, cy, 4);
+  int cx = c;                                     // lanes sharing tx: xor over the ty bits
+  cx += __shfl_xor_sync(0xffffffffu, cx, 8);
+  cx += __shfl_xor_sync(0xffffffffu, cx, 16);
+  if (tx == 0) ys[wid][ty] = cy;
+  if (ty == 0) xs[wid][tx] = cx;
+  const int cw = __reduce_add_sync(0xffffffffu, c);
+  if (lane == 0) cs[wid] = cw;
+  __syncthreads();
+  const int total = cs[0] + cs[1] + cs[2] + cs[3];
+  if (!total) return;
+  int* mr = marg + (long long)r * (g.nz + g.ny + g.nx);
+  if (t == 0) atomicAdd(&msum[r], total);
+  for (int z = w0 + t; z <= w1; z += 128)
+    if (zs[z]) atomicAdd(&mr[z], zs[z]);
+  if (t < 4) {
+    const int v = ys[0][t] + ys[1][t] + ys[2][t] + ys[3][t];
+    if (v) atomicAdd(&mr[g.nz + blockIdx.y * 4 + t], v);
+  } else if (t < 12) {
+    const int q = t - 4, v = xs[0][q] + xs[1][q] + xs[2][q] + xs[3][q];
+    if (v) atomicAdd(&mr[g.nz + g.ny + blockIdx.x * 8 + q], v);
+  }
 }
 
 // The voxels the x pass reads: each rotation's box of Geo::ez x ey x ex voxels
 // and one voxel around it (the gradient's neighbours), clipped to the volume.
 // The counts are known by then, so nothing is reduced.  At 150^3 with a
-// foreground mask the box holds 0.4 of the volume.
+// foreground mask the box holds 0.4 of the volume, and half of its voxels have
+// no mask voxel next to them: their values are never read, so with N8 (cells
+// within two of a mask corner; nullptr: all) only their mask is written.
 __global__ void __launch_bounds__(128)
-k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8,
+k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8, const uint8_t* __restrict__ N8,
                const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh, uint8_t* __restrict__ Mh) {
   constexpr int RZ = kResampleZGroups, ZB = 4 * RZ;
   const int ztiles = (g.ez + 2 + ZB - 1) / ZB;
@@ -263,7 +365,10 @@ k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8,
     if (z < 0 || z >= z_end) continue;
     float val;
     uint8_t m;
-    resample_voxel(BQ, C8, R, sr, g, z, val, m);
+    if (!resample_voxel(BQ, C8, R, sr, g, z, val, m, N8)) {
+      Mh[idx] = 0;                                // a unit step in the volume moves a sample by at most one cell
+      continue;                                   // (two, with rounding): no mask voxel is next to this one
+    }
     Bh[idx] = val;
     Mh[idx] = m;
   }

@@ -62,6 +62,9 @@ struct cs_ngf_fixed {
   uint8_t* Mh = nullptr;
   float4* BQ = nullptr;        // x-pairs of rows y, y+1 (B[i], B[i+1], B[i+sy], B[i+sy+1]) of the current call
   uint8_t* C8 = nullptr;       // corner codes of M_B of the current call
+  uint8_t* N8 = nullptr;       // cells near its mask, and a scratch volume before them [2][nvox]
+  int* mbox = nullptr;         // its mask's cell box (k_pack_floating)
+  bool near = false;           // N8 holds the current call's
   float2* F02 = nullptr;
   float2* F13 = nullptr;
   int* msum = nullptr;
@@ -103,8 +106,8 @@ namespace detail {
 cs_ngf_status fail(cs_ngf_status s, const std::string& msg);
 // host FP64 quaternions -> FP32 matrices in f->rot_h[0..R) and f->rot_d[0..R)
 cs_ngf_status upload_rotations(cs_ngf_fixed* f, const double* quats, int R, cudaStream_t st);
-// (B, M_B) -> f->BQ, f->C8 for the following score calls
-cs_ngf_status pack_floating(cs_ngf_fixed* f, const float* B, const uint8_t* MB, cudaStream_t st);
+// (B, M_B) -> f->BQ, f->C8 for the following scoring of R rotations
+cs_ngf_status pack_floating(cs_ngf_fixed* f, const float* B, const uint8_t* MB, int R, cudaStream_t st);
 // Rotations scored together: FFT lengths, box extents and shift windows per
 // axis (z, y, x), and the end of the class in the call's regrouped order.
 struct ClassGeom { int pad[3], ext[3], win[3], end; };

@@ -163,8 +163,11 @@ __device__ __forceinline__ unsigned long long make_key(float s, unsigned lin) {
 // contraction), so the decision is reproducible bit for bit.  B and M_B are
 // read as the row-pair table and corner codes k_pack_floating prepares (BQ,
 // C8: nvox entries each).
+// mbox (or nullptr): -min z, y, x and max z, y, x of the cells with a mask
+// corner, accumulated with atomicMax
 __global__ void k_pack_floating(const float* __restrict__ B, const uint8_t* __restrict__ MB, Geo g,
-                                float4* __restrict__ BQ, uint8_t* __restrict__ C8);
+                                float4* __restrict__ BQ, uint8_t* __restrict__ C8, int* __restrict__ mbox);
+__global__ void k_near_axis(const uint8_t* __restrict__ in, uint8_t* __restrict__ out, Geo g, int axis);
 // k_resample: the whole volume, mask counts into msum and marg (marg may be
 // nullptr); grid resample_grid.  k_resample_box: only the voxels the x pass
 // reads, each rotation's box and one voxel around it; grid resample_box_grid.
@@ -172,13 +175,13 @@ __global__ void k_resample(const float4* __restrict__ BQ, const uint8_t* __restr
                            const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh,
                            uint8_t* __restrict__ Mh, int* __restrict__ msum, int* __restrict__ marg);
 __global__ void k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8,
-                               const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh,
+                               const uint8_t* __restrict__ N8, const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh,
                                uint8_t* __restrict__ Mh);
 // The rotated masks alone, counted into msum and marg as k_resample counts
 // them (the same decisions from the same corner codes, no volumes written):
-// the pre-pass that bounds the shifts of a whole call.  Grid: resample_grid.
+// the pre-pass that bounds the shifts of a whole call.
 __global__ void k_mask_counts(const uint8_t* __restrict__ C8, const RotIn* __restrict__ rot, Geo g,
-                              int* __restrict__ msum, int* __restrict__ marg);
+                              const int* __restrict__ mbox, int* __restrict__ msum, int* __restrict__ marg);
 constexpr int kResampleZGroups = 8;            // z-plane groups of 4 per resample block
 inline dim3 resample_grid(const Geo& g, int nrot) {
   return dim3((unsigned)((g.nx + 7) / 8), (unsigned)((g.ny + 3) / 4),
