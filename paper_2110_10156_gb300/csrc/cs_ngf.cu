@@ -185,14 +185,10 @@ cs_ngf_status check_launch(const char* what) {
 }
 
 // ECUDA (once) if a tensor-core pass of this handle stopped on its bounded
-// wait since the last check; `st` has been synchronised by the caller
-cs_ngf_status tc_status(cs_ngf_fixed* f, cudaStream_t st) {
-  if (!f->tc_err) return CS_NGF_OK;
-  int flag = 0;
-  CS_CUDA(cudaMemcpyAsync(&flag, f->tc_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-  CS_CUDA(cudaStreamSynchronize(st));
-  if (!flag) return CS_NGF_OK;
-  CS_CUDA(cudaMemsetAsync(f->tc_err, 0, sizeof(int), st));
+// wait since the last check; the caller has synchronised its stream
+cs_ngf_status tc_status(cs_ngf_fixed* f) {
+  if (!f->tc_err || !*(volatile int*)f->tc_err) return CS_NGF_OK;
+  *f->tc_err = 0;
   return fail(CS_NGF_ECUDA, "a z pass timed out waiting for its MMAs or copies; its results are invalid");
 }
 
@@ -213,14 +209,14 @@ void free_handle(cs_ngf_fixed* f) {
   cudaFree(f->margB);
   cudaFree(f->bounds);
   cudaFree(f->keys);
-  cudaFree(f->tc_err);
+  cudaFreeHost(f->tc_err);
+  cudaFreeHost(f->fbox_h);
   cudaFree(f->zx);
   if (f->rot_ev) cudaEventSynchronize(f->rot_ev);
   if (f->order_ev) cudaEventDestroy(f->order_ev);
   for (auto& sp : f->spans) { cudaEventDestroy(sp.a); cudaEventDestroy(sp.b); }
   cudaFree(f->boxA);
   cudaFree(f->allm);
-  cudaFree(f->allb);
   cudaFreeHost(f->allb_h);
   cudaFree(f->perm_d);
   cudaFree(f->perm_score);
@@ -230,15 +226,15 @@ void free_handle(cs_ngf_fixed* f) {
   if (f->rot_ev) cudaEventDestroy(f->rot_ev);
   cudaFree(f->stage_B);
   cudaFree(f->stage_M);
-  cudaFree(f->res_score);
-  cudaFree(f->res_shift);
+  cudaFreeHost(f->res_score);
+  cudaFreeHost(f->res_shift);
   cudaFree(f->A_keep);
   cudaFree(f->MA_keep);
   delete f;
 }
 
-// upload R rotation matrices (host FP64 quaternions) to f->rot_d, boxes empty
-cs_ngf_status upload_rotations(cs_ngf_fixed* f, const double* quats, int R, cudaStream_t st) {
+// R rotation matrices (host FP64 quaternions) into f->rot_h, boxes empty
+cs_ngf_status fill_rotations(cs_ngf_fixed* f, const double* quats, int R) {
   if (!quats) return fail(CS_NGF_EINVAL, "quats is NULL");
   for (int r = 0; r < R; ++r) {
     const double* q = quats + 4 * r;
@@ -267,8 +263,6 @@ cs_ngf_status upload_rotations(cs_ngf_fixed* f, const double* quats, int R, cuda
     f->rot_h[r] = RotIn{};
     for (int i = 0; i < 9; ++i) f->rot_h[r].m.m[i] = (float)Rm[i];
   }
-  CS_CUDA(cudaMemcpyAsync(f->rot_d, f->rot_h, sizeof(RotIn) * R, cudaMemcpyHostToDevice, st));
-  CS_CUDA(cudaEventRecord(f->rot_ev, st));
   return CS_NGF_OK;
 }
 
@@ -428,13 +422,52 @@ cs_ngf_status run_transforms(cs_ngf_fixed* f, const RotIn* rot, int nb, float* m
   return CS_NGF_OK;
 }
 
-// (B, M_B) -> f->BQ, f->C8, shared by the R rotations of the call; with enough of
-// them (the three passes cost a few rotations' saving), the cells near the mask
-cs_ngf_status pack_floating(cs_ngf_fixed* f, const float* B, const uint8_t* MB, int R, cudaStream_t st) {
+cs_ngf_status ensure_rotation_buffers(cs_ngf_fixed* f, int R) {
+  if (R <= f->allb_cap) return CS_NGF_OK;
+  CS_CUDA(cudaDeviceSynchronize());              // the old buffers may still be read
+  cudaFree(f->allm);
+  cudaFreeHost(f->allb_h);
+  cudaFree(f->perm_d);
+  cudaFree(f->perm_score);
+  cudaFree(f->perm_shift);
+  f->allm = f->perm_d = nullptr;
+  f->allb_h = nullptr;
+  f->perm_score = nullptr;
+  f->perm_shift = nullptr;
+  f->allb_cap = 0;
+  const int cap = std::max(R, 64);
+  CS_CUDA(dalloc(&f->allm, (size_t)cap * (1 + (size_t)f->g.nz + f->g.ny + f->g.nx)));
+  CS_CUDA(cudaMallocHost((void**)&f->allb_h, sizeof(RotBounds) * (size_t)cap));
+  CS_CUDA(dalloc(&f->perm_d, (size_t)cap));
+  CS_CUDA(dalloc(&f->perm_score, (size_t)cap));
+  CS_CUDA(dalloc(&f->perm_shift, (size_t)cap * 3));
+  f->allb_cap = cap;
+  return CS_NGF_OK;
+}
+
+// Everything a call brings, on the device: (B, M_B) -> f->BQ, f->C8, shared by
+// its R rotations, the rotation matrices, zeroed mask counts; with enough
+// rotations (the three passes cost a few rotations' saving) the cells near the
+// mask.  One kernel does all but the last: at 32^3 the copies and memsets took
+// longer than the kernels they fed.
+cs_ngf_status stage_call_impl(cs_ngf_fixed* f, const float* B, const uint8_t* MB, const double* quats, int R,
+                              cudaStream_t st) {
   const Geo& g = f->g;
   const bool bound = f->pad_mode == CS_NGF_PAD_BOUND;
-  if (bound) CS_CUDA(cudaMemsetAsync(f->mbox, 0x80, sizeof(int) * 6, st));
-  { Stage sp(f, 0, st); k_pack_floating<<<512, 256, 0, st>>>(B, MB, g, f->BQ, f->C8, bound ? f->mbox : nullptr); }
+  if (cs_ngf_status s = fill_rotations(f, quats, R)) return s;
+  if (bound)
+    if (cs_ngf_status s = ensure_rotation_buffers(f, R)) return s;
+  CallStage cs{};
+  cs.src = reinterpret_cast<const int*>(f->rot_h);
+  cs.dst = reinterpret_cast<int*>(f->rot_d);
+  cs.words = R * (int)(sizeof(RotIn) / sizeof(int));
+  if (bound) {
+    cs.zero = f->allm;
+    cs.zeros = R * (1 + g.nz + g.ny + g.nx);
+    cs.mbox = f->mbox;
+  }
+  { Stage sp(f, 0, st); k_pack_floating<<<512, 256, 0, st>>>(B, MB, g, f->BQ, f->C8, cs); }
+  CS_CUDA(cudaEventRecord(f->rot_ev, st));
   f->near = bound && R >= 16;
   if (f->near) {
     uint8_t* tmp = f->N8;
@@ -454,16 +487,16 @@ cs_ngf_status score_batch(cs_ngf_fixed* f, int r0, int nb, float* best_score, in
                           float* map, cudaStream_t st, bool tune = false) {
   const Geo& g = f->g;
   RotIn* rot = f->rot_d + r0;
-  CS_CUDA(cudaMemsetAsync(f->keys, 0, sizeof(unsigned long long) * nb, st));
   if (f->pad_mode == CS_NGF_PAD_BOUND) {
     {
       Stage sp(f, 0, st);
       k_resample_box<<<resample_box_grid(g, nb), 128, 0, st>>>(f->BQ, f->C8, f->near ? f->N8 + g.nvox : nullptr, rot, g,
-                                                               f->Bh, f->Mh);
+                                                               f->Bh, f->Mh, f->keys);
     }
     if (cs_ngf_status s = check_launch("resample")) return s;
   } else {
     const size_t nmarg = (size_t)g.nz + g.ny + g.nx;
+    CS_CUDA(cudaMemsetAsync(f->keys, 0, sizeof(unsigned long long) * nb, st));
     CS_CUDA(cudaMemsetAsync(f->msum, 0, sizeof(int) * nb, st));
     CS_CUDA(cudaMemsetAsync(f->margB, 0, sizeof(int) * nmarg * nb, st));
     {
@@ -474,7 +507,7 @@ cs_ngf_status score_batch(cs_ngf_fixed* f, int r0, int nb, float* best_score, in
     {
       Stage sp(f, 7, st);
       k_shift_bounds<<<dim3((unsigned)nb, 3u), 512, 0, st>>>(f->margA, f->margB, f->msum, f->sumA,
-                                                             f->gamma, g, f->bounds);
+                                                             f->gamma, g, f->bounds, nullptr);
     }
     if (cs_ngf_status s = check_launch("shift bounds")) return s;
     const double pvol = (double)g.Px * (double)g.Py * (double)g.Pz;
@@ -513,31 +546,23 @@ cs_ngf_status run_spectra(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cu
   return check_launch("prep_z");
 }
 
-// a new fixed volume: slab counts of its mask, its box, and the spectra at the
-// lengths in use; synchronises st
+// a new fixed volume: slab counts of its mask, its box, copies where later
+// changes of length need them, and the spectra at the lengths in use;
+// synchronises st
 cs_ngf_status load_fixed(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cudaStream_t st) {
   const Geo& g = f->g;
-  const int n[3] = {g.nz, g.ny, g.nx};
-  std::vector<int> marg((size_t)g.nz + g.ny + g.nx);
-  CS_CUDA(cudaMemsetAsync(f->margA, 0, sizeof(int) * marg.size(), st));
-  { Stage sp(f, 6, st); k_marginals<<<(unsigned)g.nz, 256, 0, st>>>(MA, g, f->margA); }
+  CS_CUDA(cudaMemsetAsync(f->margA, 0, sizeof(int) * ((size_t)g.nz + g.ny + g.nx), st));
+  { Stage sp(f, 6, st); k_marginals<<<(unsigned)g.nz, 256, 0, st>>>(A, MA, g, f->margA, f->A_keep, f->MA_keep); }
+  { Stage sp(f, 6, st); k_fixed_box<<<1, 256, 0, st>>>(f->margA, g, f->boxed ? 1 : 0, f->fbox_h, f->boxA); }
   if (cs_ngf_status s = check_launch("marginals")) return s;
-  CS_CUDA(cudaMemcpyAsync(marg.data(), f->margA, sizeof(int) * marg.size(), cudaMemcpyDeviceToHost, st));
   CS_CUDA(cudaStreamSynchronize(st));
-  f->sumA = 0;
-  for (int z = 0; z < g.nz; ++z) f->sumA += marg[z];
-  RotIn box{};
-  const int* m = marg.data();
-  for (int a = 0; a < 3; m += n[a], ++a) {
-    int lo = 0, hi = n[a] - 1;
-    while (lo < hi && !m[lo]) ++lo;
-    while (hi > lo && !m[hi]) --hi;
-    f->a0[a] = lo;
-    f->a1[a] = hi;
-    box.b.org[a] = f->boxed ? lo : 0;
-    f->extA[a] = f->pad_mode == CS_NGF_PAD_BOUND ? hi + 1 - box.b.org[a] : n[a];
+  const int n[3] = {g.nz, g.ny, g.nx};
+  f->sumA = f->fbox_h->sum;
+  for (int a = 0; a < 3; ++a) {
+    f->a0[a] = f->fbox_h->a0[a];
+    f->a1[a] = f->fbox_h->a1[a];
+    f->extA[a] = f->pad_mode == CS_NGF_PAD_BOUND ? f->a1[a] + 1 - (f->boxed ? f->a0[a] : 0) : n[a];
   }
-  CS_CUDA(cudaMemcpyAsync(f->boxA, &box, sizeof(RotIn), cudaMemcpyHostToDevice, st));
   return run_spectra(f, A, MA, st);
 }
 
@@ -579,41 +604,14 @@ int length_for(int need, int cap) {
   return cap;
 }
 
-cs_ngf_status ensure_rotation_buffers(cs_ngf_fixed* f, int R) {
-  if (R <= f->allb_cap) return CS_NGF_OK;
-  CS_CUDA(cudaDeviceSynchronize());              // the old buffers may still be read
-  cudaFree(f->allm);
-  cudaFree(f->allb);
-  cudaFreeHost(f->allb_h);
-  cudaFree(f->perm_d);
-  cudaFree(f->perm_score);
-  cudaFree(f->perm_shift);
-  f->allm = f->perm_d = nullptr;
-  f->allb = f->allb_h = nullptr;
-  f->perm_score = nullptr;
-  f->perm_shift = nullptr;
-  f->allb_cap = 0;
-  const int cap = std::max(R, 64);
-  CS_CUDA(dalloc(&f->allm, (size_t)cap * (1 + (size_t)f->g.nz + f->g.ny + f->g.nx)));
-  CS_CUDA(dalloc(&f->allb, (size_t)cap));
-  CS_CUDA(cudaMallocHost((void**)&f->allb_h, sizeof(RotBounds) * (size_t)cap));
-  CS_CUDA(dalloc(&f->perm_d, (size_t)cap));
-  CS_CUDA(dalloc(&f->perm_score, (size_t)cap));
-  CS_CUDA(dalloc(&f->perm_shift, (size_t)cap * 3));
-  f->allb_cap = cap;
-  return CS_NGF_OK;
-}
-
 // Section 3.2 shift bounds and mask slabs of each of the R uploaded rotations
-// (from the floating volume pack_floating prepared) into f->allb_h [R];
+// (from the floating volume stage_call prepared) into f->allb_h [R];
 // synchronises st
 cs_ngf_status rotation_bounds(cs_ngf_fixed* f, int R, cudaStream_t st) {
-  if (cs_ngf_status s = ensure_rotation_buffers(f, R)) return s;
   const Geo& g = f->g;
   const size_t nmarg = (size_t)g.nz + g.ny + g.nx;
   int* msum = f->allm;
   int* marg = f->allm + R;
-  CS_CUDA(cudaMemsetAsync(f->allm, 0, sizeof(int) * (size_t)R * (1 + nmarg), st));
   for (int r0 = 0; r0 < R; r0 += 65535) {
     const dim3 grid((unsigned)((g.nx + 7) / 8), (unsigned)((g.ny + 3) / 4), (unsigned)std::min(65535, R - r0));
     Stage sp(f, 0, st);
@@ -622,10 +620,10 @@ cs_ngf_status rotation_bounds(cs_ngf_fixed* f, int R, cudaStream_t st) {
   if (cs_ngf_status s = check_launch("mask counts")) return s;
   {
     Stage sp(f, 7, st);
-    k_shift_bounds<<<dim3((unsigned)R, 3u), 512, 0, st>>>(f->margA, marg, msum, f->sumA, f->gamma, g, f->allb);
+    k_shift_bounds<<<dim3((unsigned)R, 3u), 512, 0, st>>>(f->margA, marg, msum, f->sumA, f->gamma, g, f->allb_h,
+                                                          f->mbox);
   }
   if (cs_ngf_status s = check_launch("shift bounds")) return s;
-  CS_CUDA(cudaMemcpyAsync(f->allb_h, f->allb, sizeof(RotBounds) * (size_t)R, cudaMemcpyDeviceToHost, st));
   CS_CUDA(cudaStreamSynchronize(st));
   return CS_NGF_OK;
 }
@@ -745,7 +743,7 @@ std::vector<LengthClass> length_classes(const std::vector<Need>& need, const int
 }
 
 // Classes of the R uploaded rotations (floating volume packed by
-// pack_floating): bounds (synchronises st), length classes by the overlap rule
+// stage_call): bounds (synchronises st), length classes by the overlap rule
 // (reported) and, for a boxed handle, by the boxes (scored), and the rotations
 // re-uploaded in class order with their boxes.
 cs_ngf_status plan_classes_impl(cs_ngf_fixed* f, int R, cudaStream_t st, Plan& plan) {
@@ -814,7 +812,13 @@ cs_ngf_status plan_classes_impl(cs_ngf_fixed* f, int R, cudaStream_t st, Plan& p
     f->run_pads.insert(f->run_pads.end(), q.pad, q.pad + 3);
     f->run_counts.push_back((int)c.rot.size());
   }
-  CS_CUDA(cudaMemcpyAsync(f->rot_d, f->rot_h, sizeof(RotIn) * R, cudaMemcpyHostToDevice, st));
+  const int words = R * (int)(sizeof(RotIn) / sizeof(int));
+  {
+    Stage sp(f, 7, st);
+    k_copy_words<<<std::min(64, (words + 255) / 256), 256, 0, st>>>(reinterpret_cast<const int*>(f->rot_h),
+                                                                    reinterpret_cast<int*>(f->rot_d), words);
+  }
+  if (cs_ngf_status s = check_launch("boxes")) return s;
   CS_CUDA(cudaEventRecord(f->rot_ev, st));
   return CS_NGF_OK;
 }
@@ -823,8 +827,7 @@ cs_ngf_status score_all(cs_ngf_fixed* f, const float* B, const uint8_t* MB, cons
                         int R, float* best_score, int32_t* best_shift, cudaStream_t st) {
   if (R <= 0) return fail(CS_NGF_EINVAL, "R must be positive");
   if (!best_score || !best_shift) return fail(CS_NGF_EINVAL, "output pointer is NULL");
-  if (cs_ngf_status s = upload_rotations(f, quats, R, st)) return s;
-  if (cs_ngf_status s = pack_floating(f, B, MB, R, st)) return s;
+  if (cs_ngf_status s = stage_call_impl(f, B, MB, quats, R, st)) return s;
   Plan plan;
   if (cs_ngf_status s = plan_classes_impl(f, R, st, plan)) return s;
   // classes one after another; with several, into the handle's buffers, then
@@ -905,14 +908,15 @@ Sizes sizes_for(const int32_t dims[3], const int pad[3], int measure, int precis
 cs_ngf_status ensure_results(cs_ngf_fixed* f, int R) {
   if (R <= f->res_cap) return CS_NGF_OK;
   CS_CUDA(cudaDeviceSynchronize());
-  cudaFree(f->res_score);
-  cudaFree(f->res_shift);
+  cudaFreeHost(f->res_score);
+  cudaFreeHost(f->res_shift);
   f->res_score = nullptr;
   f->res_shift = nullptr;
   f->res_cap = 0;
-  CS_CUDA(dalloc(&f->res_score, (size_t)R));
-  CS_CUDA(dalloc(&f->res_shift, (size_t)R * 3));
-  f->res_cap = R;
+  const int cap = std::max(R, 64);
+  CS_CUDA(cudaMallocHost((void**)&f->res_score, sizeof(float) * (size_t)cap));
+  CS_CUDA(cudaMallocHost((void**)&f->res_shift, sizeof(int32_t) * 3 * (size_t)cap));
+  f->res_cap = cap;
   return CS_NGF_OK;
 }
 
@@ -920,11 +924,9 @@ cs_ngf_status ensure_results(cs_ngf_fixed* f, int R) {
 
 namespace csngf {
 namespace detail {
-cs_ngf_status upload_rotations(cs_ngf_fixed* f, const double* q, int R, cudaStream_t st) {
-  return ::upload_rotations(f, q, R, st);
-}
-cs_ngf_status pack_floating(cs_ngf_fixed* f, const float* B, const uint8_t* MB, int R, cudaStream_t st) {
-  return ::pack_floating(f, B, MB, R, st);
+cs_ngf_status stage_call(cs_ngf_fixed* f, const float* B, const uint8_t* MB, const double* quats, int R,
+                         cudaStream_t st) {
+  return ::stage_call_impl(f, B, MB, quats, R, st);
 }
 cs_ngf_status score_range(cs_ngf_fixed* f, int r0, int n, float* best_score, int32_t* best_shift,
                           cudaStream_t st) {
@@ -1102,16 +1104,16 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
     g.zx = f->zx;
   }
   CS_TRYC(cudaEventCreateWithFlags(&f->order_ev, cudaEventDisableTiming));
-  CS_TRYC(dalloc(&f->tc_err, (size_t)1));
-  CS_TRYC(cudaMemsetAsync(f->tc_err, 0, sizeof(int), st));
+  CS_TRYC(cudaMallocHost((void**)&f->tc_err, sizeof(int)));
+  *f->tc_err = 0;
+  CS_TRYC(cudaMallocHost((void**)&f->fbox_h, sizeof(FixedBox)));
+  CS_TRYC(cudaMemsetAsync(f->mbox, 0, sizeof(int) * 6, st));
   g.tc_err = f->tc_err;
   f->fixed_bytes = uv_elems * sizeof(float2);
   f->workspace_bytes = (size_t)batch * per_rot + shared_ws;
   if (f->pad_mode == CS_NGF_PAD_BOUND) {
     CS_TRYC(dalloc(&f->A_keep, (size_t)g.nvox));
     CS_TRYC(dalloc(&f->MA_keep, (size_t)g.nvox));
-    CS_TRYC(cudaMemcpyAsync(f->A_keep, A, sizeof(float) * g.nvox, cudaMemcpyDeviceToDevice, st));
-    CS_TRYC(cudaMemcpyAsync(f->MA_keep, maskA, (size_t)g.nvox, cudaMemcpyDeviceToDevice, st));
     f->fixed_bytes += (size_t)g.nvox * 5;
   }
 
@@ -1154,10 +1156,10 @@ cs_ngf_status cs_ngf_score_rotations_host(cs_ngf_fixed* f, const float* B, const
   CS_CUDA(cudaMemcpyAsync(f->stage_M, maskB, (size_t)f->g.nvox, cudaMemcpyHostToDevice, st));
   if (cs_ngf_status s = score_all(f, f->stage_B, f->stage_M, quats, R, f->res_score, f->res_shift, st))
     return s;
-  CS_CUDA(cudaMemcpyAsync(best_score, f->res_score, sizeof(float) * R, cudaMemcpyDeviceToHost, st));
-  CS_CUDA(cudaMemcpyAsync(best_shift, f->res_shift, sizeof(int32_t) * 3 * R, cudaMemcpyDeviceToHost, st));
   CS_CUDA(cudaStreamSynchronize(st));
-  return tc_status(f, st);
+  std::copy(f->res_score, f->res_score + R, best_score);
+  std::copy(f->res_shift, f->res_shift + 3 * (size_t)R, best_shift);
+  return tc_status(f);
 }
 
 cs_ngf_status cs_ngf_align(cs_ngf_fixed* f, const float* B, const uint8_t* maskB,
@@ -1172,12 +1174,10 @@ cs_ngf_status cs_ngf_align(cs_ngf_fixed* f, const float* B, const uint8_t* maskB
   CS_CLAIM(f, st, true);
   if (cs_ngf_status s = ensure_results(f, R)) return s;
   if (cs_ngf_status s = score_all(f, B, maskB, quats, R, f->res_score, f->res_shift, st)) return s;
-  std::vector<float> sc(R);
-  std::vector<int32_t> sh(3 * (size_t)R);
-  CS_CUDA(cudaMemcpyAsync(sc.data(), f->res_score, sizeof(float) * R, cudaMemcpyDeviceToHost, st));
-  CS_CUDA(cudaMemcpyAsync(sh.data(), f->res_shift, sizeof(int32_t) * 3 * R, cudaMemcpyDeviceToHost, st));
   CS_CUDA(cudaStreamSynchronize(st));
-  if (cs_ngf_status s = tc_status(f, st)) return s;
+  const float* sc = f->res_score;
+  const int32_t* sh = f->res_shift;
+  if (cs_ngf_status s = tc_status(f)) return s;
   int best = -1;
   for (int r = 0; r < R; ++r)
     if (std::isfinite(sc[r]) && (best < 0 || sc[r] > sc[best])) best = r;
@@ -1202,8 +1202,7 @@ cs_ngf_status cs_ngf_score_map(cs_ngf_fixed* f, const float* B, const uint8_t* m
   cudaStream_t st = (cudaStream_t)stream;
   CS_CLAIM(f, st, true);
   if (cs_ngf_status s = ensure_results(f, 1)) return s;
-  if (cs_ngf_status s = upload_rotations(f, quat, 1, st)) return s;
-  if (cs_ngf_status s = pack_floating(f, B, maskB, 1, st)) return s;
+  if (cs_ngf_status s = stage_call_impl(f, B, maskB, quat, 1, st)) return s;
   Plan plan;
   if (cs_ngf_status s = plan_classes_impl(f, 1, st, plan)) return s;
   if (cs_ngf_status s = set_class_impl(f, plan.cls[0], st)) return s;
@@ -1218,10 +1217,9 @@ cs_ngf_status cs_ngf_resample(cs_ngf_fixed* f, const float* B, const uint8_t* ma
   DeviceGuard guard(f->device);
   cudaStream_t st = (cudaStream_t)stream;
   CS_CLAIM(f, st, true);
-  if (cs_ngf_status s = upload_rotations(f, quat, 1, st)) return s;
   CS_CUDA(cudaMemsetAsync(f->msum, 0, sizeof(int), st));
   const Geo& g = f->g;
-  if (cs_ngf_status s = pack_floating(f, B, maskB, 1, st)) return s;
+  if (cs_ngf_status s = stage_call_impl(f, B, maskB, quat, 1, st)) return s;
   k_resample<<<resample_grid(g, 1), 128, 0, st>>>(f->BQ, f->C8, f->rot_d, g, Bhat, Mhat, f->msum, nullptr);
   return check_launch("resample");
 }
@@ -1326,10 +1324,6 @@ cs_ngf_status cs_ngf_update_fixed(cs_ngf_fixed* f, const float* A, const uint8_t
   DeviceGuard guard(f->device);
   cudaStream_t st = (cudaStream_t)stream;
   CS_CLAIM(f, st, true);
-  if (f->A_keep) {                               // kept for later changes of FFT length
-    CS_CUDA(cudaMemcpyAsync(f->A_keep, A, sizeof(float) * f->g.nvox, cudaMemcpyDeviceToDevice, st));
-    CS_CUDA(cudaMemcpyAsync(f->MA_keep, maskA, (size_t)f->g.nvox, cudaMemcpyDeviceToDevice, st));
-  }
   return load_fixed(f, A, maskA, st);
 }
 

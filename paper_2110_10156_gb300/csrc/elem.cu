@@ -44,10 +44,12 @@ __device__ __forceinline__ float lerp_rn(float a, float b, float t) {
 // base is never on a far face (axis_sample clamps i0 <= n - 2); entries past
 // the volume hold 0.
 __global__ void k_pack_floating(const float* __restrict__ B, const uint8_t* __restrict__ MB, Geo g,
-                                float4* __restrict__ BQ, uint8_t* __restrict__ C8,
-                                int* __restrict__ mbox) {
+                                float4* __restrict__ BQ, uint8_t* __restrict__ C8, CallStage cs) {
   const int sy = g.nx, sz = g.nx * g.ny;          // volumes hold < 2^31 voxels
-  int b[6] = {-(1 << 30), -(1 << 30), -(1 << 30), -1, -1, -1};   // -min z, y, x and max of cells with a mask corner
+  const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+  for (int i = t0; i < cs.words; i += nt) cs.dst[i] = cs.src[i];
+  for (int i = t0; i < cs.zeros; i += nt) cs.zero[i] = 0;
+  int b[6] = {0, 0, 0, 0, 0, 0};                  // n - min and max + 1 (z, y, x) of cells with a mask corner
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.nvox;
        i += (long long)gridDim.x * blockDim.x) {
     const int x = (int)(i % g.nx), y = (int)((i / g.nx) % g.ny), z = (int)(i / sz);
@@ -62,15 +64,15 @@ __global__ void k_pack_floating(const float* __restrict__ B, const uint8_t* __re
     }
     C8[i] = (uint8_t)bits;
     if (bits) {
-      b[0] = max(b[0], -z); b[1] = max(b[1], -y); b[2] = max(b[2], -x);
-      b[3] = max(b[3], z); b[4] = max(b[4], y); b[5] = max(b[5], x);
+      b[0] = max(b[0], g.nz - z); b[1] = max(b[1], g.ny - y); b[2] = max(b[2], g.nx - x);
+      b[3] = max(b[3], z + 1); b[4] = max(b[4], y + 1); b[5] = max(b[5], x + 1);
     }
   }
-  if (!mbox) return;
+  if (!cs.mbox) return;
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const int v = __reduce_max_sync(0xffffffffu, b[k]);
-    if ((threadIdx.x & 31) == 0 && v > (k < 3 ? -(1 << 30) : -1)) atomicMax(&mbox[k], v);
+    if ((threadIdx.x & 31) == 0 && v) atomicMax(&cs.mbox[k], v);
   }
 }
 
@@ -293,7 +295,8 @@ k_mask_counts(const uint8_t* __restrict__ C8, const RotIn* __restrict__ rot, Geo
   const int x = blockIdx.x * 8 + tx, y = blockIdx.y * 4 + ty;
   const RotMat R = rot[r].m;
   const SampleRow sr = sample_row(R, g, x, y);
-  const int lo[3] = {-mbox[0], -mbox[1], -mbox[2]}, hi[3] = {mbox[3], mbox[4], mbox[5]};
+  const int lo[3] = {g.nz - mbox[0], g.ny - mbox[1], g.nx - mbox[2]};
+  const int hi[3] = {mbox[3] - 1, mbox[4] - 1, mbox[5] - 1};
   int z0 = 1 << 30, z1 = -1;
   if (x < g.nx && y < g.ny && hi[0] >= 0) z_range(R, sr, g, lo, hi, z0, z1);
   const bool some = z0 <= z1;
@@ -345,11 +348,13 @@ k_mask_counts(const uint8_t* __restrict__ C8, const RotIn* __restrict__ rot, Geo
 // within two of a mask corner; nullptr: all) only their mask is written.
 __global__ void __launch_bounds__(128)
 k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8, const uint8_t* __restrict__ N8,
-               const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh, uint8_t* __restrict__ Mh) {
+               const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh, uint8_t* __restrict__ Mh,
+               unsigned long long* __restrict__ keys) {
   constexpr int RZ = kResampleZGroups, ZB = 4 * RZ;
   const int ztiles = (g.ez + 2 + ZB - 1) / ZB;
   const int r = blockIdx.z / ztiles, zt = blockIdx.z - r * ztiles;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && zt == 0) keys[r] = 0ull;   // for the x inverse
   const RotBox& b = rot[r].b;
   const int x = b.org[2] - 1 + blockIdx.x * 8 + (lane & 7);
   const int y = b.org[1] - 1 + blockIdx.y * 4 + (lane >> 3);
@@ -374,15 +379,24 @@ k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8, co
   }
 }
 
-// block per z-plane: warps take rows; the x counts collect in shared memory
-__global__ void __launch_bounds__(256) k_marginals(const uint8_t* __restrict__ M, Geo g, int* __restrict__ marg) {
+// block per z-plane: warps take rows; the x counts collect in shared memory.  With
+// A_out, also copies of the volume and its mask
+__global__ void __launch_bounds__(256)
+k_marginals(const float* __restrict__ A, const uint8_t* __restrict__ M, Geo g, int* __restrict__ marg,
+            float* __restrict__ A_out, uint8_t* __restrict__ M_out) {
   __shared__ int xs[256];
   __shared__ int zs;
   const int t = threadIdx.x, lane = t & 31, z = blockIdx.x;
   xs[t] = 0;
   if (t == 0) zs = 0;
   __syncthreads();
-  const uint8_t* P = M + (long long)z * g.nx * g.ny;
+  const long long base = (long long)z * g.nx * g.ny;
+  const uint8_t* P = M + base;
+  if (A_out)
+    for (int i = t; i < g.nx * g.ny; i += 256) {
+      A_out[base + i] = A[base + i];
+      M_out[base + i] = P[i];
+    }
   for (int y = t >> 5; y < g.ny; y += 8) {
     int c = 0;
     for (int x = lane; x < g.nx; x += 32)
@@ -401,11 +415,45 @@ __global__ void __launch_bounds__(256) k_marginals(const uint8_t* __restrict__ M
   if (t < g.nx && xs[t]) atomicAdd(&marg[g.nz + g.ny + t], xs[t]);
 }
 
+// one block: the fixed mask's sum and the slabs that hold it, for the host (out)
+// and as the box origin of the spectra's x pass
+__global__ void __launch_bounds__(256) k_fixed_box(const int* __restrict__ marg, Geo g, int boxed,
+                                                   FixedBox* __restrict__ out, RotIn* __restrict__ box) {
+  __shared__ int sum, lo[3], hi[3];
+  const int t = threadIdx.x;
+  if (t == 0) sum = 0;
+  if (t < 3) { lo[t] = 0x7fffffff; hi[t] = -1; }
+  __syncthreads();
+  const int n[3] = {g.nz, g.ny, g.nx};
+  for (int a = 0, o = 0; a < 3; o += n[a], ++a)
+    if (t < n[a] && marg[o + t]) {
+      if (a == 0) atomicAdd(&sum, marg[t]);
+      atomicMin(&lo[a], t);
+      atomicMax(&hi[a], t);
+    }
+  __syncthreads();
+  if (t == 0) {
+    RotIn in{};
+    out->sum = sum;
+    for (int a = 0; a < 3; ++a) {
+      out->a0[a] = hi[a] < 0 ? 0 : lo[a];
+      out->a1[a] = hi[a] < 0 ? 0 : hi[a];
+      in.b.org[a] = boxed ? out->a0[a] : 0;
+    }
+    *box = in;
+  }
+}
+
+__global__ void k_copy_words(const int* __restrict__ src, int* __restrict__ dst, int n) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i];
+}
+
 // block (rotation r, axis a); thread per shift slot v, then per slab
 __global__ void k_shift_bounds(const int* __restrict__ margA, const int* __restrict__ margB,
                                const int* __restrict__ msumB, int sumA, float gamma, Geo g,
-                               RotBounds* __restrict__ bounds) {
+                               RotBounds* __restrict__ bounds, int* __restrict__ mbox) {
   const int r = blockIdx.x, a = blockIdx.y;
+  if (mbox && r == 0 && a == 0 && threadIdx.x < 6) mbox[threadIdx.x] = 0;   // counted: empty for the next call
   const int n = a == 0 ? g.nz : (a == 1 ? g.ny : g.nx);
   const int off = a == 0 ? 0 : (a == 1 ? g.nz : g.nz + g.ny);
   const int* mb = margB + (long long)r * (g.nz + g.ny + g.nx) + off;

@@ -15,6 +15,7 @@ struct cs_ngf_fixed {
   using Geo = csngf::Geo;
   using RotIn = csngf::RotIn;
   using RotBounds = csngf::RotBounds;
+  using FixedBox = csngf::FixedBox;
   int device = 0;
   Geo g{};
   float eps = 1e-5f, gamma = 0.5f;
@@ -33,8 +34,7 @@ struct cs_ngf_fixed {
   // per-rotation mask counts and bounds of a call and its rotations regrouped
   // by FFT lengths (bound-limited padding), grown on demand to the call's R
   int* allm = nullptr;         // device [R][1 + nz + ny + nx]: sums, then slab counts
-  RotBounds* allb = nullptr;   // device [R]
-  RotBounds* allb_h = nullptr; // pinned host copy
+  RotBounds* allb_h = nullptr; // [R], pinned host memory the bounds kernel writes to
   int* perm_d = nullptr;       // device: original index of each regrouped rotation
   float* perm_score = nullptr; // device results in regrouped order
   int32_t* perm_shift = nullptr;
@@ -72,9 +72,10 @@ struct cs_ngf_fixed {
   int* margB = nullptr;        // the same for each rotated mask of a batch
   RotBounds* bounds = nullptr; // per rotation of a batch (full padding)
   unsigned long long* keys = nullptr;
-  int* tc_err = nullptr;       // set by a tensor-core pass that stopped on its bounded wait
+  int* tc_err = nullptr;       // pinned host flag, set by a pass that stopped on its bounded wait
+  FixedBox* fbox_h = nullptr;  // pinned host memory k_fixed_box writes to
   float2* zx = nullptr;        // X of the tensor-core z pass (reduced-precision forms), per launch group
-  // rotation matrices: pinned host staging + device copy, grown on demand
+  // rotations: pinned host memory, copied to the device by a kernel, grown on demand
   RotIn* rot_h = nullptr;
   RotIn* rot_d = nullptr;
   int rot_cap = 0;
@@ -82,7 +83,7 @@ struct cs_ngf_fixed {
   // host-buffer entry point staging
   float* stage_B = nullptr;
   uint8_t* stage_M = nullptr;
-  float* res_score = nullptr;
+  float* res_score = nullptr;  // pinned host memory the last kernel writes results to
   int32_t* res_shift = nullptr;
   int res_cap = 0;
   size_t fixed_bytes = 0, workspace_bytes = 0;
@@ -104,10 +105,10 @@ namespace detail {
 
 // record the calling thread's error detail (cs_ngf_last_error) and return s
 cs_ngf_status fail(cs_ngf_status s, const std::string& msg);
+// a call's floating volume and rotations on the device: (B, M_B) -> f->BQ, f->C8,
 // host FP64 quaternions -> FP32 matrices in f->rot_h[0..R) and f->rot_d[0..R)
-cs_ngf_status upload_rotations(cs_ngf_fixed* f, const double* quats, int R, cudaStream_t st);
-// (B, M_B) -> f->BQ, f->C8 for the following scoring of R rotations
-cs_ngf_status pack_floating(cs_ngf_fixed* f, const float* B, const uint8_t* MB, int R, cudaStream_t st);
+cs_ngf_status stage_call(cs_ngf_fixed* f, const float* B, const uint8_t* MB, const double* quats, int R,
+                         cudaStream_t st);
 // Rotations scored together: FFT lengths, box extents and shift windows per
 // axis (z, y, x), and the end of the class in the call's regrouped order.
 struct ClassGeom { int pad[3], ext[3], win[3], end; };
@@ -116,7 +117,7 @@ struct Plan {
   std::vector<ClassGeom> cls;
 };
 // Bound-limited padding (pad_mode CS_NGF_PAD_BOUND): the R uploaded
-// rotations of the floating volume packed by pack_floating, grouped into
+// rotations of the floating volume packed by stage_call, grouped into
 // classes by the FFT lengths their admitted shifts need, their boxes uploaded
 // in class order.  Synchronises `st`.  In full mode: one class with the
 // lengths in use.

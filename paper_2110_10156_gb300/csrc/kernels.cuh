@@ -163,10 +163,21 @@ __device__ __forceinline__ unsigned long long make_key(float s, unsigned lin) {
 // contraction), so the decision is reproducible bit for bit.  B and M_B are
 // read as the row-pair table and corner codes k_pack_floating prepares (BQ,
 // C8: nvox entries each).
-// mbox (or nullptr): -min z, y, x and max z, y, x of the cells with a mask
-// corner, accumulated with atomicMax
+// What else k_pack_floating does for a call: copies its rotations from pinned host
+// memory, zeroes the mask counts and (mbox, zero before) accumulates the box of
+// the cells with a mask corner: n - min z, y, x and max + 1.  A box left by a call
+// that failed only makes the next one's larger.
+struct CallStage {
+  const int* src;
+  int* dst;
+  int words;
+  int* zero;
+  int zeros;
+  int* mbox;
+};
 __global__ void k_pack_floating(const float* __restrict__ B, const uint8_t* __restrict__ MB, Geo g,
-                                float4* __restrict__ BQ, uint8_t* __restrict__ C8, int* __restrict__ mbox);
+                                float4* __restrict__ BQ, uint8_t* __restrict__ C8, CallStage cs);
+__global__ void k_copy_words(const int* __restrict__ src, int* __restrict__ dst, int n);
 __global__ void k_near_axis(const uint8_t* __restrict__ in, uint8_t* __restrict__ out, Geo g, int axis);
 // k_resample: the whole volume, mask counts into msum and marg (marg may be
 // nullptr); grid resample_grid.  k_resample_box: only the voxels the x pass
@@ -176,7 +187,7 @@ __global__ void k_resample(const float4* __restrict__ BQ, const uint8_t* __restr
                            uint8_t* __restrict__ Mh, int* __restrict__ msum, int* __restrict__ marg);
 __global__ void k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8,
                                const uint8_t* __restrict__ N8, const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh,
-                               uint8_t* __restrict__ Mh);
+                               uint8_t* __restrict__ Mh, unsigned long long* __restrict__ keys);
 // The rotated masks alone, counted into msum and marg as k_resample counts
 // them (the same decisions from the same corner codes, no volumes written):
 // the pre-pass that bounds the shifts of a whole call.
@@ -199,10 +210,14 @@ inline dim3 resample_box_grid(const Geo& g, int nrot) {
 // axis, so shifts whose slab bound is below the Section 3.2 overlap threshold
 // are invalid; k_shift_bounds keeps, per rotation and axis, the range of shift
 // slots that can be valid and the slabs that hold mask voxels.
-__global__ void k_marginals(const uint8_t* __restrict__ M, Geo g, int* __restrict__ marg);
+__global__ void k_marginals(const float* __restrict__ A, const uint8_t* __restrict__ M, Geo g,
+                            int* __restrict__ marg, float* __restrict__ A_out, uint8_t* __restrict__ M_out);
+struct FixedBox { int sum, a0[3], a1[3]; };
+__global__ void k_fixed_box(const int* __restrict__ marg, Geo g, int boxed, FixedBox* __restrict__ out,
+                            RotIn* __restrict__ box);
 __global__ void k_shift_bounds(const int* __restrict__ margA, const int* __restrict__ margB,
                                const int* __restrict__ msumB, int sumA, float gamma, Geo g,
-                               RotBounds* __restrict__ bounds);
+                               RotBounds* __restrict__ bounds, int* __restrict__ mbox);
 // full padding: the boxes of a launch group (origin 0) from its bounds
 __global__ void k_full_boxes(const RotBounds* __restrict__ bounds, int sumA, float gamma, Geo g,
                              double pvol, int nrot, RotIn* __restrict__ rot);

@@ -237,7 +237,7 @@ extern "C" cs_ngf_status cs_ngf_score_rotations_noalloc(
   NA_DISPATCH(g.Pz, launch_prep_z<PP>(F13, UV, g, st));
   if (cs_ngf_status s = na_launched("fixed transforms")) return s;
 
-  k_pack_floating<<<64, 256, 0, st>>>(B, maskB, g, BQ, C8, nullptr);
+  k_pack_floating<<<64, 256, 0, st>>>(B, maskB, g, BQ, C8, CallStage{});
   if (cs_ngf_status s = na_launched("pack")) return s;
   const double pvol = (double)g.Px * (double)g.Py * (double)g.Pz;
   for (int r = 0; r < R; ++r) {

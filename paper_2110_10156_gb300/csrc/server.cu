@@ -196,8 +196,8 @@ cs_ngf_status setup_job(cs_ngf_server* sv, Job* j, Slot* slot, bool fresh) {
   } else if (cs_ngf_status s = cs_ngf_update_fixed(slot->f, slot->dA, slot->dMA, st)) {
     return s;
   }
-  if (cs_ngf_status s = csngf::detail::upload_rotations(slot->f, j->quats.data(), j->R, st)) return s;
-  if (cs_ngf_status s = csngf::detail::pack_floating(slot->f, slot->dB, slot->dMB, j->R, st)) return s;
+  if (cs_ngf_status s = csngf::detail::stage_call(slot->f, slot->dB, slot->dMB, j->quats.data(), j->R, st))
+    return s;
   // FFT lengths per class of rotations (bound-limited padding), first class set up
   if (cs_ngf_status s = csngf::detail::plan_classes(slot->f, j->R, st, j->plan)) return s;
   j->cls = 0;
