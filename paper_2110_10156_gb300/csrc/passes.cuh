@@ -298,99 +298,118 @@ void launch_fwd_x(const float* Bh, const uint8_t* Mh, void* F0, const RotIn* rot
 // ---------------------------------------------------------------------------
 // F0's tiles of four kx are contiguous over y, so a plane's columns arrive as
 // one bulk copy, and four planes make 128-byte pieces of F1's tiles
-// [kx][p/4][z][p%4] (one plane: 32 bytes, 31 against 28 us per rotation at 150^3).
+// [kx][p/4][z][p%4] (one plane: 32-byte pieces, 31 us per rotation at 150^3
+// against 29).  A block takes several groups of four planes, the copies of the
+// next under the current one: a block of one group waited for its copy a third
+// of its life.
 template <int P, int V> struct FwdYCfg {
   static constexpr int N1 = SplitV<P, V>::N1, N2 = SplitV<P, V>::N2, W = 16;
   static constexpr int NT = W * N2;
   // exchange [column][n2][k1]: odd rows, and columns 4 rows apart (mod 16), put
   // four columns of four rows in different banks
   static constexpr int RS = N1 | 1, CS0 = N2 * RS, CS = CS0 + ((4 * RS - CS0) % 16 + 16) % 16;
-  static constexpr size_t smem_bytes(int ey) { return ((size_t)W * CS + (size_t)W * ey) * sizeof(float2) + 16; }
+  static constexpr size_t smem_bytes(int ey) { return ((size_t)W * CS + (size_t)2 * W * ey) * sizeof(float2) + 16; }
   static constexpr int MIN_BLOCKS = pass_blocks(NT, smem_bytes(3 * P / 4), N2 > 20 ? 80 : 48);
 };
 
 template <int P, int ST, bool HALF, int V>
 __global__ void __launch_bounds__(FwdYCfg<P, V>::NT, FwdYCfg<P, V>::MIN_BLOCKS)
-k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, Geo g) {
+k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, Geo g, int groups) {
   using C = FwdYCfg<P, V>;
   constexpr int N1 = C::N1, N2 = C::N2, W = C::W, RS = C::RS, CS = C::CS, NI = HALF ? N1 / 2 : N1;
   extern __shared__ __align__(128) float2 ysm[];
-  float2* in = ysm;                                  // [4 z][ey][4 kx] (4-byte values in the 16-bit forms)
-  float2* ex = in + W * g.ey;                        // [W][CS]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(ex + W * CS + (W * CS & 1));
+  float2* in = ysm;                                  // [2][4 z][ey][4 kx] (4-byte values in the 16-bit forms)
+  float2* ex = in + 2 * W * g.ey;                    // [W][CS]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(ex + W * CS);
   const int t = threadIdx.x;
-  const int rj = blockIdx.z, z0 = 4 * blockIdx.y;    // rj = r * nf + j
+  const int rj = blockIdx.z;                         // r * nf + j
   const int r = g.nf == 4 ? rj >> 2 : rj / 3, j = rj - r * g.nf;
   const bool is_mask = j == g.nch;
   if (is_mask && (r & 1)) return;                    // paired into the even rotation's mask field
   const bool wide = ST == kStoreF32 || is_mask;
-  const int nz = min(4, g.ez - z0);
   const uint32_t bytes = (uint32_t)g.ey * 4 * (wide ? 8 : 4);   // of one plane's tile
-  if (t == 0) {
+  const int zbeg = 4 * groups * blockIdx.y, zend = min(g.ez, zbeg + 4 * groups);
+  auto fetch = [&](int z0, int s) {                  // one thread: planes z0 .. z0 + 3
+    if (z0 >= zend) return;
+    const int nz = min(4, zend - z0);
     const char* src = Fields<ST>::field(F0, g, (long long)g.ez * g.ey * g.Px, r, j);
-    tc::mbar_init(bar, 1);
-    tc::mbar_init_fence();
-    tc::mbar_expect(bar, nz * bytes);
+    tc::mbar_expect(&bar[s], nz * bytes);
     for (int z = 0; z < nz; ++z)
-      tc::bulk_load(reinterpret_cast<char*>(in) + z * bytes,
-                    src + ((long long)(z0 + z) * (g.Px / 4) + blockIdx.x) * bytes, bytes, bar);
+      tc::bulk_load(reinterpret_cast<char*>(in + s * W * g.ey) + z * bytes,
+                    src + ((long long)(z0 + z) * (g.Px / 4) + blockIdx.x) * bytes, bytes, &bar[s]);
+  };
+  if (t == 0) {
+    tc::mbar_init(&bar[0], 1);
+    tc::mbar_init(&bar[1], 1);
+    tc::mbar_init_fence();
+    fetch(zbeg, 0);
+    fetch(zbeg + 4, 1);
   }
-  __syncthreads();                                   // the barrier is initialised
-  const bool dead = !tc::mbar_wait(bar, 0, kTcWaitNs);
-  {
-    const int kxi = t & 3, n2 = (t >> 2) % N2, zz = t / (4 * N2);
-    const float isc = 1.0f / field_scale(g.scale0, j);
-    const int o = (zz * g.ey + n2) * 4 + kxi;
-    float2 v[NI];                                    // y < ey: with ey <= P/2 the upper half is zero
-    auto rows = [&](auto mc) {
+  __syncthreads();                                   // the barriers are initialised
+  bool dead = false;                                 // a wait ran out: no more waits, results invalid
+  int it = 0;
+#pragma unroll 1
+  for (int z0 = zbeg; z0 < zend; z0 += 4, ++it) {
+    const int nz = min(4, zend - z0);
+    const float2* src = in + (it & 1) * W * g.ey;
+    if (!dead && !tc::mbar_wait(&bar[it & 1], (it >> 1) & 1, kTcWaitNs)) dead = true;
+    {
+      const int kxi = t & 3, n2 = (t >> 2) % N2, zz = t / (4 * N2);
+      const float isc = 1.0f / field_scale(g.scale0, j);
+      const int o = (zz * g.ey + n2) * 4 + kxi;
+      float2 v[NI];                                  // y < ey: with ey <= P/2 the upper half is zero
+      auto rows = [&](auto mc) {
 #pragma unroll
-      for (int n1 = 0; n1 < NI; ++n1)
-        v[n1] = N2 * n1 + n2 < g.ey && zz < nz
-                    ? Fields<ST>::get(reinterpret_cast<const char*>(in), o + 4 * N2 * n1, decltype(mc)::value, isc)
-                    : make_float2(0.f, 0.f);
-    };
-    if (wide) rows(std::true_type{});
-    else rows(std::false_type{});
-    float2* e = ex + (zz * 4 + kxi) * CS + n2 * RS;
-    float2 a[N1];
-    if constexpr (HALF) {
-      dft_half<N1, -1>(v, a);
-    } else {
-#pragma unroll
-      for (int i = 0; i < N1; ++i) a[i] = v[i];
-      Dft<N1, -1>::run(a);
-    }
-#pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) {
-      const float2 w = __ldg(&kTwStep<P, N1, N2>.w[k1 * N2 + n2]);
-      e[k1] = k1 == 0 ? a[k1] : cmul(a[k1], w);
-    }
-  }
-  __syncthreads();
-  if (t < W * N1) {
-    const int k1 = t % N1, kxi = t / N1 & 3, zz = t / (4 * N1);
-    if (zz < nz) {
-      float2 u[N2];
-      const float2* s = ex + (zz * 4 + kxi) * CS + k1;
-#pragma unroll
-      for (int i = 0; i < N2; ++i) u[i] = s[i * RS];
-      Dft<N2, -1>::run(u);
-      char* dst = Fields<ST>::field(F1, g, (long long)g.ez * g.Px * ky_total(P), r, j);
-      const int row = (4 * blockIdx.x + kxi) * ky_total(P) * g.ez + 4 * (z0 + zz);
-      const KyRun<P, N1, N2> run(k1, g.ez);
-      const float sc = field_scale(g.scale1, j);
-      if (is_mask) {
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) Fields<ST>::put(dst, row + run.at(k2), u[k2], true, sc);
+        for (int n1 = 0; n1 < NI; ++n1)
+          v[n1] = N2 * n1 + n2 < g.ey && zz < nz
+                      ? Fields<ST>::get(reinterpret_cast<const char*>(src), o + 4 * N2 * n1, decltype(mc)::value, isc)
+                      : make_float2(0.f, 0.f);
+      };
+      if (wide) rows(std::true_type{});
+      else rows(std::false_type{});
+      float2* e = ex + (zz * 4 + kxi) * CS + n2 * RS;
+      float2 a[N1];
+      if constexpr (HALF) {
+        dft_half<N1, -1>(v, a);
       } else {
 #pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) Fields<ST>::put(dst, row + run.at(k2), u[k2], false, sc);
+        for (int i = 0; i < N1; ++i) a[i] = v[i];
+        Dft<N1, -1>::run(a);
+      }
+#pragma unroll
+      for (int k1 = 0; k1 < N1; ++k1) {
+        const float2 w = __ldg(&kTwStep<P, N1, N2>.w[k1 * N2 + n2]);
+        e[k1] = k1 == 0 ? a[k1] : cmul(a[k1], w);
       }
     }
+    __syncthreads();
+    if (t == 0) fetch(z0 + 8, it & 1);               // this group's inputs have been read
+    if (t < W * N1) {
+      const int k1 = t % N1, kxi = t / N1 & 3, zz = t / (4 * N1);
+      if (zz < nz) {
+        float2 u[N2];
+        const float2* s = ex + (zz * 4 + kxi) * CS + k1;
+#pragma unroll
+        for (int i = 0; i < N2; ++i) u[i] = s[i * RS];
+        Dft<N2, -1>::run(u);
+        char* dst = Fields<ST>::field(F1, g, (long long)g.ez * g.Px * ky_total(P), r, j);
+        const int row = (4 * blockIdx.x + kxi) * ky_total(P) * g.ez + 4 * (z0 + zz);
+        const KyRun<P, N1, N2> run(k1, g.ez);
+        const float sc = field_scale(g.scale1, j);
+        if (is_mask) {
+#pragma unroll
+          for (int k2 = 0; k2 < N2; ++k2) Fields<ST>::put(dst, row + run.at(k2), u[k2], true, sc);
+        } else {
+#pragma unroll
+          for (int k2 = 0; k2 < N2; ++k2) Fields<ST>::put(dst, row + run.at(k2), u[k2], false, sc);
+        }
+      }
+    }
+    __syncthreads();
   }
   if (dead) {                                        // the results are invalid; its copies end before the block does
     if (t == 0 && g.tc_err) atomicExch(g.tc_err, 1);
-    tc::mbar_wait(bar, 0, kTcWaitNs / 4);
+    for (int l = it - 1; l >= 0 && l >= it - 2; --l) tc::mbar_wait(&bar[l & 1], (l >> 1) & 1, kTcWaitNs / 4);
   }
 }
 
@@ -398,13 +417,17 @@ template <int P, int V>
 void launch_fwd_y_t(const void* F0, void* F1, Geo g, int nrot, cudaStream_t st) {
   using C = FwdYCfg<P, V>;
   const size_t smem = C::smem_bytes(g.ey);
-  const dim3 grid((unsigned)(g.Px / 4), (unsigned)((g.ez + 3) / 4), (unsigned)(nrot * g.nf));
+  // groups of four planes per block: more where there are blocks to spare
+  const int quads = (g.ez + 3) / 4;
+  int groups = 1;
+  while (groups < 4 && (long long)(g.Px / 4) * nrot * g.nf * (quads / (2 * groups)) >= 152 * C::MIN_BLOCKS * 8) groups *= 2;
+  const dim3 grid((unsigned)(g.Px / 4), (unsigned)((quads + groups - 1) / groups), (unsigned)(nrot * g.nf));
   by_store<P>(g.store, [&](auto sf) {
     constexpr int ST = decltype(sf)::value;
     by_half<P, V>(g.ey, [&](auto hc) {
       auto kern = k_fwd_y<P, ST, decltype(hc)::value, V>;
       set_smem(kern, smem);
-      kern<<<grid, C::NT, smem, st>>>(F0, F1, g);
+      kern<<<grid, C::NT, smem, st>>>(F0, F1, g, groups);
     });
   });
 }

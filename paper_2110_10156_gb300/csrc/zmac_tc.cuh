@@ -13,7 +13,7 @@
 // 16) give every frequency of every column.  The B operand is a tile of the
 // 16-bit field values as they lie in F1 ([kx][p/4][z][p%4] with (re, im) pairs):
 // N-major, its columns (field, primary / mirror, column, re / im), so that
-// the 8 primary columns of a row are two 16-byte copies, their mirrors two more.  Tensor memory lane
+// a tile of it is a bulk copy.  Tensor memory lane
 // kz then holds H at kz and P - kz of a column and of its mirror column
 // (-kx, -ky), which is all the multiply-accumulate of that frequency pair
 // needs.  The mask field (the overlap count N) and the inverse stay on the
@@ -41,7 +41,7 @@ __device__ __forceinline__ void store16(unsigned char* p, float v) {
 // k_zx_tc, per block: one kx, W = 8 columns (two tiles) and their mirrors, every
 // rotation of the launch; the cos / sin tiles and the block's weights stay
 // in shared memory.  Rotation r + 1's MMAs run while rotation r's products
-// are summed; rotation r + 2's operand is copied (cp.async) as soon as
+// are summed; rotation r + 2's operand is copied (twelve bulk copies) as soon as
 // rotation r's MMAs are done.  16 warps, four per tensor-memory lane quarter.
 // ---------------------------------------------------------------------------
 template <int P>
@@ -73,8 +73,9 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
   unsigned char* Bs = As + 2 * tileA;              // [2][KP][NB], N-major
   const uint32_t stageB = (uint32_t)NB * (uint32_t)KP * 2u;
   float2* uvs = reinterpret_cast<float2*>(Bs + 2 * stageB);   // [NUV][W][P]
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(uvs + (size_t)NUV * TILE);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 2);
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(uvs + (size_t)NUV * TILE);   // products of each buffer
+  uint64_t* bar = mbar + 2;                        // operands of each stage
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 2);
 
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int kx = blockIdx.y;
@@ -82,8 +83,11 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
   const int ntile = 2 * gridDim.x, half = ky_half(g.Py) / 4;   // tiles of four columns
   const long long E = (long long)g.ez * g.Px * 4 * ntile;
 
-  for (uint32_t q = t; q < 2 * stageB / 16; q += NT)
-    reinterpret_cast<uint4*>(Bs)[q] = make_uint4(0u, 0u, 0u, 0u);
+  // operand rows past the box stay zero
+  for (int q = t; q < 2 * (NB / 8) * (KP - g.ez); q += NT) {
+    const int n8 = q / (KP - g.ez), k = g.ez + q - n8 * (KP - g.ez);
+    reinterpret_cast<uint4*>(Bs)[n8 * KP + k] = make_uint4(0u, 0u, 0u, 0u);
+  }
   // the block's weights, [tile][field][kz][column][a, b] in HBM, transposed so that
   // kz runs over the lanes
   for (int q = t; q < NUV * TILE; q += NT) {
@@ -92,11 +96,13 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
     cp_async8(uvs + (2 * j + s) * TILE + c * P + k,
               UV + ((long long)kx * ntile + 2 * blockIdx.x + h) * (NUV + 1) * 4 * P + i);
   }
-  for (int m = warp; m < 128; m += NT / 32)
-    for (int k = lane; k < KP; k += 32) {
+  for (int m = warp; m < 128; m += NT / 32) {
+    int e = m * lane % P;                          // m k mod P
+    const int step = 32 * m % P;
+    for (int k = lane; k < KP; k += 32, e = e + step >= P ? e + step - P : e + step) {
       float cv = 0.f, sv = 0.f;
       if (m <= HF && k < g.ez) {
-        const float2 w = __ldg(&tw[(m * k) % P]);   // exp(-2 pi i m k / P)
+        const float2 w = __ldg(&tw[e]);             // exp(-2 pi i m k / P)
         cv = w.x;
         sv = -w.y;
       }
@@ -104,40 +110,41 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
       store16<ST>(As + off, cv);
       store16<ST>(As + tileA + off, sv);
     }
+  }
   if (t == 0) {
-    tc::mbar_init(&mbar[0], 1);
-    tc::mbar_init(&mbar[1], 1);
+    for (int i = 0; i < 4; ++i) tc::mbar_init(&mbar[i], 1);
     tc::mbar_init_fence();
   }
   if (warp == 0) tc::alloc(tslot, C::TMEM_COLS);
 
-  // operand copies of one (field, z) row: two tiles of primary columns and two
-  // of their mirrors, 16 bytes each (tiles that hold ky = 0 or P/2, which are
-  // their own mirrors: the four mirror values one by one)
-  const int item = t % 4, zr0 = t / 4, tile = 2 * blockIdx.x + (item & 1);
-  const bool prim = item < 2, own = tile == 0 || tile == half;
-  const int mtile = tile < half ? tile + half : tile - half;
+  // A tile's columns are N-major operand rows as they lie in F1 (16 bytes per z),
+  // so a field takes four bulk copies: the block's two tiles and the two of their
+  // mirrors.  Where a tile's first column is ky = 0 or P/2, its own mirror, that
+  // column is filled in by the threads (own_h: the tile, or -1).
+  const int own_h = blockIdx.x == 0 ? 0 : half / 2 == (int)blockIdx.x ? half & 1 : -1;
   const long long tz = 4LL * g.ez;                 // values per tile
-  const long long srow = prim ? ((long long)kx * ntile + tile) * tz : ((long long)mkx * ntile + mtile) * tz;
-  const long long sown = ((long long)mkx * ntile + tile) * tz;
-  auto fetch_b = [&](int r, int s) {
-    if (r < nrot) {
-      unsigned char* B0 = Bs + (size_t)s * stageB;
-      for (int j = 0; j < g.nch; ++j) {
-        const char* src = Fields<ST>::field(F1, g, E, r, j);
-        unsigned char* dcol = B0 + (uint32_t)(j * 4 + item) * sbo;
-        for (int z = zr0; z < g.ez; z += NT / 4) {
-          unsigned char* d = dcol + (z / 8) * 128 + (z % 8) * 16;
-          if (prim || !own) {
-            cp_async16(d, src + (srow + 4 * z) * 4);
-          } else {
-            cp_async4(d, src + (sown + 4 * z) * 4);
-#pragma unroll
-            for (int c = 1; c < 4; ++c) cp_async4(d + 4 * c, src + (srow + 4 * z + c) * 4);
-          }
-        }
+  auto fetch_b = [&](int r, int s) {               // one thread
+    if (r >= nrot) return;
+    const uint32_t bytes = (uint32_t)g.ez * 16;
+    tc::mbar_expect(&bar[s], 4 * g.nch * bytes);
+    for (int j = 0; j < g.nch; ++j) {
+      const char* src = Fields<ST>::field(F1, g, E, r, j);
+      unsigned char* d = Bs + (size_t)s * stageB + (uint32_t)(4 * j) * sbo;
+      for (int h = 0; h < 2; ++h) {
+        const int tile = 2 * blockIdx.x + h, mtile = tile < half ? tile + half : tile - half;
+        tc::bulk_load(d + h * sbo, src + ((long long)kx * ntile + tile) * tz * 4, bytes, &bar[s]);
+        tc::bulk_load(d + (2 + h) * sbo, src + ((long long)mkx * ntile + mtile) * tz * 4, bytes, &bar[s]);
       }
     }
+  };
+  auto patch_b = [&](int r, int s) {               // all threads, after the copies
+    const long long o = ((long long)mkx * ntile + 2 * blockIdx.x + own_h) * tz;
+    for (int q = t; q < g.nch * g.ez; q += NT) {
+      const int j = q / g.ez, z = q - j * g.ez;
+      *reinterpret_cast<uint32_t*>(Bs + (size_t)s * stageB + (uint32_t)(4 * j + 2 + own_h) * sbo + z * 16) =
+          reinterpret_cast<const uint32_t*>(Fields<ST>::field(F1, g, E, r, j))[o + 4 * z];
+    }
+    tc::fence_async_smem();
   };
   const uint32_t idesc = tc::idesc_f16(ST == kStoreBF16, 0, 1, 128, NB);
   auto issue = [&](uint32_t tmem, int s) {         // operand stage s -> tensor-memory buffer s
@@ -152,20 +159,28 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
     tc::commit(&mbar[s]);
   };
 
-  fetch_b(0, 0);
-  cp_async_commit();
-  fetch_b(1, 1);
-  cp_async_commit();
-  cp_async_wait_one();                             // rotation 0's operand and the weights
-  tc::fence_async_smem();
+  cp_async_wait_all();                             // the weights
+  tc::fence_async_smem();                          // the tables and zero rows, for the tensor core and the copies
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *tslot;
-  if (t == 0 && nrot > 0) issue(tmem, 0);
+  if (t == 0) {
+    fetch_b(0, 0);
+    fetch_b(1, 1);
+  }
+  // rotation r's operand has landed (and is completed): its products start
+  auto start = [&](int r) {
+    if (own_h >= 0) {
+      if (tc::mbar_wait(&bar[r & 1], (uint32_t)((r >> 1) & 1), kTcWaitNs)) patch_b(r, r & 1);
+      __syncthreads();
+    }
+    if (t == 0 && tc::mbar_wait(&bar[r & 1], (uint32_t)((r >> 1) & 1), kTcWaitNs)) issue(tmem, r & 1);
+  };
+  start(0);
 
   bool failed = false;
-  int fail_buf = 0;
+  int fail_buf = 0, fail_next = -1;
   uint32_t fail_par = 0;
   const int lq = warp & 3, cg = warp >> 2;         // lane quarter, column pair
   const int kz = lq * 32 + lane;
@@ -180,19 +195,14 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
       failed = true;
       fail_buf = s;
       fail_par = (uint32_t)((r >> 1) & 1);
+      fail_next = r + 1 < nrot ? r + 1 : r;
       break;
     }
     tc::fence_after_sync();
-    fetch_b(r + 2, s);
-    cp_async_commit();
-    // (2) rotation r + 1's operand has landed: its products start (the
-    // barrier also orders rotation r - 1's tensor-memory reads of that buffer)
-    if (r + 1 < nrot) {
-      cp_async_wait_one();
-      tc::fence_async_smem();
-    }
-    __syncthreads();
-    if (t == 0 && r + 1 < nrot) issue(tmem, (r + 1) & 1);
+    if (t == 0) fetch_b(r + 2, s);
+    // (2) rotation r + 1's products (the barrier above also orders rotation
+    // r - 1's tensor-memory reads of that buffer)
+    if (r + 1 < nrot) start(r + 1);
     // (3) Eq. 7-8: X at kz and P - kz of this thread's four primary columns
     const uint32_t trow = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(s * 2 * NB);
     float2* Xr = Xg + (((long long)r * gridDim.y + kx) * ntile + 2 * blockIdx.x + (cg >> 1)) * 4 * P + 2 * (cg & 1);
@@ -225,17 +235,16 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
               const float Sr = __uint_as_float(rs[j][2 * i]) * isc, Si = __uint_as_float(rs[j][2 * i + 1]) * isc;
               const float Smr = __uint_as_float(rsm[j][2 * i]) * isc;
               const float Smi = __uint_as_float(rsm[j][2 * i + 1]) * isc;
-              const float2 Hk = make_float2(Cr + Si, Ci - Sr);
-              const float2 Hp = make_float2(Cr - Si, Ci + Sr);
-              const float2 Mk = make_float2(Cmr + Smi, -(Cmi - Smr));   // conjugates of the
-              const float2 Mp = make_float2(Cmr - Smi, -(Cmi + Smr));   // mirror's values
+              // H = (Cr + Si, Ci - Sr) at kz and (Cr - Si, Ci + Sr) at P - kz, its mirror H'
+              // likewise; channels a = H + conj H', b = -i (H - conj H') at both
+              const float p = Cr + Cmr, q = Cr - Cmr, u = Si - Smi, v = Si + Smi;
+              const float e = Ci - Cmi, f = Ci + Cmi, g1 = Sr + Smr, h = Sr - Smr;
               const float2* Wa = uvs + (2 * j) * TILE + c * P;
               const float2* Wb = Wa + TILE;
-              // channels a = H + conj H', b = -i (H - conj H') at kz and P - kz
-              cmac(Xa[i], Wa[kz], cadd(Hk, Mp));
-              cmac(Xa[i], Wb[kz], mul_si<-1>(csub(Hk, Mp)));
-              cmac(Xb[i], Wa[kzm], cadd(Hp, Mk));
-              cmac(Xb[i], Wb[kzm], mul_si<-1>(csub(Hp, Mk)));
+              cmac(Xa[i], Wa[kz], make_float2(p + u, e - g1));
+              cmac(Xa[i], Wb[kz], make_float2(f - h, -q - v));
+              cmac(Xb[i], Wa[kzm], make_float2(p - u, e + g1));
+              cmac(Xb[i], Wb[kzm], make_float2(f + h, v - q));
             }
         }
         *reinterpret_cast<float4*>(Xr + kz * 4) = make_float4(Xa[0].x, Xa[0].y, Xa[1].x, Xa[1].y);
@@ -245,10 +254,10 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
     }
     tc::fence_before_sync();
   }
-  cp_async_wait_all();
-  if (failed) {
+  if (failed) {                                    // its products, and the next rotation's copies
     if (t == 0 && g.tc_err) atomicExch(g.tc_err, 1);
     tc::mbar_wait(&mbar[fail_buf], fail_par, kTcWaitNs / 4);
+    if (fail_next >= 0) tc::mbar_wait(&bar[fail_next & 1], (uint32_t)((fail_next >> 1) & 1), kTcWaitNs / 4);
   }
   tc::fence_before_sync();
   __syncthreads();

@@ -58,16 +58,23 @@ struct ZCfg {
   static constexpr size_t smem_bytes(int q, int ez) {
     return (size_t)(q * SEQ + P) * sizeof(c2) + (size_t)q * 2 * ez * W * sizeof(float2) + 2 * wbytes + 64;
   }
-  // as many rotations as two blocks (else one) have room for
-  static constexpr int fit(int blocks, int ez) {
-    int q = QMAX;
-    while (q > 1 && blocks * (smem_bytes(q, ez) + 1024) > 228 * 1024) q /= 2;
-    return q;
+  // registers a thread needs: in the first step the pair of transforms, with X
+  // beside it where the fields are summed here
+  static constexpr int regs0 = (4 * N1 + (MODE == kZFull ? 2 * N2 : 0) > 6 * N2 ? 4 * N1 + (MODE == kZFull ? 2 * N2 : 0) : 6 * N2) + 40;
+  static constexpr int regs = regs0 < 248 ? regs0 : 248;
+  static constexpr int blocks(int q, int ez) { return pass_blocks(q * W * N1, smem_bytes(q, ez), regs); }
+  // rotations side by side: what puts the most warps on an SM, more first
+  static constexpr int fit(int ez) {
+    int best = 1, warps = 0;
+    for (int q = QMAX; q >= 1; q /= 2) {
+      if (smem_bytes(q, ez) > 227 * 1024) continue;
+      const int w = blocks(q, ez) * ((q * W * N1 + 31) / 32);
+      if (w > warps) { warps = w; best = q; }
+    }
+    return best;
   }
-  static constexpr int fit(int ez) { return 2 * fit(2, ez) > fit(1, ez) ? fit(2, ez) : fit(1, ez); }
   static constexpr int Q = fit(2 * P / 3);        // what the registers are bounded for: typical boxes
-  static constexpr int regs = 4 * N1 + 2 * N2 + 40 < 248 ? 4 * N1 + 2 * N2 + 40 : 248;
-  static constexpr int MIN_BLOCKS = pass_blocks(Q * W * N1, smem_bytes(Q, 2 * P / 3), regs);
+  static constexpr int MIN_BLOCKS = blocks(Q, 2 * P / 3);
 };
 
 __device__ __forceinline__ void cmac(float2& x, float2 w, float2 u) {
@@ -191,16 +198,11 @@ k_zpass(const void* __restrict__ F1, float2* __restrict__ UV, const float2* __re
 
 #pragma unroll 1
   for (int r0 = rbeg; r0 < rend; r0 += Q) {
+    if constexpr (MODE == kZFull) {
 #pragma unroll
-    for (int i = 0; i < N2; ++i) X[i] = make_float2(0.f, 0.f);
-    const int r2 = r0 + q2;                       // this thread's rotation in the second step
-    if constexpr (MODE == kZFromX) {
-      if (r2 < nrot) {
-        const float2* xs = Xg + (((long long)r2 * gridDim.y + kx) * ntile + tile) * (P * W) + k1 * W + c;
-#pragma unroll
-        for (int i = 0; i < N2; ++i) X[i] = __ldg(&xs[i * N1 * W]);
-      }
+      for (int i = 0; i < N2; ++i) X[i] = make_float2(0.f, 0.f);
     }
+    const int r2 = r0 + q2;                       // this thread's rotation in the second step
 #pragma unroll 1
     for (int j = jbeg; j <= g.nch; ++j, ++f) {
       const bool mask = j == g.nch;
@@ -227,6 +229,13 @@ k_zpass(const void* __restrict__ F1, float2* __restrict__ UV, const float2* __re
         if (nr < rend) {
           fetch_inputs(nr, nj);
           if (kWeights) fetch_weights(nj, (f + 1) & 1);
+        }
+      }
+      if constexpr (MODE == kZFromX) {
+        if (r2 < nrot) {
+          const float2* xs = Xg + (((long long)r2 * gridDim.y + kx) * ntile + tile) * (P * W) + k1 * W + c;
+#pragma unroll
+          for (int i = 0; i < N2; ++i) X[i] = __ldg(&xs[i * N1 * W]);
         }
       }
       c2* e = ex + (q2 * N2 * RS + k1) * W + c;   // its column [n2] in the second step
