@@ -183,34 +183,44 @@ k_fwd_x(const float* __restrict__ Bh, const uint8_t* __restrict__ Mh, void* __re
     unsigned mb = 0, pb = 0;
 #pragma unroll
     for (int n1 = 0; n1 < NI; ++n1) {
-      const int x = N2 * n1 + n2;
+      const int x = N2 * n1 + n2;                 // box index
       if (x < nx_ok && M[row + ox + x]) mb |= 1u << n1;
       if (x < pnx && M[prow + x]) pb |= 1u << n1;
     }
+    // the first NA inputs gathered, the others zero: one branch, so that the
+    // gathers of all inputs are in flight together
+    auto gather = [&](auto na) {
+      constexpr int NA = decltype(na)::value;
 #pragma unroll
-    for (int n1 = 0; n1 < NI; ++n1) {
-      const bool in = mb >> n1 & 1;
-      // x = org + N2*n1 + n2 over ex voxels: with ex <= P/2 only n1 < N1/2 can hold data
-      const int x = ox + N2 * n1 + n2;
-      const unsigned xo = in ? 4 * x : 0;
-      const float gx = 0.5f * (vol(oc + xo + (in && x + 1 < g.nx ? 4 : 0)) - vol(oc + xo - (in && x > 0 ? 4 : 0)));
-      const float gy = 0.5f * (vol(oyp + xo) - vol(oym + xo));
-      const float gz = 0.5f * (vol(ozp + xo) - vol(ozm + xo));
-      const float inv = rsqrtf(gx * gx + gy * gy + gz * gz + g.eps2);
-      // the NGF times the mask (m^2 = m: every product of two masked components
-      // equals the product times m, bit for bit)
-      const float X = in ? gx * inv : 0.0f, Y = in ? gy * inv : 0.0f, Z = in ? gz * inv : 0.0f;
-      const float m = even && in ? 1.0f : 0.0f, m2 = pb >> n1 & 1 ? 1.0f : 0.0f;
-      // Eq. 6 products (squared measure): (xx, yy) and (zz, xy), then (xz, yz) and
-      // the mask pair; Eq. 3 (unsquared): (x, y) and (z, 0), then the mask pair
-      if (g.nch == 3) {
-        v[n1] = {make_float2(X * X, Z * Z), make_float2(Y * Y, X * Y)};
-        slot[n1 * NT] = {make_float2(X * Z, m), make_float2(Y * Z, m2)};
-      } else {
-        v[n1] = {make_float2(X, Z), make_float2(Y, 0.0f)};
-        slot[n1 * NT] = {make_float2(0.0f, m), make_float2(0.0f, m2)};
+      for (int n1 = 0; n1 < NI; ++n1) {
+        if (n1 >= NA) {
+          v[n1] = slot[n1 * NT] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+          continue;
+        }
+        const bool in = mb >> n1 & 1;
+        const int xo = in ? 4 * (ox + N2 * n1 + n2) : 0;
+        const float gx = 0.5f * (vol(oc + min(xo + 4, 4 * g.nx - 4)) - vol(oc + max(xo - 4, 0)));
+        const float gy = 0.5f * (vol(oyp + xo) - vol(oym + xo));
+        const float gz = 0.5f * (vol(ozp + xo) - vol(ozm + xo));
+        const float inv = rsqrtf(gx * gx + gy * gy + gz * gz + g.eps2);
+        // the NGF times the mask (m^2 = m: every product of two masked components
+        // equals the product times m, bit for bit)
+        const float X = in ? gx * inv : 0.0f, Y = in ? gy * inv : 0.0f, Z = in ? gz * inv : 0.0f;
+        const float m = even && in ? 1.0f : 0.0f, m2 = pb >> n1 & 1 ? 1.0f : 0.0f;
+        // Eq. 6 products (squared measure): (xx, yy) and (zz, xy), then (xz, yz) and
+        // the mask pair; Eq. 3 (unsquared): (x, y) and (z, 0), then the mask pair
+        if (g.nch == 3) {
+          v[n1] = {make_float2(X * X, Z * Z), make_float2(Y * Y, X * Y)};
+          slot[n1 * NT] = {make_float2(X * Z, m), make_float2(Y * Z, m2)};
+        } else {
+          v[n1] = {make_float2(X, Z), make_float2(Y, 0.0f)};
+          slot[n1 * NT] = {make_float2(0.0f, m), make_float2(0.0f, m2)};
+        }
       }
-    }
+    };
+    constexpr int NA = (3 * NI + 3) / 4;          // boxes of 3/4 of the length are typical
+    if (N2 * NA >= g.ex) gather(std::integral_constant<int, NA>{});
+    else gather(std::integral_constant<int, NI>{});
   }
 #pragma unroll 1
   for (int pair = 0; pair < 2; ++pair) {
