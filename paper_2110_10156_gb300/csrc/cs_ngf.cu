@@ -490,8 +490,9 @@ cs_ngf_status score_batch(cs_ngf_fixed* f, int r0, int nb, float* best_score, in
   if (f->pad_mode == CS_NGF_PAD_BOUND) {
     {
       Stage sp(f, 0, st);
-      k_resample_box<<<resample_box_grid(g, nb), 128, 0, st>>>(f->BQ, f->C8, f->near ? f->N8 + g.nvox : nullptr, rot, g,
-                                                               f->Bh, f->Mh, f->keys);
+      const int rz = resample_box_groups(g, nb);
+      k_resample_box<<<resample_box_grid(g, nb, rz), 128, 0, st>>>(f->BQ, f->C8, f->near ? f->N8 + g.nvox : nullptr, rot, g,
+                                                                   f->Bh, f->Mh, f->keys, rz);
     }
     if (cs_ngf_status s = check_launch("resample")) return s;
   } else {

@@ -349,8 +349,8 @@ k_mask_counts(const uint8_t* __restrict__ C8, const RotIn* __restrict__ rot, Geo
 __global__ void __launch_bounds__(128)
 k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8, const uint8_t* __restrict__ N8,
                const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh, uint8_t* __restrict__ Mh,
-               unsigned long long* __restrict__ keys) {
-  constexpr int RZ = kResampleZGroups, ZB = 4 * RZ;
+               unsigned long long* __restrict__ keys, int RZ) {
+  const int ZB = 4 * RZ;
   const int ztiles = (g.ez + 2 + ZB - 1) / ZB;
   const int r = blockIdx.z / ztiles, zt = blockIdx.z - r * ztiles;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;

@@ -367,7 +367,7 @@ template <int N, int V>
 struct SplitV;
 template <> struct SplitV<16, 0>  { static constexpr int N1 = 4,  N2 = 4; };
 template <> struct SplitV<32, 0>  { static constexpr int N1 = 4,  N2 = 8; };
-template <> struct SplitV<40, 0>  { static constexpr int N1 = 4,  N2 = 10; };
+template <> struct SplitV<40, 0>  { static constexpr int N1 = 5,  N2 = 8; };
 template <> struct SplitV<64, 0>  { static constexpr int N1 = 8,  N2 = 8; };
 template <> struct SplitV<80, 0>  { static constexpr int N1 = 8,  N2 = 10; };
 template <> struct SplitV<100, 0> { static constexpr int N1 = 10, N2 = 10; };

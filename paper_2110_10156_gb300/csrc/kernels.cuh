@@ -187,7 +187,7 @@ __global__ void k_resample(const float4* __restrict__ BQ, const uint8_t* __restr
                            uint8_t* __restrict__ Mh, int* __restrict__ msum, int* __restrict__ marg);
 __global__ void k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8,
                                const uint8_t* __restrict__ N8, const RotIn* __restrict__ rot, Geo g, float* __restrict__ Bh,
-                               uint8_t* __restrict__ Mh, unsigned long long* __restrict__ keys);
+                               uint8_t* __restrict__ Mh, unsigned long long* __restrict__ keys, int RZ);
 // The rotated masks alone, counted into msum and marg as k_resample counts
 // them (the same decisions from the same corner codes, no volumes written):
 // the pre-pass that bounds the shifts of a whole call.
@@ -198,9 +198,18 @@ inline dim3 resample_grid(const Geo& g, int nrot) {
   return dim3((unsigned)((g.nx + 7) / 8), (unsigned)((g.ny + 3) / 4),
               (unsigned)(((g.nz + 4 * kResampleZGroups - 1) / (4 * kResampleZGroups)) * nrot));
 }
-inline dim3 resample_box_grid(const Geo& g, int nrot) {
+// RZ: plane groups per block, 8 (the matrix and the sample row are set up once for
+// them) or fewer where the grid would not fill the SMs: a thread's voxels follow
+// one another, 12 us for a grid of 32 boxes of 34^3 that finishes in 5
+inline int resample_box_groups(const Geo& g, int nrot) {
+  const long long patches = (long long)((g.ex + 2 + 7) / 8) * ((g.ey + 2 + 3) / 4) * nrot;
+  int rz = kResampleZGroups;
+  while (rz > 1 && patches * ((g.ez + 2 + 4 * rz - 1) / (4 * rz)) < 152 * 16 * 4) rz /= 2;
+  return rz;
+}
+inline dim3 resample_box_grid(const Geo& g, int nrot, int rz) {
   return dim3((unsigned)((g.ex + 2 + 7) / 8), (unsigned)((g.ey + 2 + 3) / 4),
-              (unsigned)(((g.ez + 2 + 4 * kResampleZGroups - 1) / (4 * kResampleZGroups)) * nrot));
+              (unsigned)(((g.ez + 2 + 4 * rz - 1) / (4 * rz)) * nrot));
 }
 
 // ----------------------------------------------------------------- shift bounds

@@ -63,13 +63,15 @@ struct ZCfg {
   static constexpr int regs0 = (4 * N1 + (MODE == kZFull ? 2 * N2 : 0) > 6 * N2 ? 4 * N1 + (MODE == kZFull ? 2 * N2 : 0) : 6 * N2) + 40;
   static constexpr int regs = regs0 < 248 ? regs0 : 248;
   static constexpr int blocks(int q, int ez) { return pass_blocks(q * W * N1, smem_bytes(q, ez), regs); }
-  // rotations side by side: what puts the most warps on an SM, more first
+  // rotations side by side: the most, unless fewer put a fifth more threads on an
+  // SM (at 96 points one rotation per block counted two warps for its 48 threads
+  // and took 1.4 times as long as four)
   static constexpr int fit(int ez) {
-    int best = 1, warps = 0;
+    int best = 1, threads = 0;
     for (int q = QMAX; q >= 1; q /= 2) {
       if (smem_bytes(q, ez) > 227 * 1024) continue;
-      const int w = blocks(q, ez) * ((q * W * N1 + 31) / 32);
-      if (w > warps) { warps = w; best = q; }
+      const int n = blocks(q, ez) * q * W * N1;
+      if (5 * n > 6 * threads) { threads = n; best = q; }
     }
     return best;
   }
