@@ -319,7 +319,7 @@ template <int P, int V> struct FwdYCfg {
   // four columns of four rows in different banks
   static constexpr int RS = N1 | 1, CS0 = N2 * RS, CS = CS0 + ((4 * RS - CS0) % 16 + 16) % 16;
   static constexpr size_t smem_bytes(int ey) { return ((size_t)W * CS + (size_t)2 * W * ey) * sizeof(float2) + 16; }
-  static constexpr int MIN_BLOCKS = pass_blocks(NT, smem_bytes(3 * P / 4), N2 > 20 ? 80 : 48);
+  static constexpr int MIN_BLOCKS = pass_blocks(NT, smem_bytes(3 * P / 4), N2 > 20 ? 80 : 64);
 };
 
 template <int P, int ST, bool HALF, int V>
