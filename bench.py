@@ -157,6 +157,29 @@ def stage_bytes(dims, pad, nb, stage, nch=3, precision="fp32"):
     }.get(stage, 0)
 
 
+def box_extents(MB, quats):
+    """Mean extents (z, y, x) of the rotated mask's box over the rotations: what
+    the forward passes of the FP32 form transform.  From the mask's voxels moved
+    by x = R^T (p - c) + c, clipped to the volume."""
+    import torch
+    n = torch.tensor(MB.shape, dtype=torch.float64, device=MB.device)
+    p = torch.nonzero(MB).double() - (n - 1) / 2
+    q = torch.as_tensor(np.asarray(quats), dtype=torch.float64, device=MB.device)
+    q = q / q.norm(dim=1, keepdim=True)
+    w, x, y, z = q.unbind(1)
+    R = torch.stack([1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y),
+                     2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x),
+                     2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)], 1).reshape(-1, 3, 3)
+    R = R.flip(1, 2)                                  # on (z, y, x)
+    ext = []
+    for r in R:
+        v = p @ r
+        lo = torch.maximum(v.amin(0) + (n - 1) / 2, torch.zeros_like(n))
+        hi = torch.minimum(v.amax(0) + (n - 1) / 2, n - 1)
+        ext.append(hi.floor() - lo.ceil() + 1)
+    return tuple(int(round(float(e))) for e in torch.stack(ext).mean(0))
+
+
 PADDING = {
     "bound": "bound-limited: per call the shortest FFT lengths that keep every shift the "
              "Section 3.2 overlap bound admits alias-free (same scores as the full length)",
@@ -448,8 +471,7 @@ def run_ours(args):
             import torch.distributed as dist
             dist.barrier()
 
-    # ---------------- device-resident timed region (full launch groups replay
-    # one captured CUDA graph each)
+    # ---------------- device-resident timed region
     sampler = ClockSampler(local)
     sampler.start()
     l0 = cs_ngf.launch_count()
@@ -474,7 +496,7 @@ def run_ours(args):
     value = ws * R * args.steps / (elapsed_ms / 1000.0)
 
     # ---------------- per-kernel CUDA-event times: one more step with every
-    # launch bracketed by events on its stream (direct launches, no graph)
+    # launch bracketed by events on its stream
     f.set_profiling(True)
     f.stage_times()
     t0p = time.perf_counter()
@@ -523,21 +545,24 @@ def run_ours(args):
     stage_ms = {k: v[0] for k, v in stages.items()}
     dom = max(("resample", "fwd_x", "fwd_y", "zmac", "inv_y", "inv_x"), key=lambda k: stage_ms[k])
     classes = f.transform_classes()
+    # the FP32 form with the built-in splits transforms the masks' boxes only
+    boxed = args.precision == "fp32" and args.pad_mode == "bound" and args.autotune == "off"
+    ext = box_extents(MB, quats) if boxed else dims
     launches_of = [(cp, min(f.batch, cnt - b * f.batch)) for cp, cnt in classes
                    for b in range(-(-cnt // f.batch))]
     nbatches = len(launches_of)
-    total_bytes = sum(stage_bytes(dims, cp, nb, dom, precision=args.precision) for cp, nb in launches_of)
+    total_bytes = sum(stage_bytes(ext, cp, nb, dom, precision=args.precision) for cp, nb in launches_of)
     total_bytes *= prof_steps
     achieved = total_bytes / (stage_ms[dom] / 1000.0) / 1e9 if stage_ms[dom] > 0 else 0.0
-    tr = launch_traffic(dom, args.precision, dims, launches_of)
+    tr = launch_traffic(dom, args.precision, ext, launches_of)
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_kind": f"{peak_kind} hbm_gbs",
-                "kernel": dom,
+                "kernel": dom, "extents": list(ext),
                 "traffic": None if tr is None else tr / nbatches,
                 "algorithmic_bytes_per_launch": total_bytes / (prof_steps * nbatches),
                 "timing": "CUDA events around every launch of one profiled step after the timed region"}
     if dom == "zmac":               # the same without the F2 writes (a lower bound)
-        lo = sum(stage_bytes(dims, cp, nb, "zmac_no_f2", precision=args.precision)
+        lo = sum(stage_bytes(ext, cp, nb, "zmac_no_f2", precision=args.precision)
                  for cp, nb in launches_of) * prof_steps
         ach_lo = lo / (stage_ms[dom] / 1000.0) / 1e9 if stage_ms[dom] > 0 else 0.0
         roofline.update({"achieved_without_f2": ach_lo, "frac_without_f2": ach_lo / peak,
@@ -546,7 +571,7 @@ def run_ours(args):
     # the whole step against HBM: the ncu DRAM bytes per rotation of every
     # scoring stage (same kernel sources and precision only), times the
     # rotations, over the timed step
-    step_bytes = [launch_traffic(st, args.precision, dims, launches_of)
+    step_bytes = [launch_traffic(st, args.precision, ext, launches_of)
                   for st in ("resample", "fwd_x", "fwd_y", "zmac", "inv_y", "inv_x")]
     roofline_step = None
     if all(b is not None for b in step_bytes):
@@ -558,7 +583,7 @@ def run_ours(args):
 
     roofline_alu = None
     if dom == "zmac":
-        fl = sum(zmac_flops(dims, cp, nb) for cp, nb in launches_of) * prof_steps
+        fl = sum(zmac_flops(ext, cp, nb) for cp, nb in launches_of) * prof_steps
         ach = fl / (stage_ms[dom] / 1000.0) / 1e12 if stage_ms[dom] > 0 else 0.0
         roofline_alu = {"bound": "alu", "achieved": ach, "peak": FP32_ALU_PEAK_TFLOPS, "unit": "TFLOP/s",
                         "frac": ach / FP32_ALU_PEAK_TFLOPS, "kernel": dom,

@@ -460,10 +460,10 @@ cs_ngf_status stage_call_impl(cs_ngf_fixed* f, const float* B, const uint8_t* MB
   CallStage cs{};
   cs.src = reinterpret_cast<const int*>(f->rot_h);
   cs.dst = reinterpret_cast<int*>(f->rot_d);
-  cs.words = R * (int)(sizeof(RotIn) / sizeof(int));
+  cs.words = (long long)R * (long long)(sizeof(RotIn) / sizeof(int));
   if (bound) {
     cs.zero = f->allm;
-    cs.zeros = R * (1 + g.nz + g.ny + g.nx);
+    cs.zeros = (long long)R * (1 + g.nz + g.ny + g.nx);
     cs.mbox = f->mbox;
   }
   { Stage sp(f, 0, st); k_pack_floating<<<512, 256, 0, st>>>(B, MB, g, f->BQ, f->C8, cs); }
@@ -813,10 +813,10 @@ cs_ngf_status plan_classes_impl(cs_ngf_fixed* f, int R, cudaStream_t st, Plan& p
     f->run_pads.insert(f->run_pads.end(), q.pad, q.pad + 3);
     f->run_counts.push_back((int)c.rot.size());
   }
-  const int words = R * (int)(sizeof(RotIn) / sizeof(int));
+  const long long words = (long long)R * (long long)(sizeof(RotIn) / sizeof(int));
   {
     Stage sp(f, 7, st);
-    k_copy_words<<<std::min(64, (words + 255) / 256), 256, 0, st>>>(reinterpret_cast<const int*>(f->rot_h),
+    k_copy_words<<<(unsigned)std::min(64ll, (words + 255) / 256), 256, 0, st>>>(reinterpret_cast<const int*>(f->rot_h),
                                                                     reinterpret_cast<int*>(f->rot_d), words);
   }
   if (cs_ngf_status s = check_launch("boxes")) return s;
@@ -906,6 +906,14 @@ Sizes sizes_for(const int32_t dims[3], const int pad[3], int measure, int precis
   return z;
 }
 
+// rotations per launch group that a third of the free device memory holds, 1 .. most
+int automatic_batch(const Sizes& z, int most) {
+  size_t free_b = 0, total_b = 0;
+  cudaMemGetInfo(&free_b, &total_b);
+  const size_t uv = z.uv_elems * sizeof(float2), budget = free_b > uv ? (free_b - uv) / 3 : 0;
+  return (int)std::max<size_t>(1, std::min<size_t>((size_t)most, budget / z.per_rot));
+}
+
 cs_ngf_status ensure_results(cs_ngf_fixed* f, int R) {
   if (R <= f->res_cap) return CS_NGF_OK;
   CS_CUDA(cudaDeviceSynchronize());
@@ -941,6 +949,9 @@ cs_ngf_status set_class(cs_ngf_fixed* f, const ClassGeom& c, cudaStream_t st) {
 }
 cs_ngf_status resolve_pads(const int32_t dims[3], const cs_ngf_config& cfg, int pad[3]) {
   return ::resolve_pads_impl(dims, cfg, pad);
+}
+int auto_batch(const int32_t dims[3], const int pad[3], int measure, int precision, int tensor_cores, int most) {
+  return ::automatic_batch(::sizes_for(dims, pad, measure, precision, tensor_cores), most);
 }
 size_t handle_bytes(const int32_t dims[3], const int pad[3], int batch, int measure, int precision,
                     int tensor_cores) {
@@ -1064,12 +1075,7 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
   f->f13_elems = sz.f13_elems;
   const size_t per_rot = sz.per_rot, shared_ws = sz.shared_ws, uv_elems = sz.uv_elems;
   int batch = cfg.batch;
-  if (batch == 0) {
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
-    const size_t budget = free_b > uv_elems * sizeof(float2) ? (free_b - uv_elems * sizeof(float2)) / 3 : 0;
-    batch = (int)std::max<size_t>(1, std::min<size_t>(32, budget / per_rot));
-  }
+  if (batch == 0) batch = automatic_batch(sz, 32);
   // launch grids index (rotation, field, z-plane) and (rotation, shift plane)
   // in their y dimension, at most 65535 blocks
   batch = std::min(batch, 65535 / std::max(g.nf * g.nz, 2 * g.nz - 1));

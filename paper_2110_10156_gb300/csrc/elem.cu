@@ -47,8 +47,8 @@ __global__ void k_pack_floating(const float* __restrict__ B, const uint8_t* __re
                                 float4* __restrict__ BQ, uint8_t* __restrict__ C8, CallStage cs) {
   const int sy = g.nx, sz = g.nx * g.ny;          // volumes hold < 2^31 voxels
   const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-  for (int i = t0; i < cs.words; i += nt) cs.dst[i] = cs.src[i];
-  for (int i = t0; i < cs.zeros; i += nt) cs.zero[i] = 0;
+  for (long long i = t0; i < cs.words; i += nt) cs.dst[i] = cs.src[i];
+  for (long long i = t0; i < cs.zeros; i += nt) cs.zero[i] = 0;
   int b[6] = {0, 0, 0, 0, 0, 0};                  // n - min and max + 1 (z, y, x) of cells with a mask corner
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.nvox;
        i += (long long)gridDim.x * blockDim.x) {
@@ -444,8 +444,8 @@ __global__ void __launch_bounds__(256) k_fixed_box(const int* __restrict__ marg,
   }
 }
 
-__global__ void k_copy_words(const int* __restrict__ src, int* __restrict__ dst, int n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i];
+__global__ void k_copy_words(const int* __restrict__ src, int* __restrict__ dst, long long n) {
+  for (long long i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i];
 }
 
 // block (rotation r, axis a); thread per shift slot v, then per slab

@@ -131,6 +131,8 @@ cs_ngf_status score_range(cs_ngf_fixed* f, int r0, int n, float* best_score, int
                           cudaStream_t st);
 // validate dims / cfg and return the FFT lengths; EINVAL / EUNSUPPORTED on error
 cs_ngf_status resolve_pads(const int32_t dims[3], const cs_ngf_config& cfg, int pad[3]);
+// the automatic launch group: what a third of the free device memory holds, 1 .. most
+int auto_batch(const int32_t dims[3], const int pad[3], int measure, int precision, int tensor_cores, int most);
 // device bytes a handle of these dims, FFT lengths and batch allocates
 size_t handle_bytes(const int32_t dims[3], const int pad[3], int batch, int measure, int precision,
                     int tensor_cores);

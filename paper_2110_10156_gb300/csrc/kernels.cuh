@@ -170,14 +170,14 @@ __device__ __forceinline__ unsigned long long make_key(float s, unsigned lin) {
 struct CallStage {
   const int* src;
   int* dst;
-  int words;
+  long long words;
   int* zero;
-  int zeros;
+  long long zeros;
   int* mbox;
 };
 __global__ void k_pack_floating(const float* __restrict__ B, const uint8_t* __restrict__ MB, Geo g,
                                 float4* __restrict__ BQ, uint8_t* __restrict__ C8, CallStage cs);
-__global__ void k_copy_words(const int* __restrict__ src, int* __restrict__ dst, int n);
+__global__ void k_copy_words(const int* __restrict__ src, int* __restrict__ dst, long long n);
 __global__ void k_near_axis(const uint8_t* __restrict__ in, uint8_t* __restrict__ out, Geo g, int axis);
 // k_resample: the whole volume, mask counts into msum and marg (marg may be
 // nullptr); grid resample_grid.  k_resample_box: only the voxels the x pass

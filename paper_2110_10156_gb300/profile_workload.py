@@ -17,8 +17,9 @@ import sys
 import numpy as np
 
 
-STAGE_OF = {"k_resample": "resample", "k_mask_counts": "resample", "k_fwd_x": "fwd_x",
-            "k_fwd_y": "fwd_y", "k_zmac": "zmac", "k_inv_y": "inv_y", "k_inv_x": "inv_x"}
+STAGE_OF = {"k_resample": "resample", "k_resample_box": "resample", "k_mask_counts": "resample",
+            "k_fwd_x": "fwd_x", "k_fwd_y": "fwd_y", "k_zmac": "zmac", "k_zpass": "zmac", "k_inv_y": "inv_y",
+            "k_inv_x": "inv_x"}
 
 
 def _stage_bytes(csv_paths) -> dict:
@@ -41,7 +42,7 @@ def _stage_bytes(csv_paths) -> dict:
             lines = [ln for ln in fh if ln.startswith('"')]
         rows = list(csv.DictReader(lines))
         first = min((int(r["ID"]) for r in rows if r.get("Kernel Name", "").split("(")[0].split("<")[0]
-                     .endswith("k_resample")), default=0)
+                     .endswith(("k_resample", "k_resample_box"))), default=0)
         for r in rows:
             stage = stage_of(r.get("Kernel Name", ""))
             if stage is None or int(r["ID"]) < first:
