@@ -548,8 +548,12 @@ def run_ours(args):
     # the FP32 form with the built-in splits transforms the masks' boxes only
     boxed = args.precision == "fp32" and args.pad_mode == "bound" and args.autotune == "off"
     ext = box_extents(MB, quats) if boxed else dims
-    launches_of = [(cp, min(f.batch, cnt - b * f.batch)) for cp, cnt in classes
-                   for b in range(-(-cnt // f.batch))]
+    # launch groups: as many as were launched, shared out over the classes
+    per = R / max(1, stages["zmac"][1])
+    launches_of = []
+    for cp, cnt in classes:
+        k = max(1, round(cnt / per))
+        launches_of += [(cp, cnt // k + (b < cnt % k)) for b in range(k)]
     nbatches = len(launches_of)
     total_bytes = sum(stage_bytes(ext, cp, nb, dom, precision=args.precision) for cp, nb in launches_of)
     total_bytes *= prof_steps

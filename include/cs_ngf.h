@@ -134,7 +134,8 @@ typedef struct {
   float gamma;       /* minimum overlap fraction in (0, 1]; the paper uses 0.5 */
   int32_t pad[3];    /* FFT lengths (z, y, x); 0 = automatic */
   int32_t batch;     /* rotations per launch group; 0 = automatic (memory-sized, at
-                        most 32); a value above 65535 / (fields x nz) is lowered to
+                        most 32 at the longest lengths, up to 128 where a call's
+                        are shorter); a value above 65535 / (fields x nz) is lowered to
                         that (4 fields for the squared measure, 3 unsquared);
                         an odd value above 1 is rounded down to even, since the
                         masks of rotations 2k and 2k+1 share one transform.
@@ -172,7 +173,7 @@ typedef struct {
 typedef struct {
   int32_t dims[3];              /* nz, ny, nx */
   int32_t pad[3];               /* FFT lengths (those the last call's shift ranges give) */
-  int32_t batch;                /* rotations per launch group */
+  int32_t batch;                /* rotations per launch group at the longest lengths */
   int64_t sum_mask_a;           /* sum of M_A */
   int64_t fixed_bytes;          /* device bytes of the fixed spectra */
   int64_t workspace_bytes;      /* device bytes of the per-batch workspace */

@@ -666,13 +666,36 @@ cs_ngf_status check_volume_args(const cs_ngf_fixed* f, const float* B, const uin
   return CS_NGF_OK;
 }
 
-// rotations [r0_begin, r0_begin + n) of the uploaded set in launch groups
+// Rotations per launch group at the lengths in use.  The fields' buffers hold
+// f->batch rotations at the longest lengths, so more at shorter ones; every pass
+// fills the SMs better with more (32 -> 128 rotations, us per rotation: 32^3 4.6
+// -> 3.5, 64^3 11.0 -> 10.0, 150^3 101.4 -> 99.9).  Fewer, to keep the fields
+// within L2, was slower everywhere (64^3: 15.0 with 8).  Always even above one.
+int group_size(const cs_ngf_fixed* f) {
+  if (f->group_cap <= f->batch) return f->batch;
+  const Geo& g = f->g;
+  const size_t cb = g.store == kStoreF32 ? 8 : 4, field = g.nch * cb + 8;
+  const size_t row = (size_t)g.Px * ky_total(g.Py);
+  const size_t f02 = (std::max(field * g.ez * g.ey * g.Px, (size_t)g.wz * row * 8) + 7) / 8;
+  const size_t f13 = (std::max(field * g.ez * row, (size_t)g.wz * g.wy * g.Px * 8) + 7) / 8;
+  size_t n = std::min({(size_t)f->group_cap, f->batch * f->f02_elems / f02, f->batch * f->f13_elems / f13});
+  if (f->zx) n = std::min(n, f->batch * f->zx_elems / ((size_t)(g.Px / 2 + 1) * ky_total(g.Py) * g.Pz));
+  return std::max((int)n / 2 * 2, f->batch);
+}
+
+// rotations [r0_begin, r0_begin + n) of the uploaded set in launch groups of
+// about the same size (a short last one would leave SMs idle)
 cs_ngf_status score_range_impl(cs_ngf_fixed* f, int r0_begin, int n, float* best_score,
                                int32_t* best_shift, cudaStream_t st) {
   const int end = r0_begin + n;
-  for (int r0 = r0_begin; r0 < end; r0 += f->batch) {
+  int group = group_size(f);
+  if (f->group_cap > f->batch) {
+    const int groups = (n + group - 1) / group;
+    group = std::min(group, ((n + groups - 1) / groups + 1) / 2 * 2);
+  }
+  for (int r0 = r0_begin; r0 < end; r0 += group) {
     // the first group at new lengths times the splits (autotuning)
-    if (cs_ngf_status s = score_batch(f, r0, std::min(f->batch, end - r0), best_score, best_shift, nullptr, st,
+    if (cs_ngf_status s = score_batch(f, r0, std::min(group, end - r0), best_score, best_shift, nullptr, st,
                                       needs_tuning(f)))
       return s;
   }
@@ -1083,6 +1106,14 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
   // keeps every pair inside one launch group, so results do not depend on it
   if (batch > 1 && (batch & 1)) --batch;
   f->batch = batch;
+  // the volumes of a launch group at shorter lengths (group_size): up to 128, and
+  // up to 1 GB where that is more than the batch; a workspace that free memory
+  // cut short stays as it is
+  f->group_cap = batch;
+  if (cfg.batch == 0 && batch == 32 && cfg.pad_mode == CS_NGF_PAD_BOUND)
+    f->group_cap = std::max(batch, (int)std::min<long long>({128, (1ll << 30) / (5 * g.nvox),
+                                                             65535 / std::max(g.nf * g.nz, 2 * g.nz - 1)}) / 2 * 2);
+  f->zx_elems = sz.zx_elems;
 
   cudaStream_t st = (cudaStream_t)stream;
   auto bail = [&](cs_ngf_status s) { std::string m = g_last_error; free_handle(f); g_last_error = m; return s; };
@@ -1091,8 +1122,8 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
     e_ == cudaErrorMemoryAllocation ? CS_NGF_ENOMEM : CS_NGF_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_))); } while (0)
 
   CS_TRYC(dalloc(&f->UV, uv_elems));
-  CS_TRYC(dalloc(&f->Bh, (size_t)batch * g.nvox));
-  CS_TRYC(dalloc(&f->Mh, (size_t)batch * g.nvox));
+  CS_TRYC(dalloc(&f->Bh, (size_t)f->group_cap * g.nvox));
+  CS_TRYC(dalloc(&f->Mh, (size_t)f->group_cap * g.nvox));
   CS_TRYC(dalloc(&f->BQ, (size_t)g.nvox));
   CS_TRYC(dalloc(&f->C8, (size_t)g.nvox));
   CS_TRYC(dalloc(&f->N8, (size_t)g.nvox * 2));
@@ -1105,7 +1136,7 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
   CS_TRYC(dalloc(&f->margB, (size_t)batch * nmarg));
   CS_TRYC(dalloc(&f->bounds, (size_t)batch));
   CS_TRYC(dalloc(&f->boxA, (size_t)1));
-  CS_TRYC(dalloc(&f->keys, (size_t)batch));
+  CS_TRYC(dalloc(&f->keys, (size_t)f->group_cap));
   if (sz.zx_elems) {
     CS_TRYC(dalloc(&f->zx, (size_t)batch * sz.zx_elems));
     g.zx = f->zx;
@@ -1117,7 +1148,7 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
   CS_TRYC(cudaMemsetAsync(f->mbox, 0, sizeof(int) * 6, st));
   g.tc_err = f->tc_err;
   f->fixed_bytes = uv_elems * sizeof(float2);
-  f->workspace_bytes = (size_t)batch * per_rot + shared_ws;
+  f->workspace_bytes = (size_t)batch * per_rot + (size_t)(f->group_cap - batch) * g.nvox * 5 + shared_ws;
   if (f->pad_mode == CS_NGF_PAD_BOUND) {
     CS_TRYC(dalloc(&f->A_keep, (size_t)g.nvox));
     CS_TRYC(dalloc(&f->MA_keep, (size_t)g.nvox));

@@ -19,7 +19,8 @@ struct cs_ngf_fixed {
   int device = 0;
   Geo g{};
   float eps = 1e-5f, gamma = 0.5f;
-  int batch = 1;
+  int batch = 1;               // rotations the workspace holds at the longest lengths
+  int group_cap = 1;           // most rotations of a launch group: B_hat, M_hat and keys are sized for them
   int sumA = 0;
   // FFT lengths the buffers are sized for (the automatic or requested ones);
   // g.Pz/Py/Px are the lengths in use, which bound-limited padding
@@ -56,7 +57,7 @@ struct cs_ngf_fixed {
   // the alternatives are requested outright (autotune 2)
   int autotune = 0;
   int vars[5] = {0, 0, 0, 0, 0};
-  size_t f02_elems = 0, f13_elems = 0;
+  size_t f02_elems = 0, f13_elems = 0, zx_elems = 0;   // per rotation at the longest lengths
   float2* UV = nullptr;
   float* Bh = nullptr;
   uint8_t* Mh = nullptr;

@@ -235,9 +235,8 @@ cs_ngf_status cs_ngf_global_align(const float* A, const uint8_t* maskA, const fl
     // and unmap than they take to score (search of a 150^3 pair: 95.9 -> 91.4 ms,
     // with the other changes to small calls)
     int pad[3];
-    if (lc.batch == 0 && !csngf::detail::resolve_pads(ld, lc, pad))
-      lc.batch = csngf::detail::auto_batch(ld, pad, lc.measure, lc.precision, lc.tensor_cores,
-                                           std::min(32, (R + 1) / 2 * 2));
+    if (lc.batch == 0 && R < 32 && !csngf::detail::resolve_pads(ld, lc, pad))
+      lc.batch = csngf::detail::auto_batch(ld, pad, lc.measure, lc.precision, lc.tensor_cores, (R + 1) / 2 * 2);
     cs_ngf_fixed* h = nullptr;
     if (cs_ngf_status s = cs_ngf_prepare_fixed(la.as<float>(), lma.as<uint8_t>(), ld, &lc, st, &h)) return s;
     cudaFree(rsc.p);

@@ -148,3 +148,17 @@ def test_box_only_lengths_match_oracle(cs, P, axis):
     sc, sh = [t.cpu().numpy() for t in f.score_rotations(dev(p.B), dev(p.MB), p.quats)]
     for r, q in enumerate(p.quats):
         check_best_against_map(O.score_map(p.A, p.MA, p.B, p.MB, q)[0], sc[r], sh[r])
+
+
+@pytest.mark.parametrize("dims,R,kw", [((20, 23, 18), 131, {}), ((20, 23, 18), 65, dict(precision="bf16")),
+                                       ((33, 30, 36), 290, dict(measure="unsquared"))])
+def test_automatic_launch_groups_match_small_ones(cs, dims, R, kw):
+    """Automatic handles score more than 32 rotations per launch group at short
+    lengths: bit for bit what groups of eight give, for a class's odd rest too."""
+    p = synth.small_pair(410 + R, dims, masks="full", n_rot=R)
+    MA, MB = box_mask(dims, (4, 5, 3), (14, 17, 15)), box_mask(dims, (2, 6, 4), (15, 19, 14))
+    a = cs.prepare_fixed(dev(p.A), dev(MA), **kw)
+    b = cs.prepare_fixed(dev(p.A), dev(MA), batch=8, **kw)
+    assert a.batch == 32
+    for x, y in zip(a.score_rotations(dev(p.B), dev(MB), p.quats), b.score_rotations(dev(p.B), dev(MB), p.quats)):
+        np.testing.assert_array_equal(x.cpu().numpy(), y.cpu().numpy())
