@@ -134,7 +134,11 @@ struct FwdXCfg {
   // put eight consecutive lanes of either step in different 16-byte banks
   static constexpr int RS = N1 | 1, CS0 = N2 * RS, CS = CS0 + ((N1 - CS0) % 8 + 8) % 8;
   static constexpr size_t smem_bytes = ((size_t)ROWS * CS + (size_t)NI * NT) * sizeof(c2);
-  static constexpr int regs = 4 * (N1 > N2 ? N1 : N2) + 56 < 248 ? 4 * (N1 > N2 ? N1 : N2) + 56 : 248;
+  // registers: the larger step's pair of values and the gather's addresses, fewer
+  // where half of the inputs are zero (320 points: 51.4 -> 48.2 us per rotation of
+  // 120x144x132 with full padding; whole inputs at 160 and 300 spill with as few,
+  // 150^3 25.4 -> 30.3, 256^3 149 -> 166)
+  static constexpr int regs0 = 4 * (N1 > N2 ? N1 : N2) + (HALF ? 40 : 56), regs = regs0 < 248 ? regs0 : 248;
   static constexpr int MIN_BLOCKS = pass_blocks(NT, smem_bytes, regs);
 };
 

@@ -59,8 +59,10 @@ struct ZCfg {
     return (size_t)(q * SEQ + P) * sizeof(c2) + (size_t)q * 2 * ez * W * sizeof(float2) + 2 * wbytes + 64;
   }
   // registers a thread needs: in the first step the pair of transforms, with X
-  // beside it where the fields are summed here
-  static constexpr int regs0 = (4 * N1 + (MODE == kZFull ? 2 * N2 : 0) > 6 * N2 ? 4 * N1 + (MODE == kZFull ? 2 * N2 : 0) : 6 * N2) + 40;
+  // beside it where the fields are summed here (with 40 more instead of 24 there:
+  // 96x128x128 19.2 -> 20.1 us per rotation; with 24 in the other modes: 150^3 BF16
+  // 84.9 -> 90.4)
+  static constexpr int regs0 = (4 * N1 + (MODE == kZFull ? 2 * N2 : 0) > 6 * N2 ? 4 * N1 + (MODE == kZFull ? 2 * N2 : 0) : 6 * N2) + (MODE == kZFull ? 24 : 40);
   static constexpr int regs = regs0 < 248 ? regs0 : 248;
   static constexpr int blocks(int q, int ez) { return pass_blocks(q * W * N1, smem_bytes(q, ez), regs); }
   // rotations side by side: the most, unless fewer put a fifth more threads on an
