@@ -54,7 +54,7 @@ struct Geo {
   // 1 in the other forms and for the mask field (j = nch)
   float scale0[4], scale1[4];
   // 1: in the BF16 and FP16 forms the z pass runs the forward z-axis DFT of
-  // the channel fields on the tensor cores (k_zmac_tc) where its length allows
+  // the channel fields on the tensor cores (k_zx_tc) where its length allows
   int tc;
   // set to 1 by a z pass whose bounded wait for its own MMAs or copies ran out
   // (it then stops and returns); nullptr: not reported
