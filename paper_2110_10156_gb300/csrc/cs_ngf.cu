@@ -466,7 +466,9 @@ cs_ngf_status stage_call_impl(cs_ngf_fixed* f, const float* B, const uint8_t* MB
     cs.zeros = (long long)R * (1 + g.nz + g.ny + g.nx);
     cs.mbox = f->mbox;
   }
-  { Stage sp(f, 0, st); k_pack_floating<<<512, 256, 0, st>>>(B, MB, g, f->BQ, f->C8, cs); }
+  const long long items = std::max({g.nvox, cs.words, cs.zeros});
+  const unsigned blocks = (unsigned)std::min(1216ll, (items + 255) / 256);   // eight per SM
+  { Stage sp(f, 0, st); k_pack_floating<<<blocks, 256, 0, st>>>(B, MB, g, f->BQ, f->C8, cs); }
   CS_CUDA(cudaEventRecord(f->rot_ev, st));
   f->near = bound && R >= 16;
   if (f->near) {
@@ -553,7 +555,7 @@ cs_ngf_status run_spectra(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cu
 cs_ngf_status load_fixed(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cudaStream_t st) {
   const Geo& g = f->g;
   CS_CUDA(cudaMemsetAsync(f->margA, 0, sizeof(int) * ((size_t)g.nz + g.ny + g.nx), st));
-  { Stage sp(f, 6, st); k_marginals<<<(unsigned)g.nz, 256, 0, st>>>(A, MA, g, f->margA, f->A_keep, f->MA_keep); }
+  { Stage sp(f, 6, st); k_marginals<<<dim3((unsigned)g.nz, (unsigned)((g.ny + 31) / 32)), 256, 0, st>>>(A, MA, g, f->margA, f->A_keep, f->MA_keep); }
   { Stage sp(f, 6, st); k_fixed_box<<<1, 256, 0, st>>>(f->margA, g, f->boxed ? 1 : 0, f->fbox_h, f->boxA); }
   if (cs_ngf_status s = check_launch("marginals")) return s;
   CS_CUDA(cudaStreamSynchronize(st));
