@@ -196,8 +196,10 @@ void cs_ngf_default_config(cs_ngf_config* cfg);
  *   dims   host {nz, ny, nx}
  *   cfg    host, NULL = defaults
  *   out    host; receives the handle (NULL on failure)
- * Synchronises `stream` before returning (the handle's sum of M_A is read
- * back).  Errors: EINVAL, EUNSUPPORTED, ENOMEM, ECUDA. */
+ * Synchronises `stream` after its last read of A and maskA, which the caller
+ * may then write or free (with bound-limited padding the spectra come from the
+ * handle's own copies and may still be running).  Errors: EINVAL,
+ * EUNSUPPORTED, ENOMEM, ECUDA. */
 cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const int32_t dims[3],
                                    const cs_ngf_config* cfg, void* stream, cs_ngf_fixed** out);
 
@@ -244,7 +246,8 @@ cs_ngf_status cs_ngf_resample(cs_ngf_fixed* f, const float* B, const uint8_t* ma
                               const double* quat, float* Bhat, uint8_t* Mhat, void* stream);
 
 /* Recompute the fixed-volume spectra of an existing handle from a new A and
- * maskA of the same dims (no reallocation).  Synchronises `stream`.
+ * maskA of the same dims (no reallocation).  Synchronises `stream` after its
+ * last read of A and maskA, as cs_ngf_prepare_fixed.
  * Errors: EINVAL, EBUSY, ECUDA. */
 cs_ngf_status cs_ngf_update_fixed(cs_ngf_fixed* f, const float* A, const uint8_t* maskA,
                                   void* stream);

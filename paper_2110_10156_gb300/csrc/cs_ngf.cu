@@ -550,8 +550,8 @@ cs_ngf_status run_spectra(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cu
 }
 
 // a new fixed volume: slab counts of its mask, its box, copies where later
-// changes of length need them, and the spectra at the lengths in use;
-// synchronises st
+// changes of length need them, and the spectra at the lengths in use, from the
+// copies where there are some; synchronises st after the last read of A and MA
 cs_ngf_status load_fixed(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cudaStream_t st) {
   const Geo& g = f->g;
   CS_CUDA(cudaMemsetAsync(f->margA, 0, sizeof(int) * ((size_t)g.nz + g.ny + g.nx), st));
@@ -566,7 +566,11 @@ cs_ngf_status load_fixed(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cud
     f->a1[a] = f->fbox_h->a1[a];
     f->extA[a] = f->pad_mode == CS_NGF_PAD_BOUND ? f->a1[a] + 1 - (f->boxed ? f->a0[a] : 0) : n[a];
   }
-  return run_spectra(f, A, MA, st);
+  // the caller may write A and MA again once this has returned
+  if (f->A_keep) return run_spectra(f, f->A_keep, f->MA_keep, st);
+  if (cs_ngf_status s = run_spectra(f, A, MA, st)) return s;
+  CS_CUDA(cudaStreamSynchronize(st));
+  return CS_NGF_OK;
 }
 
 // switch the handle to a class's FFT lengths (each <= alloc_pad), box extents
