@@ -30,7 +30,10 @@ def test_fixed_volume_overwritten_on_another_stream(cs, pad_mode, call):
     ref = cs.prepare_fixed(A, M, pad_mode=pad_mode)
     want = [t.cpu().numpy() for t in ref.score_rotations(B, M, q)]
     ref.release()
-    other = torch.cuda.Stream()
+    other, busy = torch.cuda.Stream(priority=-1), torch.cuda.Stream()
+    X = torch.rand(8192, 8192, device="cuda").bfloat16()
+    with torch.cuda.stream(busy):
+        X @ X
     if call == "update_fixed":
         f = cs.prepare_fixed(first, M, pad_mode=pad_mode)
         f.score_rotations(B, M, q)               # the lengths the next call keeps
@@ -40,6 +43,9 @@ def test_fixed_volume_overwritten_on_another_stream(cs, pad_mode, call):
         M2.copy_(M)
         M.clone().zero_()
     torch.cuda.synchronize()
+    with torch.cuda.stream(busy):                # about 50 ms: what the call leaves running takes its time
+        for _ in range(80):
+            X @ X
     if call == "update_fixed":
         f.update_fixed(A2, M2)
     else:
