@@ -360,13 +360,13 @@ k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, Geo g, int groups) {
     fetch(zbeg + 4, 1);
   }
   __syncthreads();                                   // the barriers are initialised
-  bool dead = false;                                 // a wait ran out: no more waits, results invalid
+  int dead = -1;                                     // the group whose wait ran out: no more waits, results invalid
   int it = 0;
 #pragma unroll 1
   for (int z0 = zbeg; z0 < zend; z0 += 4, ++it) {
     const int nz = min(4, zend - z0);
     const float2* src = in + (it & 1) * W * g.ey;
-    if (!dead && !tc::mbar_wait(&bar[it & 1], (it >> 1) & 1, kTcWaitNs)) dead = true;
+    if (dead < 0 && !tc::mbar_wait(&bar[it & 1], (it >> 1) & 1, kTcWaitNs)) dead = it;
     {
       const int kxi = t & 3, n2 = (t >> 2) % N2, zz = t / (4 * N2);
       const float isc = 1.0f / field_scale(g.scale0, j);
@@ -397,7 +397,9 @@ k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, Geo g, int groups) {
       }
     }
     __syncthreads();
-    if (t == 0) fetch(z0 + 8, it & 1);               // this group's inputs have been read
+    // this group's inputs have been read (dead: its phase is still open, and a
+    // second arrival on it would be undefined)
+    if (t == 0 && dead < 0) fetch(z0 + 8, it & 1);
     if (t < W * N1) {
       const int k1 = t % N1, kxi = t / N1 & 3, zz = t / (4 * N1);
       if (zz < nz) {
@@ -421,9 +423,10 @@ k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, Geo g, int groups) {
     }
     __syncthreads();
   }
-  if (dead) {                                        // the results are invalid; its copies end before the block does
-    if (t == 0 && g.tc_err) atomicExch(g.tc_err, 1);
-    for (int l = it - 1; l >= 0 && l >= it - 2; --l) tc::mbar_wait(&bar[l & 1], (l >> 1) & 1, kTcWaitNs / 4);
+  if (dead >= 0) {                                   // the copies still in flight end before the block does
+    if (g.tc_err) atomicExch(g.tc_err, 1);
+    if (t == 0)
+      for (int l = dead; l < it && l < dead + 2; ++l) tc::mbar_wait(&bar[l & 1], (l >> 1) & 1, kTcWaitNs / 4);
   }
 }
 

@@ -161,9 +161,10 @@ k_zpass(const void* __restrict__ F1, float2* __restrict__ UV, const float2* __re
 
   float2 X[N2];
   int f = 0;                                      // fields so far: buffers and phases of the barriers
-  bool dead = false;                              // a wait ran out: no more waits, results invalid
+  int dead = -1;                                  // 2 field + (inputs: 0, weights: 1) of a wait that ran out: no more
+                                                  // waits, results invalid
   auto wait = [&](int b, int phase) {
-    if (!dead && !tc::mbar_wait(&bar[b], phase & 1, kTcWaitNs)) dead = true;
+    if (dead < 0 && !tc::mbar_wait(&bar[b], phase & 1, kTcWaitNs)) dead = 2 * f + (b > 0);
   };
   // channels a', b' at this thread's z; zero past the box
   auto load = [&](c2 (&v)[NI], const float2* s, int r, int j) {
@@ -228,7 +229,9 @@ k_zpass(const void* __restrict__ F1, float2* __restrict__ UV, const float2* __re
         for (int k = 0; k < N1; ++k) e[k * W] = k == 0 ? v[k] : cmul(v[k], tw2[n2 * k]);
       }
       __syncthreads();
-      if (t == 0) {                               // the inputs have been read, the other weights' products summed
+      // the inputs have been read, the other weights' products summed (dead: a phase
+      // is still open, and a second arrival on it would be undefined)
+      if (t == 0 && dead < 0) {
         const int nr = mask ? r0 + Q : r0, nj = mask ? jbeg : j + 1;
         if (nr < rend) {
           fetch_inputs(nr, nj);
@@ -316,11 +319,15 @@ k_zpass(const void* __restrict__ F1, float2* __restrict__ UV, const float2* __re
       }
     }
   }
-  if (dead && g.tc_err) atomicExch(g.tc_err, 1);
-  if (dead) {                                     // copies that were not waited for, before the block ends
-    tc::mbar_wait(&bar[0], (f - 1) & 1, kTcWaitNs / 4);
-    if (kWeights)
-      for (int l = f - 1; l >= 0 && l >= f - 2; --l) tc::mbar_wait(&bar[1 + (l & 1)], (l >> 1) & 1, kTcWaitNs / 4);
+  if (dead >= 0) {
+    if (g.tc_err) atomicExch(g.tc_err, 1);
+    if (t == 0) {                                 // the copies still in flight end before the block does: inputs and
+      const int d = dead >> 1;                    // weights of field d, or its weights and all of field d + 1
+      const bool in = !(dead & 1);
+      tc::mbar_wait(&bar[0], (in ? d : d + 1) & 1, kTcWaitNs / 4);
+      if (kWeights)
+        for (int l = d; l <= d + !in; ++l) tc::mbar_wait(&bar[1 + (l & 1)], (l >> 1) & 1, kTcWaitNs / 4);
+    }
   }
 }
 
