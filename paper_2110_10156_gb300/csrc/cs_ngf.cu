@@ -716,16 +716,20 @@ cs_ngf_status score_range_impl(cs_ngf_fixed* f, int r0_begin, int n, float* best
 // more than kMaxClasses; kMaxBoxClasses for the closer spaced box lengths).  Rotations admitting no shift join the first
 // class.  The classes do not depend on the launch-group size, so results
 // stay the same for every even batch.
-constexpr double kClassCost = 4.0;
+// A class also costs its launches, whatever their size: about 40 us, the time of
+// kClassPoints transform points, below which a box class's volume counts as that
+// (us per call with and without: 26 rotations at 20x23x18 121, 185;
+// 64 at 26x24x30 196, 273; from 80^3 on the same classes).
+constexpr double kClassCost = 4.0, kClassPoints = 1.6e6;
 constexpr size_t kMaxClasses = 8, kMaxBoxClasses = 16;
 struct LengthClass { int pad[3]; std::vector<int> rot; };
 
 double class_volume(const int* p) { return (double)p[0] * p[1] * p[2]; }
 
 // cur: the lengths in use (their class goes first); none: lengths when no
-// rotation admits a shift
+// rotation admits a shift; least: what a class costs at least, in points
 std::vector<LengthClass> length_classes(const std::vector<Need>& need, const int none_pad[3], const int cur[3],
-                                        size_t max_classes = kMaxClasses) {
+                                        size_t max_classes = kMaxClasses, double least = 0.0) {
   std::vector<LengthClass> cls;
   std::vector<int> none;
   for (int r = 0; r < (int)need.size(); ++r) {
@@ -753,7 +757,7 @@ std::vector<LengthClass> length_classes(const std::vector<Need>& need, const int
           std::copy(m, m + 3, bm);
         }
       }
-    const double keep = kClassCost * std::min(class_volume(cls[bc].pad), class_volume(cls[bd].pad));
+    const double keep = std::max(kClassCost * std::min(class_volume(cls[bc].pad), class_volume(cls[bd].pad)), least);
     if (best >= keep && cls.size() <= max_classes) break;
     std::copy(bm, bm + 3, cls[bc].pad);
     cls[bc].rot.insert(cls[bc].rot.end(), cls[bd].rot.begin(), cls[bd].rot.end());
@@ -808,7 +812,7 @@ cs_ngf_status plan_classes_impl(cs_ngf_fixed* f, int R, cudaStream_t st, Plan& p
   if (f->boxed) {
     const int cur[3] = {g.Pz, g.Py, g.Px};
     for (int r = 0; r < R; ++r) need[r] = box_need(f, bounds[r]);
-    cls = length_classes(need, none_pad, cur, kMaxBoxClasses);
+    cls = length_classes(need, none_pad, cur, kMaxBoxClasses, kClassPoints);
   }
   f->run_pads.clear();
   f->run_counts.clear();
