@@ -28,4 +28,4 @@ def test_results_do_not_depend_on_the_empty_slots(kw):
         k = n // 2 * 2                           # an odd last mask is transformed alone: its last bits may differ
         np.testing.assert_array_equal(got[0][:k], want[0][:k])
         np.testing.assert_array_equal(got[1], want[1][:n])
-        np.testing.assert_allclose(got[0][k:], want[0][k:n], rtol=1e-6)
+        np.testing.assert_allclose(got[0][k:], want[0][k:n], rtol=1e-5)
