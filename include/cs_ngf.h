@@ -57,6 +57,11 @@
  * call's (an event recorded on the previous call's stream), so they never
  * overlap on the handle's buffers.  No function aborts the process: each
  * returns a status.
+ *   A transform pass that waits more than 2 s for its own copies or MMAs gives
+ * up and returns.  The results that depend on it are then NaN scores with zero
+ * shifts (a map of NaN), and a call that waits for its results returns ECUDA.
+ * With bound-limited padding the next call works again; with full padding, if
+ * the pass was one of the fixed volume's spectra, after cs_ngf_update_fixed.
  */
 #ifndef CS_NGF_H
 #define CS_NGF_H
@@ -165,9 +170,7 @@ typedef struct {
                         mask field and every inverse transform stay FP32 on the CUDA cores.
                         The handle then holds one more per-rotation buffer (the spectral sum
                         X, (Px/2+1) Py Pz complex values).  0: the CUDA-core FFT for every
-                        field.  Ignored in the FP32 form.  A tensor-core pass that waits more
-                        than 2 s for its own MMAs stops; the next synchronous call
-                        (cs_ngf_align, cs_ngf_score_rotations_host) then returns ECUDA. */
+                        field.  Ignored in the FP32 form. */
 } cs_ngf_config;
 
 typedef struct {

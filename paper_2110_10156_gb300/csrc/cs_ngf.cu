@@ -184,12 +184,11 @@ cs_ngf_status check_launch(const char* what) {
   return CS_NGF_OK;
 }
 
-// ECUDA (once) if a tensor-core pass of this handle stopped on its bounded
-// wait since the last check; the caller has synchronised its stream
-cs_ngf_status tc_status(cs_ngf_fixed* f) {
-  if (!f->tc_err || !*(volatile int*)f->tc_err) return CS_NGF_OK;
-  *f->tc_err = 0;
-  return fail(CS_NGF_ECUDA, "a z pass timed out waiting for its MMAs or copies; its results are invalid");
+// ECUDA if a pass of the handle's last call, or of the spectra it used, stopped
+// on its bounded wait; the caller has synchronised its stream
+cs_ngf_status wait_status_impl(const cs_ngf_fixed* f) {
+  if (*(volatile int*)f->wait_h != f->call_id) return CS_NGF_OK;
+  return fail(CS_NGF_ECUDA, "a transform pass timed out waiting for its copies or MMAs; the results are invalid");
 }
 
 void free_handle(cs_ngf_fixed* f) {
@@ -208,8 +207,8 @@ void free_handle(cs_ngf_fixed* f) {
   cudaFree(f->margA);
   cudaFree(f->margB);
   cudaFree(f->bounds);
-  cudaFree(f->keys);
-  cudaFreeHost(f->tc_err);
+  if (f->keys) cudaFree(f->keys - 1);
+  cudaFreeHost(f->wait_h);
   cudaFreeHost(f->fbox_h);
   cudaFree(f->zx);
   if (f->rot_ev) cudaEventSynchronize(f->rot_ev);
@@ -455,6 +454,7 @@ cs_ngf_status stage_call_impl(cs_ngf_fixed* f, const float* B, const uint8_t* MB
   const Geo& g = f->g;
   const bool bound = f->pad_mode == CS_NGF_PAD_BOUND;
   if (cs_ngf_status s = fill_rotations(f, quats, R)) return s;
+  f->call_id = f->call_id % 0x40000000 + 1;
   if (bound)
     if (cs_ngf_status s = ensure_rotation_buffers(f, R)) return s;
   CallStage cs{};
@@ -499,7 +499,7 @@ cs_ngf_status score_batch(cs_ngf_fixed* f, int r0, int nb, float* best_score, in
     if (cs_ngf_status s = check_launch("resample")) return s;
   } else {
     const size_t nmarg = (size_t)g.nz + g.ny + g.nx;
-    CS_CUDA(cudaMemsetAsync(f->keys, 0, sizeof(unsigned long long) * nb, st));
+    CS_CUDA(cudaMemsetAsync(g.wait_err, 0, sizeof(int) + sizeof(unsigned long long) * nb, st));   // and the keys
     CS_CUDA(cudaMemsetAsync(f->msum, 0, sizeof(int) * nb, st));
     CS_CUDA(cudaMemsetAsync(f->margB, 0, sizeof(int) * nmarg * nb, st));
     {
@@ -527,7 +527,8 @@ cs_ngf_status score_batch(cs_ngf_fixed* f, int r0, int nb, float* best_score, in
   if (cs_ngf_status s = run_transforms(f, rot, nb, map, st, tune)) return s;
   {
     Stage sp(f, 7, st);
-    k_finalize<<<(nb + 127) / 128, 128, 0, st>>>(f->keys, nb, g, best_score + r0, best_shift + 3 * (size_t)r0);
+    k_finalize<<<(nb + 127) / 128, 128, 0, st>>>(f->keys, nb, g, best_score + r0, best_shift + 3 * (size_t)r0, map,
+                                                 f->wait_h, f->call_id);
   }
   return check_launch("finalize");
 }
@@ -537,6 +538,7 @@ cs_ngf_status score_batch(cs_ngf_fixed* f, int r0, int nb, float* best_score, in
 cs_ngf_status run_spectra(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cudaStream_t st) {
   Geo g = f->g;
   g.store = kStoreF32;            // the fixed spectra are always computed in FP32
+  --g.wait_err;                   // their flag stays set for every call that uses them
   for (int j = 0; j < 4; ++j) g.scale0[j] = g.scale1[j] = 1.0f;
   g.ez = f->extA[0]; g.ey = f->extA[1]; g.ex = f->extA[2];
   f->spectra_ok = g.ez <= g.Pz && g.ey <= g.Py && g.ex <= g.Px;
@@ -579,6 +581,11 @@ cs_ngf_status set_class_impl(cs_ngf_fixed* f, const ClassGeom& c, cudaStream_t s
   Geo& g = f->g;
   g.ez = c.ext[0]; g.ey = c.ext[1]; g.ex = c.ext[2];
   g.wz = c.win[0]; g.wy = c.win[1];
+  if (f->A_keep && ((volatile int*)f->wait_h)[1]) {   // a call found the spectra invalid: again, from the copies
+    f->wait_h[1] = 0;
+    f->spectra_ok = false;
+    CS_CUDA(cudaMemsetAsync(g.wait_err - 1, 0, sizeof(int), st));
+  }
   if (f->spectra_ok && g.Pz == c.pad[0] && g.Py == c.pad[1] && g.Px == c.pad[2]) return CS_NGF_OK;
   g.Pz = c.pad[0];
   g.Py = c.pad[1];
@@ -980,6 +987,7 @@ cs_ngf_status plan_classes(cs_ngf_fixed* f, int R, cudaStream_t st, Plan& plan) 
 cs_ngf_status set_class(cs_ngf_fixed* f, const ClassGeom& c, cudaStream_t st) {
   return ::set_class_impl(f, c, st);
 }
+cs_ngf_status wait_status(const cs_ngf_fixed* f) { return ::wait_status_impl(f); }
 cs_ngf_status resolve_pads(const int32_t dims[3], const cs_ngf_config& cfg, int pad[3]) {
   return ::resolve_pads_impl(dims, cfg, pad);
 }
@@ -1146,17 +1154,18 @@ cs_ngf_status cs_ngf_prepare_fixed(const float* A, const uint8_t* maskA, const i
   CS_TRYC(dalloc(&f->margB, (size_t)batch * nmarg));
   CS_TRYC(dalloc(&f->bounds, (size_t)batch));
   CS_TRYC(dalloc(&f->boxA, (size_t)1));
-  CS_TRYC(dalloc(&f->keys, (size_t)f->group_cap));
+  CS_TRYC(dalloc(&f->keys, (size_t)f->group_cap + 1));
+  g.wait_err = reinterpret_cast<int*>(++f->keys) - 1;
+  CS_TRYC(cudaMemsetAsync(g.wait_err, 0, sizeof(int), st));
   if (sz.zx_elems) {
     CS_TRYC(dalloc(&f->zx, (size_t)batch * sz.zx_elems));
     g.zx = f->zx;
   }
   CS_TRYC(cudaEventCreateWithFlags(&f->order_ev, cudaEventDisableTiming));
-  CS_TRYC(cudaMallocHost((void**)&f->tc_err, sizeof(int)));
-  *f->tc_err = 0;
+  CS_TRYC(cudaMallocHost((void**)&f->wait_h, sizeof(int) * 2));
+  f->wait_h[0] = f->wait_h[1] = 0;
   CS_TRYC(cudaMallocHost((void**)&f->fbox_h, sizeof(FixedBox)));
   CS_TRYC(cudaMemsetAsync(f->mbox, 0, sizeof(int) * 6, st));
-  g.tc_err = f->tc_err;
   f->fixed_bytes = uv_elems * sizeof(float2);
   f->workspace_bytes = (size_t)batch * per_rot + (size_t)(f->group_cap - batch) * g.nvox * 5 + shared_ws;
   if (f->pad_mode == CS_NGF_PAD_BOUND) {
@@ -1207,7 +1216,7 @@ cs_ngf_status cs_ngf_score_rotations_host(cs_ngf_fixed* f, const float* B, const
   CS_CUDA(cudaStreamSynchronize(st));
   std::copy(f->res_score, f->res_score + R, best_score);
   std::copy(f->res_shift, f->res_shift + 3 * (size_t)R, best_shift);
-  return tc_status(f);
+  return wait_status_impl(f);
 }
 
 cs_ngf_status cs_ngf_align(cs_ngf_fixed* f, const float* B, const uint8_t* maskB,
@@ -1225,7 +1234,7 @@ cs_ngf_status cs_ngf_align(cs_ngf_fixed* f, const float* B, const uint8_t* maskB
   CS_CUDA(cudaStreamSynchronize(st));
   const float* sc = f->res_score;
   const int32_t* sh = f->res_shift;
-  if (cs_ngf_status s = tc_status(f)) return s;
+  if (cs_ngf_status s = wait_status_impl(f)) return s;
   int best = -1;
   for (int r = 0; r < R; ++r)
     if (std::isfinite(sc[r]) && (best < 0 || sc[r] > sc[best])) best = r;

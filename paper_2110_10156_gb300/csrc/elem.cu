@@ -361,7 +361,10 @@ k_resample_box(const float4* __restrict__ BQ, const uint8_t* __restrict__ C8, co
   const int ztiles = (g.ez + 2 + ZB - 1) / ZB;
   const int r = blockIdx.z / ztiles, zt = blockIdx.z - r * ztiles;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && zt == 0) keys[r] = 0ull;   // for the x inverse
+  if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && zt == 0) {
+    keys[r] = 0ull;                               // for the x inverse
+    if (r == 0) g.wait_err[0] = 0;                // a new launch group
+  }
   const RotBox& b = rot[r].b;
   const int x = b.org[2] - 1 + blockIdx.x * 8 + (lane & 7);
   const int y = b.org[1] - 1 + blockIdx.y * 4 + (lane >> 3);
@@ -443,6 +446,7 @@ __global__ void __launch_bounds__(256) k_fixed_box(const int* __restrict__ marg,
   __syncthreads();
   if (t == 0) {
     RotIn in{};
+    g.wait_err[-1] = 0;                           // new spectra follow
     out->sum = sum;
     for (int a = 0; a < 3; ++a) {
       out->a0[a] = hi[a] < 0 ? 0 : lo[a];
@@ -546,8 +550,22 @@ __global__ void k_mask_sum(const uint8_t* __restrict__ M, long long n, int* __re
 }
 
 __global__ void k_finalize(const unsigned long long* __restrict__ keys, int nrot, Geo g,
-                           float* __restrict__ best_score, int32_t* __restrict__ best_shift) {
+                           float* __restrict__ best_score, int32_t* __restrict__ best_shift,
+                           float* __restrict__ map, int* __restrict__ host, int call) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g.wait_err[0] | g.wait_err[-1]) {
+    const float nan = __int_as_float(0x7fc00000);
+    if (map)
+      for (long long i = r; i < (long long)g.vz * g.vy * g.vx; i += (long long)gridDim.x * blockDim.x) map[i] = nan;
+    if (r >= nrot) return;
+    best_score[r] = nan;
+    for (int a = 0; a < 3; ++a) best_shift[3 * r + a] = 0;
+    if (host && r == 0) {
+      host[0] = call;
+      if (g.wait_err[-1]) host[1] = 1;
+    }
+    return;
+  }
   if (r >= nrot) return;
   const unsigned long long k = keys[r];
   if (k == 0ull) {

@@ -72,8 +72,9 @@ struct cs_ngf_fixed {
   int* margA = nullptr;        // slab counts of M_A per axis [nz | ny | nx]
   int* margB = nullptr;        // the same for each rotated mask of a batch
   RotBounds* bounds = nullptr; // per rotation of a batch (full padding)
-  unsigned long long* keys = nullptr;
-  int* tc_err = nullptr;       // pinned host flag, set by a pass that stopped on its bounded wait
+  unsigned long long* keys = nullptr;   // per rotation; Geo::wait_err[-1, 0] is the entry before them
+  int* wait_h = nullptr;       // pinned: [0] the last call whose passes' waits ran out, [1] spectra among them
+  int call_id = 0;             // number of the last call staged
   FixedBox* fbox_h = nullptr;  // pinned host memory k_fixed_box writes to
   float2* zx = nullptr;        // X of the tensor-core z pass (reduced-precision forms), per launch group
   // rotations: pinned host memory, copied to the device by a kernel, grown on demand
@@ -130,6 +131,9 @@ cs_ngf_status set_class(cs_ngf_fixed* f, const ClassGeom& c, cudaStream_t st);
 // (device, indexed from r0), in launch groups of f->batch
 cs_ngf_status score_range(cs_ngf_fixed* f, int r0, int n, float* best_score, int32_t* best_shift,
                           cudaStream_t st);
+// ECUDA if a wait of the last call's passes ran out; the caller has
+// synchronised its stream
+cs_ngf_status wait_status(const cs_ngf_fixed* f);
 // validate dims / cfg and return the FFT lengths; EINVAL / EUNSUPPORTED on error
 cs_ngf_status resolve_pads(const int32_t dims[3], const cs_ngf_config& cfg, int pad[3]);
 // the automatic launch group: what a third of the free device memory holds, 1 .. most

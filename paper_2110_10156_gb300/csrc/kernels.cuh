@@ -56,9 +56,11 @@ struct Geo {
   // 1: in the BF16 and FP16 forms the z pass runs the forward z-axis DFT of
   // the channel fields on the tensor cores (k_zx_tc) where its length allows
   int tc;
-  // set to 1 by a z pass whose bounded wait for its own MMAs or copies ran out
-  // (it then stops and returns); nullptr: not reported
-  int* tc_err;
+  // device flags set to 1 by a pass whose bounded wait for its own MMAs or copies
+  // ran out (its results are invalid): [0] a pass of the current launch group,
+  // cleared where the group begins; [-1] a pass of the fixed spectra (which is
+  // launched with wait_err one lower)
+  int* wait_err;
   // X of the tensor-core z pass, [r][kx <= Px/2][p/4][kz][p%4] per launch group
   // (the handle allocates it with the tensor-core forms); nullptr: the z pass
   // runs as one kernel
@@ -248,9 +250,12 @@ __host__ __device__ inline float overlap_threshold(int sumA, int sumB, float gam
   return (float)((t - 0.5) * pvol);
 }
 
-// decode per-rotation keys into (score, shift)
+// decode per-rotation keys into (score, shift).  With a wait_err flag set the
+// results are invalid: NaN scores, zero shifts, a map of NaN, and (host: pinned
+// memory, may be nullptr) host[0] = call, host[1] |= the spectra's flag.
 __global__ void k_finalize(const unsigned long long* __restrict__ keys, int nrot, Geo g,
-                           float* __restrict__ best_score, int32_t* __restrict__ best_shift);
+                           float* __restrict__ best_score, int32_t* __restrict__ best_shift,
+                           float* __restrict__ map, int* __restrict__ host, int call);
 
 // copy a float volume / mask into the rotation-0 slot (fixed-volume prepare)
 __global__ void k_copy_in(const float* __restrict__ A, const uint8_t* __restrict__ MA,

@@ -41,7 +41,7 @@ constexpr size_t kVolBytes = align256((size_t)kNaMaxDim * kNaMaxDim * kNaMaxDim 
 constexpr size_t kMaskBytes = align256((size_t)kNaMaxDim * kNaMaxDim * kNaMaxDim);
 constexpr size_t kBQBytes = align256((size_t)kNaMaxDim * kNaMaxDim * kNaMaxDim * 16);
 constexpr size_t kC8Bytes = align256((size_t)kNaMaxDim * kNaMaxDim * kNaMaxDim);
-constexpr size_t kMiscBytes = 256;   // msum[2] (A, B), thr, key, rotation matrix
+constexpr size_t kMiscBytes = 256;   // Misc
 
 constexpr size_t kOffUV = 0;
 constexpr size_t kOffF02 = kOffUV + kUVBytes;
@@ -61,6 +61,7 @@ static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
 struct Misc {
   int msum[2];                 // [0] sum of M_A, [1] sum of the rotated M_B
+  int wait_err[2];             // Geo::wait_err[-1], of the fixed spectra, and [0], of the current rotation
   unsigned long long key;      // best (score, shift) key of the current rotation
   RotIn rot;                   // the current rotation; its box is the whole volume, every shift
 };
@@ -86,6 +87,7 @@ cs_ngf_status na_fail(cs_ngf_status s, const std::string& m) {
 __global__ void k_na_set_rot(RotIn in, Misc* misc) {
   misc->rot = in;
   misc->msum[1] = 0;
+  misc->wait_err[1] = 0;
   misc->key = 0ull;
 }
 
@@ -224,6 +226,7 @@ extern "C" cs_ngf_status cs_ngf_score_rotations_noalloc(
   float4* BQ = (float4*)(base + kOffBQ);
   uint8_t* C8 = (uint8_t*)(base + kOffC8);
   Misc* misc = (Misc*)(base + kOffMisc);
+  g.wait_err = misc->wait_err + 1;
   cudaStream_t st = (cudaStream_t)stream;
 
   // fixed volume: mask sum, forward transforms, weights (all in scratch)
@@ -232,9 +235,11 @@ extern "C" cs_ngf_status cs_ngf_score_rotations_noalloc(
   if (cs_ngf_status s = na_launched("copy_in")) return s;
   k_mask_sum<<<64, 256, 0, st>>>(Mh, g.nvox, &misc->msum[0]);
   if (cs_ngf_status s = na_launched("mask_sum")) return s;
-  NA_DISPATCH(g.Px, launch_fwd_x<PP>(Bh, Mh, F02, &misc->rot, g, 1, st));
-  NA_DISPATCH(g.Py, launch_fwd_y<PP>(F02, F13, g, 1, st));
-  NA_DISPATCH(g.Pz, launch_prep_z<PP>(F13, UV, g, st));
+  Geo ga = g;
+  ga.wait_err = misc->wait_err;
+  NA_DISPATCH(g.Px, launch_fwd_x<PP>(Bh, Mh, F02, &misc->rot, ga, 1, st));
+  NA_DISPATCH(g.Py, launch_fwd_y<PP>(F02, F13, ga, 1, st));
+  NA_DISPATCH(g.Pz, launch_prep_z<PP>(F13, UV, ga, st));
   if (cs_ngf_status s = na_launched("fixed transforms")) return s;
 
   k_pack_floating<<<64, 256, 0, st>>>(B, maskB, g, BQ, C8, CallStage{});
@@ -258,7 +263,7 @@ extern "C" cs_ngf_status cs_ngf_score_rotations_noalloc(
     NA_DISPATCH(g.Pz, launch_zmac<PP>(F13, UV, F02, g, 1, &misc->rot, st));
     NA_DISPATCH(g.Py, launch_inv_y<PP>(F02, F13, g, 1, &misc->rot, st));
     NA_DISPATCH(g.Px, launch_inv_x<PP>(F13, &misc->key, nullptr, g, 1, &misc->rot, st));
-    k_finalize<<<1, 32, 0, st>>>(&misc->key, 1, g, best_score + r, best_shift + 3 * (size_t)r);
+    k_finalize<<<1, 32, 0, st>>>(&misc->key, 1, g, best_score + r, best_shift + 3 * (size_t)r, nullptr, nullptr, 0);
     if (cs_ngf_status s = na_launched("rotation")) return s;
   }
   return CS_NGF_OK;

@@ -424,7 +424,7 @@ k_fwd_y(const void* __restrict__ F0, void* __restrict__ F1, Geo g, int groups) {
     __syncthreads();
   }
   if (dead >= 0) {                                   // the copies still in flight end before the block does
-    if (g.tc_err) atomicExch(g.tc_err, 1);
+    atomicExch(g.wait_err, 1);
     if (t == 0)
       for (int l = dead; l < it && l < dead + 2; ++l) tc::mbar_wait(&bar[l & 1], (l >> 1) & 1, kTcWaitNs / 4);
   }

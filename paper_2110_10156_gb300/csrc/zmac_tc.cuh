@@ -255,7 +255,7 @@ k_zx_tc(const void* __restrict__ F1, const float2* __restrict__ UV, float2* __re
     tc::fence_before_sync();
   }
   if (failed) {                                    // its copies and products, and the next rotation's copies
-    if (t == 0 && g.tc_err) atomicExch(g.tc_err, 1);
+    if (t == 0) atomicExch(g.wait_err, 1);
     tc::mbar_wait(&bar[fail_buf], fail_par, kTcWaitNs / 4);
     tc::mbar_wait(&mbar[fail_buf], fail_par, kTcWaitNs / 4);
     if (fail_next >= 0) tc::mbar_wait(&bar[fail_next & 1], (uint32_t)((fail_next >> 1) & 1), kTcWaitNs / 4);

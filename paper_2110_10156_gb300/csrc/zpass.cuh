@@ -323,7 +323,7 @@ k_zpass(const void* __restrict__ F1, float2* __restrict__ UV, const float2* __re
     }
   }
   if (dead >= 0) {
-    if (g.tc_err) atomicExch(g.tc_err, 1);
+    atomicExch(g.wait_err, 1);
     if (t == 0) {                                 // the copies still in flight end before the block does: inputs and
       const int d = dead >> 1;                    // weights of field d, or its weights and all of field d + 1
       const bool in = !(dead & 1);

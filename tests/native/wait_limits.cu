@@ -1,20 +1,5 @@
-// The y and z passes with one bulk copy left out, so that a block's wait for it
-// runs out: the wait limit is 20 ms here, and the copy with number g_drop is not
-// issued (its bytes never arrive).  Every wait stays bounded.
-#include "tc.cuh"
-
-namespace csngf {
-namespace tc {
-constexpr unsigned long long kShortWaitNs = 20000000ull;
-__device__ int g_copies, g_drop;
-__device__ __forceinline__ void bulk_load_or_drop(void* dst, const void* src, uint32_t bytes, uint64_t* mbar) {
-  if (atomicAdd(&g_copies, 1) != g_drop) bulk_load(dst, src, bytes, mbar);
-}
-}  // namespace tc
-}  // namespace csngf
-#define bulk_load bulk_load_or_drop
-#define kTcWaitNs tc::kShortWaitNs
-#include "passes.cuh"
+// The y and z passes with one bulk copy left out; see wait_limits.h.
+#include "wait_limits.h"
 
 using namespace csngf;
 
@@ -34,23 +19,23 @@ extern "C" int run_pass(int pass, int drop, int* flag) {
   const size_t n2 = (size_t)R * P * g.wz * ky_total(P), nuv = (size_t)7 * (P / 2 + 1) * ky_total(P) * 32;
   float2 *F0 = nullptr, *F1 = nullptr, *F2 = nullptr, *UV = nullptr;
   RotIn* rot = nullptr;
-  int* err = nullptr;
+  int* err = nullptr;                               // [spectra, group]
   const int zero = 0;
   cudaMalloc(&F0, n0 * sizeof(float2));
   cudaMalloc(&F1, n0 * sizeof(float2));
   cudaMalloc(&F2, n2 * sizeof(float2));
   cudaMalloc(&UV, nuv * sizeof(float2));
   cudaMalloc(&rot, R * sizeof(RotIn));
-  cudaMalloc(&err, sizeof(int));
+  cudaMalloc(&err, 2 * sizeof(int));
   if (cudaError_t e = cudaGetLastError()) return e;
   cudaMemset(F0, 0, n0 * sizeof(float2));
   cudaMemset(F1, 0, n0 * sizeof(float2));
   cudaMemset(UV, 0, nuv * sizeof(float2));
   cudaMemset(rot, 0, R * sizeof(RotIn));            // window of one slot
-  cudaMemset(err, 0, sizeof(int));
+  cudaMemset(err, 0, 2 * sizeof(int));
   cudaMemcpyToSymbol(tc::g_copies, &zero, sizeof(int));
   cudaMemcpyToSymbol(tc::g_drop, &drop, sizeof(int));
-  g.tc_err = err;
+  g.wait_err = err + 1;
   if (pass == 0) {
     using C = FwdYCfg<P, 0>;
     k_fwd_y<P, kStoreF32, true, 0><<<dim3(P / 4, 1, R * g.nf), C::NT, C::smem_bytes(g.ey)>>>(F0, F1, g, 4);
@@ -64,7 +49,7 @@ extern "C" int run_pass(int pass, int drop, int* flag) {
   }
   cudaError_t e = cudaGetLastError();
   if (!e) e = cudaDeviceSynchronize();
-  if (!e) e = cudaMemcpy(flag, err, sizeof(int), cudaMemcpyDeviceToHost);
+  if (!e) e = cudaMemcpy(flag, err + 1, sizeof(int), cudaMemcpyDeviceToHost);
   cudaFree(F0); cudaFree(F1); cudaFree(F2); cudaFree(UV); cudaFree(rot); cudaFree(err);
   return e;
 }
