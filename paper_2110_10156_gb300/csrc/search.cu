@@ -256,7 +256,7 @@ cs_ngf_status cs_ngf_global_align(const float* A, const uint8_t* maskA, const fl
       cudaError_t e = cudaMemcpyAsync(hs.data(), rsc.p, sizeof(float) * R, cudaMemcpyDeviceToHost, st);
       if (e == cudaSuccess) e = cudaMemcpyAsync(hh.data(), rsh.p, sizeof(int32_t) * 3 * R, cudaMemcpyDeviceToHost, st);
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) s = fail(CS_NGF_ECUDA, cudaGetErrorString(e));
+      s = e != cudaSuccess ? fail(CS_NGF_ECUDA, cudaGetErrorString(e)) : csngf::detail::wait_status(h);
     }
     cs_ngf_release(h);
     if (s) return s;

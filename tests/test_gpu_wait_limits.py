@@ -2,6 +2,8 @@
 stays usable and the error reaches the caller."""
 import ctypes
 import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -12,6 +14,9 @@ from tests import native_util
 pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CALLS = ["search"]
 
 
 @pytest.fixture(scope="module")
@@ -121,3 +126,35 @@ def test_allocation_free_results_say_that_a_wait_ran_out(noalloc):
     assert np.isnan(sc[-1]) and (sh[-1] == 0).all()
     again, _, _ = run(-1)
     np.testing.assert_array_equal(again, want)
+
+
+CHILD = """
+import numpy as np, torch
+from paper_2110_10156_gb300 import cs_ngf as cs, synth
+p = synth.small_pair(19, (12, 14, 13), n_rot=5)
+dev = lambda v: torch.from_numpy(np.ascontiguousarray(v)).cuda()
+if %r == "search":
+    try:
+        cs.global_align(dev(p.A), dev(p.MA), dev(p.B), dev(p.MB), schedule=[(1.0, 1, 20.0, 5, 1)], seed=1)
+        print("status", 0)
+    except cs.CsNgfError as e:
+        print("status", e.status, e)
+else:
+    srv = cs.Server()
+    print("status", srv.wait(srv.submit(p.A, p.MA, p.B, p.MB, p.quats))["status"])
+    srv.close()
+"""
+
+
+@pytest.mark.parametrize("call", CALLS)
+def test_handles_made_inside_the_library(call, tmp_path):
+    """The search and the server prepare handles of their own: a child process whose
+    library finds their flag raised."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2110_10156_gb300 import cs_ngf as cs
+    lib = native_util.compile_shared("handle_flags.cu", tmp_path, ["-ldl"])
+    env = dict(os.environ, LD_PRELOAD=lib, CS_NGF_LIB=build.LIB)
+    out = subprocess.run([sys.executable, "-c", CHILD % call], cwd=ROOT, env=env, capture_output=True, text=True, timeout=120)
+    assert out.returncode == 0, out.stderr
+    assert f"status {cs.ECUDA}" in out.stdout, out.stdout
