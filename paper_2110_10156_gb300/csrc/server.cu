@@ -390,6 +390,9 @@ void worker_loop(cs_ngf_server* sv) {
           j->status = CS_NGF_ECUDA;
           j->error = "device error while scoring";
         }
+        // (its groups are done) a wait of their passes that ran out
+        if (!j->status && j->cursor > 0 && (j->status = csngf::detail::wait_status(j->slot->f)))
+          j->error = cs_ngf_last_error();
         const int n = j->cursor;
         Slot* s = j->slot;
         if (j->plan.perm.empty()) {

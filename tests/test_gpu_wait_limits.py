@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-CALLS = ["search"]
+CALLS = ["search", "server"]
 
 
 @pytest.fixture(scope="module")
