@@ -2,6 +2,9 @@
 // Included by one translation unit per FFT length (passes_<P>.cu).
 #pragma once
 
+#include <atomic>
+#include <mutex>
+
 #include "kernels.cuh"
 #include "tc.cuh"
 
@@ -63,10 +66,27 @@ static void by_half_z(int e, F&& f) {
   f(std::false_type{});
 }
 
-template <class K>
-static void set_smem(K kern, size_t bytes) {
-  if (bytes > 48 * 1024)
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+// Kernel K may take `bytes` of dynamic shared memory on the current device.  The
+// limit is the kernel's own, shared by every handle and host thread, and sizes
+// follow the boxes: it is only ever raised, under a lock, or a launch that needs
+// more would fail between another thread's setting and its own.
+template <auto K>
+static void set_smem(size_t bytes) {
+  if (bytes <= 48 * 1024) return;
+  constexpr int kDevices = 64;
+  static std::atomic<size_t> high[kDevices];
+  static std::mutex mu;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= kDevices) {                             // not remembered: the most a block can have
+    cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    return;
+  }
+  if (bytes <= high[dev].load(std::memory_order_acquire)) return;
+  std::lock_guard<std::mutex> lk(mu);
+  if (bytes <= high[dev].load(std::memory_order_relaxed)) return;
+  if (cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess)
+    high[dev].store(bytes, std::memory_order_release);
 }
 
 // Offsets of a second step's outputs in a tiled axis: tiles of four consecutive
@@ -290,7 +310,7 @@ void launch_fwd_x_t(const float* Bh, const uint8_t* Mh, void* F0, const RotIn* r
   const dim3 grid((unsigned)((g.ey + C::ROWS - 1) / C::ROWS), (unsigned)g.ez, (unsigned)nrot);
   by_store<P>(g.store, [&](auto sf) {
     constexpr int ST = decltype(sf)::value;
-    set_smem(k_fwd_x<P, ST, HALF, V>, C::smem_bytes);
+    set_smem<k_fwd_x<P, ST, HALF, V>>(C::smem_bytes);
     k_fwd_x<P, ST, HALF, V><<<grid, C::NT, C::smem_bytes, st>>>(Bh, Mh, F0, rot, g);
   });
 }
@@ -442,9 +462,9 @@ void launch_fwd_y_t(const void* F0, void* F1, Geo g, int nrot, cudaStream_t st) 
   by_store<P>(g.store, [&](auto sf) {
     constexpr int ST = decltype(sf)::value;
     by_half<P, V>(g.ey, [&](auto hc) {
-      auto kern = k_fwd_y<P, ST, decltype(hc)::value, V>;
-      set_smem(kern, smem);
-      kern<<<grid, C::NT, smem, st>>>(F0, F1, g, groups);
+      constexpr bool HALF = decltype(hc)::value;
+      set_smem<k_fwd_y<P, ST, HALF, V>>(smem);
+      k_fwd_y<P, ST, HALF, V><<<grid, C::NT, smem, st>>>(F0, F1, g, groups);
     });
   });
 }
@@ -543,7 +563,7 @@ void launch_inv_y(const float2* F2, float2* F3, Geo g, int nrot, const RotIn* ro
     constexpr int V = decltype(vc)::value;
     constexpr int W = 16, N2 = SplitV<P, V>::N2;
     const size_t smem = (size_t)W * FourStep<P, true, V>::CS * sizeof(float2);
-    set_smem(k_inv_y<P, W, V>, smem);
+    set_smem<k_inv_y<P, W, V>>(smem);
     dim3 grid((unsigned)(nrot * g.wz), (unsigned)((g.Px + W - 1) / W));
     k_inv_y<P, W, V><<<grid, W * N2, smem, st>>>(F2, F3, g, rot);
   });
@@ -631,7 +651,7 @@ void launch_inv_x(const float2* F3, unsigned long long* keys, float* map, Geo g,
     constexpr int N2 = SplitV<P, V>::N2;
     constexpr int ROWS = (256 / N2) > 0 ? (256 / N2) : 1;
     const size_t smem = (size_t)ROWS * FourStep<P, true, V>::CS * sizeof(float2);
-    set_smem(k_inv_x<P, ROWS, V>, smem);
+    set_smem<k_inv_x<P, ROWS, V>>(smem);
     dim3 grid((unsigned)((g.wy + ROWS - 1) / ROWS), (unsigned)(nrot * g.wz));
     k_inv_x<P, ROWS, V><<<grid, (ROWS * N2 + 31) / 32 * 32, smem, st>>>(F3, keys, map, g, rot);
   });

@@ -279,7 +279,7 @@ bool launch_zx_tc(const void* F1, const float2* UV, Geo g, int nrot, cudaStream_
     if (NB > 128 || NB % 16 != 0) return false;
     if (C1::bytes((g.nz + 15) / 16 * 16, NB, 2 * g.nch) > 232448) return false;
     const size_t s1 = std::max<size_t>(C1::bytes(KP, NB, 2 * g.nch), 120 * 1024);   // one block per SM: all of its tensor memory
-    set_smem(k_zx_tc<P, ST>, s1);
+    set_smem<k_zx_tc<P, ST>>(s1);
     dim3 grid((unsigned)(ky_total(g.Py) / C1::W), (unsigned)(g.Px / 2 + 1));
     k_zx_tc<P, ST><<<grid, C1::NT, s1, st>>>(F1, UV, g.zx, g, nrot, KP);
     return true;

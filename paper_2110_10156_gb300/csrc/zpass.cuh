@@ -348,7 +348,7 @@ void launch_zpass_t(const void* F1, float2* UV, const float2* Xg, float2* F2, Ge
   int rpb = q;
   while (rpb < 16 && cols * ((nrot + 2 * rpb - 1) / (2 * rpb)) >= 152 * C::MIN_BLOCKS * 16) rpb *= 2;
   const size_t smem = C::smem_bytes(q, g.ez);
-  set_smem(k_zpass<P, ST, HALF, V, MODE>, smem);
+  set_smem<k_zpass<P, ST, HALF, V, MODE>>(smem);
   k_zpass<P, ST, HALF, V, MODE><<<dim3(tiles, nkx, (unsigned)((nrot + rpb - 1) / rpb)), q * C::W * C::N1, smem, st>>>(
       F1, UV, Xg, F2, g, nrot, rpb, rot);
 }

@@ -43,7 +43,7 @@ extern "C" int run_pass(int pass, int drop, int* flag) {
     using C = ZCfg<32, 0, kZFull>;
     const int q = std::min(C::Q, C::fit(g.ez));
     const size_t smem = C::smem_bytes(q, g.ez);
-    set_smem(k_zpass<32, kStoreF32, true, 0, kZFull>, smem);
+    set_smem<k_zpass<32, kStoreF32, true, 0, kZFull>>(smem);
     k_zpass<32, kStoreF32, true, 0, kZFull><<<dim3(ky_total(P) / 4, P / 2 + 1, 1), q * C::W * C::N1, smem>>>(
         F1, UV, nullptr, F2, g, R, R, rot);
   }
