@@ -179,7 +179,9 @@ typedef struct {
   int32_t batch;                /* rotations per launch group at the longest lengths */
   int64_t sum_mask_a;           /* sum of M_A */
   int64_t fixed_bytes;          /* device bytes of the fixed spectra */
-  int64_t workspace_bytes;      /* device bytes of the per-batch workspace */
+  int64_t workspace_bytes;      /* device bytes of the per-batch workspace (not of a call's
+                                   rotations: 108 bytes each, and with bound-limited padding the
+                                   mask counts of up to 8192, 4 (1 + nz + ny + nx) bytes each) */
   int32_t max_pad[3];           /* largest FFT lengths (buffers are sized for them) */
   int32_t pad_mode;             /* cs_ngf_pad_mode */
   int32_t length_sets;          /* sets of FFT lengths the last scoring call used */

@@ -421,6 +421,10 @@ cs_ngf_status run_transforms(cs_ngf_fixed* f, const RotIn* rot, int nb, float* m
   return CS_NGF_OK;
 }
 
+// Mask counts of a call are taken this many rotations at a time, so that their
+// memory (25 MB at 256^3) does not grow with the call
+constexpr int kCountRotations = 8192;
+
 cs_ngf_status ensure_rotation_buffers(cs_ngf_fixed* f, int R) {
   if (R <= f->allb_cap) return CS_NGF_OK;
   CS_CUDA(cudaDeviceSynchronize());              // the old buffers may still be read
@@ -433,14 +437,15 @@ cs_ngf_status ensure_rotation_buffers(cs_ngf_fixed* f, int R) {
   f->allb_h = nullptr;
   f->perm_score = nullptr;
   f->perm_shift = nullptr;
-  f->allb_cap = 0;
-  const int cap = std::max(R, 64);
-  CS_CUDA(dalloc(&f->allm, (size_t)cap * (1 + (size_t)f->g.nz + f->g.ny + f->g.nx)));
+  f->allb_cap = f->allm_cap = 0;
+  const int cap = std::max(R, 64), mcap = std::min(cap, kCountRotations);
+  CS_CUDA(dalloc(&f->allm, (size_t)mcap * (1 + (size_t)f->g.nz + f->g.ny + f->g.nx)));
   CS_CUDA(cudaMallocHost((void**)&f->allb_h, sizeof(RotBounds) * (size_t)cap));
   CS_CUDA(dalloc(&f->perm_d, (size_t)cap));
   CS_CUDA(dalloc(&f->perm_score, (size_t)cap));
   CS_CUDA(dalloc(&f->perm_shift, (size_t)cap * 3));
   f->allb_cap = cap;
+  f->allm_cap = mcap;
   return CS_NGF_OK;
 }
 
@@ -463,7 +468,7 @@ cs_ngf_status stage_call_impl(cs_ngf_fixed* f, const float* B, const uint8_t* MB
   cs.words = (long long)R * (long long)(sizeof(RotIn) / sizeof(int));
   if (bound) {
     cs.zero = f->allm;
-    cs.zeros = (long long)R * (1 + g.nz + g.ny + g.nx);
+    cs.zeros = (long long)std::min(R, f->allm_cap) * (1 + g.nz + g.ny + g.nx);
     cs.mbox = f->mbox;
   }
   const long long items = std::max({g.nvox, cs.words, cs.zeros});
@@ -624,20 +629,24 @@ int length_for(int need, int cap) {
 cs_ngf_status rotation_bounds(cs_ngf_fixed* f, int R, cudaStream_t st) {
   const Geo& g = f->g;
   const size_t nmarg = (size_t)g.nz + g.ny + g.nx;
-  int* msum = f->allm;
-  int* marg = f->allm + R;
-  for (int r0 = 0; r0 < R; r0 += 65535) {
-    const dim3 grid((unsigned)((g.nx + 7) / 8), (unsigned)((g.ny + 3) / 4), (unsigned)std::min(65535, R - r0));
-    Stage sp(f, 0, st);
-    k_mask_counts<<<grid, 128, 0, st>>>(f->C8, f->rot_d + r0, g, f->mbox, msum + r0, marg + nmarg * r0);
+  for (int r0 = 0; r0 < R; r0 += f->allm_cap) {
+    const int n = std::min(f->allm_cap, R - r0);
+    int* msum = f->allm;
+    int* marg = f->allm + n;
+    if (r0) CS_CUDA(cudaMemsetAsync(f->allm, 0, sizeof(int) * (1 + nmarg) * n, st));   // the first are zero
+    const dim3 grid((unsigned)((g.nx + 7) / 8), (unsigned)((g.ny + 3) / 4), (unsigned)n);
+    {
+      Stage sp(f, 0, st);
+      k_mask_counts<<<grid, 128, 0, st>>>(f->C8, f->rot_d + r0, g, f->mbox, msum, marg);
+    }
+    if (cs_ngf_status s = check_launch("mask counts")) return s;
+    {
+      Stage sp(f, 7, st);
+      k_shift_bounds<<<dim3((unsigned)n, 3u), 512, 0, st>>>(f->margA, marg, msum, f->sumA, f->gamma, g, f->allb_h + r0,
+                                                            r0 + n == R ? f->mbox : nullptr);
+    }
+    if (cs_ngf_status s = check_launch("shift bounds")) return s;
   }
-  if (cs_ngf_status s = check_launch("mask counts")) return s;
-  {
-    Stage sp(f, 7, st);
-    k_shift_bounds<<<dim3((unsigned)R, 3u), 512, 0, st>>>(f->margA, marg, msum, f->sumA, f->gamma, g, f->allb_h,
-                                                          f->mbox);
-  }
-  if (cs_ngf_status s = check_launch("shift bounds")) return s;
   CS_CUDA(cudaStreamSynchronize(st));
   return CS_NGF_OK;
 }

@@ -34,12 +34,12 @@ struct cs_ngf_fixed {
   int a0[3] = {0, 0, 0}, a1[3] = {-1, -1, -1};
   // per-rotation mask counts and bounds of a call and its rotations regrouped
   // by FFT lengths (bound-limited padding), grown on demand to the call's R
-  int* allm = nullptr;         // device [R][1 + nz + ny + nx]: sums, then slab counts
+  int* allm = nullptr;         // device, of up to kCountRotations: sums, then slab counts [nz + ny + nx]
   RotBounds* allb_h = nullptr; // [R], pinned host memory the bounds kernel writes to
   int* perm_d = nullptr;       // device: original index of each regrouped rotation
   float* perm_score = nullptr; // device results in regrouped order
   int32_t* perm_shift = nullptr;
-  int allb_cap = 0;
+  int allb_cap = 0, allm_cap = 0;
   // lengths the overlap rule gives (n + max(-lo, hi)): those of the last class
   // reported, the sets of the last scoring call and their rotation counts
   int rule_pad[3] = {0, 0, 0};
