@@ -453,11 +453,11 @@ cs_ngf_status ensure_rotation_buffers(cs_ngf_fixed* f, int R) {
 // its R rotations, the rotation matrices, zeroed mask counts; with enough
 // rotations (the three passes cost a few rotations' saving) the cells near the
 // mask.  One kernel does all but the last: at 32^3 the copies and memsets took
-// longer than the kernels they fed.
+// longer than the kernels they fed.  Without `counts` no mask counts follow.
 cs_ngf_status stage_call_impl(cs_ngf_fixed* f, const float* B, const uint8_t* MB, const double* quats, int R,
-                              cudaStream_t st) {
+                              cudaStream_t st, bool counts = true) {
   const Geo& g = f->g;
-  const bool bound = f->pad_mode == CS_NGF_PAD_BOUND;
+  const bool bound = counts && f->pad_mode == CS_NGF_PAD_BOUND;
   if (cs_ngf_status s = fill_rotations(f, quats, R)) return s;
   f->call_id = f->call_id % 0x40000000 + 1;
   if (bound)
@@ -1285,7 +1285,7 @@ cs_ngf_status cs_ngf_resample(cs_ngf_fixed* f, const float* B, const uint8_t* ma
   CS_CLAIM(f, st, true);
   CS_CUDA(cudaMemsetAsync(f->msum, 0, sizeof(int), st));
   const Geo& g = f->g;
-  if (cs_ngf_status s = stage_call_impl(f, B, maskB, quat, 1, st)) return s;
+  if (cs_ngf_status s = stage_call_impl(f, B, maskB, quat, 1, st, false)) return s;
   k_resample<<<resample_grid(g, 1), 128, 0, st>>>(f->BQ, f->C8, f->rot_d, g, Bhat, Mhat, f->msum, nullptr);
   return check_launch("resample");
 }

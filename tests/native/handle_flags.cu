@@ -7,6 +7,12 @@ extern "C" int raise_spectra_flag(cs_ngf_fixed* f) {
   return cudaMemcpy(f->g.wait_err - 1, &one, sizeof(int), cudaMemcpyHostToDevice);
 }
 
+// The floating mask's cell box as the next call finds it.
+extern "C" int read_mask_box(cs_ngf_fixed* f, int* box) {
+  if (cudaError_t e = cudaDeviceSynchronize()) return e;
+  return cudaMemcpy(box, f->mbox, 6 * sizeof(int), cudaMemcpyDeviceToHost);
+}
+
 // Preloaded: every handle that the library itself prepares comes with the flag raised.
 #include <dlfcn.h>
 #include <cstdlib>
