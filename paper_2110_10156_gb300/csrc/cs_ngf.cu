@@ -301,13 +301,14 @@ void split_of(int P, int v, int32_t* n1, int32_t* n2) {
   CS_DISPATCH(P, split_into<PP>(v, n1, n2));
 }
 
-// the key of pass k at the handle's lengths in use
+// the key of pass k at the handle's lengths and extents in use (which say whether the
+// pass takes a half-filled input)
 TuneKey tune_key(const cs_ngf_fixed* f, int k) {
   const Geo& g = f->g;
   switch (k) {
-    case 0: return {0, g.Px, 2 * g.nx <= g.Px, g.store};
-    case 1: return {1, g.Py, 2 * g.ny <= g.Py, g.store};
-    case 2: return {2, g.Pz, 2 * g.nz <= g.Pz, g.store};
+    case 0: return {0, g.Px, 2 * g.ex <= g.Px, g.store};
+    case 1: return {1, g.Py, 2 * g.ey <= g.Py, g.store};
+    case 2: return {2, g.Pz, 2 * g.ez <= g.Pz, g.store};
     case 3: return {3, g.Py, 0, 0};
     default: return {4, g.Px, 0, 0};
   }
@@ -591,7 +592,10 @@ cs_ngf_status set_class_impl(cs_ngf_fixed* f, const ClassGeom& c, cudaStream_t s
     f->spectra_ok = false;
     CS_CUDA(cudaMemsetAsync(g.wait_err - 1, 0, sizeof(int), st));
   }
-  if (f->spectra_ok && g.Pz == c.pad[0] && g.Py == c.pad[1] && g.Px == c.pad[2]) return CS_NGF_OK;
+  if (f->spectra_ok && g.Pz == c.pad[0] && g.Py == c.pad[1] && g.Px == c.pad[2]) {
+    if (f->autotune == 1) resolve_variants(f);      // the extents choose too
+    return CS_NGF_OK;
+  }
   g.Pz = c.pad[0];
   g.Py = c.pad[1];
   g.Px = c.pad[2];
