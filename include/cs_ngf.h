@@ -38,6 +38,9 @@
  *   - A shift is valid iff N(chi) >= max(1, ceil(gamma * min(sum M_A,
  *     sum M_hat))), the product taken in FP64 from the FP32 gamma given.
  *     Masks are 0/1 bytes (nonzero counts as 1).
+ *   - Voxels that no gradient under a mask reads have no influence, whatever
+ *     they hold, NaN and infinities included.  A NaN or an infinity that such a
+ *     gradient does read leaves the rotation without a valid shift.
  *   - Ties: the larger score wins; equal scores go to the smallest
  *     (chi_z, chi_y, chi_x), then to the smallest rotation index.
  *   - FFT lengths: per axis the smallest of {16, 32, 40, 64, 80, 100, 128,
