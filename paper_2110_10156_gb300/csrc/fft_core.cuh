@@ -103,7 +103,6 @@ __device__ __forceinline__ float2 csub(float2 a, float2 b) {
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
-__device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 
 // asynchronous global -> shared copies (cp.async, L1-allocating); the copies a
 // thread issued are visible to that thread after cp_async_wait_all()
@@ -111,18 +110,8 @@ __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gsrc) {
   const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
-__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
-  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {   // L2 only
-  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 // (wait_group 0 would not wait for copies that no commit_group closed)
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 // a * (S i)
 template <int S>
@@ -417,8 +406,6 @@ constexpr bool box_only(int N) {
   return N == 24 || N == 48 || N == 56 || N == 72 || N == 96 || N == 112 || N == 120 || N == 144 ||
          N == 168 || N == 180 || N == 240 || N == 280 || N == 300;
 }
-template <int N>
-using Split = SplitV<N, 0>;
 
 template <int N, bool PAD_ROWS = true, int V = 0>
 struct FourStep {
@@ -433,20 +420,14 @@ struct FourStep {
   static constexpr int CS = (CS0 % 2 == 0) ? CS0 + 1 : CS0;
   static_assert(CS >= N, "sequence stride must hold N natural-order values");
 
-  // twiddle table read: shared memory (TS) or the read-only global path
-  template <bool TS>
-  __device__ __forceinline__ static float2 twl(const float2* p) {
-    if constexpr (TS) return *p; else return __ldg(p);
-  }
-
   // v holds x[N2*n1 + n2] for n1 = 0..N1-1; writes twiddled N1-point outputs
-  template <int S, bool TS = false>
+  template <int S>
   __device__ __forceinline__ static void step1(float2 (&v)[N1], float2* ex_seq, int n2,
                                                const float2* __restrict__ twN) {
     Dft<N1, S>::run(v);
 #pragma unroll
     for (int k1 = 0; k1 < N1; ++k1) {
-      float2 w = twl<TS>(&twN[n2 * k1]);
+      float2 w = __ldg(&twN[n2 * k1]);
       if (S > 0) w.y = -w.y;
       ex_seq[n2 * RS + k1] = (k1 == 0) ? v[k1] : cmul(v[k1], w);
     }

@@ -149,8 +149,6 @@ __device__ __forceinline__ int window_index(int m, int m0, int P) {
   return d < 0 ? d + P : d;
 }
 
-__device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
-
 // orderable key: larger score -> larger key; equal score -> smaller index wins
 __device__ __forceinline__ unsigned long long make_key(float s, unsigned lin) {
   unsigned u = __float_as_uint(s);

@@ -81,24 +81,8 @@ __device__ __forceinline__ void commit(uint64_t* mbar) {
                ::"r"(smem_addr(mbar)) : "memory");
 }
 
-// 16 consecutive FP32 columns of this warp's 32 lanes (lane i of the warp's
-// quarter reads row i); complete after wait_ld()
-__device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-               "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                 "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-                 "=r"(r[14]), "=r"(r[15])
-               : "r"(taddr));
-}
-// 8 consecutive FP32 columns of this warp's 32 lanes
-__device__ __forceinline__ void ld8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                 "=r"(r[7])
-               : "r"(taddr));
-}
-// 4 consecutive FP32 columns of this warp's 32 lanes
+// 4 consecutive FP32 columns of this warp's 32 lanes (lane i of the warp's quarter
+// reads row i); complete after wait_ld()
 __device__ __forceinline__ void ld4(uint32_t taddr, uint32_t (&r)[4]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
