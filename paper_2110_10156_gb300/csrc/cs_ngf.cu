@@ -547,14 +547,16 @@ cs_ngf_status run_spectra(cs_ngf_fixed* f, const float* A, const uint8_t* MA, cu
   --g.wait_err;                   // their flag stays set for every call that uses them
   for (int j = 0; j < 4; ++j) g.scale0[j] = g.scale1[j] = 1.0f;
   g.ez = f->extA[0]; g.ey = f->extA[1]; g.ex = f->extA[2];
-  f->spectra_ok = g.ez <= g.Pz && g.ey <= g.Py && g.ex <= g.Px;
-  if (!f->spectra_ok) return CS_NGF_OK;   // lengths of another volume: the next call sets its own
+  f->spectra_ok = false;
+  if (g.ez > g.Pz || g.ey > g.Py || g.ex > g.Px) return CS_NGF_OK;   // lengths of another volume: the next call sets its own
   { Stage sp(f, 6, st); CS_DISPATCH(g.Px, launch_fwd_x<PP>(A, MA, f->F02, f->boxA, g, 1, st)); }
   if (cs_ngf_status s = check_launch("fwd_x (fixed)")) return s;
   { Stage sp(f, 6, st); CS_DISPATCH(g.Py, launch_fwd_y<PP>(f->F02, f->F13, g, 1, st)); }
   if (cs_ngf_status s = check_launch("fwd_y (fixed)")) return s;
   { Stage sp(f, 6, st); CS_DISPATCH(g.Pz, launch_prep_z<PP>(f->F13, f->UV, g, st)); }
-  return check_launch("prep_z");
+  if (cs_ngf_status s = check_launch("prep_z")) return s;
+  f->spectra_ok = true;
+  return CS_NGF_OK;
 }
 
 // a new fixed volume: slab counts of its mask, its box, copies where later
@@ -596,6 +598,7 @@ cs_ngf_status set_class_impl(cs_ngf_fixed* f, const ClassGeom& c, cudaStream_t s
     if (f->autotune == 1) resolve_variants(f);      // the extents choose too
     return CS_NGF_OK;
   }
+  if (!f->A_keep) return fail(CS_NGF_ECUDA, "the fixed volume's spectra were not computed; call cs_ngf_update_fixed");
   g.Pz = c.pad[0];
   g.Py = c.pad[1];
   g.Px = c.pad[2];
