@@ -349,7 +349,7 @@ def l2_note(roofline_step, R, batch):
         return (f"inputs larger than L2: each launch group's FFT intermediates exceed the 129 MB L2; "
                 f"about {tb:.2f} TB of DRAM traffic per step (ncu bytes per rotation x {R})")
     return ("inputs larger than L2: each launch group's FFT intermediates "
-            f"({batch} rotations) exceed the 129 MB L2")
+            f"({batch} rotations and more) exceed the 129 MB L2")
 
 
 def time_form(cs_ngf, A, MA, B, MB, quats, precision, args, fp32_value, tensor_cores=True):

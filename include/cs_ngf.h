@@ -155,6 +155,9 @@ typedef struct {
   int32_t pad_mode;  /* cs_ngf_pad_mode; cs_ngf_default_config sets CS_NGF_PAD_BOUND.  The
                         lengths from pad (or automatic) are then the largest a call uses */
   int32_t autotune;  /* 0 (default): every FFT pass uses its built-in radix split.
+                        Any other value keeps the lengths of the overlap rule, also where
+                        the masks' boxes allow shorter ones (cs_ngf_pad_mode): on masked
+                        pairs that costs far more than a split gains.
                         1: the first launch group at a new set of FFT lengths times each
                         pass with each split its length offers (e.g. 200 = 10 x 20 or
                         8 x 25) and keeps the faster for the rest of the process

@@ -317,7 +317,8 @@ TuneKey tune_key(const cs_ngf_fixed* f, int k) {
 // the built-in split of pass k at length P: variant 0, except in the x and z
 // passes at 160, where 10 x 16 keeps more of a block busy in both steps and its
 // pairs of transforms within 128 registers (x forward: 32.5 -> 27.9 us per
-// rotation of the 150^3 workload)
+// rotation of the 150^3 workload; the other lengths with two splits have not been
+// measured since both passes took pairs of transforms)
 int default_variant(int k, int P) { return (k == 0 || k == 2) && P == 160 ? 1 : 0; }
 
 // the variants the handle uses at its lengths in use: the table's choices
@@ -734,11 +735,11 @@ cs_ngf_status score_range_impl(cs_ngf_fixed* f, int r0_begin, int n, float* best
 // Bound-limited padding per rotation: each rotation's own shortest lengths;
 // rotations that need the same lengths form one class, scored together.  A
 // class costs a fixed-spectra recomputation and a partial launch group, about
-// kClassCost rotations of its own size; so two classes merge, with lengths raised to cover both, while the
-// cheapest merge adds less transform volume than that (and while there are
-// more than kMaxClasses; kMaxBoxClasses for the closer spaced box lengths).  Rotations admitting no shift join the first
-// class.  The classes do not depend on the launch-group size, so results
-// stay the same for every even batch.
+// kClassCost rotations of its own size; so two classes merge, with lengths raised
+// to cover both, while the cheapest merge adds less transform volume than that (and
+// while there are more than kMaxClasses; kMaxBoxClasses for the closer spaced box
+// lengths).  Rotations admitting no shift join the first class.  The classes do not
+// depend on the launch-group size, so results stay the same for every even batch.
 // A class also costs its launches, whatever their size: about 40 us, the time of
 // kClassPoints transform points, below which a box class's volume counts as that
 // (us per call with and without: 26 rotations at 20x23x18 121, 185;

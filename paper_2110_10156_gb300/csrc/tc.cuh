@@ -18,7 +18,7 @@
 
 namespace csngf {
 
-// wait limit of a z pass for its own MMAs and copies (they take microseconds)
+// wait limit of a y or z pass for its own MMAs and copies (they take microseconds)
 constexpr unsigned long long kTcWaitNs = 2000000000ull;
 
 namespace tc {
