@@ -111,6 +111,8 @@ def score_rotations_resumable(f, B, MB, quats, path: str, chunk: int = 1000,
         end = min(R, done + chunk)
         s, c = f.score_rotations(B, MB, q[done:end])
         scores[done:end] = _to_numpy(s)
+        if np.isnan(scores[done:end]).any():      # the library's mark of invalid results: not saved
+            raise RuntimeError(f"rotations {done} to {end - 1}: a transform pass timed out; the results are invalid")
         shifts[done:end] = _to_numpy(c)
         done = end
         _save(path, fp, done, scores, shifts)
