@@ -28,6 +28,8 @@ def local_best(scores, shifts, offset: int):
     (-inf, -1, (0, 0, 0)) if none is valid."""
     scores = np.asarray(scores, dtype=np.float64)
     shifts = np.asarray(shifts).reshape(-1, 3)
+    if np.isnan(scores).any():                # the library's mark of invalid results
+        raise RuntimeError("a transform pass timed out; the scores are invalid")
     fin = np.isfinite(scores)
     if not fin.any():
         return -math.inf, -1, (0, 0, 0)

@@ -3,7 +3,7 @@ job neither saves nor returns them, and a rank does not merge past them."""
 import numpy as np
 import pytest
 
-from paper_2110_10156_gb300 import resume
+from paper_2110_10156_gb300 import resume, shard
 from paper_2110_10156_gb300.synth import random_quaternions
 
 
@@ -29,3 +29,10 @@ def test_resumable_job_scores_an_invalid_chunk_again(tmp_path):
     rest = Scorer()
     s, _ = resume.score_rotations_resumable(rest, None, None, q, path, chunk=4)
     assert rest.calls == 2 and not np.isnan(s).any()
+
+
+def test_a_rank_does_not_merge_invalid_scores():
+    ok = np.array([0.1, -np.inf, 0.3])
+    assert shard.local_best(ok, np.zeros((3, 3), int), 5) == (0.3, 7, (0, 0, 0))
+    with pytest.raises(RuntimeError, match="invalid"):
+        shard.local_best(np.array([0.1, np.nan, 0.3]), np.zeros((3, 3), int), 5)
